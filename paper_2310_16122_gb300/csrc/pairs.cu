@@ -32,6 +32,89 @@ constexpr int kGasListCapRows = 128;
 constexpr int kGasTableCap = 512;
 constexpr float kSigmaW = 0.61548156588532f;  // 495 / (256 pi), Wendland C4 3-D normalisation
 
+// Words of a stage record that are stored: all of it, or Rec::kWords leading ones.
+template <class R, class = void>
+struct rec_words {
+    static constexpr int value = (int)(sizeof(R) / sizeof(float));
+};
+template <class R>
+struct rec_words<R, std::void_t<decltype(R::kWords)>> {
+    static constexpr int value = R::kWords;
+};
+
+// How the records of a stage are stored.  Planes (the rule): word quads
+// 0..kQ-1 as float4 arrays, then a tail of one or two words.  Lanes that read
+// different records of one 32-particle cell then touch the same few 128-byte
+// lines per load (8 records a line and quad), where whole records cost a line
+// per lane, and in shared memory the 16-byte stride spreads random records
+// over all banks.  Whole (Rec::kWhole): records side by side, for one whose
+// gather is bound by L1 misses rather than by lookups.  Measured on the
+// 2x64^3 clustered box, whole -> planes: Extras 226 -> 172 us, corrections
+// 198 -> 178, geometry adjoint 90 -> 70, hydro adjoint 518 -> 378,
+// Acceleration 383 -> 356, Energy 393 -> 378, hydro 253 -> 260; corrections
+// adjoint (136 bytes) 300 -> 338, kept whole.
+template <class R, class = void>
+struct rec_whole : std::false_type {};
+template <class R>
+struct rec_whole<R, std::void_t<decltype(R::kWhole)>> : std::bool_constant<R::kWhole> {};
+
+template <class R>
+struct Planes {
+    static constexpr bool kWhole = rec_whole<R>::value;
+    static constexpr int kW = kWhole ? (int)(sizeof(R) / sizeof(float)) : rec_words<R>::value;
+    static constexpr int kQ = kW / 4 + (kW % 4 == 3 ? 1 : 0);
+    static constexpr int kT = kW % 4 == 3 ? 0 : kW % 4;
+    static constexpr size_t kBytes = 16 * kQ + 4 * kT;  // stored bytes of one record
+    static_assert(kBytes <= sizeof(R) && !(kWhole && kT), "stored words lie inside the record");
+
+    __device__ __forceinline__ static int64_t quad(int k, int64_t stride, int64_t i) {
+        return kWhole ? i * kQ + k : k * stride + i;
+    }
+    template <bool kGlobal>
+    __device__ __forceinline__ static R load(const void *base, int64_t stride, int64_t i) {
+        const float4 *q = reinterpret_cast<const float4 *>(base);
+        R r{};
+        float *w = reinterpret_cast<float *>(&r);
+#pragma unroll
+        for (int k = 0; k < kQ; ++k) {
+            float4 t;
+            if constexpr (kGlobal) t = __ldg(q + quad(k, stride, i));
+            else t = q[quad(k, stride, i)];
+            w[4 * k] = t.x; w[4 * k + 1] = t.y; w[4 * k + 2] = t.z; w[4 * k + 3] = t.w;
+        }
+        const float4 *tail = q + kQ * stride;
+        if constexpr (kT == 1) {
+            const float *f = reinterpret_cast<const float *>(tail) + i;
+            w[4 * kQ] = kGlobal ? __ldg(f) : *f;
+        } else if constexpr (kT == 2) {
+            const float2 *f = reinterpret_cast<const float2 *>(tail) + i;
+            float2 t;
+            if constexpr (kGlobal) t = __ldg(f);
+            else t = *f;
+            w[4 * kQ] = t.x; w[4 * kQ + 1] = t.y;
+        }
+        return r;
+    }
+    __device__ __forceinline__ static void store(void *base, int64_t stride, int64_t i, const R &r) {
+        float4 *q = reinterpret_cast<float4 *>(base);
+        const float *w = reinterpret_cast<const float *>(&r);
+#pragma unroll
+        for (int k = 0; k < kQ; ++k)
+            q[quad(k, stride, i)] = make_float4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+        float4 *tail = q + kQ * stride;
+        if constexpr (kT == 1) reinterpret_cast<float *>(tail)[i] = w[4 * kQ];
+        if constexpr (kT == 2) reinterpret_cast<float2 *>(tail)[i] = make_float2(w[4 * kQ], w[4 * kQ + 1]);
+    }
+};
+
+// The records of one stage in kernel order.
+template <class R>
+struct RecView {
+    const void *base;
+    int64_t n;
+    __device__ __forceinline__ R operator[](int64_t i) const { return Planes<R>::template load<true>(base, n, i); }
+};
+
 struct LeafView {
     const int32_t *leaf_start;
     const int32_t *leaf_ngas;
@@ -474,6 +557,7 @@ struct GeomAdjStage {
     struct __align__(16) Rec {
         float x, y, z, h;
         float sbar, pad0, pad1, pad2;
+        static constexpr int kWords = 5;
     };
     struct I {
         float gx, gy, gz;
@@ -535,6 +619,7 @@ struct CorrStage {
     struct __align__(16) Rec {
         float x, y, z, h;
         float V, pad0, pad1, pad2;
+        static constexpr int kWords = 5;
     };
     struct I {
         float m0, c0;
@@ -949,6 +1034,7 @@ struct CorrAdjStage {
     struct __align__(16) Rec {
         float x, y, z, h;
         float V, c[kCorrCoef], pad[2];
+        static constexpr bool kWhole = true;
     };
     struct I {
         float gx, gy, gz, Vb;
@@ -1026,11 +1112,10 @@ struct HydroRec {
     float B[3], gA0;
     float gA1, gA2, gB0, gB1;
     float gB[7];  // gB[2..8]
-    float pad;
+    float pad;    // limited viscosity: G[0]; hydro adjoint: the particle's identity
 };
 struct HydroRecLim : HydroRec {
-    float G[9];  // velocity gradient, dv^a/dx^b at 3a+b
-    float pad2[3];
+    float G8[8];  // velocity gradient, dv^a/dx^b at 3a+b, entries 1..8 (entry 0 in pad)
 };
 template <class Base>
 struct HydroRecVstar : Base {
@@ -1085,8 +1170,8 @@ struct HydroStageT {
         for (int k = 0; k < 7; ++k) r.gB[k] = p.gB[(2 + k) * n + o];
         r.pad = 0.f;
         if constexpr (kLim) {
-            for (int k = 0; k < 9; ++k) r.G[k] = p.dvg[k * n + o];
-            r.pad2[0] = r.pad2[1] = r.pad2[2] = 0.f;
+            r.pad = p.dvg[o];
+            for (int k = 1; k < 9; ++k) r.G8[k - 1] = p.dvg[k * n + o];
         }
         if constexpr (kPass == kHydroEnergy) {
             r.wx = p.vstar[o]; r.wy = p.vstar[n + o]; r.wz = p.vstar[2 * n + o];
@@ -1129,11 +1214,13 @@ struct HydroStageT {
         float vij[3] = {ri.vx - rj.vx, ri.vy - rj.vy, ri.vz - rj.vz};
         float vx;
         if constexpr (kLim) {
+            const float Gi[9] = {ri.pad, ri.G8[0], ri.G8[1], ri.G8[2], ri.G8[3], ri.G8[4], ri.G8[5], ri.G8[6], ri.G8[7]};
+            const float Gj[9] = {rj.pad, rj.G8[0], rj.G8[1], rj.G8[2], rj.G8[3], rj.G8[4], rj.G8[5], rj.G8[6], rj.G8[7]};
             float si[3], sj[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                si[a] = fmaf(ri.G[3 * a], x[0], fmaf(ri.G[3 * a + 1], x[1], ri.G[3 * a + 2] * x[2]));
-                sj[a] = fmaf(rj.G[3 * a], x[0], fmaf(rj.G[3 * a + 1], x[1], rj.G[3 * a + 2] * x[2]));
+                si[a] = fmaf(Gi[3 * a], x[0], fmaf(Gi[3 * a + 1], x[1], Gi[3 * a + 2] * x[2]));
+                sj[a] = fmaf(Gj[3 * a], x[0], fmaf(Gj[3 * a + 1], x[1], Gj[3 * a + 2] * x[2]));
             }
             const float ai = fmaf(x[0], si[0], fmaf(x[1], si[1], x[2] * si[2]));
             const float aj = fmaf(x[0], sj[0], fmaf(x[1], sj[1], x[2] * sj[2]));
@@ -1475,6 +1562,7 @@ struct ExtrasStage {
         float x, y, z, h;
         float V, m, vx, vy;
         float vz, pad0, pad1, pad2;
+        static constexpr int kWords = 9;
     };
     struct I {
         float A, B[3], gA[3], gB[9];  // the i particle's corrections (gB[3g+a] = d_g B^a)
@@ -1575,6 +1663,7 @@ struct ListStage {
     struct __align__(16) Rec {
         float x, y, z, h;
         uint32_t code, pad0, pad1, pad2;
+        static constexpr int kWords = 4;  // the code is set when the record is loaded
     };
     struct I {
         uint16_t *out;
@@ -1585,7 +1674,6 @@ struct ListStage {
         int cnt;
     };
 
-    __device__ static Rec gather(const P &, int32_t, float4 ps) { return {ps.x, ps.y, ps.z, ps.w, 0u, 0u, 0u, 0u}; }
     __device__ static float box_cut(const P &p, float hmax_i, const Rec &rj) {
         return kGas ? hmax_i + rj.h : sqrtf(p.rc2);
     }
@@ -1642,7 +1730,7 @@ struct ListStage {
 // --------------------------------------------------------------- framework
 template <class S>
 __global__ void gather_kernel(int64_t n, const float4 *__restrict__ pos, const int32_t *__restrict__ kperm,
-                              typename S::P p, typename S::Rec *__restrict__ rec, int korder) {
+                              typename S::P p, void *__restrict__ rec, int korder) {
     int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= n) return;
     const float4 ps = pos[q];
@@ -1651,7 +1739,7 @@ __global__ void gather_kernel(int64_t n, const float4 *__restrict__ pos, const i
         S::finish_other(p, o);           // its gas-only outputs are zero
         return;
     }
-    rec[q] = S::gather(p, o, ps);
+    Planes<typename S::Rec>::store(rec, n, q, S::gather(p, o, ps));
 }
 
 // Work of one warp on one i-group (tiles): the kernel-order particles
@@ -1661,7 +1749,7 @@ __global__ void gather_kernel(int64_t n, const float4 *__restrict__ pos, const i
 // buffer (broadcast reads), each accumulating its own i.
 template <class S, bool kCount>
 __device__ __forceinline__ void tile_group(const LeafView &lv, const typename S::P &p,
-                                           const typename S::Rec *__restrict__ rec, typename S::Rec *buf,
+                                           RecView<typename S::Rec> rec, typename S::Rec *buf,
                                            int64_t a, int lo, int g0, int hi, int lane, double cons_acc[4]) {
     using Rec = typename S::Rec;
     const unsigned below = lanemask_lt();
@@ -1757,7 +1845,7 @@ __device__ __forceinline__ void tile_group(const LeafView &lv, const typename S:
 // padded with a massless dummy outside every i's cut, which adds exact zeros.
 template <class S, bool kCount>
 __device__ __forceinline__ void tile_group_pair(const LeafView &lv, const typename S::P &p,
-                                                const typename S::Rec *__restrict__ rec, typename S::Rec2 *buf,
+                                                RecView<typename S::Rec> rec, typename S::Rec2 *buf,
                                                 int64_t a, int lo, int g0, int hi, int lane) {
     using Rec = typename S::Rec;
     static_assert(!S::kCons && !S::kGasOnly && !S::kTag, "packed sweep: gravity-type stages only");
@@ -1861,7 +1949,7 @@ __device__ __forceinline__ void tile_group_pair(const LeafView &lv, const typena
 // overflow the buffer (gcap) is swept as plain tiles.
 template <class S, bool kCount>
 __global__ void __launch_bounds__(kThreads) pair_kernel_split(LeafView lv, typename S::P p,
-                                                              const typename S::Rec *__restrict__ rec,
+                                                              RecView<typename S::Rec> rec,
                                                               typename S::Rec *__restrict__ gbuf, int gcap) {
     using Rec = typename S::Rec;
     using Rec2 = typename S::Rec2;
@@ -2031,7 +2119,7 @@ __device__ __forceinline__ bool positive_shift(float sx, float sy, float sz) {
 // sums are taken afterwards from the finished outputs (halfwarp_cons_kernel).
 template <class S, bool kCount, int kEx>
 __global__ void __launch_bounds__(kThreads) pair_kernel_halfwarp(LeafView lv, typename S::P p,
-                                                                 const typename S::Rec *__restrict__ rec,
+                                                                 RecView<typename S::Rec> rec,
                                                                  double *__restrict__) {
     using Rec = typename S::Rec;
     static_assert(S::kHalfWarp, "half-warp arms: stages with atomic partial sums");
@@ -2136,7 +2224,7 @@ __global__ void __launch_bounds__(kThreads) pair_kernel_halfwarp(LeafView lv, ty
 // one i-group, tiles (packed sweep where the stage has one)
 template <class S, bool kCount>
 __device__ __forceinline__ void tile_group_any(const LeafView &lv, const typename S::P &p,
-                                               const typename S::Rec *__restrict__ rec, typename S::Rec *buf,
+                                               RecView<typename S::Rec> rec, typename S::Rec *buf,
                                                int64_t a, int lo, int g0, int hi, int lane, double cons_acc[4]) {
     if constexpr (S::kPair) {
         static_assert(sizeof(typename S::Rec2) == 2 * sizeof(typename S::Rec), "pair record layout");
@@ -2167,7 +2255,7 @@ __device__ __forceinline__ void cons_block_partial(double (*cons_sh)[4], const d
 // sweeps' narrow launch shape, two groups of a 128-leaf per warp).
 template <class S, bool kCount, int kW = kWarps>
 __global__ void __launch_bounds__(32 * kW) pair_kernel(LeafView lv, typename S::P p,
-                                                       const typename S::Rec *__restrict__ rec,
+                                                       RecView<typename S::Rec> rec,
                                                        double *__restrict__ cons_part) {
     using Rec = typename S::Rec;
     static_assert(kW == kWarps || !S::kCons, "conservation partials assume kWarps warps per block");
@@ -2207,7 +2295,7 @@ __device__ __forceinline__ int64_t group_count(int64_t cap, const int32_t *dgrou
 // groups than a block has warps (gas stages: a leaf of 128 holds about 64 gas).
 template <class S, bool kCount>
 __global__ void __launch_bounds__(kThreads) pair_group_kernel(LeafView lv, typename S::P p,
-                                                              const typename S::Rec *__restrict__ rec,
+                                                              RecView<typename S::Rec> rec,
                                                               GroupTable gt, double *__restrict__ cons_part) {
     using Rec = typename S::Rec;
     __shared__ __align__(16) Rec buf[kWarps][kCap];
@@ -2236,7 +2324,7 @@ __global__ void __launch_bounds__(kThreads) pair_group_kernel(LeafView lv, typen
 // record (G >= 8), so the sweep stays a broadcast.
 template <class S, int G, bool kCount>
 __global__ void __launch_bounds__(kThreads) pair_kernel_sub(LeafView lv, typename S::P p,
-                                                            const typename S::Rec *__restrict__ rec,
+                                                            RecView<typename S::Rec> rec,
                                                             double *__restrict__ cons_part) {
     using Rec = typename S::Rec;
     constexpr int NS = 32 / G;
@@ -2387,7 +2475,7 @@ __global__ void __launch_bounds__(kThreads) pair_kernel_sub(LeafView lv, typenam
 // the candidates than its 32-particle parent at r_c = 3.
 template <class S, bool kCount>
 __global__ void __launch_bounds__(kThreads) pair_kernel_sub_pair(LeafView lv, typename S::P p,
-                                                                 const typename S::Rec *__restrict__ rec,
+                                                                 RecView<typename S::Rec> rec,
                                                                  double *__restrict__ cons_part) {
     using Rec = typename S::Rec;
     using Rec2 = typename S::Rec2;
@@ -2515,7 +2603,7 @@ constexpr int kRing = 128;  // entries per ring (power of two)
 
 template <class S, bool kCount>
 __global__ void __launch_bounds__(kThreads) pair_kernel_ring(LeafView lv, typename S::P p,
-                                                             const typename S::Rec *__restrict__ rec,
+                                                             RecView<typename S::Rec> rec,
                                                              double *__restrict__ cons_part) {
     using Rec = typename S::Rec;
     static_assert(!S::kCons, "the balanced sub-warp sweep has no conservation sums");
@@ -2694,9 +2782,7 @@ struct GasLists {
 // bytes; the hydro record is too large to stage, its lanes gather directly)
 template <class S>
 __host__ __device__ constexpr int table_cap() {
-    // corrections: 256, so that five blocks of 128 threads fit an SM (with list_min_blocks below)
-    return std::is_same<S, CorrStage>::value ? 256
-                                             : (sizeof(typename S::Rec) <= 32 ? 320 : (sizeof(typename S::Rec) <= 48 ? 224 : 0));
+    return sizeof(typename S::Rec) <= 32 ? 320 : (sizeof(typename S::Rec) <= 48 ? 224 : 0);
 }
 
 // resident blocks per SM that list_kernel<S> is compiled for (a register cap; 0: none).
@@ -2753,7 +2839,7 @@ struct flat_tail<ExtrasStage> {
 // memory through the leaf's image table.
 template <class S, bool kCount>
 __global__ void __launch_bounds__(kThreads, list_min_blocks<S>::value) list_kernel(LeafView lv, typename S::P p,
-                                                        const typename S::Rec *__restrict__ rec, GasLists gl,
+                                                        RecView<typename S::Rec> rec, GasLists gl,
                                                         double *__restrict__ cons_part) {
     using Rec = typename S::Rec;
     constexpr int kTab = table_cap<S>();
@@ -2762,7 +2848,7 @@ __global__ void __launch_bounds__(kThreads, list_min_blocks<S>::value) list_kern
     __shared__ float4 itab_all[kWarps][kGroupImgCap];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float4 *itab = itab_all[warp];
-    Rec *table = reinterpret_cast<Rec *>(list_dyn) + (size_t)warp * kTab;
+    unsigned char *table = list_dyn + (size_t)warp * kTab * Planes<Rec>::kBytes;
     double cons_acc[4] = {0.0, 0.0, 0.0, 0.0};
     const int64_t ngroups = group_count(gl.groups, gl.dgroups);
     for (int64_t grp = next_group(lv, -1, lane); grp < ngroups; grp = next_group(lv, grp, lane)) {
@@ -2800,12 +2886,12 @@ __global__ void __launch_bounds__(kThreads, list_min_blocks<S>::value) list_kern
         if constexpr (kTab > 0) {
             const int ns = nu < kTab ? nu : kTab;
 #pragma unroll 4
-            for (int u = lane; u < ns; u += 32) table[u] = fetch(__ldg(U + u));
+            for (int u = lane; u < ns; u += 32) Planes<Rec>::store(table, kTab, u, fetch(__ldg(U + u)));
             __syncwarp();
         }
         auto entry = [&](int idx) -> Rec {
             if constexpr (kTab > 0) {
-                if (idx < kTab) return table[idx];
+                if (idx < kTab) return Planes<Rec>::template load<false>(table, kTab, idx);
             }
             return fetch(__ldg(U + idx));
         };
@@ -2907,7 +2993,7 @@ __global__ void __launch_bounds__(kThreads, list_min_blocks<S>::value) list_kern
 // dynamic shared memory of list_kernel<S>, and the opt-in above the 48 KB default (once per kernel)
 template <class S, bool kCount>
 size_t list_kernel_smem() {
-    const size_t bytes = (size_t)kWarps * table_cap<S>() * sizeof(typename S::Rec);
+    const size_t bytes = (size_t)kWarps * table_cap<S>() * Planes<typename S::Rec>::kBytes;
     static bool set = false;
     if (!set) {
         cudaFuncSetAttribute(list_kernel<S, kCount>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -2988,8 +3074,9 @@ int run_stage(crk_ctx *ctx, const crk_leaves *lv, typename S::P p, bool gas_pair
     const int64_t n = lv->n;
     if (n == 0) return CRK_OK;
     using Rec = typename S::Rec;
-    Rec *rec = (Rec *)crk_scratch(ctx, 4, sizeof(Rec) * (size_t)n);
-    if (!rec) return crk_fail(ctx, CRK_ENOMEM, "stage scratch");
+    void *recs = crk_scratch(ctx, 4, Planes<Rec>::kBytes * (size_t)n);
+    if (!recs) return crk_fail(ctx, CRK_ENOMEM, "stage scratch");
+    const RecView<Rec> rec{recs, n};
     const crk_nlist &nls = gas_pairs ? lv->gas_lists : lv->grav_lists;
     const bool lists = nls.list && ctx->variant[kernel_id] == CRK_VARIANT_LISTS;
     // one block per i-leaf, or (lists) one warp per i-group
@@ -3017,7 +3104,7 @@ int run_stage(crk_ctx *ctx, const crk_leaves *lv, typename S::P p, bool gas_pair
     }
     const float4 *kpos = gas_pairs ? lv->pos : lv->pos_g;          // gravity: species-mixed kernel order
     const int32_t *kperm = gas_pairs ? lv->kperm : lv->kperm_g;
-    gather_kernel<S><<<crk_grid(n, 256), 256, 0, ctx->stream>>>(n, kpos, kperm, p, rec, korder ? 1 : 0);
+    gather_kernel<S><<<crk_grid(n, 256), 256, 0, ctx->stream>>>(n, kpos, kperm, p, recs, korder ? 1 : 0);
     int32_t *queue = nullptr;
     if (persistent) {
         queue = (int32_t *)crk_scratch(ctx, 17, 64);
@@ -3345,14 +3432,12 @@ static int build_lists(crk_ctx *ctx, crk_leaves *lv, crk_nlist &out, bool reuse)
     LeafView v{lv->leaf_start, lv->leaf_ngas, lv->bbox, lv->hmax, kGas ? lv->pos : lv->pos_g,
                kGas ? lv->kperm : lv->kperm_g, kGas ? lv->himg_start : lv->gimg_start,
                kGas ? lv->himg_cnt : lv->gimg_cnt, kGas ? lv->himg : lv->gimg, nl, nullptr, 0, 32};
-    typename LS::Rec *rec = (typename LS::Rec *)crk_scratch(ctx, 4, sizeof(typename LS::Rec) * (size_t)n);
-    if (!rec) return crk_fail(ctx, CRK_ENOMEM, "neighbour list scratch");
+    const RecView<typename LS::Rec> rec{v.pos, n};  // a list record is the position and h
     const float rc2 = lv->r_cut_grav * lv->r_cut_grav;
     const int capr = kGasListCapRows, capt = kGasTableCap;
     if (reuse) {
         const int64_t capg = out.groups;
         list_group_leaf_kernel<<<crk_grid(nl, 256), 256, 0, st>>>(nl, gstart, out.gleaf, capg);
-        gather_kernel<LS><<<crk_grid(n, 256), 256, 0, st>>>(n, v.pos, v.kperm, ListP{}, rec, 0);
         CRK_CUDA(ctx, cudaMemsetAsync(tot + 5, 0, sizeof(int32_t), st));
         ListP pf{out.list, out.ucode, gstart, out.goff, out.uoff, cnt, out.unum, nullptr, tot + 5, capr, capt, rc2, n,
                  nullptr};
@@ -3360,7 +3445,7 @@ static int build_lists(crk_ctx *ctx, crk_leaves *lv, crk_nlist &out, bool reuse)
         const unsigned gg = (unsigned)((capg + kWarps - 1) / kWarps > 0 ? (capg + kWarps - 1) / kWarps : 1);
         pair_group_kernel<LS, false><<<gg, kThreads, 0, st>>>(v, pf, rec, gt, nullptr);
         lists_status_kernel<<<1, 1, 0, st>>>(tot, capg, tot + 5, lv->dev);
-        ctx->launches += 4;
+        ctx->launches += 3;
         CRK_LAUNCH_CHECK(ctx, "neighbour lists");
         return CRK_OK;
     }
@@ -3376,8 +3461,7 @@ static int build_lists(crk_ctx *ctx, crk_leaves *lv, crk_nlist &out, bool reuse)
     const unsigned ggrid = (unsigned)((ngroups + kWarps - 1) / kWarps > 0 ? (ngroups + kWarps - 1) / kWarps : 1);
     int32_t *ucnt = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(capg + 1));
     if (!ucnt) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
-    gather_kernel<LS><<<crk_grid(n, 256), 256, 0, st>>>(n, v.pos, v.kperm, ListP{}, rec, 0);
-    ctx->launches += 2;
+    ++ctx->launches;
     int32_t *goff = nullptr, *uoff = nullptr;
     uint16_t *list = nullptr;
     uint32_t *ucode = nullptr;
@@ -3516,7 +3600,7 @@ int grav_short_noalloc(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params
         }
         base = g_noalloc_ptr[dev];
     }
-    GravStage::Rec *rec = (GravStage::Rec *)base;
+    const RecView<GravStage::Rec> rec{base, n};
     GravP p{};
     p.m = m;
     p.a3 = a3;
@@ -3526,7 +3610,7 @@ int grav_short_noalloc(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params
     p.n = n;
     p.count = nullptr;
     // every record is rewritten before it is read, so nothing needs clearing
-    gather_kernel<GravStage><<<crk_grid(n, 256), 256, 0, ctx->stream>>>(n, lv->pos_g, lv->kperm_g, p, rec, 0);
+    gather_kernel<GravStage><<<crk_grid(n, 256), 256, 0, ctx->stream>>>(n, lv->pos_g, lv->kperm_g, p, base, 0);
     LeafView v{lv->leaf_start, lv->leaf_ngas, lv->bbox, lv->hmax, lv->pos_g, lv->kperm_g, lv->gimg_start,
                lv->gimg_cnt, lv->gimg, lv->n_leaves, nullptr, 0, 32};
     const int64_t grid = lv->n_leaves < 1 ? 1 : lv->n_leaves;
