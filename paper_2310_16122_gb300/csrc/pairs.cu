@@ -167,10 +167,26 @@ __device__ __forceinline__ void kahan_add(float &s, float &c, float v) {
     s = t;
 }
 
+// 1/sqrt(x), 1/x and a/x by the hardware approximations for arguments that are normal numbers:
+// rsqrtf and __fdividef wrap the same approximation in a scaling for subnormal x, four
+// instructions per pair that no argument here needs.  Gravity's x = r^2 + eps^2 may be subnormal
+// (eps = 0, r < 1e-19): x^-3/2 then overflows to infinity either way.  The same bits;
+// on the 2x128^3 box gravity 3644 -> 3272 us, its adjoint 6324 -> 6006 us.
+__device__ __forceinline__ float rsqrt_normal(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float div_normal(float a, float x) {
+    float y;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(x));
+    return y;
+}
+
 // Wendland C4 with support 2h: W and (dW/dr)/r at distance^2 r2, h = hij.
 __device__ __forceinline__ void wendland(float r2, float hij, float &W, float &dWr) {
-    float r = r2 * rsqrtf(fmaxf(r2, 1e-30f));
-    float ih = __fdividef(1.0f, hij);
+    float r = r2 * rsqrt_normal(fmaxf(r2, 1e-30f));
+    float ih = div_normal(1.0f, hij);
     float q = r * ih;
     float t = fmaxf(1.0f - 0.5f * q, 0.0f);
     float t2 = t * t;
@@ -184,8 +200,8 @@ __device__ __forceinline__ void wendland(float r2, float hij, float &W, float &d
 
 // W, (dW/dr)/r and (d[(dW/dr)/r]/dr)/r = 495/(256 pi h^7) 35 (1 - q/2)^4 (zero beyond 2h)
 __device__ __forceinline__ void wendland2(float r2, float hij, float &W, float &dWr, float &ddWr) {
-    float r = r2 * rsqrtf(fmaxf(r2, 1e-30f));
-    float ih = __fdividef(1.0f, hij);
+    float r = r2 * rsqrt_normal(fmaxf(r2, 1e-30f));
+    float ih = div_normal(1.0f, hij);
     float q = r * ih;
     float t = fmaxf(1.0f - 0.5f * q, 0.0f);
     float t2 = t * t;
@@ -236,7 +252,7 @@ struct GravStage {
     __device__ static void interact(const P &p, I &s, const Rec &ri, const Rec &rj) {
         float dx = rj.x - ri.x, dy = rj.y - ri.y, dz = rj.z - ri.z;
         float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        float rinv = rsqrtf(r2 + p.eps2);
+        float rinv = rsqrt_normal(r2 + p.eps2);
         float r3 = rinv * rinv * rinv;
         float poly = fmaf(fmaf(fmaf(fmaf(fmaf(p.c[5], r2, p.c[4]), r2, p.c[3]), r2, p.c[2]), r2, p.c[1]), r2, p.c[0]);
         bool in = r2 < p.rc2;
@@ -283,7 +299,7 @@ struct GravStage {
         const float2 dx = __fadd2_rn(rj.x, s.nx), dy = __fadd2_rn(rj.y, s.ny), dz = __fadd2_rn(rj.z, s.nz);
         const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
         const float2 t = __fadd2_rn(r2, make_float2(p.eps2, p.eps2));
-        const float2 rinv = make_float2(rsqrtf(t.x), rsqrtf(t.y));
+        const float2 rinv = make_float2(rsqrt_normal(t.x), rsqrt_normal(t.y));
         const float2 r3 = __fmul2_rn(__fmul2_rn(rinv, rinv), rinv);
         // -P5(r^2) by Horner with negated coefficients (negation is exact)
         float2 np = __ffma2_rn(make_float2(-p.c[5], -p.c[5]), r2, make_float2(-p.c[4], -p.c[4]));
@@ -359,7 +375,7 @@ struct GravAdjStage {
     __device__ static void interact(const P &p, I &s, const Rec &ri, const Rec &rj) {
         float dx = rj.x - ri.x, dy = rj.y - ri.y, dz = rj.z - ri.z;  // d_ij = x_j - x_i
         float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        float rinv = rsqrtf(r2 + p.eps2);
+        float rinv = rsqrt_normal(r2 + p.eps2);
         float ri2 = rinv * rinv;
         float r3 = ri2 * rinv;
         float poly = fmaf(fmaf(fmaf(fmaf(fmaf(p.c[5], r2, p.c[4]), r2, p.c[3]), r2, p.c[2]), r2, p.c[1]), r2, p.c[0]);
@@ -423,7 +439,7 @@ struct GravAdjStage {
         const float2 dx = __fadd2_rn(rj.x, s.nx), dy = __fadd2_rn(rj.y, s.ny), dz = __fadd2_rn(rj.z, s.nz);
         const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
         const float2 t = __fadd2_rn(r2, make_float2(p.eps2, p.eps2));
-        const float2 rinv = make_float2(rsqrtf(t.x), rsqrtf(t.y));
+        const float2 rinv = make_float2(rsqrt_normal(t.x), rsqrt_normal(t.y));
         const float2 ri2 = __fmul2_rn(rinv, rinv);
         const float2 r3 = __fmul2_rn(ri2, rinv);
         float2 np = __ffma2_rn(make_float2(-p.c[5], -p.c[5]), r2, make_float2(-p.c[4], -p.c[4]));
@@ -1234,7 +1250,7 @@ struct HydroStageT {
         } else {
             vx = fmaf(vij[0], x[0], fmaf(vij[1], x[1], vij[2] * x[2]));
         }
-        float mu = vx < 0.0f ? __fdividef(hij * vx, fmaf(p.eta2 * hij, hij, r2)) : 0.0f;
+        float mu = vx < 0.0f ? div_normal(hij * vx, fmaf(p.eta2 * hij, hij, r2)) : 0.0f;
         float Q = 0.5f * (ri.rho + rj.rho) * mu * fmaf(-p.alpha * 0.5f, ri.c + rj.c, p.beta * mu);
         float pre = in ? -0.5f * ri.V * rj.V * (ri.P + rj.P + Q) : 0.0f;
         float f[3] = {pre * (gi[0] - gj[0]), pre * (gi[1] - gj[1]), pre * (gi[2] - gj[2])};
@@ -1462,7 +1478,7 @@ struct HydroAdjStage {
         const float vx = fmaf(vij[0], x[0], fmaf(vij[1], x[1], vij[2] * x[2]));
         const float den = fmaf(p.eta2 * hij, hij, r2);
         const bool visc = vx < 0.0f && in;
-        const float mu = visc ? __fdividef(hij * vx, den) : 0.0f;
+        const float mu = visc ? div_normal(hij * vx, den) : 0.0f;
         const float rbar = 0.5f * (ri.rho + rj.rho), cbar = 0.5f * (ri.c + rj.c);
         const float Q = rbar * mu * fmaf(-p.alpha, cbar, p.beta * mu);
         const float Pi = ri.P + rj.P + Q;
@@ -1483,8 +1499,8 @@ struct HydroAdjStage {
             const float mub = Pib * rbar * fmaf(-p.alpha, cbar, 2.0f * p.beta * mu);
             s.rb = fmaf(Pib * 0.5f * mu, fmaf(-p.alpha, cbar, p.beta * mu), s.rb);
             s.cb = fmaf(Pib * rbar * mu, -0.5f * p.alpha, s.cb);
-            const float vxb = __fdividef(mub * hij, den);
-            const float r2b2 = -2.0f * vxb * __fdividef(vx, den);
+            const float vxb = div_normal(mub * hij, den);
+            const float r2b2 = -2.0f * vxb * div_normal(vx, den);
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 s.xb[c] = fmaf(vxb, vij[c], fmaf(r2b2, x[c], s.xb[c]));
@@ -3419,6 +3435,8 @@ static int build_lists(crk_ctx *ctx, crk_leaves *lv, crk_nlist &out, bool reuse)
     using LS = ListStage<kGas>;
     int32_t *gstart = reuse ? out.gstart : (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(nl + 1));
     int32_t *cnt = reuse ? out.cnt : (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)n);
+    // room for the records of the light stages, so that the first pair kernel need not allocate
+    if (!reuse && !crk_scratch(ctx, 4, 32 * (size_t)n)) return crk_fail(ctx, CRK_ENOMEM, "neighbour list scratch");
     int32_t *ng = (int32_t *)crk_scratch(ctx, 6, sizeof(int32_t) * (size_t)(nl + 1));
     int32_t *tot = (int32_t *)crk_scratch(ctx, 7, 64);  // [0] groups, [1] rows, [2] table entries, [4] largest table
     if (!gstart || !cnt || !ng || !tot) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
