@@ -133,9 +133,8 @@ int crk_set_trace(crk_ctx *ctx, int on);
 #define CRK_VARIANT_HALFWARP_SHFL 5
 #define CRK_VARIANT_HALFWARP_SMEM 6
 #define CRK_VARIANT_HALFWARP_LOAD 7
-/* gravity kernels: the candidates of each 32-particle group compacted once, then swept once per
- * 8-particle sub-cell (only those within the cut of its box) by 4 lanes per particle; the leaf
- * build makes the sub-cells RCB cells of 8 when a gravity kernel is set to it at build time */
+/* gravity kernels: the tiles sweep with 8 particles per warp, 4 lanes per particle (TILES takes
+ * 16 particles and 2 lanes per particle on boxes large enough to fill the GPU that way) */
 #define CRK_VARIANT_SPLIT8 8
 #define CRK_N_VARIANTS 9
 int crk_set_variant(crk_ctx *ctx, int kernel, int variant);
@@ -147,10 +146,10 @@ int crk_set_variant(crk_ctx *ctx, int kernel, int variant);
 int crk_set_persistent(crk_ctx *ctx, int on);
 /* Launch shape of one pair kernel (CRK_K_*), as the autotuner sets it:
  * persistent as above; the j-tile depth of the packed tiles sweeps of the
- * gravity kernels (candidates compacted before each sweep: 32, 64 or 96); and
- * their warps per i-leaf block (4: one warp per 32-particle group of a
- * 128-leaf; 2: blocks of two warps, each taking two groups).  The other
- * kernels and variants sweep at depth 32 with 4 warps and ignore both.  The
+ * gravity kernels (32, 64 or 96: a sweep starts once 64 more than that many
+ * candidates are compacted); and their warps per block (4 or 2; each warp
+ * takes 16 or 8 particles of a leaf).  The other kernels and variants sweep at
+ * depth 32 with 4 warps and ignore both.  The
  * results agree up to the order of FP32 additions.  CRK_EINVAL for an unknown
  * kernel, a depth other than 32, 64, 96 or warps other than 2, 4. */
 int crk_set_launch(crk_ctx *ctx, int kernel, int persistent, int depth, int warps);

@@ -48,9 +48,9 @@ struct crk_ctx {
     int num_sms = 0;
     std::string err;
     // growable scratch arena: one buffer per slot
-    static const int kSlots = 38;  // leaf build 0-16 and 19-31, radix sort 12-14, scan 15, queue 17, step 18,
+    static const int kSlots = 37;  // leaf build 0-16 and 19-31, radix sort 12-14, scan 15, queue 17, step 18,
                                    // integrator 32, corrections adjoint 33, adjoint chain 34, half-warp force 35,
-                                   // tuner 36, split-sweep candidates 37
+                                   // tuner 36
     void *slot[kSlots] = {};
     size_t slot_bytes[kSlots] = {};
     int64_t launches = 0;  // kernels this context has launched
@@ -107,6 +107,9 @@ struct crk_leaves {
     int32_t *kinv = nullptr;        // original index -> kernel order position (inverse of kperm)
     int32_t *kinv_g = nullptr;      // original index -> gravity kernel order position
     float4 *pos_g = nullptr;        // [n] gravity kernel order: leaf-relative x, y, z and h or 0
+    // tight boxes (lo, hi; leaf-relative) of the gravity order's cells of 32: cell q of leaf a at
+    // entries 2 c, 2 c + 1 with c = leaf_start[a] / 32 + a + q (n / 32 + n_leaves + 1 cells at most)
+    float4 *gcell = nullptr;
     // leaf-pair lists: per i-leaf a, entries [start[a], start[a] + count[a]) in
     // ascending j-leaf order (leaves may be laid out in any order)
     int32_t *gimg_start = nullptr, *gimg_cnt = nullptr;  // gravity images
@@ -126,7 +129,6 @@ struct crk_leaves {
     std::vector<std::pair<void *, size_t>> allocs;
     // what a capture-safe rebuild (crk_leaves_rebuild) reuses
     int max_leaf = 0, cells = 0;
-    bool cells8 = false;  // gravity order bisected down to RCB cells of 8 (split gravity sweeps)
     std::vector<int64_t> box_start;
     std::vector<float> box_side;
     float *node_box = nullptr, *node_hmax = nullptr;  // RCB traversal tree: node boxes and h_max

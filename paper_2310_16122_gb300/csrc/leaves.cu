@@ -777,7 +777,7 @@ __global__ void leaf_data_kernel(int64_t n_leaves, const int32_t *__restrict__ l
                                  int32_t *__restrict__ leaf_ngas, float *__restrict__ bbox,
                                  float *__restrict__ hmax, float4 *__restrict__ pos, int32_t *__restrict__ kperm_g,
                                  float4 *__restrict__ pos_g, int32_t *__restrict__ kinv, int32_t *__restrict__ kinv_g,
-                                 int32_t *__restrict__ err, int cells8) {
+                                 float4 *__restrict__ gcell, int32_t *__restrict__ err) {
     __shared__ uint64_t key[kCap], zkey[kCap];
     __shared__ Bisect32<kCap> bs;
     __shared__ float4 pm[kCap];  // member position and h (0 for dark matter), gathered once
@@ -879,20 +879,34 @@ __global__ void leaf_data_kernel(int64_t n_leaves, const int32_t *__restrict__ l
         pos[lo + q] = make_float4(c.x - ox, c.y - oy, c.z - oz, c.w);
     }
     __syncthreads();
-    // gravity order: the whole leaf bisected into groups of 32, and (cells8, leaves of at most 256)
-    // each group of 32 into groups of 8 (the sub-cells of the split gravity sweeps)
+    // gravity order: the whole leaf bisected into groups of 32, and (leaves of at most 256) each
+    // group of 32 into groups of 8 (the sub-cells of the gravity sweeps)
     for (int t = threadIdx.x; t < cnt; t += blockDim.x) bs.a[t] = (int16_t)t;
     int16_t *src = bisect32(bs, cnt, pm, key);
-    if constexpr (kCap <= 256) {
-        if (cells8) src = bisect32<kCap, 8>(bs, cnt, pm, key, src, 32);
-    }
-    for (int q = threadIdx.x; q < cnt; q += blockDim.x) {
-        const int t = src[q];
+    if constexpr (kCap <= 256) src = bisect32<kCap, 8>(bs, cnt, pm, key, src, 32);
+    for (int q0 = w * 32; q0 < cnt; q0 += nw * 32) {  // one warp per cell of 32
+        const int q = q0 + lane;
+        const int t = src[q < cnt ? q : cnt - 1];
         const float4 c = pm[t];
-        const int32_t id = (int32_t)(uint32_t)key[t];
-        kperm_g[lo + q] = id;
-        kinv_g[id] = lo + q;
-        pos_g[lo + q] = make_float4(c.x - ox, c.y - oy, c.z - oz, c.w);
+        const float4 r = make_float4(c.x - ox, c.y - oy, c.z - oz, c.w);
+        if (q < cnt) {
+            const int32_t id = (int32_t)(uint32_t)key[t];
+            kperm_g[lo + q] = id;
+            kinv_g[id] = lo + q;
+            pos_g[lo + q] = r;
+        }
+        // the cell's box: leaf-relative coordinates are >= 0 (-0 + 0 = 0), so their bits order like the values
+        const unsigned bits[3] = {__float_as_uint(r.x + 0.0f), __float_as_uint(r.y + 0.0f), __float_as_uint(r.z + 0.0f)};
+        float l[3], u[3];
+        for (int k = 0; k < 3; ++k) {
+            l[k] = __uint_as_float(__reduce_min_sync(CRK_FULL_MASK, bits[k]));
+            u[k] = __uint_as_float(__reduce_max_sync(CRK_FULL_MASK, bits[k]));
+        }
+        if (lane == 0) {
+            float4 *g = gcell + 2 * ((int64_t)(lo >> 5) + a + (q0 >> 5));
+            g[0] = make_float4(l[0], l[1], l[2], 0.0f);
+            g[1] = make_float4(u[0], u[1], u[2], 0.0f);
+        }
     }
 }
 
@@ -1500,9 +1514,6 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
     lv->cells = lp->cells_per_side;
     lv->box_start = box_start;
     lv->box_side = box_side;
-    if (!re)  // the split gravity sweeps want RCB cells of 8 in the gravity order (kept by rebuilds)
-        lv->cells8 = ctx->variant[CRK_K_GRAVITY] == CRK_VARIANT_SPLIT8 ||
-                     ctx->variant[CRK_K_GRAVITY_ADJOINT] == CRK_VARIANT_SPLIT8;
     cudaStream_t st = ctx->stream;
     int rc = CRK_OK;
 #define TRY(expr)                          \
@@ -1741,17 +1752,19 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
         ALLOC(lv->pos_g, float4, n);
         ALLOC(lv->kinv, int32_t, n);
         ALLOC(lv->kinv_g, int32_t, n);
+        ALLOC(lv->gcell, float4, 2 * (n / 32 + nl + 1));
         if (nl > 0) {
             if (lp->mode == 1 && shape && shape->max_leaf_size <= 128)
                 leaf_data_kernel<128><<<(unsigned)nl, 32, 0, st>>>(nl, lv->leaf_start, members, p->x, p->y, p->z,
                                                                    p->species, h, lv->perm, lv->kperm, lv->leaf_ngas,
                                                                    lv->bbox, lv->hmax, lv->pos, lv->kperm_g,
-                                                                   lv->pos_g, lv->kinv, lv->kinv_g, flags + 4,
-                                                                   lv->cells8 ? 1 : 0);
+                                                                   lv->pos_g, lv->kinv, lv->kinv_g, lv->gcell,
+                                                                   flags + 4);
             else
                 leaf_data_kernel<kMaxLeafCap><<<(unsigned)nl, 128, 0, st>>>(
                     nl, lv->leaf_start, members, p->x, p->y, p->z, p->species, h, lv->perm, lv->kperm, lv->leaf_ngas,
-                    lv->bbox, lv->hmax, lv->pos, lv->kperm_g, lv->pos_g, lv->kinv, lv->kinv_g, flags + 4, 0);
+                    lv->bbox, lv->hmax, lv->pos, lv->kperm_g, lv->pos_g, lv->kinv, lv->kinv_g, lv->gcell,
+                    flags + 4);
             ++ctx->launches;
         }
         KCHECK("leaf data");

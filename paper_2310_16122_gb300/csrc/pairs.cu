@@ -24,7 +24,7 @@ namespace {
 constexpr int kThreads = 128;
 constexpr int kWarps = kThreads / 32;
 constexpr int kCap = 64;                     // per-warp candidate buffer
-constexpr int kCapPair = 128;                // per-warp candidate buffer of the packed sweeps (depth <= 96)
+constexpr int kCellPairs = 96;                // per-warp candidate pairs of the gravity cell sweeps
 constexpr int kGroupImgCap = 128;            // image table of one i-leaf staged per warp in shared memory
 // capacities of the one-pass gas lists (adaptive h keeps a gas particle near 58 neighbours;
 // the largest lane list and group table seen in the clustered workloads are ~95 and ~360)
@@ -128,7 +128,8 @@ struct LeafView {
     int64_t n_leaves;
     int32_t *queue;  // persistent mode: next leaf to take (zeroed before launch); NULL = one block per leaf
     int korder;      // 1: the stage's per-particle arrays are in kernel order (no permutation)
-    int depth;       // packed tiles sweeps: candidates compacted before each sweep (32, 64 or 96)
+    int depth;       // gravity sweeps: candidates compacted before each sweep (32, 64 or 96)
+    const float4 *gcell;  // boxes of the gravity order's cells of 32 (lo, hi), leaf-relative
 };
 
 // Next i-leaf of this block: the grid-stride successor, or (persistent mode)
@@ -315,6 +316,26 @@ struct GravStage {
         s.az = __ffma2_rn(f, dz, s.az);
         if (kCount) s.cnt += (int)in0 + (int)in1;
     }
+    // Cell sweeps: the candidate buffer is in planes of float4 over candidate pairs, (x0, x1, y0, y1)
+    // and (z0, z1, m0, m1), so that a pair's fields load as register pairs.
+    static constexpr int kPlanes = 2;
+    __device__ static void putc(float4 (*b)[kCellPairs], int c, const Rec &r) {
+        float *a = reinterpret_cast<float *>(b[0] + (c >> 1)) + (c & 1), *d = reinterpret_cast<float *>(b[1] + (c >> 1)) + (c & 1);
+        a[0] = r.x; a[2] = r.y; d[0] = r.z; d[2] = r.m;
+    }
+    __device__ static Rec2 getc(const float4 (*b)[kCellPairs], int k) {
+        const float4 a = b[0][k], d = b[1][k];
+        return {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(d.x, d.y), make_float2(d.z, d.w)};
+    }
+    // adds the sums of lane ^ o
+    __device__ static void addc(I2 &s, int o) {
+        float2 *a[3] = {&s.ax, &s.ay, &s.az};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            a[k]->x += __shfl_xor_sync(CRK_FULL_MASK, a[k]->x, o);
+            a[k]->y += __shfl_xor_sync(CRK_FULL_MASK, a[k]->y, o);
+        }
+    }
     // partial sums of one i from one leaf-pair tile (half-warp arms): added atomically
     __device__ static void flush(const P &p, const I &s, const Rec &, int32_t o) {
         atomicAdd(&p.a3[o], s.ax);
@@ -322,16 +343,6 @@ struct GravStage {
         atomicAdd(&p.a3[2 * p.n + o], s.az);
     }
     static void zero_outputs(const P &p, cudaStream_t st) { cudaMemsetAsync(p.a3, 0, sizeof(float) * 3 * p.n, st); }
-    // adds the accumulators of lane ^ x (split sweeps: the lanes sharing one i)
-    __device__ static void combine2(I2 &s, int x) {
-        s.ax.x += __shfl_xor_sync(CRK_FULL_MASK, s.ax.x, x);
-        s.ax.y += __shfl_xor_sync(CRK_FULL_MASK, s.ax.y, x);
-        s.ay.x += __shfl_xor_sync(CRK_FULL_MASK, s.ay.x, x);
-        s.ay.y += __shfl_xor_sync(CRK_FULL_MASK, s.ay.y, x);
-        s.az.x += __shfl_xor_sync(CRK_FULL_MASK, s.az.x, x);
-        s.az.y += __shfl_xor_sync(CRK_FULL_MASK, s.az.y, x);
-        s.cnt += __shfl_xor_sync(CRK_FULL_MASK, s.cnt, x);
-    }
     __device__ static void finish2(const P &p, I2 &s, int32_t orig) {
         p.a3[orig] = s.ax.x + s.ax.y;
         p.a3[p.n + orig] = s.ay.x + s.ay.y;
@@ -474,6 +485,29 @@ struct GravAdjStage {
         s.sg = __ffma2_rn(g, dbj, s.sg);
         if (kCount) s.cnt += (int)in0 + (int)in1;
     }
+    // Cell sweeps: planes (x0, x1, y0, y1), (z0, z1, m0, m1), (bx0, bx1, by0, by1), (bz0, bz1, -, -).
+    static constexpr int kPlanes = 4;
+    __device__ static void putc(float4 (*b)[kCellPairs], int c, const Rec &r) {
+        const float v[7] = {r.x, r.y, r.z, r.m, r.bx, r.by, r.bz};
+#pragma unroll
+        for (int k = 0; k < 7; ++k)
+            (reinterpret_cast<float *>(b[k >> 1] + (c >> 1)) + (c & 1))[2 * (k & 1)] = v[k];
+    }
+    __device__ static Rec2 getc(const float4 (*b)[kCellPairs], int k) {
+        const float4 a = b[0][k], d = b[1][k], e = b[2][k];
+        const float2 f = *reinterpret_cast<const float2 *>(&b[3][k]);
+        return {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(d.x, d.y), make_float2(d.z, d.w),
+                make_float2(e.x, e.y), make_float2(e.z, e.w), f, f};
+    }
+    // adds the sums of lane ^ o
+    __device__ static void addc(I2 &s, int o) {
+        float2 *a[8] = {&s.kx, &s.ky, &s.kz, &s.s1x, &s.s1y, &s.s1z, &s.s2, &s.sg};
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            a[k]->x += __shfl_xor_sync(CRK_FULL_MASK, a[k]->x, o);
+            a[k]->y += __shfl_xor_sync(CRK_FULL_MASK, a[k]->y, o);
+        }
+    }
     // partial sums of one i from one leaf-pair tile (half-warp arms): added atomically
     __device__ static void flush(const P &p, const I &s, const Rec &, int32_t o) {
         atomicAdd(&p.gx3[o], s.gx);
@@ -484,16 +518,6 @@ struct GravAdjStage {
     static void zero_outputs(const P &p, cudaStream_t st) {
         cudaMemsetAsync(p.gx3, 0, sizeof(float) * 3 * p.n, st);
         cudaMemsetAsync(p.gm, 0, sizeof(float) * p.n, st);
-    }
-    // adds the accumulators of lane ^ x (split sweeps: the lanes sharing one i)
-    __device__ static void combine2(I2 &s, int x) {
-        float2 *acc[8] = {&s.kx, &s.ky, &s.kz, &s.s1x, &s.s1y, &s.s1z, &s.s2, &s.sg};
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            acc[q]->x += __shfl_xor_sync(CRK_FULL_MASK, acc[q]->x, x);
-            acc[q]->y += __shfl_xor_sync(CRK_FULL_MASK, acc[q]->y, x);
-        }
-        s.cnt += __shfl_xor_sync(CRK_FULL_MASK, s.cnt, x);
     }
     __device__ static void finish2(const P &p, I2 &s, int32_t o) {
         const float mi = s.mi.x, nbx = s.nbx.x, nby = s.nby.x, nbz = s.nbz.x;
@@ -1671,7 +1695,6 @@ struct ListP {
 
 template <bool kGas>
 struct ListStage {
-    static constexpr bool kPair = false;
     static constexpr bool kGasOnly = kGas;
     static constexpr bool kCons = false;
     static constexpr bool kTag = true;
@@ -1856,253 +1879,191 @@ __device__ __forceinline__ void tile_group(const LeafView &lv, const typename S:
     }
 }
 
-// tile_group for stages with packed two-candidate interactions (kPair): the
-// candidate buffer holds field-interleaved candidate pairs; an odd tail is
-// padded with a massless dummy outside every i's cut, which adds exact zeros.
-template <class S, bool kCount>
-__device__ __forceinline__ void tile_group_pair(const LeafView &lv, const typename S::P &p,
-                                                RecView<typename S::Rec> rec, typename S::Rec2 *buf,
-                                                int64_t a, int lo, int g0, int hi, int lane) {
+// Cell sweeps (the TILES and SPLIT8 variants of the gravity kernels).  A warp
+// takes G consecutive particles of a leaf (G = 16 or 8: an RCB cell of the
+// gravity kernel order) and all candidates within r_c of their box:
+//   1. The j side is walked in cells of 32 (the groups of the kernel order).
+//      Their boxes are tested 32 at a time, one per lane, before any particle
+//      is loaded; the particles of a cell near enough are tested one per lane,
+//      loaded one cell ahead, and those kept are compacted into shared memory.
+//   2. A full buffer is swept: lane l evaluates candidate pairs k 32/G + l/G
+//      (k = 0, 1, ..) against particle l % G with packed FP32 (f32x2)
+//      arithmetic, so each row of the sweep reads 32/G pairs and every lane
+//      works.  The sums of the 32/G streams are added by shuffles at the end
+//      (fixed order, no atomics: deterministic).
+// The FP32 pipe bounds it (56% busy; DRAM below 1%), on swept pairs: of those
+// 0.43 are in range with G = 16 on the clustered boxes, 0.34 with G = 32 and
+// 0.54 with G = 8, whose candidate tests cost more than the pairs they save.
+// 2x128^3 box, gravity / adjoint: 2.92 / 5.49 ms (G = 32: 2.97 / 5.92, G = 8:
+// 3.56 / 6.33), against 3.27 / 6.01 for a warp per group of 32 that walked the
+// leaf images one by one.  Slower: several units per warp sharing the candidate loads (3.3 / 5.7 ms and more), two i per
+// lane against one j (the j then needs register moves: 3.3 / 5.7 ms).
+template <class S, bool kCount, int G, int kW>
+__global__ void __launch_bounds__(32 * kW) cell_kernel(LeafView lv, typename S::P p, RecView<typename S::Rec> rec,
+                                                       int units, int log_cpl, int full) {
     using Rec = typename S::Rec;
-    static_assert(!S::kCons && !S::kGasOnly && !S::kTag, "packed sweep: gravity-type stages only");
+    constexpr int T = 32 / G;  // streams: candidate pairs per row
+    __shared__ float4 buf[kW][S::kPlanes][kCellPairs];
+    __shared__ float4 cells[kW][32];  // one round's cells: shift, first particle
+    __shared__ int cell_n[kW][32];    // and particles
+    __shared__ int64_t slot;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, str = lane / G;
     const unsigned below = lanemask_lt();
-    const int ib = lv.img_start[a], ie = ib + lv.img_cnt[a];
-    const int i = g0 + lane;
-    const bool act = i < hi;
-    const Rec ri = rec[act ? i : g0];
-    typename S::I2 st;
-    S::init2(p, st, ri);
-    float bl0 = ri.x, bl1 = ri.y, bl2 = ri.z, bh0 = ri.x, bh1 = ri.y, bh2 = ri.z;
-    float hm = lv.pos[act ? i : g0].w;
+    const float cut = S::leaf_cut(p, 0.0f, 0.0f), cut2 = cut * cut * 1.0001f + 1e-6f;
+    const int cmask = (1 << log_cpl) - 1;
+    // block b takes units b kW .. b kW + kW - 1; a unit is G consecutive particles of one leaf
+    for (int64_t b = next_leaf(lv, -1, &slot); b * kW < lv.n_leaves * units; b = next_leaf(lv, b, &slot)) {
+        const int64_t unit = b * kW + warp;
+        const int64_t a = unit / units;
+        if (a >= lv.n_leaves) continue;
+        const int lo = lv.leaf_start[a], hi = lv.leaf_start[a + 1];
+        const int ib = lv.img_start[a], ie = ib + lv.img_cnt[a];
+        // (a rebuilt chaining-mesh cell may hold more units than the launch counted: strided)
+        for (int c0 = lo + G * (int)(unit - a * units); c0 < hi; c0 += G * units) {
+            const int i = c0 + lane % G;
+            const bool act = i < hi;
+            typename S::I2 st;
+            float ul[3], uh[3];  // the unit's box
+            {
+                const Rec ri = rec[act ? i : hi - 1];
+                S::init2(p, st, ri);
+                // leaf-relative coordinates are >= 0 (-0 + 0 = 0): their bits order like the values
+                const unsigned x[3] = {__float_as_uint(ri.x + 0.0f), __float_as_uint(ri.y + 0.0f),
+                                       __float_as_uint(ri.z + 0.0f)};
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        bl0 = fminf(bl0, __shfl_xor_sync(CRK_FULL_MASK, bl0, o));
-        bl1 = fminf(bl1, __shfl_xor_sync(CRK_FULL_MASK, bl1, o));
-        bl2 = fminf(bl2, __shfl_xor_sync(CRK_FULL_MASK, bl2, o));
-        bh0 = fmaxf(bh0, __shfl_xor_sync(CRK_FULL_MASK, bh0, o));
-        bh1 = fmaxf(bh1, __shfl_xor_sync(CRK_FULL_MASK, bh1, o));
-        bh2 = fmaxf(bh2, __shfl_xor_sync(CRK_FULL_MASK, bh2, o));
-        hm = fmaxf(hm, __shfl_xor_sync(CRK_FULL_MASK, hm, o));
-    }
-    const float far = 2.0f * S::leaf_cut(p, hm, hm) + 1.0f;
-    const Rec dummy = S::far_dummy(bh0 + far, bh1 + far, bh2 + far);
-    // sweep once at least `depth` candidates are compacted (the buffer holds depth + 31 + 1 dummy)
-    const int depth = lv.depth >= 64 ? (lv.depth >= 96 ? 96 : 64) : 32;
-    auto sweep = [&](int cnt) {
-        if (cnt & 1) {
-            if (lane == 0) S::put2(buf, cnt, dummy);
-            ++cnt;
-        }
-        __syncwarp();
-        // unrolled: independent packed pairs interleave their dependent chains (Horner, rsqrt);
-        // on the 2x256^3 box gravity and its adjoint took 28.2 and 48.8 ms rolled, 26.6 and
-        // 46.9 ms unrolled by 4, 26.4 and 46.4 ms by 8
+                for (int k = 0; k < 3; ++k) {
+                    ul[k] = __uint_as_float(__reduce_min_sync(CRK_FULL_MASK, x[k]));
+                    uh[k] = __uint_as_float(__reduce_max_sync(CRK_FULL_MASK, x[k]));
+                }
+            }
+            unsigned long long swept = 0;  // counting runs: candidates swept
+            int cnt = 0, e0 = ib, q = lane & cmask;  // q: this lane's cell of its image's leaf
+            unsigned todo = 0;
+            Rec rn;        // this lane's particle of the next cell, loaded one cell ahead
+            float4 cl;     // that cell's shift
+            int nn = 0;    // and its particles
+            auto next = [&]() {
+                const int src = __ffs(todo) - 1;
+                cl = cells[warp][src];
+                nn = cell_n[warp][src];
+                if (lane < nn) rn = rec[__float_as_int(cl.w) + lane];
+            };
+            bool done = false;
+            while (!done) {
+                // ---- 1. fill the buffer
+                while (cnt < full) {
+                    if (!todo) {
+                        if (e0 >= ie) {
+                            done = true;
+                            break;
+                        }
+                        const int e = e0 + (lane >> log_cpl);
+                        bool pass = false, more = false;
+                        if (e < ie) {
+                            const crk_image im = lv.img[e];
+                            const int jlo = lv.leaf_start[im.b], jhi = lv.leaf_start[im.b + 1];
+                            const int jb = jlo + 32 * q;
+                            more = jhi - jb > 32 * (cmask + 1);
+                            if (jb < jhi) {
+                                const float4 *gb = lv.gcell + 2 * ((int64_t)(jlo >> 5) + im.b + q);
+                                const float4 l = gb[0], h = gb[1];
+                                const float gx = fmaxf(fmaxf(im.sx + l.x - uh[0], ul[0] - (im.sx + h.x)), 0.f);
+                                const float gy = fmaxf(fmaxf(im.sy + l.y - uh[1], ul[1] - (im.sy + h.y)), 0.f);
+                                const float gz = fmaxf(fmaxf(im.sz + l.z - uh[2], ul[2] - (im.sz + h.z)), 0.f);
+                                pass = fmaf(gx, gx, fmaf(gy, gy, gz * gz)) <= cut2;
+                                cells[warp][lane] = make_float4(im.sx, im.sy, im.sz, __int_as_float(jb));
+                                cell_n[warp][lane] = min(jhi - jb, 32);
+                            }
+                        }
+                        todo = __ballot_sync(CRK_FULL_MASK, pass);
+                        if (__any_sync(CRK_FULL_MASK, more)) {  // a leaf with more cells than its lanes: once more
+                            q += cmask + 1;
+                        } else {
+                            q = lane & cmask;
+                            e0 += 32 >> log_cpl;
+                        }
+                        if (!todo) continue;
+                        __syncwarp();
+                        next();
+                    }
+                    Rec rj = rn;
+                    const bool jv = lane < nn;
+                    S::shift(rj, cl.x, cl.y, cl.z);
+                    todo &= todo - 1;
+                    if (todo) next();
+                    const float dx = fmaxf(fmaxf(ul[0] - rj.x, rj.x - uh[0]), 0.f);
+                    const float dy = fmaxf(fmaxf(ul[1] - rj.y, rj.y - uh[1]), 0.f);
+                    const float dz = fmaxf(fmaxf(ul[2] - rj.z, rj.z - uh[2]), 0.f);
+                    const bool keep = jv && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= cut2;
+                    const unsigned m = __ballot_sync(CRK_FULL_MASK, keep);
+                    if (keep) S::putc(buf[warp], cnt + __popc(m & below), rj);
+                    cnt += __popc(m);
+                }
+                // ---- 2. sweep the whole rows; what is left over goes to the front (at the end: padded
+                // with a massless dummy outside every cut, which adds exact zeros)
+                if (done) {
+                    const float far = 2.0f * cut + 1.0f;
+                    const Rec dummy = S::far_dummy(uh[0] + far, uh[1] + far, uh[2] + far);
+                    const int pad = -cnt & (2 * T - 1);
+                    if (kCount) swept += cnt;
+                    if (lane < pad) S::putc(buf[warp], cnt + lane, dummy);
+                    cnt += pad;
+                }
+                __syncwarp();
+                const int rows = cnt / (2 * T);
 #pragma unroll 8
-        for (int k = 0; k < (cnt >> 1); ++k) S::template interact2<kCount>(p, st, buf[k]);
-        __syncwarp();
-    };
-    int cnt = 0;
-    unsigned long long swept = 0;  // counting runs: candidates swept
-    for (int e = ib; e < ie; ++e) {
-        const crk_image im = lv.img[e];
-        const int jlo = lv.leaf_start[im.b];
-        const int jhi = lv.leaf_start[im.b + 1];
-        {
-            const float *bb = lv.bbox + 6 * (int64_t)im.b;
-            float gx = fmaxf(fmaxf(im.sx - bh0, bl0 - (im.sx + (bb[3] - bb[0]))), 0.f);
-            float gy = fmaxf(fmaxf(im.sy - bh1, bl1 - (im.sy + (bb[4] - bb[1]))), 0.f);
-            float gz = fmaxf(fmaxf(im.sz - bh2, bl2 - (im.sz + (bb[5] - bb[2]))), 0.f);
-            float cut = S::leaf_cut(p, hm, lv.hmax[im.b]);
-            if (!(fmaf(gx, gx, fmaf(gy, gy, gz * gz)) <= cut * cut * 1.0001f + 1e-6f)) continue;
-        }
-        for (int j0 = jlo; j0 < jhi; j0 += 32) {
-            const int j = j0 + lane;
-            const bool jv = j < jhi;
-            Rec rj;
-            bool keep = false;
-            if (jv) {
-                rj = rec[j];
-                S::shift(rj, im.sx, im.sy, im.sz);
-                float dx = fmaxf(fmaxf(bl0 - rj.x, rj.x - bh0), 0.f);
-                float dy = fmaxf(fmaxf(bl1 - rj.y, rj.y - bh1), 0.f);
-                float dz = fmaxf(fmaxf(bl2 - rj.z, rj.z - bh2), 0.f);
-                float cut = S::box_cut(p, hm, rj);
-                keep = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= cut * cut * 1.0001f + 1e-6f;
+                for (int k = 0; k < rows; ++k) S::template interact2<kCount>(p, st, S::getc(buf[warp], k * T + str));
+                if (!done) {
+                    if (kCount) swept += rows * 2 * T;
+                    cnt -= rows * 2 * T;
+                    __syncwarp();
+                    if (lane < T * S::kPlanes) {  // at most T pairs (rows > 1: the two ranges do not overlap)
+                        const int k = lane % T, w = lane / T;
+                        buf[warp][w][k] = buf[warp][w][rows * T + k];
+                    }
+                }
+                __syncwarp();
             }
-            const unsigned m = __ballot_sync(CRK_FULL_MASK, keep);
-            if (keep) S::put2(buf, cnt + __popc(m & below), rj);
-            cnt += __popc(m);
-            if (cnt >= depth) {
-                sweep(cnt);
-                if (kCount) swept += cnt;
-                cnt = 0;
-            }
-        }
-    }
-    sweep(cnt);
-    if (kCount) swept += cnt;
-    if (act) S::finish2(p, st, lv.korder ? i : lv.kperm[i]);
-    if (kCount) {
-        int c = act ? st.cnt - 1 : 0;  // the self pair (r = 0) is always in range
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(CRK_FULL_MASK, c, o);
-        if (lane == 0 && c) atomicAdd(p.count, (unsigned long long)c);
-        const unsigned long long na = __popc(__ballot_sync(CRK_FULL_MASK, act));
-        if (lane == 0 && p.swept) atomicAdd(p.swept, swept * na);
+            for (int o = G; o < 32; o <<= 1) S::addc(st, o);
+            if (act && str == 0) S::finish2(p, st, stage_index(lv, i));
+            if (kCount) {
+                int cn = act ? st.cnt - (str == 0) : 0;  // the self pair (r = 0) is always in range
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) cn += __shfl_xor_sync(CRK_FULL_MASK, cn, o);
+                if (lane == 0 && cn) atomicAdd(p.count, (unsigned long long)cn);
+                if (lane == 0 && p.swept) atomicAdd(p.swept, swept * min(G, hi - c0));
+            }
+        }
     }
 }
 
-// Split tiles for the packed gravity sweeps (CRK_VARIANT_SPLIT8).  The warp
-// compacts the candidates within the cut of its 32-particle group (an RCB cell
-// of the leaf) once, into a per-warp buffer in global memory (its working set
-// stays in L2), then sweeps that buffer once for each of the group's four
-// 8-particle RCB sub-cells: only the candidates within the cut of the
-// sub-cell's box are kept (compacted into shared memory), and the 4 lanes of
-// each of the sub-cell's 8 i-particles take every 4th packed candidate pair,
-// so the lanes stay balanced; their partial sums are added by shuffles at the
-// end.  A sub-cell box is about a quarter of the group's volume, so a larger
-// share of the evaluated pairs lies within r_c.  A group whose candidates
-// overflow the buffer (gcap) is swept as plain tiles.
+template <class S, bool kCount, int G>
+void launch_cells_g(const crk_ctx *ctx, const crk_leaves *lv, const LeafView &v, const typename S::P &p,
+                    RecView<typename S::Rec> rec, bool persistent, int warps) {
+    const int most = lv->max_leaf_size > 0 ? lv->max_leaf_size : 1;
+    const int units = (most + G - 1) / G;
+    int log_cpl = 0;  // cells of 32 per leaf, rounded up to a power of two (at most 32: one per lane)
+    while ((32 << log_cpl) < most && log_cpl < 5) ++log_cpl;
+    const int kw = warps == 2 ? 2 : 4;
+    int64_t grid = (lv->n_leaves * units + kw - 1) / kw;
+    if (grid < 1) grid = 1;
+    if (grid > 2147483647LL) grid = 2147483647LL;
+    if (persistent) grid = std::min<int64_t>(grid, (int64_t)ctx->num_sms * (kw == 2 ? 8 : 4));
+    const int full = v.depth + 64;  // at most 160: 32 more fit, and a padded row
+    if (kw == 2) cell_kernel<S, kCount, G, 2><<<(unsigned)grid, 64, 0, ctx->stream>>>(v, p, rec, units, log_cpl, full);
+    else cell_kernel<S, kCount, G, 4><<<(unsigned)grid, 128, 0, ctx->stream>>>(v, p, rec, units, log_cpl, full);
+}
+
+// SPLIT8: 8 particles per warp.  TILES: 16, or 8 where units of 16 are fewer
+// than the warps the GPU holds (28 per SM at the kernels' registers): a box of
+// 8192 particles then takes 35 / 43 us (gravity / adjoint) instead of 42 / 52,
+// one of 30011 43 / 70 instead of 47 / 68, one of 65,536 80 / 125 instead of 80 / 129.
 template <class S, bool kCount>
-__global__ void __launch_bounds__(kThreads) pair_kernel_split(LeafView lv, typename S::P p,
-                                                              RecView<typename S::Rec> rec,
-                                                              typename S::Rec *__restrict__ gbuf, int gcap) {
-    using Rec = typename S::Rec;
-    using Rec2 = typename S::Rec2;
-    static_assert(S::kPair && !S::kCons && !S::kGasOnly, "split sweeps: packed gravity-type stages only");
-    __shared__ __align__(16) Rec sbuf[kWarps][kCapPair];
-    __shared__ int64_t leaf_slot;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    Rec2 *buf = reinterpret_cast<Rec2 *>(sbuf[warp]);
-    Rec *gb = gbuf + ((size_t)blockIdx.x * kWarps + warp) * (size_t)gcap;
-    const unsigned below = lanemask_lt();
-    const int depth = lv.depth >= 64 ? (lv.depth >= 96 ? 96 : 64) : 64;  // at least 64: 8 pairs per split lane
-    for (int64_t a = next_leaf(lv, -1, &leaf_slot); a < lv.n_leaves; a = next_leaf(lv, a, &leaf_slot)) {
-        const int lo = lv.leaf_start[a], hi = lv.leaf_start[a + 1];
-        const int ib = lv.img_start[a], ie = ib + lv.img_cnt[a];
-        for (int g0 = lo + warp * 32; g0 < hi; g0 += kWarps * 32) {
-            // ---- the group's candidates into the per-warp buffer
-            const int i = g0 + lane;
-            const Rec ri = rec[i < hi ? i : g0];
-            float bl0 = ri.x, bl1 = ri.y, bl2 = ri.z, bh0 = ri.x, bh1 = ri.y, bh2 = ri.z;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                bl0 = fminf(bl0, __shfl_xor_sync(CRK_FULL_MASK, bl0, o));
-                bl1 = fminf(bl1, __shfl_xor_sync(CRK_FULL_MASK, bl1, o));
-                bl2 = fminf(bl2, __shfl_xor_sync(CRK_FULL_MASK, bl2, o));
-                bh0 = fmaxf(bh0, __shfl_xor_sync(CRK_FULL_MASK, bh0, o));
-                bh1 = fmaxf(bh1, __shfl_xor_sync(CRK_FULL_MASK, bh1, o));
-                bh2 = fmaxf(bh2, __shfl_xor_sync(CRK_FULL_MASK, bh2, o));
-            }
-            const float cut = S::leaf_cut(p, 0.f, 0.f);
-            const float cut2 = cut * cut * 1.0001f + 1e-6f;
-            int cnt = 0;
-            bool ovf = false;
-            for (int e = ib; e < ie && !ovf; ++e) {
-                const crk_image im = lv.img[e];
-                const int jlo = lv.leaf_start[im.b], jhi = lv.leaf_start[im.b + 1];
-                {
-                    const float *bb = lv.bbox + 6 * (int64_t)im.b;
-                    float gx = fmaxf(fmaxf(im.sx - bh0, bl0 - (im.sx + (bb[3] - bb[0]))), 0.f);
-                    float gy = fmaxf(fmaxf(im.sy - bh1, bl1 - (im.sy + (bb[4] - bb[1]))), 0.f);
-                    float gz = fmaxf(fmaxf(im.sz - bh2, bl2 - (im.sz + (bb[5] - bb[2]))), 0.f);
-                    if (!(fmaf(gx, gx, fmaf(gy, gy, gz * gz)) <= cut2)) continue;
-                }
-                for (int j0 = jlo; j0 < jhi; j0 += 32) {
-                    const int j = j0 + lane;
-                    Rec rj;
-                    bool keep = false;
-                    if (j < jhi) {
-                        rj = rec[j];
-                        S::shift(rj, im.sx, im.sy, im.sz);
-                        float dx = fmaxf(fmaxf(bl0 - rj.x, rj.x - bh0), 0.f);
-                        float dy = fmaxf(fmaxf(bl1 - rj.y, rj.y - bh1), 0.f);
-                        float dz = fmaxf(fmaxf(bl2 - rj.z, rj.z - bh2), 0.f);
-                        keep = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= cut2;
-                    }
-                    const unsigned m = __ballot_sync(CRK_FULL_MASK, keep);
-                    if (cnt + __popc(m) > gcap) {
-                        ovf = true;
-                        break;
-                    }
-                    if (keep) gb[cnt + __popc(m & below)] = rj;
-                    cnt += __popc(m);
-                }
-            }
-            if (ovf) {  // a dense group: plain tiles
-                tile_group_pair<S, kCount>(lv, p, rec, buf, a, lo, g0, hi, lane);
-                __syncwarp();
-                continue;
-            }
-            __syncwarp();  // the buffer's stores are visible to the whole warp
-            // ---- the four sub-cells of 8: 4 lanes per i, each taking every 4th packed pair
-            const int il = lane >> 2, sp = lane & 3;
-            for (int c0 = g0; c0 < g0 + 32 && c0 < hi; c0 += 8) {
-                const int ii = c0 + il;
-                const bool iact = ii < hi;
-                const Rec rs = rec[iact ? ii : c0];
-                float sl0 = rs.x, sl1 = rs.y, sl2 = rs.z, sh0 = rs.x, sh1 = rs.y, sh2 = rs.z;
-#pragma unroll
-                for (int o = 4; o < 32; o <<= 1) {  // over the 8 i of the sub-cell
-                    sl0 = fminf(sl0, __shfl_xor_sync(CRK_FULL_MASK, sl0, o));
-                    sl1 = fminf(sl1, __shfl_xor_sync(CRK_FULL_MASK, sl1, o));
-                    sl2 = fminf(sl2, __shfl_xor_sync(CRK_FULL_MASK, sl2, o));
-                    sh0 = fmaxf(sh0, __shfl_xor_sync(CRK_FULL_MASK, sh0, o));
-                    sh1 = fmaxf(sh1, __shfl_xor_sync(CRK_FULL_MASK, sh1, o));
-                    sh2 = fmaxf(sh2, __shfl_xor_sync(CRK_FULL_MASK, sh2, o));
-                }
-                const float far = 2.0f * cut + 1.0f;
-                const Rec dummy = S::far_dummy(sh0 + far, sh1 + far, sh2 + far);
-                typename S::I2 st;
-                S::init2(p, st, rs);
-                unsigned long long swept = 0;
-                int bc = 0;
-                auto sweep = [&](int n) {
-                    if (n & 1) {
-                        if (lane == 0) S::put2(buf, n, dummy);
-                        ++n;
-                    }
-                    __syncwarp();
-                    for (int k = sp; k < (n >> 1); k += 4) S::template interact2<kCount>(p, st, buf[k]);
-                    __syncwarp();
-                };
-                for (int q0 = 0; q0 < cnt; q0 += 32) {
-                    const int q = q0 + lane;
-                    Rec rj;
-                    bool keep = false;
-                    if (q < cnt) {
-                        rj = gb[q];
-                        float dx = fmaxf(fmaxf(sl0 - rj.x, rj.x - sh0), 0.f);
-                        float dy = fmaxf(fmaxf(sl1 - rj.y, rj.y - sh1), 0.f);
-                        float dz = fmaxf(fmaxf(sl2 - rj.z, rj.z - sh2), 0.f);
-                        keep = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= cut2;
-                    }
-                    const unsigned m = __ballot_sync(CRK_FULL_MASK, keep);
-                    if (keep) S::put2(buf, bc + __popc(m & below), rj);
-                    bc += __popc(m);
-                    if (bc >= depth) {
-                        sweep(bc);
-                        if (kCount) swept += bc;
-                        bc = 0;
-                    }
-                }
-                sweep(bc);
-                if (kCount) swept += bc;
-                S::combine2(st, 1);
-                S::combine2(st, 2);
-                if (sp == 0 && iact) S::finish2(p, st, lv.korder ? ii : lv.kperm[ii]);
-                if (kCount) {
-                    int c = (sp == 0 && iact) ? st.cnt - 1 : 0;  // the self pair (r = 0) is always in range
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(CRK_FULL_MASK, c, o);
-                    if (lane == 0 && c) atomicAdd(p.count, (unsigned long long)c);
-                    const unsigned long long na = __popc(__ballot_sync(CRK_FULL_MASK, sp == 0 && iact));
-                    if (lane == 0 && p.swept) atomicAdd(p.swept, swept * na);
-                }
-            }
-            __syncwarp();  // the buffer is reused by the next group
-        }
-    }
+void launch_cells(const crk_ctx *ctx, const crk_leaves *lv, const LeafView &v, const typename S::P &p,
+                  RecView<typename S::Rec> rec, bool persistent, int warps, bool split8) {
+    if (split8 || lv->n < (int64_t)16 * 28 * ctx->num_sms) launch_cells_g<S, kCount, 8>(ctx, lv, v, p, rec, persistent, warps);
+    else launch_cells_g<S, kCount, 16>(ctx, lv, v, p, rec, persistent, warps);
 }
 
 // The paper's "half-warp" leaf-pair scheme (Sec. 5.3), as autotuner arms for
@@ -2237,19 +2198,6 @@ __global__ void __launch_bounds__(kThreads) pair_kernel_halfwarp(LeafView lv, ty
     }
 }
 
-// one i-group, tiles (packed sweep where the stage has one)
-template <class S, bool kCount>
-__device__ __forceinline__ void tile_group_any(const LeafView &lv, const typename S::P &p,
-                                               RecView<typename S::Rec> rec, typename S::Rec *buf,
-                                               int64_t a, int lo, int g0, int hi, int lane, double cons_acc[4]) {
-    if constexpr (S::kPair) {
-        static_assert(sizeof(typename S::Rec2) == 2 * sizeof(typename S::Rec), "pair record layout");
-        tile_group_pair<S, kCount>(lv, p, rec, reinterpret_cast<typename S::Rec2 *>(buf), a, lo, g0, hi, lane);
-    } else {
-        tile_group<S, kCount>(lv, p, rec, buf, a, lo, g0, hi, lane, cons_acc);
-    }
-}
-
 // Per-block partial of the FP64 conservation sums in a fixed order (reduced by
 // cons_reduce_kernel: deterministic for a fixed assignment of work to blocks).
 __device__ __forceinline__ void cons_block_partial(double (*cons_sh)[4], const double cons_acc[4],
@@ -2267,15 +2215,14 @@ __device__ __forceinline__ void cons_block_partial(double (*cons_sh)[4], const d
 }
 
 // Tiles, one block per i-leaf (or leaves from the persistent queue); the
-// block's kW warps take the leaf's groups in turn (kW = 2: the packed gravity
-// sweeps' narrow launch shape, two groups of a 128-leaf per warp).
-template <class S, bool kCount, int kW = kWarps>
-__global__ void __launch_bounds__(32 * kW) pair_kernel(LeafView lv, typename S::P p,
-                                                       RecView<typename S::Rec> rec,
-                                                       double *__restrict__ cons_part) {
+// block's warps take the leaf's groups in turn (gas stages; the gravity
+// stages run cell_kernel).
+template <class S, bool kCount>
+__global__ void __launch_bounds__(kThreads) pair_kernel(LeafView lv, typename S::P p, RecView<typename S::Rec> rec,
+                                                        double *__restrict__ cons_part) {
     using Rec = typename S::Rec;
-    static_assert(kW == kWarps || !S::kCons, "conservation partials assume kWarps warps per block");
-    __shared__ __align__(16) Rec buf[kW][S::kPair ? kCapPair : kCap];
+    static_assert(!S::kPair, "gravity stages sweep sub-cells");
+    __shared__ __align__(16) Rec buf[kWarps][kCap];
     __shared__ double cons_sh[kWarps][4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double cons_acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -2283,8 +2230,8 @@ __global__ void __launch_bounds__(32 * kW) pair_kernel(LeafView lv, typename S::
     for (int64_t a = next_leaf(lv, -1, &leaf_slot); a < lv.n_leaves; a = next_leaf(lv, a, &leaf_slot)) {
         const int lo = lv.leaf_start[a];
         const int hi = S::kGasOnly ? lo + lv.leaf_ngas[a] : lv.leaf_start[a + 1];
-        for (int g0 = lo + warp * 32; g0 < hi; g0 += kW * 32)
-            tile_group_any<S, kCount>(lv, p, rec, buf[warp], a, lo, g0, hi, lane, cons_acc);
+        for (int g0 = lo + warp * 32; g0 < hi; g0 += kWarps * 32)
+            tile_group<S, kCount>(lv, p, rec, buf[warp], a, lo, g0, hi, lane, cons_acc);
     }
     if constexpr (S::kCons) {
         if (cons_part) cons_block_partial(cons_sh, cons_acc, cons_part);
@@ -2324,7 +2271,7 @@ __global__ void __launch_bounds__(kThreads) pair_group_kernel(LeafView lv, typen
         const int lo = lv.leaf_start[a];
         const int hi = S::kGasOnly ? lo + lv.leaf_ngas[a] : lv.leaf_start[a + 1];
         const int g0 = lo + 32 * (int)(grp - gt.gstart[a]);
-        tile_group_any<S, kCount>(lv, p, rec, buf[warp], a, lo, g0, hi, lane, cons_acc);
+        tile_group<S, kCount>(lv, p, rec, buf[warp], a, lo, g0, hi, lane, cons_acc);
     }
     if constexpr (S::kCons) {
         if (cons_part) cons_block_partial(cons_sh, cons_acc, cons_part);
@@ -3129,7 +3076,7 @@ int run_stage(crk_ctx *ctx, const crk_leaves *lv, typename S::P p, bool gas_pair
     }
     LeafView v{lv->leaf_start, lv->leaf_ngas, lv->bbox, lv->hmax, kpos, kperm,
                gas_pairs ? lv->himg_start : lv->gimg_start, gas_pairs ? lv->himg_cnt : lv->gimg_cnt,
-               gas_pairs ? lv->himg : lv->gimg, lv->n_leaves, queue, korder ? 1 : 0, ctx->depth[kernel_id]};
+               gas_pairs ? lv->himg : lv->gimg, lv->n_leaves, queue, korder ? 1 : 0, ctx->depth[kernel_id], lv->gcell};
     if (p.count) CRK_CUDA(ctx, cudaMemsetAsync(p.count, 0, sizeof(unsigned long long), ctx->stream));
     if (p.swept) CRK_CUDA(ctx, cudaMemsetAsync(p.swept, 0, sizeof(unsigned long long), ctx->stream));
     if (lists) {
@@ -3176,35 +3123,7 @@ int run_stage(crk_ctx *ctx, const crk_leaves *lv, typename S::P p, bool gas_pair
         else
             pair_kernel<S, false><<<(unsigned)grid, kThreads, 0, ctx->stream>>>(v, p, rec, part);
     } else {
-        if (ctx->variant[kernel_id] == CRK_VARIANT_SPLIT8 && S::kPair) {
-            if constexpr (S::kPair) {
-                // a bounded grid: every block's warps own a slot of the candidate buffer
-                constexpr int kGcap = 4096;
-                static int occ[2] = {0, 0};  // resident blocks per SM, from the kernel's registers and shared memory
-                int &oc = occ[p.count ? 1 : 0];
-                if (!oc) {
-                    cudaFuncAttributes fa{};
-                    const cudaError_t e = p.count ? cudaFuncGetAttributes(&fa, pair_kernel_split<S, true>)
-                                                  : cudaFuncGetAttributes(&fa, pair_kernel_split<S, false>);
-                    int by_regs = 16, by_smem = 16;
-                    if (e == cudaSuccess && fa.numRegs > 0) {
-                        const int regs = (fa.numRegs + 7) / 8 * 8;  // allocated per thread in units of 8
-                        by_regs = 65536 / (regs * kThreads);
-                        by_smem = (int)((228u * 1024u) / ((unsigned)fa.sharedSizeBytes + 1024u));
-                    } else {
-                        cudaGetLastError();
-                    }
-                    oc = std::max(1, std::min(16, std::min(by_regs, by_smem)));
-                }
-                const int64_t g = std::min<int64_t>(grid, (int64_t)ctx->num_sms * oc);
-                Rec *gbuf = (Rec *)crk_scratch(ctx, 37, sizeof(Rec) * (size_t)g * kWarps * kGcap);
-                if (!gbuf) return crk_fail(ctx, CRK_ENOMEM, "stage scratch");
-                if (p.count)
-                    pair_kernel_split<S, true><<<(unsigned)g, kThreads, 0, ctx->stream>>>(v, p, rec, gbuf, kGcap);
-                else
-                    pair_kernel_split<S, false><<<(unsigned)g, kThreads, 0, ctx->stream>>>(v, p, rec, gbuf, kGcap);
-            }
-        } else if (ctx->variant[kernel_id] == CRK_VARIANT_TILES16) {
+        if (ctx->variant[kernel_id] == CRK_VARIANT_TILES16) {
             if constexpr (S::kPair) {  // gravity stages: packed two-candidate sweeps
                 if (p.count)
                     pair_kernel_sub_pair<S, true><<<(unsigned)grid, kThreads, 0, ctx->stream>>>(v, p, rec, part);
@@ -3228,14 +3147,11 @@ int run_stage(crk_ctx *ctx, const crk_leaves *lv, typename S::P p, bool gas_pair
                 pair_kernel_sub<S, 8, true><<<(unsigned)grid, kThreads, 0, ctx->stream>>>(v, p, rec, part);
             else
                 pair_kernel_sub<S, 8, false><<<(unsigned)grid, kThreads, 0, ctx->stream>>>(v, p, rec, part);
-        } else if (S::kPair && ctx->warps[kernel_id] == 2) {
-            if constexpr (S::kPair) {  // two warps per i-leaf (persistent: twice the blocks per SM)
-                const unsigned g2 = (unsigned)(persistent ? std::min<int64_t>(lv->n_leaves, 2 * grid) : grid);
-                if (p.count)
-                    pair_kernel<S, true, 2><<<g2, 64, 0, ctx->stream>>>(v, p, rec, part);
-                else
-                    pair_kernel<S, false, 2><<<g2, 64, 0, ctx->stream>>>(v, p, rec, part);
-            }
+        } else if constexpr (S::kPair) {
+            const bool one = ctx->variant[kernel_id] == CRK_VARIANT_SPLIT8;
+            const int w = ctx->warps[kernel_id];
+            if (p.count) launch_cells<S, true>(ctx, lv, v, p, rec, persistent, w, one);
+            else launch_cells<S, false>(ctx, lv, v, p, rec, persistent, w, one);
         } else if (p.count) {
             pair_kernel<S, true><<<(unsigned)grid, kThreads, 0, ctx->stream>>>(v, p, rec, part);
         } else {
@@ -3449,7 +3365,7 @@ static int build_lists(crk_ctx *ctx, crk_leaves *lv, crk_nlist &out, bool reuse)
     CRK_CUDA(ctx, cudaMemcpyAsync(dgroups, tot, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     LeafView v{lv->leaf_start, lv->leaf_ngas, lv->bbox, lv->hmax, kGas ? lv->pos : lv->pos_g,
                kGas ? lv->kperm : lv->kperm_g, kGas ? lv->himg_start : lv->gimg_start,
-               kGas ? lv->himg_cnt : lv->gimg_cnt, kGas ? lv->himg : lv->gimg, nl, nullptr, 0, 32};
+               kGas ? lv->himg_cnt : lv->gimg_cnt, kGas ? lv->himg : lv->gimg, nl, nullptr, 0, 32, nullptr};
     const RecView<typename LS::Rec> rec{v.pos, n};  // a list record is the position and h
     const float rc2 = lv->r_cut_grav * lv->r_cut_grav;
     const int capr = kGasListCapRows, capt = kGasTableCap;
@@ -3630,8 +3546,7 @@ int grav_short_noalloc(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params
     // every record is rewritten before it is read, so nothing needs clearing
     gather_kernel<GravStage><<<crk_grid(n, 256), 256, 0, ctx->stream>>>(n, lv->pos_g, lv->kperm_g, p, base, 0);
     LeafView v{lv->leaf_start, lv->leaf_ngas, lv->bbox, lv->hmax, lv->pos_g, lv->kperm_g, lv->gimg_start,
-               lv->gimg_cnt, lv->gimg, lv->n_leaves, nullptr, 0, 32};
-    const int64_t grid = lv->n_leaves < 1 ? 1 : lv->n_leaves;
+               lv->gimg_cnt, lv->gimg, lv->n_leaves, nullptr, 0, 32, lv->gcell};
     const crk_nlist &nls = lv->grav_lists;
     if (nls.list && ctx->variant[CRK_K_GRAVITY] == CRK_VARIANT_LISTS) {
         GasLists gl{nls.gstart, nls.goff, nls.cnt, nls.list, nls.uoff, nls.unum, nls.ucode, nls.gleaf, nls.groups,
@@ -3640,7 +3555,7 @@ int grav_short_noalloc(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params
         list_kernel<GravStage, false><<<(unsigned)(lgrid > 0 ? lgrid : 1), kThreads,
                                         list_kernel_smem<GravStage, false>(), ctx->stream>>>(v, p, rec, gl, nullptr);
     } else {
-        pair_kernel<GravStage, false><<<(unsigned)grid, kThreads, 0, ctx->stream>>>(v, p, rec, nullptr);
+        launch_cells<GravStage, false>(ctx, lv, v, p, rec, false, 4, false);
     }
     ctx->launches += 2;
     return cudaGetLastError() == cudaSuccess ? CRK_OK : CRK_ECUDA;
