@@ -13,6 +13,7 @@
 // tree depends on n alone, so the host precomputes every level's segments.
 #include <algorithm>
 #include <chrono>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 
@@ -1844,7 +1845,19 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             for (int q = 0; q < 8; ++q) ALLOC(se[q], int32_t, nl);
             // the list cursors live with the leaves (a rebuild refreshes the counts from them later)
             unsigned long long *cur = (unsigned long long *)(lv->dev + 16);
-            int64_t cap[4] = {48 * nl + 64, 32 * nl + 64, 48 * nl + 64, 32 * nl + 64};
+            // first capacities: 1.5 times the leaves of the mean size within the cut of one (clustered
+            // boxes hold 34 images a leaf and list, cubes of 128 particles at r_c = 3 an estimated 38),
+            // the hydro cut taken at the largest h but at most 128 a leaf
+            double vol = 0.0;
+            for (float side : box_side) vol += (double)side * side * side;
+            const double ls = nl > 0 ? cbrt(vol / (double)nl) : 1.0;
+            auto images = [&](double cut, double most) {
+                const double w = 2.0 * ls;  // leaf boxes nearer than cut: Minkowski sum of two leaves and a ball
+                const double v = w * w * w + 6.0 * w * w * cut + 9.42 * w * cut * cut + 4.19 * cut * cut * cut;
+                return nl * (int64_t)std::min(most, 1.5 * v / (ls * ls * ls) + 16.0) + 64;
+            };
+            const int64_t cg = images((double)lp->r_cut_grav, (double)kCandCap), ch = images(2.0 * lv->hmax_all, 128.0);
+            int64_t cap[4] = {cg, cg, ch, ch};
             if (re)
                 for (int k = 0; k < 4; ++k) cap[k] = lv->img_cap[k];
             crk_image *gimg = lv->gimg, *himg = lv->himg;
