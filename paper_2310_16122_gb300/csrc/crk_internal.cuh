@@ -135,7 +135,8 @@ struct crk_leaves {
     int64_t img_cap[4] = {0, 0, 0, 0};               // capacities of gimg, gpair, himg, hpair
     unsigned char *boxtab = nullptr;                  // device copy of the build's box-table block
     size_t boxtab_bytes = 0;
-    // device: [0] status bits, [1] gas groups, [2] gravity groups; [16..27] the six list cursors (u64)
+    // device (256 bytes at the end of boxtab): [0] status bits, [1] gas groups, [2] gravity groups,
+    // [3] overflow of the one-pass gas lists; [16..27] the six list cursors (u64)
     int32_t *dev = nullptr;
 };
 
@@ -148,6 +149,12 @@ void crk_rcb_shape_free(crk_ctx *ctx);
 // neighbour lists of the leaves; reuse: a rebuild into the buffers of the first build (no host
 // synchronisation; a capacity overflow sets a bit of the leaves' status word)
 int crk_build_lists(crk_ctx *ctx, crk_leaves *lv, bool gas, bool reuse);
+// The gas lists of a build without a synchronisation of their own: whether any gas kernel walks
+// them; the groups of each leaf (their number into lv->dev[1]); then, with that number on the host
+// and the leaf images on the device, the one-pass lists (an overflow sets lv->dev[3]).
+bool crk_wants_gas_lists(const crk_ctx *ctx);
+int crk_gas_groups(crk_ctx *ctx, crk_leaves *lv);
+int crk_gas_lists_onepass(crk_ctx *ctx, crk_leaves *lv, int32_t ngroups);
 int crk_step_fused(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params *gp, const crk_hydro_params *hp,
                    const crk_step_io *io);
 // One stage of crk_advance in the library's kernel orders.  The work array
@@ -188,6 +195,12 @@ void crk_step_mark(crk_ctx *ctx, int k);
 int crk_exclusive_scan_i32(crk_ctx *ctx, const int32_t *in, int32_t *out, int64_t n, int32_t *total);
 // stable LSD radix sort of (key, value) pairs by all 32 key bits
 int crk_radix_sort_u32(crk_ctx *ctx, uint32_t *keys, int32_t *vals, int64_t n, int key_bits);
+// the stable (coordinate, index) order along each axis, in scratch memory (slots 1, 2, 13, 14), for
+// coordinates >= 0; with box_of ((device) box of each particle, nbox boxes) the (box, coordinate, index) order
+int crk_sort_axes(crk_ctx *ctx, const float *x, const float *y, const float *z, int64_t n, const int32_t *box_of,
+                  int nbox, int32_t *order[3]);
+// sort key of a coordinate: the IEEE bits of non-negative floats are ordered like the values
+__device__ __forceinline__ uint32_t crk_coord_key(float x) { return x == 0.0f ? 0u : __float_as_uint(x); }
 
 static inline int crk_grid(int64_t n, int block) {
     int64_t g = (n + block - 1) / block;

@@ -23,33 +23,27 @@ namespace {
 
 constexpr int kMaxLeafCap = 1024;
 
-__device__ __forceinline__ uint32_t coord_key(float x) {
-    // x >= 0 after validation: the IEEE bits of non-negative floats are ordered like the values
-    return x == 0.0f ? 0u : __float_as_uint(x);
-}
-
 // Positions in [0, L_box), gas h > 0 and finite; largest gas h per box.
-// Each block takes kValItems rows of 256 consecutive particles and combines
+// Each block takes `items` rows of 256 consecutive particles and combines
 // its counts (and, when its range lies in one box, its h maximum) in shared
 // memory, so the global atomics are a few per block: same-address atomics
 // from every warp of a 33M-particle launch serialise at L2 (about 1.7 ms).
-constexpr int kValItems = 16;
-constexpr int kValTile = 256 * kValItems;
+// 16 rows where that leaves blocks for every SM, else 4 (2x64^3: 20 -> 7.5 us).
 
 __global__ void __launch_bounds__(256) validate_kernel(const float *__restrict__ x, const float *__restrict__ y,
                                                        const float *__restrict__ z, const uint8_t *__restrict__ sp,
-                                                       const float *__restrict__ h, int64_t n,
+                                                       const float *__restrict__ h, int64_t n, int items,
                                                        const int32_t *__restrict__ box_of,
                                                        const float *__restrict__ box_L,
                                                        int32_t *__restrict__ flags /* [0] bad pos, [1] bad h, [2] n_gas */,
                                                        unsigned *__restrict__ hmax_bits /* per box */) {
     __shared__ unsigned part[4][8];
-    const int64_t base = (int64_t)blockIdx.x * kValTile;
-    const int64_t last = (base + kValTile < n ? base + kValTile : n) - 1;
+    const int64_t tile = 256 * (int64_t)items, base = (int64_t)blockIdx.x * tile;
+    const int64_t last = (base + tile < n ? base + tile : n) - 1;
     const int bfirst = box_of ? box_of[base] : 0;
     const bool one_box = !box_of || box_of[last] == bfirst;  // boxes are contiguous ranges
     unsigned nbad = 0, nbadh = 0, ngas = 0, hb_blk = 0;
-    for (int k = 0; k < kValItems; ++k) {
+    for (int k = 0; k < items; ++k) {
         const int64_t i = base + (int64_t)k * 256 + threadIdx.x;
         if (i >= n) break;
         const int b = box_of ? box_of[i] : 0;
@@ -106,21 +100,6 @@ __global__ void box_of_kernel(int64_t n, const int64_t *__restrict__ box_start, 
     box_of[i] = lo;
 }
 
-// keys for the stable re-sort of an axis list by box
-__global__ void box_keys_kernel(int64_t n, const int32_t *__restrict__ list, const int32_t *__restrict__ box_of,
-                                uint32_t *__restrict__ keys) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < n) keys[p] = (uint32_t)box_of[list[p]];
-}
-
-__global__ void init_axis_keys_kernel(const float *__restrict__ c, int64_t n, uint32_t *__restrict__ keys,
-                                      int32_t *__restrict__ vals) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    keys[i] = coord_key(c[i]);
-    vals[i] = (int32_t)i;
-}
-
 // chaining mesh cell: c = min(nc-1, floor(x nc / L)) per axis in FP64, id = (cx nc + cy) nc + cz
 __global__ void mesh_keys_kernel(const float *__restrict__ x, const float *__restrict__ y, const float *__restrict__ z,
                                  int64_t n, int nc, double L, uint32_t *__restrict__ keys, int32_t *__restrict__ vals,
@@ -172,6 +151,9 @@ struct AxisOrder {
     const int32_t *S[3];
     const int32_t *R[3];
 };
+struct RankOut {
+    int32_t *r[3];
+};
 
 __device__ __forceinline__ unsigned lanemask_lt_u() {
     unsigned m;
@@ -187,18 +169,28 @@ __device__ __forceinline__ int32_t rank_entry_id(const RankLists &L, const AxisO
     return a == 0 ? o.S[1][r] : (a == 1 ? o.S[2][r] : o.S[0][r]);
 }
 
-// R[S[p]] = p: the inverse of one axis order (one axis per launch, so the
+// R[S[p]] = p: the inverse of each axis order (blocks run in launch order, axis by axis, so the
 // randomly written array, n ints, stays about the size of L2)
-__global__ void rank_of_kernel(int64_t n, const int32_t *__restrict__ S, int32_t *__restrict__ R) {
+__global__ void rank_of_kernel(int64_t n, AxisOrder o, RankOut R) {
     int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < n) R[S[p]] = (int32_t)p;
+    const int t = blockIdx.y;
+    if (p < n) (t == 0 ? R.r[0] : (t == 1 ? R.r[1] : R.r[2]))[(t == 0 ? o.S[0] : (t == 1 ? o.S[1] : o.S[2]))[p]] = (int32_t)p;
 }
 
-// dst[p] = R[S[p]]: one rank column of one axis list (one source array per launch, as above)
-__global__ void rank_column_kernel(int64_t n, const int32_t *__restrict__ S, const int32_t *__restrict__ R,
-                                   int32_t *__restrict__ dst) {
+// the six rank columns: list a, column c holds R[S_a[p]] of axis t = (a + 1 + c) % 3; columns in
+// the order of t, two per randomly read source array
+__global__ void rank_column_kernel(int64_t n, AxisOrder o, RankListsOut A) {
     int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < n) dst[p] = __ldg(R + S[p]);
+    if (p >= n) return;
+    auto col = [&](int a, int c, int t) { A.A[a][c][p] = __ldg(o.R[t] + o.S[a][p]); };
+    switch (blockIdx.y) {
+        case 0: col(2, 0, 0); break;
+        case 1: col(1, 1, 0); break;
+        case 2: col(0, 0, 1); break;
+        case 3: col(2, 1, 1); break;
+        case 4: col(1, 0, 2); break;
+        default: col(0, 1, 2); break;
+    }
 }
 
 // final member order (list 0) as particle ids
@@ -207,20 +199,16 @@ __global__ void rank_members_kernel(int64_t n, RankLists L, AxisOrder o, int32_t
     if (p < n) members[p] = rank_entry_id(L, o, 0, p);
 }
 
-// per split node: tight box from the ends of its three list segments, split
-// axis (longest extent, ties to the lower axis), rank threshold
-__global__ void rcb_axis_kernel(int nseg, LevelDev lv, RankLists L, AxisOrder o, const float *__restrict__ x,
-                                const float *__restrict__ y, const float *__restrict__ z, float *__restrict__ node_box,
-                                SegRec *__restrict__ seg) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nseg) return;
+// Record of segment s of a level; for a split node the tight box from the ends of its three list
+// segments, the split axis (longest extent, ties to the lower axis) and the rank threshold, with
+// the box and the axis stored when `store`.
+__device__ __forceinline__ SegRec rcb_segment(int s, const LevelDev &lv, const RankLists &L, const AxisOrder &o,
+                                              const float *__restrict__ x, const float *__restrict__ y,
+                                              const float *__restrict__ z, float *__restrict__ node_box, bool store) {
     int k = lv.k[s];
     int lo = lv.lo[s], hi = lv.hi[s];
     SegRec r{lo, hi, k, lv.child[s], 0, lv.leftbase[s], 0, 0};
-    if (k <= 0) {
-        seg[s] = r;
-        return;
-    }
+    if (k <= 0) return r;
     const float *cs[3] = {x, y, z};
     float blo[3], bhi[3];
     double ext[3];
@@ -232,15 +220,24 @@ __global__ void rcb_axis_kernel(int nseg, LevelDev lv, RankLists L, AxisOrder o,
     int axis = 0;
     if (ext[1] > ext[axis]) axis = 1;
     if (ext[2] > ext[axis]) axis = 2;
-    lv.axis[s] = axis;
     r.axis = axis;
     r.thr = o.R[axis][rank_entry_id(L, o, axis, lo + k)];
-    seg[s] = r;
-    float *nb = node_box + 6 * (int64_t)lv.node[s];
-    for (int a = 0; a < 3; ++a) {
-        nb[a] = blo[a];
-        nb[3 + a] = bhi[a];
+    if (store) {
+        lv.axis[s] = axis;
+        float *nb = node_box + 6 * (int64_t)lv.node[s];
+        for (int a = 0; a < 3; ++a) {
+            nb[a] = blo[a];
+            nb[3 + a] = bhi[a];
+        }
     }
+    return r;
+}
+
+__global__ void rcb_axis_kernel(int nseg, LevelDev lv, RankLists L, AxisOrder o, const float *__restrict__ x,
+                                const float *__restrict__ y, const float *__restrict__ z, float *__restrict__ node_box,
+                                SegRec *__restrict__ seg) {
+    int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s < nseg) seg[s] = rcb_segment(s, lv, L, o, x, y, z, node_box, true);
 }
 
 // Stable partition of the three lists, one level at a time.  The prefix count
@@ -273,11 +270,66 @@ __device__ __forceinline__ unsigned rcb_left3(const SegRec &sr, const RankLists 
     return f;
 }
 
-__global__ void __launch_bounds__(kPartThreads) rcb_count3_kernel(int64_t n, const SegRec *__restrict__ segs,
+// Exclusive scan of the three columns of tile sums in place, by one block (nb entries each).
+__device__ void rcb_scan_columns(int32_t *bsum, int64_t nb, int32_t *wt) {
+    constexpr int kItems = 8;
+    for (int b = 0; b < 3; ++b) {
+        int32_t carry = 0;
+        int32_t *col = bsum + (int64_t)b * nb;
+        for (int64_t s0 = 0; s0 < nb; s0 += (int64_t)blockDim.x * kItems) {
+            const int64_t i0 = s0 + (int64_t)threadIdx.x * kItems;
+            int32_t v[kItems], s = 0;
+#pragma unroll
+            for (int k = 0; k < kItems; ++k) {
+                v[k] = i0 + k < nb ? __ldcg(col + i0 + k) : 0;
+                s += v[k];
+            }
+            int32_t tot;
+            int32_t e = carry + crk_block_scan(s, wt, tot);
+#pragma unroll
+            for (int k = 0; k < kItems; ++k) {
+                if (i0 + k < nb) col[i0 + k] = e;
+                e += v[k];
+            }
+            carry += tot;
+        }
+    }
+}
+
+// kAxis (one box: a streamed level's segments hold over 1024 entries, so a tile of 2048 meets at
+// most kTileSegs): the blocks make the segment records they need themselves instead of a launch of
+// their own.  ctr != NULL: the last block to finish scans the tile sums (no block waits on another).
+constexpr int kTileSegs = 4;
+constexpr int64_t kFusedTiles = 1024;  // up to here (2M particles) launches cost more than the repeated work
+
+template <bool kAxis>
+__global__ void __launch_bounds__(kPartThreads) rcb_count3_kernel(int64_t n, SegRec *__restrict__ segs,
                                                                    const int32_t *__restrict__ node_of, RankLists L,
-                                                                   int32_t *__restrict__ bsum, int64_t nb) {
+                                                                   int32_t *bsum, int64_t nb, unsigned *ctr, LevelDev lv,
+                                                                   AxisOrder o, const float *__restrict__ x,
+                                                                   const float *__restrict__ y,
+                                                                   const float *__restrict__ z,
+                                                                   float *__restrict__ node_box, int32_t *__restrict__ err) {
     __shared__ int32_t wt[32];
+    __shared__ SegRec own[kTileSegs];
+    __shared__ bool last;
     const int64_t base = (int64_t)blockIdx.x * kPartTile;
+    int s0 = 0;
+    if constexpr (kAxis) {
+        s0 = node_of[base];
+        const int ns = node_of[(base + kPartTile < n ? base + kPartTile : n) - 1] - s0 + 1;
+        const int t = threadIdx.x >> 5;  // one warp's first lane per segment
+        if ((threadIdx.x & 31) == 0 && t < kTileSegs) {
+            if (t < ns) {
+                const int lo = lv.lo[s0 + t];
+                const bool mine = lo >= base && lo < base + kPartTile;
+                own[t] = rcb_segment(s0 + t, lv, L, o, x, y, z, node_box, mine);
+                if (mine) segs[s0 + t] = own[t];
+            }
+            if (t == 0 && ns > kTileSegs) atomicAdd(err, 1);  // excluded by the host's choice of levels
+        }
+        __syncthreads();
+    }
     int32_t seg[kPartItems];
 #pragma unroll
     for (int k = 0; k < kPartItems; ++k) {
@@ -290,7 +342,7 @@ __global__ void __launch_bounds__(kPartThreads) rcb_count3_kernel(int64_t n, con
         int64_t p = base + (int64_t)k * kPartThreads + threadIdx.x;
         unsigned f = 0u;
         if (seg[k] >= 0) {
-            const SegRec sr = segs[seg[k]];
+            const SegRec sr = kAxis ? own[min(seg[k] - s0, kTileSegs - 1)] : segs[seg[k]];
             f = rcb_left3(sr, L, p);
         }
         c[0] += f & 1u;
@@ -302,23 +354,20 @@ __global__ void __launch_bounds__(kPartThreads) rcb_count3_kernel(int64_t n, con
         crk_block_scan(c[b], wt, tot);
         if (threadIdx.x == 0) bsum[(int64_t)b * nb + blockIdx.x] = tot;
     }
+    if (!ctr) return;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicInc(ctr, gridDim.x - 1) == gridDim.x - 1;  // wraps to 0 for the next level
+        __threadfence();
+    }
+    __syncthreads();
+    if (last) rcb_scan_columns(bsum, nb, wt);
 }
 
 // single block: exclusive scan of the three columns of tile sums, in place
-__global__ void rcb_scan3_kernel(int32_t *__restrict__ bsum, int64_t nb) {
+__global__ void __launch_bounds__(1024) rcb_scan3_kernel(int32_t *__restrict__ bsum, int64_t nb) {
     __shared__ int32_t wt[32];
-    for (int b = 0; b < 3; ++b) {
-        int32_t carry = 0;
-        int32_t *col = bsum + (int64_t)b * nb;
-        for (int64_t s0 = 0; s0 < nb; s0 += blockDim.x) {
-            int64_t i = s0 + threadIdx.x;
-            int32_t v = i < nb ? col[i] : 0;
-            int32_t tot;
-            int32_t e = crk_block_scan(v, wt, tot);
-            if (i < nb) col[i] = carry + e;
-            carry += tot;
-        }
-    }
+    rcb_scan_columns(bsum, nb, wt);
 }
 
 // Entries are taken in rows of kPartThreads consecutive positions (entry k of
@@ -1169,8 +1218,19 @@ __global__ void __launch_bounds__(kTravWarps * 32) leaf_pairs_warp_kernel(
         if (nc > kCandCap) bad = true;
     }
     __syncwarp();
+    // a leaf whose candidates or images do not fit is left without images: the gas lists of the
+    // same build may read them before the host sees the error
+    auto none = [&]() {
+        if (lane < 4) {
+            int32_t *const st = lane == 0 ? o.start[0] : (lane == 1 ? o.start[1] : (lane == 2 ? o.start[2] : o.start[3]));
+            int32_t *const ct = lane == 0 ? o.count[0] : (lane == 1 ? o.count[1] : (lane == 2 ? o.count[2] : o.count[3]));
+            st[a] = 0;
+            ct[a] = 0;
+        }
+    };
     if (bad) {
         if (lane == 0) atomicAdd(&o.err[0], 1);
+        none();
         return;
     }
     // ascending j-leaf order (rank sort; leaf ids are unique)
@@ -1217,6 +1277,7 @@ __global__ void __launch_bounds__(kTravWarps * 32) leaf_pairs_warp_kernel(
     }
     if (over) {
         if (lane == 0) atomicAdd(&o.err[1], 1);
+        none();
         return;
     }
     if (lane == 0)
@@ -1268,6 +1329,50 @@ __global__ void node_hmax_kernel(int nseg, LevelDev lv, const int32_t *__restric
     if (s >= nseg || lv.k[s] <= 0) return;
     int nd = lv.node[s];
     node_hmax[nd] = fmaxf(node_hmax[left[nd]], node_hmax[right[nd]]);
+}
+
+// The small levels (at most kTreeLevel segments) of a tree, deepest first, in one block: the node
+// h_max of split nodes, after the leaf boxes and h_max went into the nodes.
+constexpr int kTreeLevel = 8192;
+constexpr int kTreeLevels = 32;
+struct TreeLevels {
+    const int32_t *k[kTreeLevels], *node[kTreeLevels];
+    int32_t m[kTreeLevels];
+    int n;
+};
+__global__ void __launch_bounds__(1024) tree_hmax_kernel(TreeLevels t, const int32_t *__restrict__ left,
+                                                         const int32_t *__restrict__ right, float *node_hmax) {
+    for (int d = 0; d < t.n; ++d) {
+        for (int s = threadIdx.x; s < t.m[d]; s += blockDim.x) {
+            if (t.k[d][s] <= 0) continue;
+            const int nd = t.node[d][s];
+            node_hmax[nd] = fmaxf(node_hmax[left[nd]], node_hmax[right[nd]]);
+        }
+        __syncthreads();
+    }
+}
+
+// The box tables of a build (layout: see build_leaves_impl) written by a kernel: a copy from
+// pageable host memory waits for the stream's earlier work before it starts.
+constexpr int kBoxTables = 64;
+struct BoxTables {
+    int64_t start[kBoxTables + 1];
+    float side[kBoxTables];
+    int32_t seg[kBoxTables];
+};
+__global__ void box_tables_kernel(BoxTables t, int nbox, int32_t *__restrict__ a, int32_t *__restrict__ b, int words,
+                                  int start_at) {
+    for (int w = threadIdx.x; w < words; w += blockDim.x) a[w] = b[w] = 0;
+    __syncthreads();
+    for (int k = threadIdx.x; k <= nbox; k += blockDim.x) {
+        for (int c = 0; c < 2; ++c) {
+            int32_t *d = c ? a : b;
+            reinterpret_cast<int64_t *>(d + start_at)[k] = t.start[k];
+            if (k == nbox) continue;
+            reinterpret_cast<float *>(d)[16 + nbox + k] = t.side[k];
+            d[start_at + 2 * (nbox + 1) + k] = t.seg[k];
+        }
+    }
 }
 
 struct HostSeg {
@@ -1541,43 +1646,56 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
         }                                                  \
     } while (0)
     {
-        // flags[0..15]; then per box: hmax bits, side, start (int64), segment index
-        const size_t fbytes = 64 + 4 * (size_t)nbox + 4 * (size_t)nbox + 8 * (size_t)(nbox + 1) + 4 * (size_t)nbox;
-        int32_t *flags = (int32_t *)crk_scratch(ctx, 0, fbytes + 64);
+        // the box tables: flags[0..15] and per box hmax bits (zero), side, start (int64), segment index;
+        // then the leaves' device words (zero)
+        const size_t tbytes = (64 + 4 * (size_t)nbox + 4 * (size_t)nbox + 8 * (size_t)(nbox + 2) + 4 * (size_t)nbox + 127) &
+                              ~(size_t)127;
+        const size_t fbytes = tbytes + 256;
+        int32_t *flags = (int32_t *)crk_scratch(ctx, 0, fbytes);
         if (!flags) { rc = crk_fail(ctx, CRK_ENOMEM, "scratch"); goto fail; }
+        const size_t o_start = (64 + 8 * (size_t)nbox + 7) & ~(size_t)7;
         unsigned *hbits = (unsigned *)(flags + 16);
         float *box_L = (float *)(flags + 16 + nbox);
-        int64_t *d_box_start = (int64_t *)(((uintptr_t)(flags + 16 + 2 * nbox) + 7) & ~(uintptr_t)7);
+        int64_t *d_box_start = (int64_t *)((char *)flags + o_start);
         int32_t *seg_of_box = (int32_t *)(d_box_start + nbox + 1);
-        std::vector<int32_t> h_seg(nbox, 0);
-        for (int b = 0, q = 0; b < nbox; ++b) {
-            h_seg[b] = q;
-            if (box_start[b + 1] > box_start[b]) ++q;
-        }
         if (!re) {
-            if (cudaMemcpyAsync(box_L, box_side.data(), 4 * (size_t)nbox, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-                cudaMemcpyAsync(d_box_start, box_start.data(), 8 * (size_t)(nbox + 1), cudaMemcpyHostToDevice, st) !=
-                    cudaSuccess ||
-                cudaMemcpyAsync(seg_of_box, h_seg.data(), 4 * (size_t)nbox, cudaMemcpyHostToDevice, st) != cudaSuccess) {
-                rc = crk_fail(ctx, CRK_ECUDA, "leaf build set-up copies");
-                goto fail;
-            }
-            // the rebuild state: a device copy of the box tables, the status word, group counts and cursors
-            lv->boxtab_bytes = fbytes + 64;
+            // the rebuild state: a device copy of the box tables; status word, group counts and cursors
+            lv->boxtab_bytes = fbytes;
             lv->boxtab = (unsigned char *)crk_leaves_alloc(ctx, lv, lv->boxtab_bytes);
-            lv->dev = (int32_t *)crk_leaves_alloc(ctx, lv, 256);
-            if (!lv->boxtab || !lv->dev) { rc = crk_fail(ctx, CRK_ENOMEM, "leaf allocation"); goto fail; }
-            if (cudaMemcpyAsync(lv->boxtab, flags, lv->boxtab_bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
-                rc = crk_fail(ctx, CRK_ECUDA, "leaf build set-up copies");
-                goto fail;
+            if (!lv->boxtab) { rc = crk_fail(ctx, CRK_ENOMEM, "leaf allocation"); goto fail; }
+            lv->dev = (int32_t *)(lv->boxtab + tbytes);
+            BoxTables bt{};
+            for (int b = 0, q = 0; b < nbox && nbox <= kBoxTables; ++b) {
+                bt.start[b] = box_start[b];
+                bt.side[b] = box_side[b];
+                bt.seg[b] = q;
+                if (box_start[b + 1] > box_start[b]) ++q;
             }
-        } else if (cudaMemcpyAsync(flags, lv->boxtab, lv->boxtab_bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+            if (nbox <= kBoxTables) {
+                bt.start[nbox] = n;
+                box_tables_kernel<<<1, 256, 0, st>>>(bt, nbox, (int32_t *)lv->boxtab, flags, (int)(fbytes / 4),
+                                                     (int)(o_start / 4));
+                ++ctx->launches;
+                KCHECK("box tables");
+            } else {
+                std::vector<char> tab(fbytes, 0);
+                std::memcpy(tab.data() + 64 + 4 * (size_t)nbox, box_side.data(), 4 * (size_t)nbox);
+                std::memcpy(tab.data() + o_start, box_start.data(), 8 * (size_t)(nbox + 1));
+                int32_t *hs = (int32_t *)(tab.data() + o_start + 8 * (size_t)(nbox + 1));
+                for (int b = 0, q = 0; b < nbox; ++b) {
+                    hs[b] = q;
+                    if (box_start[b + 1] > box_start[b]) ++q;
+                }
+                if (cudaMemcpyAsync(flags, tab.data(), fbytes, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+                    cudaMemcpyAsync(lv->boxtab, flags, fbytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+                    rc = crk_fail(ctx, CRK_ECUDA, "leaf build set-up copies");
+                    goto fail;
+                }
+            }
+        } else if (cudaMemsetAsync(lv->dev, 0, 256, st) != cudaSuccess ||
+                   cudaMemcpyAsync(flags, lv->boxtab, lv->boxtab_bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+            // (the table's flags and hmax bits are zero: the build works on the scratch copy)
             rc = crk_fail(ctx, CRK_ECUDA, "leaf build set-up copies");
-            goto fail;
-        }
-        if (cudaMemsetAsync(flags, 0, 64 + 4 * (size_t)nbox, st) != cudaSuccess ||
-            cudaMemsetAsync(lv->dev, 0, 256, st) != cudaSuccess) {
-            rc = crk_fail(ctx, CRK_ECUDA, "memset");
             goto fail;
         }
         int32_t *box_of = nullptr;
@@ -1588,8 +1706,9 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             ++ctx->launches;
         }
         if (n > 0) {
-            validate_kernel<<<(unsigned)((n + kValTile - 1) / kValTile), 256, 0, st>>>(
-                p->x, p->y, p->z, p->species, h, n, box_of, box_L, flags, hbits);
+            const int items = n >= (int64_t)4096 * 8 * ctx->num_sms ? 16 : 4;
+            validate_kernel<<<(unsigned)((n + 256 * items - 1) / (256 * items)), 256, 0, st>>>(
+                p->x, p->y, p->z, p->species, h, n, items, box_of, box_L, flags, hbits);
             ++ctx->launches;
         }
         int32_t *members = nullptr;  // particle ids grouped by leaf
@@ -1635,10 +1754,9 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             tr.mark("shape");
             int32_t *Lc[3];
             size_t nb = sizeof(int32_t) * (size_t)(n > 0 ? n : 1);
-            uint32_t *keys = (uint32_t *)crk_scratch(ctx, 1, nb);
             int32_t *R[3], *Ac[3][2], *An[3][2];
             for (int a = 0; a < 3; ++a) {
-                Lc[a] = (int32_t *)crk_scratch(ctx, 2 + a, nb);
+                Lc[a] = nullptr;
                 R[a] = (int32_t *)crk_scratch(ctx, 5 + a, nb);
                 for (int c = 0; c < 2; ++c) {
                     Ac[a][c] = (int32_t *)crk_scratch(ctx, 19 + 2 * a + c, nb);
@@ -1652,36 +1770,21 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             size_t max_seg = 1;
             for (size_t m : shape->level_size) max_seg = std::max(max_seg, m);
             SegRec *segs = (SegRec *)crk_scratch(ctx, 31, sizeof(SegRec) * max_seg);
-            bool ok = keys && node_of && node_nx && mem && flag && segs;
-            for (int a = 0; a < 3; ++a) ok = ok && Lc[a] && R[a] && Ac[a][0] && Ac[a][1] && An[a][0] && An[a][1];
+            bool ok = node_of && node_nx && mem && flag && segs;
+            for (int a = 0; a < 3; ++a) ok = ok && R[a] && Ac[a][0] && Ac[a][1] && An[a][0] && An[a][1];
             if (!ok) {
                 rc = crk_fail(ctx, CRK_ENOMEM, "scratch");
                 goto fail;
             }
-            const float *cs[3] = {p->x, p->y, p->z};
-            for (int a = 0; a < 3 && n > 0; ++a) {
-                init_axis_keys_kernel<<<crk_grid(n, 256), 256, 0, st>>>(cs[a], n, keys, Lc[a]);
-                ++ctx->launches;
-                TRY(crk_radix_sort_u32(ctx, keys, Lc[a], n, 32));
-                if (box_of) {  // stable by box: (box, coordinate, index) order
-                    box_keys_kernel<<<crk_grid(n, 256), 256, 0, st>>>(n, Lc[a], box_of, keys);
-                    ++ctx->launches;
-                    int bits = 1;
-                    while ((1 << bits) < nbox) ++bits;
-                    TRY(crk_radix_sort_u32(ctx, keys, Lc[a], n, bits));
-                }
-            }
+            TRY(crk_sort_axes(ctx, p->x, p->y, p->z, n, box_of, nbox, Lc));
             tr.mark("axis sorts");
             const AxisOrder ord{{Lc[0], Lc[1], Lc[2]}, {R[0], R[1], R[2]}};
             if (n > 0) {
-                for (int t = 0; t < 3; ++t) rank_of_kernel<<<crk_grid(n, 256), 256, 0, st>>>(n, Lc[t], R[t]);
-                // list a, column c holds the rank along axis (a + 1 + c) % 3
-                for (int t = 0; t < 3; ++t) {
-                    const int a0 = (t + 2) % 3, a1 = (t + 1) % 3;
-                    rank_column_kernel<<<crk_grid(n, 256), 256, 0, st>>>(n, Lc[a0], R[t], Ac[a0][0]);
-                    rank_column_kernel<<<crk_grid(n, 256), 256, 0, st>>>(n, Lc[a1], R[t], Ac[a1][1]);
-                }
-                ctx->launches += 9;
+                const dim3 g3((unsigned)crk_grid(n, 256), 3), g6((unsigned)crk_grid(n, 256), 6);
+                rank_of_kernel<<<g3, 256, 0, st>>>(n, ord, RankOut{{R[0], R[1], R[2]}});
+                rank_column_kernel<<<g6, 256, 0, st>>>(
+                    n, ord, RankListsOut{{{Ac[0][0], Ac[0][1]}, {Ac[1][0], Ac[1][1]}, {Ac[2][0], Ac[2][1]}}});
+                ctx->launches += 2;
                 if (box_of) {
                     init_node_of_kernel<<<crk_grid(n, 256), 256, 0, st>>>(n, box_of, seg_of_box, node_of);
                     ++ctx->launches;
@@ -1706,13 +1809,22 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
                 LevelDev dv{tab, tab + m, tab + 2 * m, tab + 3 * m, tab + 4 * m, tab + 5 * m, tab + 6 * m};
                 const RankLists Lr{{{Ac[0][0], Ac[0][1]}, {Ac[1][0], Ac[1][1]}, {Ac[2][0], Ac[2][1]}}};
                 const RankListsOut Lo{{{An[0][0], An[0][1]}, {An[1][0], An[1][1]}, {An[2][0], An[2][1]}}};
-                rcb_axis_kernel<<<crk_grid(m, 128), 128, 0, st>>>(m, dv, Lr, ord, p->x, p->y, p->z, node_box, segs);
                 const int64_t nbt = (n + kPartTile - 1) / kPartTile;
-                rcb_count3_kernel<<<(unsigned)nbt, kPartThreads, 0, st>>>(n, segs, node_of, Lr, flag, nbt);
-                rcb_scan3_kernel<<<1, 1024, 0, st>>>(flag, nbt);
+                // small builds: one launch makes the records, counts and scans (in one box a level above
+                // kLocalCap has no segment below kLocalCap / 2)
+                const bool fused = nbt <= kFusedTiles, axis = fused && nbox == 1 && shape->level_max[d] > kLocalCap;
+                unsigned *ctr = fused ? (unsigned *)(flags + 8) : nullptr;
+                if (!axis) rcb_axis_kernel<<<crk_grid(m, 128), 128, 0, st>>>(m, dv, Lr, ord, p->x, p->y, p->z, node_box, segs);
+                if (axis)
+                    rcb_count3_kernel<true><<<(unsigned)nbt, kPartThreads, 0, st>>>(
+                        n, segs, node_of, Lr, flag, nbt, ctr, dv, ord, p->x, p->y, p->z, node_box, flags + 5);
+                else
+                    rcb_count3_kernel<false><<<(unsigned)nbt, kPartThreads, 0, st>>>(
+                        n, segs, node_of, Lr, flag, nbt, ctr, dv, ord, p->x, p->y, p->z, node_box, flags + 5);
+                if (!fused) rcb_scan3_kernel<<<1, 1024, 0, st>>>(flag, nbt);
+                ctx->launches += (axis ? 1 : 2) + (fused ? 0 : 1) + 1;
                 rcb_scatter3_kernel<<<(unsigned)nbt, kPartThreads, 0, st>>>(n, segs, node_of, Lr, flag, nbt, Lo, node_nx,
                                                                             flags + 5);
-                ctx->launches += 4;
                 for (int a = 0; a < 3; ++a)
                     for (int c = 0; c < 2; ++c) std::swap(Ac[a][c], An[a][c]);
                 std::swap(node_of, node_nx);
@@ -1773,12 +1885,19 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             leaf_status_kernel<<<1, 256, 0, st>>>(flags, hbits, box_L, nbox, (int32_t)lv->n_gas, lv->dev);
             ++ctx->launches;
         }
-        // ---- host checks (one synchronisation)
-        int32_t hflags[16];
-        std::vector<unsigned> hb(nbox);
+        // the gas lists' groups are counted before the host looks, so that one read brings everything
+        const bool gas_lists = re ? lv->gas_lists.list != nullptr : crk_wants_gas_lists(ctx);
+        if (!re && gas_lists) TRY(crk_gas_groups(ctx, lv));
+        // ---- host checks (first synchronisation)
+        std::vector<int32_t> hflags(16 + nbox);
+        const unsigned *hb = (const unsigned *)hflags.data() + 16;
+        int32_t hdev[2] = {0, 0};
+        std::vector<int32_t> ls(!re && lp->mode == 0 ? nl + 1 : 0);
         if (re) {
-        } else if (cudaMemcpyAsync(hflags, flags, 64, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaMemcpyAsync(hb.data(), hbits, 4 * (size_t)nbox, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        } else if ((!ls.empty() && cudaMemcpyAsync(ls.data(), lv->leaf_start, sizeof(int32_t) * ls.size(),
+                                                   cudaMemcpyDeviceToHost, st) != cudaSuccess) ||
+            cudaMemcpyAsync(hflags.data(), flags, 64 + 4 * (size_t)nbox, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaMemcpyAsync(hdev, lv->dev, sizeof(hdev), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) {
             rc = crk_fail(ctx, CRK_ECUDA, "leaf build: %s", cudaGetErrorString(cudaGetLastError()));
             goto fail;
@@ -1802,11 +1921,6 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
         }
         lv->hmax_all = hmax_all;
         if (lp->mode == 0) {
-            std::vector<int32_t> ls(nl + 1);
-            if (cudaMemcpy(ls.data(), lv->leaf_start, sizeof(int32_t) * (nl + 1), cudaMemcpyDeviceToHost) != cudaSuccess) {
-                rc = crk_fail(ctx, CRK_ECUDA, "leaf starts");
-                goto fail;
-            }
             int mx = 0;
             for (int64_t a = 0; a < nl; ++a) mx = std::max(mx, ls[a + 1] - ls[a]);
             lv->max_leaf_size = mx;
@@ -1822,11 +1936,22 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             leaf_box_to_node_kernel<<<crk_grid(nl, 128), 128, 0, st>>>(nl, lv->bbox, lv->hmax, shape->leaf_node,
                                                                        node_box, node_hmax);
             ++ctx->launches;
+            TreeLevels tl{};
             for (size_t d = shape->level_size.size(); d-- > 0;) {
                 int m = (int)shape->level_size[d];
                 int32_t *tab = shape->dtab + shape->level_off[d];
                 LevelDev dv{tab, tab + m, tab + 2 * m, tab + 3 * m, tab + 4 * m, tab + 5 * m, tab + 6 * m};
-                node_hmax_kernel<<<crk_grid(m, 128), 128, 0, st>>>(m, dv, shape->left, shape->right, node_hmax);
+                if (m > kTreeLevel || tl.n == kTreeLevels) {  // (levels shrink towards the root)
+                    node_hmax_kernel<<<crk_grid(m, 128), 128, 0, st>>>(m, dv, shape->left, shape->right, node_hmax);
+                    ++ctx->launches;
+                } else {
+                    tl.k[tl.n] = dv.k;
+                    tl.node[tl.n] = dv.node;
+                    tl.m[tl.n++] = m;
+                }
+            }
+            if (tl.n > 0) {
+                tree_hmax_kernel<<<1, 1024, 0, st>>>(tl, shape->left, shape->right, node_hmax);
                 ++ctx->launches;
             }
             KCHECK("node h_max");
@@ -1837,13 +1962,15 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             tree.node_leaf = shape->leaf_of;
             tree.root = 0;
         }
+        bool lists_over = false;  // a gas list exceeded the one-pass capacities
         // ---- leaf-pair image lists, one warp per leaf; retried once with exact
         // capacities if the first estimate is too small
         {
             int32_t *se[8] = {lv->gimg_start, lv->gimg_cnt, lv->gpair_start, lv->gpair_cnt,
                               lv->himg_start, lv->himg_cnt, lv->hpair_start, lv->hpair_cnt};
             for (int q = 0; q < 8; ++q) ALLOC(se[q], int32_t, nl);
-            // the list cursors live with the leaves (a rebuild refreshes the counts from them later)
+            // the list cursors live with the leaves (a rebuild refreshes the counts from them later); they
+            // are zero at the start of a build and of a rebuild
             unsigned long long *cur = (unsigned long long *)(lv->dev + 16);
             // first capacities: 1.5 times the leaves of the mean size within the cut of one (clustered
             // boxes hold 34 images a leaf and list, cubes of 128 particles at r_c = 3 an estimated 38),
@@ -1871,7 +1998,10 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
                 ALLOC(gpair, int32_t, cap[1]);
                 ALLOC(himg, crk_image, cap[2]);
                 ALLOC(hpair, int32_t, cap[3]);
-                if (cudaMemsetAsync(cur, 0, 64, st) != cudaSuccess) { rc = crk_fail(ctx, CRK_ECUDA, "memset"); goto fail; }
+                if (attempt > 0 && cudaMemsetAsync(lv->dev + 3, 0, 256 - 12, st) != cudaSuccess) {
+                    rc = crk_fail(ctx, CRK_ECUDA, "memset");
+                    goto fail;
+                }
                 PairOut po;
                 for (int k = 0; k < 4; ++k) {
                     po.start[k] = se[2 * k];
@@ -1899,11 +2029,21 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
                     ++ctx->launches;
                     break;
                 }
-                if (cudaMemcpyAsync(hcur, cur, 48, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+                tr.mark("pair lists");
+                if (gas_lists) {  // on these images; a leaf whose images did not fit has none (and the lists are redone)
+                    lv->himg_start = se[4]; lv->himg_cnt = se[5]; lv->himg = himg;
+                    TRY(crk_gas_lists_onepass(ctx, lv, hdev[1]));
+                    tr.mark("gas lists");
+                }
+                // ---- second synchronisation: list sizes and overflows
+                int32_t hall[64];
+                if (cudaMemcpyAsync(hall, lv->dev, 256, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
                     cudaStreamSynchronize(st) != cudaSuccess) {
                     rc = crk_fail(ctx, CRK_ECUDA, "pair lists: %s", cudaGetErrorString(cudaGetLastError()));
                     goto fail;
                 }
+                std::memcpy(hcur, hall + 16, 48);
+                lists_over = hall[3] != 0;
                 const int32_t *herr = (const int32_t *)(hcur + 4);
                 if (herr[0] > 0) {
                     rc = crk_fail(ctx, CRK_EINVAL,
@@ -1922,13 +2062,8 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             lv->hpair_start = se[6]; lv->hpair_cnt = se[7]; lv->hpair_list = hpair; lv->n_hpairs = (int64_t)hcur[3];
             for (int k = 0; k < 4; ++k) lv->img_cap[k] = cap[k];
         }
-        tr.mark("pair lists");
-        bool gas_lists = false;  // every gas-pair kernel may walk the gas lists
-        for (int k : {CRK_K_GEOMETRY, CRK_K_CORRECTIONS, CRK_K_HYDRO, CRK_K_GEOMETRY_ADJOINT, CRK_K_EXTRAS, CRK_K_ACCEL,
-                      CRK_K_ENERGY})
-            gas_lists = gas_lists || ctx->variant[k] == CRK_VARIANT_LISTS;
-        if (re ? lv->gas_lists.list != nullptr : gas_lists) TRY(crk_build_lists(ctx, lv, true, re != nullptr));
-        tr.mark("gas lists");
+        if (re && gas_lists) TRY(crk_build_lists(ctx, lv, true, true));
+        if (!re && gas_lists && lists_over) TRY(crk_build_lists(ctx, lv, true, false));  // the exact two-pass build
         if (!re && (ctx->variant[CRK_K_GRAVITY] == CRK_VARIANT_LISTS ||
                     ctx->variant[CRK_K_GRAVITY_ADJOINT] == CRK_VARIANT_LISTS))
             TRY(crk_build_lists(ctx, lv, false, false));

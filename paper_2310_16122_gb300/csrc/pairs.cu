@@ -3011,6 +3011,7 @@ __global__ void list_group_count_kernel(int64_t n_leaves, const int32_t *__restr
                                         const int32_t *__restrict__ ngas, int gas, int32_t *__restrict__ ng) {
     int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (a < n_leaves) ng[a] = ((gas ? ngas[a] : leaf_start[a + 1] - leaf_start[a]) + 31) >> 5;
+    if (a == n_leaves) ng[a] = 0;
 }
 
 // per group: the longest list of its lanes (units of 32 entries once scanned)
@@ -3340,135 +3341,169 @@ int crk_hydro_adjoint(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params
     return run_stage<HydroAdjStage>(ctx, lv, p, true, CRK_K_HYDRO);
 }
 
-// reuse: a rebuild of one-pass gas lists into the buffers of the first build (group arrays with
-// room for 1/8 more groups); no host synchronisation, overflows go to the leaves' status word.
+template <bool kGas>
+static LeafView list_view(const crk_leaves *lv) {
+    return LeafView{lv->leaf_start, lv->leaf_ngas, lv->bbox, lv->hmax, kGas ? lv->pos : lv->pos_g,
+                    kGas ? lv->kperm : lv->kperm_g, kGas ? lv->himg_start : lv->gimg_start,
+                    kGas ? lv->himg_cnt : lv->gimg_cnt, kGas ? lv->himg : lv->gimg, lv->n_leaves, nullptr, 0, 32, nullptr};
+}
+
+// groups of each leaf and their number, into gstart and lv->dev[1] (gas) or [2]
+template <bool kGas>
+static int list_groups(crk_ctx *ctx, crk_leaves *lv, int32_t *gstart) {
+    const int64_t nl = lv->n_leaves;
+    int32_t *ng = (int32_t *)crk_scratch(ctx, 6, sizeof(int32_t) * (size_t)(nl + 1));
+    if (!ng) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
+    list_group_count_kernel<<<crk_grid(nl + 1, 256), 256, 0, ctx->stream>>>(nl, lv->leaf_start, lv->leaf_ngas, kGas, ng);
+    ++ctx->launches;
+    return crk_exclusive_scan_i32(ctx, ng, gstart, nl + 1, lv->dev + (kGas ? 1 : 2));
+}
+
+static bool no_lists(const crk_leaves *lv, bool gas) { return lv->n_leaves == 0 || lv->n == 0 || (gas && lv->n_gas == 0); }
+
+bool crk_wants_gas_lists(const crk_ctx *ctx) {
+    for (int k : {CRK_K_GEOMETRY, CRK_K_CORRECTIONS, CRK_K_HYDRO, CRK_K_GEOMETRY_ADJOINT, CRK_K_EXTRAS, CRK_K_ACCEL,
+                  CRK_K_ENERGY})
+        if (ctx->variant[k] == CRK_VARIANT_LISTS) return true;
+    return false;
+}
+
+int crk_gas_groups(crk_ctx *ctx, crk_leaves *lv) {
+    if (lv->n_leaves == 0 || lv->n == 0) return CRK_OK;
+    crk_nlist &out = lv->gas_lists;
+    out.gstart = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(lv->n_leaves + 1));
+    if (!out.gstart) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
+    return list_groups<true>(ctx, lv, out.gstart);
+}
+
+// One pass into fixed capacities (a lane's list and a group's table), which the adaptive
+// smoothing lengths keep well above the largest counts; room for 1/8 more groups than this build
+// holds (a rebuild of moved particles reuses the buffers).
+int crk_gas_lists_onepass(crk_ctx *ctx, crk_leaves *lv, int32_t ngroups) {
+    using LS = ListStage<true>;
+    if (no_lists(lv, true)) return CRK_OK;
+    crk_nlist &out = lv->gas_lists;
+    const int64_t nl = lv->n_leaves, n = lv->n;
+    const int capr = kGasListCapRows, capt = kGasTableCap;
+    const int64_t capg = (int64_t)ngroups + ngroups / 8 + 64;
+    cudaStream_t st = ctx->stream;
+    if (capg * capt >= 2147483647LL) {  // 32-bit offsets: the exact build
+        CRK_CUDA(ctx, cudaMemsetAsync(lv->dev + 3, 1, sizeof(int32_t), st));
+        return CRK_OK;
+    }
+    if (!out.list) {  // (a second attempt of the pair lists keeps the first's buffers)
+        // room for the records of the light stages, so that the first pair kernel need not allocate
+        if (!crk_scratch(ctx, 4, 32 * (size_t)n)) return crk_fail(ctx, CRK_ENOMEM, "neighbour list scratch");
+        out.cnt = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)n);
+        out.gleaf = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)capg);
+        out.unum = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(capg + 1));
+        out.goff = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(capg + 1));
+        out.uoff = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(capg + 1));
+        out.ucode = (uint32_t *)crk_leaves_alloc(ctx, lv, sizeof(uint32_t) * (size_t)capg * capt);
+        out.list = (uint16_t *)crk_leaves_alloc(ctx, lv, sizeof(uint16_t) * (size_t)capg * capr * 32);
+        if (!out.cnt || !out.gleaf || !out.unum || !out.goff || !out.uoff || !out.list || !out.ucode)
+            return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
+    }
+    out.groups = capg;
+    out.dgroups = lv->dev + 1;
+    out.onepass = true;
+    out.entries = capg * capr * 32;
+    out.table = capg * capt;
+    const LeafView v = list_view<true>(lv);
+    list_group_leaf_kernel<<<crk_grid(nl, 256), 256, 0, st>>>(nl, out.gstart, out.gleaf, capg);
+    strided_offsets_kernel<<<crk_grid(capg + 1, 256), 256, 0, st>>>(capg + 1, capr, capt, out.goff, out.uoff);
+    ListP pf{out.list, out.ucode, out.gstart, out.goff, out.uoff, out.cnt, out.unum, nullptr, lv->dev + 3, capr, capt,
+             lv->r_cut_grav * lv->r_cut_grav, n, nullptr};
+    const GroupTable gt{out.gstart, out.gleaf, ngroups, nullptr};
+    const unsigned gg = (unsigned)std::max<int64_t>(1, ((int64_t)ngroups + kWarps - 1) / kWarps);
+    pair_group_kernel<LS, false><<<gg, kThreads, 0, st>>>(v, pf, RecView<LS::Rec>{v.pos, n}, gt, nullptr);
+    ctx->launches += 3;
+    CRK_LAUNCH_CHECK(ctx, "neighbour lists");
+    return CRK_OK;
+}
+
+// reuse: a rebuild of one-pass gas lists into the buffers of the first build; no host
+// synchronisation, overflows go to the leaves' status word.  Otherwise the exact two-pass build
+// (count, scan, fill): gravity lists, and gas lists beyond the one-pass capacities.
 template <bool kGas>
 static int build_lists(crk_ctx *ctx, crk_leaves *lv, crk_nlist &out, bool reuse) {
     const int64_t nl = lv->n_leaves, n = lv->n;
-    if (nl == 0 || n == 0 || (kGas && lv->n_gas == 0)) return CRK_OK;
+    if (no_lists(lv, kGas)) return CRK_OK;
     if (reuse && (!kGas || !out.onepass)) return crk_fail(ctx, CRK_ESTATE, "rebuild: lists without fixed capacities");
     cudaStream_t st = ctx->stream;
     using LS = ListStage<kGas>;
-    int32_t *gstart = reuse ? out.gstart : (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(nl + 1));
-    int32_t *cnt = reuse ? out.cnt : (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)n);
-    // room for the records of the light stages, so that the first pair kernel need not allocate
-    if (!reuse && !crk_scratch(ctx, 4, 32 * (size_t)n)) return crk_fail(ctx, CRK_ENOMEM, "neighbour list scratch");
-    int32_t *ng = (int32_t *)crk_scratch(ctx, 6, sizeof(int32_t) * (size_t)(nl + 1));
-    int32_t *tot = (int32_t *)crk_scratch(ctx, 7, 64);  // [0] groups, [1] rows, [2] table entries, [4] largest table
-    if (!gstart || !cnt || !ng || !tot) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
-    CRK_CUDA(ctx, cudaMemsetAsync(ng, 0, sizeof(int32_t) * (size_t)(nl + 1), st));
-    list_group_count_kernel<<<crk_grid(nl, 256), 256, 0, st>>>(nl, lv->leaf_start, lv->leaf_ngas, kGas, ng);
-    ++ctx->launches;
-    int rc = crk_exclusive_scan_i32(ctx, ng, gstart, nl + 1, tot);
-    if (rc) return rc;
-    int32_t *dgroups = lv->dev + (kGas ? 1 : 2);  // this build's group count, for the kernels
-    CRK_CUDA(ctx, cudaMemcpyAsync(dgroups, tot, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
-    LeafView v{lv->leaf_start, lv->leaf_ngas, lv->bbox, lv->hmax, kGas ? lv->pos : lv->pos_g,
-               kGas ? lv->kperm : lv->kperm_g, kGas ? lv->himg_start : lv->gimg_start,
-               kGas ? lv->himg_cnt : lv->gimg_cnt, kGas ? lv->himg : lv->gimg, nl, nullptr, 0, 32, nullptr};
+    const LeafView v = list_view<kGas>(lv);
     const RecView<typename LS::Rec> rec{v.pos, n};  // a list record is the position and h
     const float rc2 = lv->r_cut_grav * lv->r_cut_grav;
-    const int capr = kGasListCapRows, capt = kGasTableCap;
+    int32_t *dgroups = lv->dev + (kGas ? 1 : 2);  // this build's group count, for the kernels
+    int rc;
     if (reuse) {
+        if ((rc = list_groups<kGas>(ctx, lv, out.gstart))) return rc;
         const int64_t capg = out.groups;
-        list_group_leaf_kernel<<<crk_grid(nl, 256), 256, 0, st>>>(nl, gstart, out.gleaf, capg);
-        CRK_CUDA(ctx, cudaMemsetAsync(tot + 5, 0, sizeof(int32_t), st));
-        ListP pf{out.list, out.ucode, gstart, out.goff, out.uoff, cnt, out.unum, nullptr, tot + 5, capr, capt, rc2, n,
-                 nullptr};
-        const GroupTable gt{gstart, out.gleaf, capg, dgroups};
+        list_group_leaf_kernel<<<crk_grid(nl, 256), 256, 0, st>>>(nl, out.gstart, out.gleaf, capg);
+        ListP pf{out.list, out.ucode, out.gstart, out.goff, out.uoff, out.cnt, out.unum, nullptr, lv->dev + 3,
+                 kGasListCapRows, kGasTableCap, rc2, n, nullptr};
+        const GroupTable gt{out.gstart, out.gleaf, capg, dgroups};
         const unsigned gg = (unsigned)((capg + kWarps - 1) / kWarps > 0 ? (capg + kWarps - 1) / kWarps : 1);
         pair_group_kernel<LS, false><<<gg, kThreads, 0, st>>>(v, pf, rec, gt, nullptr);
-        lists_status_kernel<<<1, 1, 0, st>>>(tot, capg, tot + 5, lv->dev);
+        lists_status_kernel<<<1, 1, 0, st>>>(dgroups, capg, lv->dev + 3, lv->dev);
         ctx->launches += 3;
         CRK_LAUNCH_CHECK(ctx, "neighbour lists");
         return CRK_OK;
     }
+    if (kGas && ctx->trace) fprintf(stderr, "[crk] gas lists: a list or table exceeded its capacity, exact build\n");
+    out = crk_nlist{};
+    int32_t *gstart = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(nl + 1));
+    int32_t *cnt = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)n);
+    int32_t *tot = (int32_t *)crk_scratch(ctx, 7, 64);  // [1] rows, [2] table entries, [4] largest table
+    if (!gstart || !cnt || !tot) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
+    if ((rc = list_groups<kGas>(ctx, lv, gstart))) return rc;
     int32_t ngroups = 0;
-    CRK_CUDA(ctx, cudaMemcpyAsync(&ngroups, tot, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    CRK_CUDA(ctx, cudaMemcpyAsync(&ngroups, dgroups, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CRK_CUDA(ctx, cudaStreamSynchronize(st));
-    // one-pass lists: room for 1/8 more groups than this build holds (a rebuild of moved particles reuses them)
-    const int64_t capg = (int64_t)ngroups + ngroups / 8 + 64;
-    int32_t *gleaf = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)capg);
-    if (!gleaf) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
-    list_group_leaf_kernel<<<crk_grid(nl, 256), 256, 0, st>>>(nl, gstart, gleaf, capg);
+    int32_t *gleaf = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)std::max(ngroups, 1));
+    int32_t *ucnt = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(ngroups + 1));
+    int32_t *goff = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(ngroups + 1));
+    int32_t *uoff = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(ngroups + 1));
+    int32_t *gk = (int32_t *)crk_scratch(ctx, 8, sizeof(int32_t) * (size_t)(ngroups + 1));
+    if (!gleaf || !ucnt || !goff || !uoff || !gk) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
+    list_group_leaf_kernel<<<crk_grid(nl, 256), 256, 0, st>>>(nl, gstart, gleaf, ngroups);
     const GroupTable gt{gstart, gleaf, ngroups, nullptr};
     const unsigned ggrid = (unsigned)((ngroups + kWarps - 1) / kWarps > 0 ? (ngroups + kWarps - 1) / kWarps : 1);
-    int32_t *ucnt = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(capg + 1));
-    if (!ucnt) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
+    CRK_CUDA(ctx, cudaMemsetAsync(ucnt, 0, sizeof(int32_t) * (size_t)(ngroups + 1), st));
+    CRK_CUDA(ctx, cudaMemsetAsync(tot + 4, 0, sizeof(int32_t), st));
+    ListP pc{nullptr, nullptr, gstart, nullptr, nullptr, cnt, ucnt, tot + 4, nullptr, 2147483647, 2147483647,
+             rc2, n, nullptr};
+    pair_group_kernel<LS, false><<<ggrid, kThreads, 0, st>>>(v, pc, rec, gt, nullptr);
+    CRK_LAUNCH_CHECK(ctx, "neighbour counts");
+    CRK_CUDA(ctx, cudaMemsetAsync(gk, 0, sizeof(int32_t) * (size_t)(ngroups + 1), st));
+    list_group_k_kernel<<<(unsigned)nl, kThreads, 0, st>>>(nl, lv->leaf_start, lv->leaf_ngas, kGas, gstart, cnt, gk);
+    ctx->launches += 3;
+    rc = crk_exclusive_scan_i32(ctx, gk, goff, ngroups + 1, tot + 1);
+    if (rc) return rc;
+    rc = crk_exclusive_scan_i32(ctx, ucnt, uoff, ngroups + 1, tot + 2);
+    if (rc) return rc;
+    int32_t sizes[5] = {0, 0, 0, 0, 0};
+    CRK_CUDA(ctx, cudaMemcpyAsync(sizes, tot, sizeof(sizes), cudaMemcpyDeviceToHost, st));
+    CRK_CUDA(ctx, cudaStreamSynchronize(st));
+    const int32_t rows = sizes[1], umax = sizes[4];
+    const int64_t tsize = (int64_t)(uint32_t)sizes[2];
+    // table indices are 16-bit, and the offsets 32-bit: without lists the kernels use tiles
+    if (umax > 65535 || rows < 0 || sizes[2] < 0) {
+        if (ctx->trace)
+            fprintf(stderr, "[crk] %s lists skipped (largest group table %d)\n", kGas ? "gas" : "gravity", umax);
+        return CRK_OK;
+    }
+    const int64_t entries = (int64_t)rows * 32;
+    uint16_t *list = (uint16_t *)crk_leaves_alloc(ctx, lv, sizeof(uint16_t) * (size_t)(entries > 0 ? entries : 1));
+    uint32_t *ucode = (uint32_t *)crk_leaves_alloc(ctx, lv, sizeof(uint32_t) * (size_t)(tsize > 0 ? tsize : 1));
+    if (!list || !ucode)
+        return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation (%lld entries)", (long long)entries);
+    ListP pf{list, ucode, gstart, goff, uoff, nullptr, nullptr, nullptr, nullptr, 2147483647, 2147483647,
+             rc2, n, nullptr};
+    pair_group_kernel<LS, false><<<ggrid, kThreads, 0, st>>>(v, pf, rec, gt, nullptr);
     ++ctx->launches;
-    int32_t *goff = nullptr, *uoff = nullptr;
-    uint16_t *list = nullptr;
-    uint32_t *ucode = nullptr;
-    int64_t entries = 0, tsize = 0;
-    // Gas lists: one pass into fixed capacities (a lane's list and a group's table), which the
-    // adaptive smoothing lengths keep well above the largest counts; the exact two-pass build
-    // (count, scan, fill) runs only if something overflowed.
-    bool done = false;
-    if (kGas && capg * capt < 2147483647LL) {
-        goff = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(capg + 1));
-        uoff = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(capg + 1));
-        list = (uint16_t *)crk_leaves_alloc(ctx, lv, sizeof(uint16_t) * (size_t)capg * capr * 32);
-        ucode = (uint32_t *)crk_leaves_alloc(ctx, lv, sizeof(uint32_t) * (size_t)capg * capt);
-        if (!goff || !uoff || !list || !ucode) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
-        strided_offsets_kernel<<<crk_grid(capg + 1, 256), 256, 0, st>>>(capg + 1, capr, capt, goff, uoff);
-        CRK_CUDA(ctx, cudaMemsetAsync(tot + 5, 0, sizeof(int32_t), st));
-        ListP pf{list, ucode, gstart, goff, uoff, cnt, ucnt, nullptr, tot + 5, capr, capt, rc2, n, nullptr};
-        pair_group_kernel<LS, false><<<ggrid, kThreads, 0, st>>>(v, pf, rec, gt, nullptr);
-        ctx->launches += 2;
-        CRK_LAUNCH_CHECK(ctx, "neighbour lists");
-        int32_t ovf = 1;
-        CRK_CUDA(ctx, cudaMemcpyAsync(&ovf, tot + 5, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        CRK_CUDA(ctx, cudaStreamSynchronize(st));
-        if (ovf == 0) {
-            done = true;
-            entries = (int64_t)capg * capr * 32;
-            tsize = (int64_t)capg * capt;
-        } else if (ctx->trace) {
-            fprintf(stderr, "[crk] gas lists: a list or table exceeded its capacity, exact build\n");
-        }
-    }
-    if (!done) {
-        CRK_CUDA(ctx, cudaMemsetAsync(ucnt, 0, sizeof(int32_t) * (size_t)(ngroups + 1), st));
-        CRK_CUDA(ctx, cudaMemsetAsync(tot + 4, 0, sizeof(int32_t), st));
-        ListP pc{nullptr, nullptr, gstart, nullptr, nullptr, cnt, ucnt, tot + 4, nullptr, 2147483647, 2147483647,
-                 rc2, n, nullptr};
-        pair_group_kernel<LS, false><<<ggrid, kThreads, 0, st>>>(v, pc, rec, gt, nullptr);
-        ++ctx->launches;
-        CRK_LAUNCH_CHECK(ctx, "neighbour counts");
-        goff = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(ngroups + 1));
-        uoff = (int32_t *)crk_leaves_alloc(ctx, lv, sizeof(int32_t) * (size_t)(ngroups + 1));
-        int32_t *gk = (int32_t *)crk_scratch(ctx, 8, sizeof(int32_t) * (size_t)(ngroups + 1));
-        if (!goff || !uoff || !gk) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
-        CRK_CUDA(ctx, cudaMemsetAsync(gk, 0, sizeof(int32_t) * (size_t)(ngroups + 1), st));
-        list_group_k_kernel<<<(unsigned)nl, kThreads, 0, st>>>(nl, lv->leaf_start, lv->leaf_ngas, kGas, gstart, cnt,
-                                                               gk);
-        ++ctx->launches;
-        rc = crk_exclusive_scan_i32(ctx, gk, goff, ngroups + 1, tot + 1);
-        if (rc) return rc;
-        rc = crk_exclusive_scan_i32(ctx, ucnt, uoff, ngroups + 1, tot + 2);
-        if (rc) return rc;
-        int32_t sizes[5] = {0, 0, 0, 0, 0};
-        CRK_CUDA(ctx, cudaMemcpyAsync(sizes, tot, sizeof(sizes), cudaMemcpyDeviceToHost, st));
-        CRK_CUDA(ctx, cudaStreamSynchronize(st));
-        const int32_t rows = sizes[1], umax = sizes[4];
-        tsize = (int64_t)(uint32_t)sizes[2];
-        // table indices are 16-bit, and the offsets 32-bit: without lists the kernels use tiles
-        if (umax > 65535 || rows < 0 || sizes[2] < 0) {
-            if (ctx->trace)
-                fprintf(stderr, "[crk] %s lists skipped (largest group table %d)\n", kGas ? "gas" : "gravity", umax);
-            return CRK_OK;
-        }
-        entries = (int64_t)rows * 32;
-        list = (uint16_t *)crk_leaves_alloc(ctx, lv, sizeof(uint16_t) * (size_t)(entries > 0 ? entries : 1));
-        ucode = (uint32_t *)crk_leaves_alloc(ctx, lv, sizeof(uint32_t) * (size_t)(tsize > 0 ? tsize : 1));
-        if (!list || !ucode)
-            return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation (%lld entries)", (long long)entries);
-        ListP pf{list, ucode, gstart, goff, uoff, nullptr, nullptr, nullptr, nullptr, 2147483647, 2147483647,
-                 rc2, n, nullptr};
-        pair_group_kernel<LS, false><<<ggrid, kThreads, 0, st>>>(v, pf, rec, gt, nullptr);
-        ++ctx->launches;
-        CRK_LAUNCH_CHECK(ctx, "neighbour lists");
-    }
+    CRK_LAUNCH_CHECK(ctx, "neighbour lists");
     out.unum = ucnt;
     out.uoff = uoff;
     out.ucode = ucode;
@@ -3478,9 +3513,9 @@ static int build_lists(crk_ctx *ctx, crk_leaves *lv, crk_nlist &out, bool reuse)
     out.goff = goff;
     out.cnt = cnt;
     out.list = list;
-    out.groups = done ? capg : ngroups;
+    out.groups = ngroups;
     out.dgroups = dgroups;
-    out.onepass = done;
+    out.onepass = false;
     out.entries = entries;
     return CRK_OK;
 }
