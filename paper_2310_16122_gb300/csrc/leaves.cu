@@ -500,6 +500,8 @@ __global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) rcb_local_kernel(
                                                                        const float *__restrict__ z,
                                                                        float *__restrict__ node_box,
                                                                        int32_t *__restrict__ members,
+                                                                       int32_t *__restrict__ rank_y,
+                                                                       int32_t *__restrict__ rank_z,
                                                                        int32_t *__restrict__ err) {
     extern __shared__ int4 local_smem[];
     int32_t *cur = reinterpret_cast<int32_t *>(local_smem);  // [6][kLocalCap]: column 2b + c of list b
@@ -657,7 +659,12 @@ __global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) rcb_local_kernel(
     }
     __syncthreads();
     if (t == 0 && bad) atomicAdd(err, 1);
-    for (int q = t; q < cnt; q += kLocalThreads) members[lo + q] = o.S[1][rk(cur[q])];  // list 0, column 0
+    for (int q = t; q < cnt; q += kLocalThreads) {  // list 0: its columns are the ranks along y and z
+        const int32_t ry = cur[q];
+        members[lo + q] = o.S[1][rk(ry)];
+        rank_y[lo + q] = ry;
+        rank_z[lo + q] = cur[kLocalCap + q];
+    }
 }
 
 // --- per-leaf data ------------------------------------------------------------
@@ -670,11 +677,26 @@ __device__ __forceinline__ uint32_t spread10(uint32_t v) {
     return v;
 }
 
-// Shared state of bisect32 (one per block) for leaves of at most kCap members
-// (parts of 8 for leaves of at most 256, parts of 32 above).
+// box of the 32 leaf-relative positions r of a warp into cell[0] (lo), cell[1] (hi): the
+// coordinates are >= 0 (-0 + 0 = 0), so their bits order like the values
+__device__ __forceinline__ void store_cell(float4 *cell, const float4 &r, int lane) {
+    const unsigned bits[3] = {__float_as_uint(r.x + 0.0f), __float_as_uint(r.y + 0.0f), __float_as_uint(r.z + 0.0f)};
+    float l[3], u[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        l[k] = __uint_as_float(__reduce_min_sync(CRK_FULL_MASK, bits[k]));
+        u[k] = __uint_as_float(__reduce_max_sync(CRK_FULL_MASK, bits[k]));
+    }
+    if (lane == 0) {
+        cell[0] = make_float4(l[0], l[1], l[2], 0.0f);
+        cell[1] = make_float4(u[0], u[1], u[2], 0.0f);
+    }
+}
+
+// Shared state of bisect32 (one per block) for leaves of at most kCap members.
 template <int kCap>
 struct Bisect32 {
-    static constexpr int kMaxSeg = kCap <= 256 ? kCap / 8 : kCap / 32;
+    static constexpr int kMaxSeg = kCap / 32;
     int16_t a[kCap], b[kCap];  // orders (member slots), double-buffered
     float cax[kCap];           // coordinate of the member at each position on its part's axis
     uint32_t cid[kCap];        // its particle index (ties)
@@ -682,35 +704,24 @@ struct Bisect32 {
     int nseg, more;
 };
 
-// Bisects positions [0, m) of the order src (bs.a or bs.b; member slots; m <= kCap)
-// into groups of U: each part above U is ranked along the longest extent of
-// its members in (coordinate, index) order and split with U ceil(g/2) of its
-// g groups of U on the left, until every part holds at most U; then every run
-// of U positions starting at a multiple of U is an RCB cell.  The parts start
-// as the runs of `start` positions (start = m: the whole range; start = 32
-// with U = 8: the RCB cells of 32, each bisected into cells of 8).  At most
-// ceil(m/U) <= 32 parts, one per lane of warp 0.  All threads call it; returns
+// Bisects positions [0, m) of the order bs.a (member slots; m <= kCap) into
+// groups of 32: each part above 32 is ranked along the longest extent of its
+// members in (coordinate, index) order and split with 32 ceil(g/2) of its g
+// groups of 32 on the left, until every part holds at most 32; then every run
+// of 32 positions starting at a multiple of 32 is an RCB cell.  At most
+// ceil(m/32) <= 32 parts, one per lane of warp 0.  All threads call it; returns
 // the array (bs.a or bs.b) holding the result in [0, m).
-template <int kCap, int U = 32>
-__device__ int16_t *bisect32(Bisect32<kCap> &bs, int m, const float4 *pm, const uint64_t *key,
-                             int16_t *src_in = nullptr, int start = 0) {
+template <int kCap>
+__device__ int16_t *bisect32(Bisect32<kCap> &bs, int m, const float4 *pm, const uint64_t *key) {
+    constexpr int U = 32;
     static_assert(kCap / U <= Bisect32<kCap>::kMaxSeg && kCap / U <= 32, "parts per leaf");
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int16_t *src = src_in ? src_in : bs.a, *dst = src == bs.a ? bs.b : bs.a;
-    if (start <= 0 || start > m) start = m;
+    int16_t *src = bs.a, *dst = bs.b;
     if (threadIdx.x == 0) {
-        bs.nseg = 0;
-        bs.more = 0;
-        for (int l = 0; l < m; l += start) {
-            bs.lo[bs.nseg] = l;
-            bs.hi[bs.nseg] = l + start < m ? l + start : m;
-            bs.more |= bs.hi[bs.nseg] - l > U;
-            ++bs.nseg;
-        }
-        if (m == 0) {
-            bs.nseg = 1;
-            bs.lo[0] = bs.hi[0] = 0;
-        }
+        bs.nseg = 1;
+        bs.lo[0] = 0;
+        bs.hi[0] = m;
+        bs.more = m > U;
     }
     __syncthreads();
     while (bs.more) {
@@ -816,8 +827,7 @@ __device__ int16_t *bisect32(Bisect32<kCap> &bs, int m, const float4 *pm, const 
 // candidates within r_c of a group's box: at r_c = 3 such cells cut the
 // candidates per in-range pair from ~4.0 to ~3.3 against Z-order groups); and
 // the leaf-relative positions in both kernel orders.
-// kCap: the largest leaf the launch may meet (1024 with blocks of 128 threads; 128 with one
-// warp per block for RCB leaves of at most 128, whose shared arrays then fit 32 blocks per SM).
+// kCap: the largest leaf the launch may meet (RCB leaves of at most 128 have a kernel of their own below).
 template <int kCap>
 __global__ void leaf_data_kernel(int64_t n_leaves, const int32_t *__restrict__ leaf_start,
                                  const int32_t *__restrict__ members, const float *__restrict__ x,
@@ -929,11 +939,9 @@ __global__ void leaf_data_kernel(int64_t n_leaves, const int32_t *__restrict__ l
         pos[lo + q] = make_float4(c.x - ox, c.y - oy, c.z - oz, c.w);
     }
     __syncthreads();
-    // gravity order: the whole leaf bisected into groups of 32, and (leaves of at most 256) each
-    // group of 32 into groups of 8 (the sub-cells of the gravity sweeps)
+    // gravity order: the whole leaf bisected into groups of 32
     for (int t = threadIdx.x; t < cnt; t += blockDim.x) bs.a[t] = (int16_t)t;
     int16_t *src = bisect32(bs, cnt, pm, key);
-    if constexpr (kCap <= 256) src = bisect32<kCap, 8>(bs, cnt, pm, key, src, 32);
     for (int q0 = w * 32; q0 < cnt; q0 += nw * 32) {  // one warp per cell of 32
         const int q = q0 + lane;
         const int t = src[q < cnt ? q : cnt - 1];
@@ -945,18 +953,257 @@ __global__ void leaf_data_kernel(int64_t n_leaves, const int32_t *__restrict__ l
             kinv_g[id] = lo + q;
             pos_g[lo + q] = r;
         }
-        // the cell's box: leaf-relative coordinates are >= 0 (-0 + 0 = 0), so their bits order like the values
-        const unsigned bits[3] = {__float_as_uint(r.x + 0.0f), __float_as_uint(r.y + 0.0f), __float_as_uint(r.z + 0.0f)};
-        float l[3], u[3];
-        for (int k = 0; k < 3; ++k) {
-            l[k] = __uint_as_float(__reduce_min_sync(CRK_FULL_MASK, bits[k]));
-            u[k] = __uint_as_float(__reduce_max_sync(CRK_FULL_MASK, bits[k]));
+        store_cell(gcell + 2 * ((int64_t)(lo >> 5) + a + (q0 >> 5)), r, lane);
+    }
+}
+
+// The same for RCB leaves of at most kRcbLeaf members, with the gravity order bisected down to
+// cells of 8.  Members arrive in x order with their ranks along y and z (integers, all different,
+// ordered like (coordinate, index)), so every order inside the leaf follows from one ranking per
+// axis (7-bit local ranks) and no coordinate is compared again:
+//   * the ranking counts smaller 32-bit keys, four to a shared-memory load;
+//   * a part's extents are the coordinates of its lowest and highest ranks (warp min and max);
+//   * the rank inside a part counts the smaller local ranks four to a word: with 7-bit values the
+//     byte differences of (rank | 0x80) - w never borrow, and bit 7 says rank >= w.
+// What bounds it is issue and the chain of levels.  33.5M particles: 8.4 ms for the general kernel
+// above with cells of 8, 5.2 here; 2x64^3: 156 -> 72 us; 30,011 particles: 71 -> 12.5 us.
+constexpr int kRcbLeaf = 128;
+struct LeafParts {
+    int lo[2][kRcbLeaf / 8], hi[2][kRcbLeaf / 8];  // bounds of the parts, double-buffered
+    int ax[kRcbLeaf / 8], left[kRcbLeaf / 8];      // split axis (-1: none), members that go left
+    unsigned split[2];                             // parts that split
+    uint8_t part[2][kRcbLeaf];                     // part of each position
+    __align__(8) uint8_t ab[kRcbLeaf];             // local rank of each position's member on its part's axis
+    uint8_t rk[3][kRcbLeaf], ord[3][kRcbLeaf];     // local rank of a member, member of a local rank
+};
+
+// Bisects positions [0, m) of the order src: parts above 32 with a multiple of 32 on the left, then
+// (cells8) parts above 8 with a multiple of 8; returns the buffer (src or dst) with the result.
+__device__ uint8_t *bisect_ranks(LeafParts &lp, int m, const float4 *pm, uint8_t *src, uint8_t *dst, bool cells8) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        lp.lo[0][0] = 0;
+        lp.hi[0][0] = m;
+        lp.split[0] = 0u;
+    }
+    for (int q = threadIdx.x; q < kRcbLeaf; q += blockDim.x) {
+        lp.part[0][q] = 0;
+        if (q >= m) lp.ab[q] = 0;  // (a 7-bit value: the differences never borrow)
+    }
+    int np = 1, b = 0;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) lp.split[b ^ 1] = 0u;
+        bool any = false;
+        for (int p = w; p < np; p += nw) {
+            const int l = lp.lo[b][p], h = lp.hi[b][p], len = h - l;
+            const int U = len > 32 ? 32 : (cells8 && len > 8 ? 8 : 0);
+            if (U == 0) {
+                if (lane == 0) lp.ax[p] = -1;
+                continue;
+            }
+            unsigned mn[3] = {255u, 255u, 255u}, mx[3] = {0u, 0u, 0u};
+            for (int q = l + lane; q < h; q += 32) {
+                const int t = src[q];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const unsigned v = lp.rk[a][t];
+                    mn[a] = min(mn[a], v);
+                    mx[a] = max(mx[a], v);
+                }
+            }
+            float e[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const float4 c0 = pm[lp.ord[a][__reduce_min_sync(CRK_FULL_MASK, mn[a])]];
+                const float4 c1 = pm[lp.ord[a][__reduce_max_sync(CRK_FULL_MASK, mx[a])]];
+                e[a] = a == 0 ? c1.x - c0.x : (a == 1 ? c1.y - c0.y : c1.z - c0.z);
+            }
+            any = true;
+            if (lane == 0) {
+                lp.ax[p] = (e[0] >= e[1] && e[0] >= e[2]) ? 0 : (e[1] >= e[2] ? 1 : 2);
+                lp.left[p] = U * (((len + U - 1) / U + 1) / 2);
+                atomicOr(&lp.split[b], 1u << p);
+            }
         }
-        if (lane == 0) {
-            float4 *g = gcell + 2 * ((int64_t)(lo >> 5) + a + (q0 >> 5));
-            g[0] = make_float4(l[0], l[1], l[2], 0.0f);
-            g[1] = make_float4(u[0], u[1], u[2], 0.0f);
+        if (!__syncthreads_or(any)) return src;
+        const unsigned split = lp.split[b];
+        for (int q = threadIdx.x; q < m; q += blockDim.x) {
+            const int ax = lp.ax[lp.part[b][q]];
+            if (ax >= 0) lp.ab[q] = lp.rk[ax][src[q]];
         }
+        if (threadIdx.x < np) {  // the children's bounds
+            const int p = threadIdx.x, c = p + __popc(split & ((1u << p) - 1u));
+            const int l = lp.lo[b][p], h = lp.hi[b][p];
+            lp.lo[b ^ 1][c] = l;
+            lp.hi[b ^ 1][c] = h;
+            if (split >> p & 1u) {
+                lp.hi[b ^ 1][c] = l + lp.left[p];
+                lp.lo[b ^ 1][c + 1] = l + lp.left[p];
+                lp.hi[b ^ 1][c + 1] = h;
+            }
+        }
+        __syncthreads();
+        for (int q = threadIdx.x; q < m; q += blockDim.x) {
+            const int p = lp.part[b][q], c = p + __popc(split & ((1u << p) - 1u));
+            int to = q, cp = c;
+            if (split >> p & 1u) {
+                const unsigned r = (unsigned)lp.ab[q] * 0x01010101u | 0x80808080u;
+                const int l = lp.lo[b][p], h = lp.hi[b][p];
+                unsigned n4 = 0u;  // four byte counters
+                for (int u = l; u < h; u += 8) {  // parts start at multiples of 8; only the last may end inside a word
+                    const uint2 v = *reinterpret_cast<const uint2 *>(lp.ab + u);
+                    unsigned c0 = (r - v.x) >> 7 & 0x01010101u, c1 = (r - v.y) >> 7 & 0x01010101u;
+                    if (u + 8 > h) {  // the bytes past the end do not count
+                        c0 &= h - u >= 4 ? ~0u : (1u << (8 * (h - u))) - 1u;
+                        c1 &= h - u <= 4 ? 0u : (1u << (8 * (h - u - 4))) - 1u;
+                    }
+                    n4 += c0 + c1;
+                }
+                const int rank = (int)((n4 * 0x01010101u) >> 24) - 1;  // (the member itself counted)
+                to = l + rank;
+                cp = c + (rank >= lp.left[p]);
+            }
+            dst[to] = src[q];
+            lp.part[b ^ 1][to] = (uint8_t)cp;
+        }
+        np += __popc(split);
+        b ^= 1;
+        uint8_t *t = src;
+        src = dst;
+        dst = t;
+    }
+}
+
+__global__ void __launch_bounds__(128) leaf_data_rcb_kernel(
+    const int32_t *__restrict__ leaf_start, const int32_t *__restrict__ members, const int32_t *__restrict__ rank_y,
+    const int32_t *__restrict__ rank_z, const float *__restrict__ x, const float *__restrict__ y,
+    const float *__restrict__ z, const uint8_t *__restrict__ sp, const float *__restrict__ h, int32_t *__restrict__ perm,
+    int32_t *__restrict__ kperm, int32_t *__restrict__ leaf_ngas, float *__restrict__ bbox, float *__restrict__ hmax,
+    float4 *__restrict__ pos, int32_t *__restrict__ kperm_g, float4 *__restrict__ pos_g, int32_t *__restrict__ kinv,
+    int32_t *__restrict__ kinv_g, float4 *__restrict__ gcell, int32_t *__restrict__ err) {
+    __shared__ float4 pm[kRcbLeaf];                                  // member position and h (0 for dark matter)
+    __shared__ uint4 key4[3][kRcbLeaf / 4];                          // dark matter << 31 | id; ranks along y, z
+    __shared__ LeafParts lp;
+    __shared__ uint8_t can[kRcbLeaf], oa[kRcbLeaf], ob[kRcbLeaf];    // canonical order; working orders
+    __shared__ float red[6][4], hms[4];
+    __shared__ int ngs[4];
+    uint32_t *const key = reinterpret_cast<uint32_t *>(key4[0]), *const gy = reinterpret_cast<uint32_t *>(key4[1]),
+                   *const gz = reinterpret_cast<uint32_t *>(key4[2]);
+    const int64_t a = blockIdx.x;
+    const int lo = leaf_start[a], m = leaf_start[a + 1] - lo;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (m > kRcbLeaf) {  // excluded by the tree's shape
+        if (threadIdx.x == 0) atomicAdd(err, 1);
+        return;
+    }
+    float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
+    int ng = 0;
+    float hm = 0.0f;
+    for (int t = threadIdx.x; t < kRcbLeaf; t += blockDim.x) {
+        if (t >= m) {
+            key[t] = gy[t] = gz[t] = 0xffffffffu;
+            continue;
+        }
+        // (every order starts as one of valid members: a partition found inconsistent, which is
+        // reported through err, may leave ranks that are not all different)
+        can[t] = oa[t] = ob[t] = lp.ord[0][t] = lp.ord[1][t] = lp.ord[2][t] = lp.rk[0][t] = (uint8_t)t;
+        const int32_t id = members[lo + t];
+        gy[t] = (uint32_t)rank_y[lo + t];
+        gz[t] = (uint32_t)rank_z[lo + t];
+        const bool gas = sp[id] == 0;
+        key[t] = (gas ? 0u : 0x80000000u) | (uint32_t)id;  // ids are below 2^31
+        const float c[3] = {x[id], y[id], z[id]};
+        const float hh = gas ? h[id] : 0.0f;
+        pm[t] = make_float4(c[0], c[1], c[2], hh);
+        for (int q = 0; q < 3; ++q) {
+            mn[q] = fminf(mn[q], c[q]);
+            mx[q] = fmaxf(mx[q], c[q]);
+        }
+        if (gas) {
+            ++ng;
+            hm = fmaxf(hm, hh);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        for (int q = 0; q < 3; ++q) {
+            mn[q] = fminf(mn[q], __shfl_xor_sync(CRK_FULL_MASK, mn[q], o));
+            mx[q] = fmaxf(mx[q], __shfl_xor_sync(CRK_FULL_MASK, mx[q], o));
+        }
+        hm = fmaxf(hm, __shfl_xor_sync(CRK_FULL_MASK, hm, o));
+    }
+    ng = __reduce_add_sync(CRK_FULL_MASK, ng);
+    if (lane == 0) {
+        for (int q = 0; q < 3; ++q) {
+            red[q][w] = mn[q];
+            red[3 + q][w] = mx[q];
+        }
+        ngs[w] = ng;
+        hms[w] = hm;
+    }
+    __syncthreads();
+    // the leaf's box, gas count and h_max, and its members' ranks: canonical, along y, along z
+    float ox = red[0][0], oy = red[1][0], oz = red[2][0], ux = red[3][0], uy = red[4][0], uz = red[5][0];
+    ng = ngs[0];
+    hm = hms[0];
+    for (int v = 1; v < nw; ++v) {
+        ox = fminf(ox, red[0][v]); oy = fminf(oy, red[1][v]); oz = fminf(oz, red[2][v]);
+        ux = fmaxf(ux, red[3][v]); uy = fmaxf(uy, red[4][v]); uz = fmaxf(uz, red[5][v]);
+        ng += ngs[v];
+        hm = fmaxf(hm, hms[v]);
+    }
+    if (threadIdx.x == 0) {
+        bbox[6 * a] = ox; bbox[6 * a + 1] = oy; bbox[6 * a + 2] = oz;
+        bbox[6 * a + 3] = ux; bbox[6 * a + 4] = uy; bbox[6 * a + 5] = uz;
+        leaf_ngas[a] = ng;
+        hmax[a] = hm;
+    }
+    const int m4 = (m + 3) >> 2;
+    for (int t = threadIdx.x; t < m; t += blockDim.x) {
+        const uint32_t k = key[t], ky = gy[t], kz = gz[t];
+        int r = 0, ry = 0, rz = 0;
+#pragma unroll 4
+        for (int u = 0; u < m4; ++u) {
+            const uint4 c = key4[0][u], cy = key4[1][u], cz = key4[2][u];
+            r += (c.x < k) + (c.y < k) + (c.z < k) + (c.w < k);
+            ry += (cy.x < ky) + (cy.y < ky) + (cy.z < ky) + (cy.w < ky);
+            rz += (cz.x < kz) + (cz.y < kz) + (cz.z < kz) + (cz.w < kz);
+        }
+        can[r] = (uint8_t)t;
+        oa[r] = ob[r] = (uint8_t)t;
+        perm[lo + r] = (int32_t)(k & 0x7fffffffu);
+        lp.rk[1][t] = (uint8_t)ry;
+        lp.rk[2][t] = (uint8_t)rz;
+        lp.ord[1][ry] = (uint8_t)t;
+        lp.ord[2][rz] = (uint8_t)t;
+    }
+    // gas order: gas first, bisected into groups of 32, then dark matter in canonical order
+    const uint8_t *gsrc = bisect_ranks(lp, ng, pm, oa, ob, false);
+    for (int q = threadIdx.x; q < m; q += blockDim.x) {
+        const int t = q < ng ? gsrc[q] : can[q];
+        const float4 c = pm[t];
+        const int32_t id = (int32_t)(key[t] & 0x7fffffffu);
+        kperm[lo + q] = id;
+        kinv[id] = lo + q;
+        pos[lo + q] = make_float4(c.x - ox, c.y - oy, c.z - oz, c.w);
+    }
+    __syncthreads();
+    // gravity order: every member, down to cells of 8
+    for (int t = threadIdx.x; t < m; t += blockDim.x) oa[t] = (uint8_t)t;
+    const uint8_t *src = bisect_ranks(lp, m, pm, oa, ob, true);
+    for (int q0 = w * 32; q0 < m; q0 += nw * 32) {  // one warp per cell of 32
+        const int q = q0 + lane;
+        const int t = src[q < m ? q : m - 1];
+        const float4 c = pm[t];
+        const float4 r = make_float4(c.x - ox, c.y - oy, c.z - oz, c.w);
+        if (q < m) {
+            const int32_t id = (int32_t)(key[t] & 0x7fffffffu);
+            kperm_g[lo + q] = id;
+            kinv_g[id] = lo + q;
+            pos_g[lo + q] = r;
+        }
+        store_cell(gcell + 2 * ((int64_t)(lo >> 5) + a + (q0 >> 5)), r, lane);
     }
 }
 
@@ -1712,6 +1959,7 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             ++ctx->launches;
         }
         int32_t *members = nullptr;  // particle ids grouped by leaf
+        int32_t *rank_yz[2] = {nullptr, nullptr};  // RCB: the members' ranks along y and z (members are in x order)
         int64_t nl = 0;
         const crk_rcb_shape *shape = nullptr;
         float *node_box = nullptr, *node_hmax = nullptr;
@@ -1844,11 +2092,15 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
                     ls.m[l] = (int32_t)shape->level_size[d_local + l];
                 }
                 rcb_local_kernel<<<(unsigned)shape->level_size[d_local], kLocalThreads, kLocalSmem, st>>>(
-                    n, ls, Lfin, ord, p->x, p->y, p->z, node_box, mem, flags + 5);
+                    n, ls, Lfin, ord, p->x, p->y, p->z, node_box, mem, An[0][0], An[0][1], flags + 5);
+                rank_yz[0] = An[0][0];
+                rank_yz[1] = An[0][1];
                 ++ctx->launches;
                 KCHECK("rcb local levels");
             } else if (n > 0) {
                 rank_members_kernel<<<crk_grid(n, 256), 256, 0, st>>>(n, Lfin, ord, mem);
+                rank_yz[0] = Ac[0][0];
+                rank_yz[1] = Ac[0][1];
                 ++ctx->launches;
             }
             tr.mark("rcb levels");
@@ -1867,12 +2119,12 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
         ALLOC(lv->kinv_g, int32_t, n);
         ALLOC(lv->gcell, float4, 2 * (n / 32 + nl + 1));
         if (nl > 0) {
-            if (lp->mode == 1 && shape && shape->max_leaf_size <= 128)
-                leaf_data_kernel<128><<<(unsigned)nl, 32, 0, st>>>(nl, lv->leaf_start, members, p->x, p->y, p->z,
-                                                                   p->species, h, lv->perm, lv->kperm, lv->leaf_ngas,
-                                                                   lv->bbox, lv->hmax, lv->pos, lv->kperm_g,
-                                                                   lv->pos_g, lv->kinv, lv->kinv_g, lv->gcell,
-                                                                   flags + 4);
+            if (lp->mode == 1 && shape && shape->max_leaf_size <= kRcbLeaf)
+                // two warps a leaf; four where the leaves are too few to fill the GPU
+                leaf_data_rcb_kernel<<<(unsigned)nl, nl < (int64_t)32 * ctx->num_sms ? 128 : 64, 0, st>>>(
+                    lv->leaf_start, members, rank_yz[0], rank_yz[1], p->x, p->y, p->z, p->species, h, lv->perm,
+                    lv->kperm, lv->leaf_ngas, lv->bbox, lv->hmax, lv->pos, lv->kperm_g, lv->pos_g, lv->kinv,
+                    lv->kinv_g, lv->gcell, flags + 4);
             else
                 leaf_data_kernel<kMaxLeafCap><<<(unsigned)nl, 128, 0, st>>>(
                     nl, lv->leaf_start, members, p->x, p->y, p->z, p->species, h, lv->perm, lv->kperm, lv->leaf_ngas,
