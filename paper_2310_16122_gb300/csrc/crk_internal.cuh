@@ -48,9 +48,9 @@ struct crk_ctx {
     int num_sms = 0;
     std::string err;
     // growable scratch arena: one buffer per slot
-    static const int kSlots = 37;  // leaf build 0-16 and 19-31, radix sort 12-14, scan 15, queue 17, step 18,
+    static const int kSlots = 38;  // leaf build 0-16 and 19-31, radix sort 12-14, scan 15, queue 17, step 18,
                                    // integrator 32, corrections adjoint 33, adjoint chain 34, half-warp force 35,
-                                   // tuner 36
+                                   // tuner 36, single calls' kernel-order columns 37
     void *slot[kSlots] = {};
     size_t slot_bytes[kSlots] = {};
     int64_t launches = 0;  // kernels this context has launched

@@ -3165,6 +3165,142 @@ int run_stage(crk_ctx *ctx, const crk_leaves *lv, typename S::P p, bool gas_pair
     return CRK_OK;
 }
 
+// ------------------------------------------------------- columns in another order
+// One column through a permutation: dst[o] = src[perm[o]] (o in the
+// destination order).  One column per launch keeps the randomly read source
+// (n floats) about the size of L2, so each 32-byte sector is fetched from DRAM
+// about once; gathering many columns at once thrashes L2 (measured slower).
+__global__ void permute_col_kernel(int64_t n, const int32_t *__restrict__ perm, const float *__restrict__ src,
+                                   float *__restrict__ dst) {
+    int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (o < n) dst[o] = __ldg(src + perm[o]);
+}
+
+// Several columns through one permutation in two streaming passes: the columns
+// are interleaved into rows of 4 Q floats (through shared memory, both sides
+// coalesced), then each destination reads its whole row, so a random access
+// brings 16 Q useful bytes instead of 4.  33.5M particles: 0.33 ms a column by
+// permute_col_kernel, 0.16 ms in rows of 5 to 8 (the step's 20 columns: 6.5 ->
+// 3.2 ms); 524,288 particles: 168 -> 60 us for 38 columns.
+constexpr int kBundle = 36;  // columns of one bundle (the limited Energy pass reads 35)
+struct Bundle {
+    const float *src[kBundle];
+    float *dst[kBundle];
+    int k = 0;
+    void add(const float *s, float *d, int comps, int64_t n) {
+        for (int c = 0; c < comps; ++c, ++k) {
+            src[k] = s + (size_t)c * n;
+            dst[k] = d + (size_t)c * n;
+        }
+    }
+};
+constexpr int kRowTile = 128;  // particles per block of the interleaving pass
+
+template <int Q>
+__global__ void __launch_bounds__(kRowTile) interleave_kernel(int64_t n, Bundle b, float4 *__restrict__ rows) {
+    __shared__ float tile[4 * Q][kRowTile + 1];
+    const int64_t base = (int64_t)blockIdx.x * kRowTile;
+    const int t = threadIdx.x, m = (int)(n - base < kRowTile ? n - base : kRowTile);
+    if (t < m) {
+#pragma unroll
+        for (int c = 0; c < 4 * Q; ++c)
+            if (c < b.k) tile[c][t] = __ldg(b.src[c] + base + t);
+    }
+    __syncthreads();
+    for (int j = t; j < m * Q; j += kRowTile) {
+        const int r = j / Q, c = 4 * (j % Q);
+        rows[base * Q + j] = make_float4(tile[c][r], tile[c + 1][r], tile[c + 2][r], tile[c + 3][r]);
+    }
+}
+
+template <int Q>
+__global__ void __launch_bounds__(256) deal_rows_kernel(int64_t n, const int32_t *__restrict__ perm, Bundle b,
+                                                        const float4 *__restrict__ rows) {
+    const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (o >= n) return;
+    const float4 *r = rows + (int64_t)perm[o] * Q;
+    float4 v[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) v[q] = __ldg(r + q);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        if (4 * q < b.k) b.dst[4 * q][o] = v[q].x;
+        if (4 * q + 1 < b.k) b.dst[4 * q + 1][o] = v[q].y;
+        if (4 * q + 2 < b.k) b.dst[4 * q + 2][o] = v[q].z;
+        if (4 * q + 3 < b.k) b.dst[4 * q + 3][o] = v[q].w;
+    }
+}
+
+template <int Q>
+int permute_rows(crk_ctx *ctx, int64_t n, const int32_t *perm, const Bundle &b) {
+    if constexpr (Q > 1) {
+        if (b.k <= 4 * (Q - 1)) return permute_rows<Q - 1>(ctx, n, perm, b);
+    }
+    // the rows live in the stages' record scratch, which holds nothing between two stages
+    float4 *rows = (float4 *)crk_scratch(ctx, 4, sizeof(float4) * Q * (size_t)n);
+    if (!rows) return crk_fail(ctx, CRK_ENOMEM, "permutation scratch");
+    interleave_kernel<Q><<<crk_grid(n, kRowTile), kRowTile, 0, ctx->stream>>>(n, b, rows);
+    deal_rows_kernel<Q><<<crk_grid(n, 256), 256, 0, ctx->stream>>>(n, perm, b, rows);
+    ctx->launches += 2;
+    CRK_LAUNCH_CHECK(ctx, "column permutation");
+    return CRK_OK;
+}
+
+// dst = src[perm] for every column of the bundle
+int permute_bundle(crk_ctx *ctx, int64_t n, const int32_t *perm, const Bundle &b) {
+    if (b.k >= 3) return permute_rows<kBundle / 4>(ctx, n, perm, b);
+    for (int c = 0; c < b.k; ++c) {
+        permute_col_kernel<<<crk_grid(n, 256), 256, 0, ctx->stream>>>(n, perm, b.src[c], b.dst[c]);
+        ++ctx->launches;
+    }
+    CRK_LAUNCH_CHECK(ctx, "column permutation");
+    return CRK_OK;
+}
+
+// Single calls of the gas stages on large boxes: the caller's columns are
+// permuted into the kernel order, the stage runs there and its outputs are
+// permuted back, instead of gathering and scattering every column at random
+// 4-byte places inside the stage's kernels.  Geometry, corrections and hydro,
+// direct -> permuted: 0.62 -> 0.64 ms on 524,288 particles, 1.13 -> 1.12 on
+// 1.02M, 2.17 -> 1.83 on 1.77M, 6.47 -> 4.22 on 4.19M; with Extras,
+// Acceleration and Energy 1.36 -> 1.42, 2.61 -> 2.50, 4.89 -> 4.16, 13.8 -> 9.8.
+// (The gravity calls, four columns each way, gain nothing: 8.33 -> 8.42 ms on
+// 4.19M, 68.3 -> 68.1 on 33.5M.)
+constexpr int64_t kKorderMin = 900000;
+struct KernelOrder {
+    crk_ctx *ctx;
+    const crk_leaves *lv;
+    bool on;
+    float *next = nullptr;
+    Bundle in, out;
+    // cols: columns the call will ask for
+    KernelOrder(crk_ctx *c, const crk_leaves *l, int cols) : ctx(c), lv(l) {
+        on = lv->n >= kKorderMin;
+        if (!on) return;
+        next = (float *)crk_scratch(ctx, 37, sizeof(float) * (size_t)cols * (size_t)lv->n);
+        on = next != nullptr;  // without room for the columns: the direct form
+    }
+    float *take(int comps) {
+        float *r = next;
+        next += (size_t)comps * lv->n;
+        return r;
+    }
+    const float *input(const float *p, int comps) {
+        if (!on || !p) return p;
+        float *r = take(comps);
+        in.add(p, r, comps, lv->n);
+        return r;
+    }
+    float *output(float *p, int comps) {
+        if (!on || !p) return p;
+        float *r = take(comps);
+        out.add(r, p, comps, lv->n);
+        return r;
+    }
+    int begin() { return on ? permute_bundle(ctx, lv->n, lv->kperm, in) : CRK_OK; }
+    int end(int rc) { return rc || !on ? rc : permute_bundle(ctx, lv->n, lv->kinv, out); }
+};
+
 }  // namespace
 
 int grav_short(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params *gp, const float *m, float *a3,
@@ -3216,8 +3352,11 @@ int crk_geometry_adjoint(crk_ctx *ctx, const crk_leaves *lv, const float *m, con
     if (!ctx) return CRK_EINVAL;
     if (!lv) return crk_fail(ctx, CRK_EINVAL, "null leaves");
     if (lv->n > 0 && (!m || !V || !rhobar || !gx3 || !gm)) return crk_fail(ctx, CRK_EINVAL, "null array");
-    GeomAdjP p{m, V, rhobar, Vbar, gx3, gm, lv->n, nullptr};
-    return run_stage<GeomAdjStage>(ctx, lv, p, true, CRK_K_GEOMETRY_ADJOINT);
+    KernelOrder ko(ctx, lv, 4 + 4);
+    GeomAdjP p{ko.input(m, 1), ko.input(V, 1), ko.input(rhobar, 1), ko.input(Vbar, 1), ko.output(gx3, 3),
+               ko.output(gm, 1), lv->n, nullptr};
+    const int rc = ko.begin();
+    return rc ? rc : ko.end(run_stage<GeomAdjStage>(ctx, lv, p, true, CRK_K_GEOMETRY_ADJOINT, nullptr, ko.on));
 }
 
 int crk_corrections(crk_ctx *ctx, const crk_leaves *lv, const float *V, float *A, float *B, float *gradA,
@@ -3226,8 +3365,11 @@ int crk_corrections(crk_ctx *ctx, const crk_leaves *lv, const float *V, float *A
     if (!lv) return crk_fail(ctx, CRK_EINVAL, "null leaves");
     if (lv->n > 0 && (!V || !A || !B || !gradA || !gradB)) return crk_fail(ctx, CRK_EINVAL, "null array");
     if (n_singular) CRK_CUDA(ctx, cudaMemsetAsync(n_singular, 0, sizeof(int32_t), ctx->stream));
-    CorrP p{V, A, B, gradA, gradB, n_singular, lv->n, nullptr};
-    return run_stage<CorrStage>(ctx, lv, p, true, CRK_K_CORRECTIONS);
+    KernelOrder ko(ctx, lv, 1 + 16);
+    CorrP p{ko.input(V, 1), ko.output(A, 1), ko.output(B, 3), ko.output(gradA, 3), ko.output(gradB, 9), n_singular,
+            lv->n, nullptr};
+    const int rc = ko.begin();
+    return rc ? rc : ko.end(run_stage<CorrStage>(ctx, lv, p, true, CRK_K_CORRECTIONS, nullptr, ko.on));
 }
 
 int crk_hydro(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params *hp, const float *m, const float *v3,
@@ -3237,9 +3379,12 @@ int crk_hydro(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params *hp, co
     if (!lv || !hp) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvdt3 || !dudt))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    HydroP p{m, v3, u, V, rho, A, B, gradA, gradB, dvdt3, dudt, conservation,
+    KernelOrder ko(ctx, lv, 23 + 4);
+    HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
+             ko.input(gradA, 3), ko.input(gradB, 9), ko.output(dvdt3, 3), ko.output(dudt, 1), conservation,
              hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count};
-    return run_stage<HydroStage>(ctx, lv, p, true, CRK_K_HYDRO, conservation);
+    const int rc = ko.begin();
+    return rc ? rc : ko.end(run_stage<HydroStage>(ctx, lv, p, true, CRK_K_HYDRO, conservation, ko.on));
 }
 
 int crk_extras(crk_ctx *ctx, const crk_leaves *lv, const float *m, const float *v3, const float *V, const float *A,
@@ -3249,8 +3394,11 @@ int crk_extras(crk_ctx *ctx, const crk_leaves *lv, const float *m, const float *
     if (!lv) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !V || !A || !B || !gradA || !gradB || !rho_r || !dvdx))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    ExtrasP p{m, v3, V, A, B, gradA, gradB, rho_r, dvdx, lv->n, (unsigned long long *)pair_count};
-    return run_stage<ExtrasStage>(ctx, lv, p, true, CRK_K_EXTRAS);
+    KernelOrder ko(ctx, lv, 21 + 10);
+    ExtrasP p{ko.input(m, 1), ko.input(v3, 3), ko.input(V, 1), ko.input(A, 1), ko.input(B, 3), ko.input(gradA, 3),
+              ko.input(gradB, 9), ko.output(rho_r, 1), ko.output(dvdx, 9), lv->n, (unsigned long long *)pair_count};
+    const int rc = ko.begin();
+    return rc ? rc : ko.end(run_stage<ExtrasStage>(ctx, lv, p, true, CRK_K_EXTRAS, nullptr, ko.on));
 }
 
 int crk_hydro_limited(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params *hp, const float *m,
@@ -3261,9 +3409,12 @@ int crk_hydro_limited(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params
     if (!lv || !hp) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvdx || !dvdt3 || !dudt))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    HydroP p{m, v3, u, V, rho, A, B, gradA, gradB, dvdt3, dudt, conservation,
-             hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, dvdx};
-    return run_stage<HydroLimStage>(ctx, lv, p, true, CRK_K_HYDRO, conservation);
+    KernelOrder ko(ctx, lv, 32 + 4);
+    HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
+             ko.input(gradA, 3), ko.input(gradB, 9), ko.output(dvdt3, 3), ko.output(dudt, 1), conservation,
+             hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, ko.input(dvdx, 9)};
+    const int rc = ko.begin();
+    return rc ? rc : ko.end(run_stage<HydroLimStage>(ctx, lv, p, true, CRK_K_HYDRO, conservation, ko.on));
 }
 
 int crk_hydro_accel(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params *hp, const float *m, const float *v3,
@@ -3275,12 +3426,16 @@ int crk_hydro_accel(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params *
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvdt3))
         return crk_fail(ctx, CRK_EINVAL, "null array");
     if (!(sig_beta >= 0.0f)) return crk_fail(ctx, CRK_EINVAL, "sig_beta must be >= 0");
-    HydroP p{m, v3, u, V, rho, A, B, gradA, gradB, dvdt3, nullptr, conservation,
-             hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, dvdx};
+    KernelOrder ko(ctx, lv, 32 + 3);
+    HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
+             ko.input(gradA, 3), ko.input(gradB, 9), ko.output(dvdt3, 3), nullptr, conservation,
+             hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, ko.input(dvdx, 9)};
     p.vsig_h = vsig_h_max;
     p.sig_beta = sig_beta;
-    if (dvdx) return run_stage<HydroAccelStage<true>>(ctx, lv, p, true, CRK_K_ACCEL, conservation);
-    return run_stage<HydroAccelStage<false>>(ctx, lv, p, true, CRK_K_ACCEL, conservation);
+    const int rc = ko.begin();
+    if (rc) return rc;
+    if (dvdx) return ko.end(run_stage<HydroAccelStage<true>>(ctx, lv, p, true, CRK_K_ACCEL, conservation, ko.on));
+    return ko.end(run_stage<HydroAccelStage<false>>(ctx, lv, p, true, CRK_K_ACCEL, conservation, ko.on));
 }
 
 int crk_hydro_energy(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params *hp, const float *m, const float *v3,
@@ -3291,11 +3446,15 @@ int crk_hydro_energy(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params 
     if (!lv || !hp) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !vstar3 || !dudt))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    HydroP p{m, v3, u, V, rho, A, B, gradA, gradB, nullptr, dudt, conservation,
-             hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, dvdx};
-    p.vstar = vstar3;
-    if (dvdx) return run_stage<HydroEnergyStage<true>>(ctx, lv, p, true, CRK_K_ENERGY, conservation);
-    return run_stage<HydroEnergyStage<false>>(ctx, lv, p, true, CRK_K_ENERGY, conservation);
+    KernelOrder ko(ctx, lv, 35 + 1);
+    HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
+             ko.input(gradA, 3), ko.input(gradB, 9), nullptr, ko.output(dudt, 1), conservation,
+             hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, ko.input(dvdx, 9)};
+    p.vstar = vstar3 == v3 ? p.v3 : ko.input(vstar3, 3);
+    const int rc = ko.begin();
+    if (rc) return rc;
+    if (dvdx) return ko.end(run_stage<HydroEnergyStage<true>>(ctx, lv, p, true, CRK_K_ENERGY, conservation, ko.on));
+    return ko.end(run_stage<HydroEnergyStage<false>>(ctx, lv, p, true, CRK_K_ENERGY, conservation, ko.on));
 }
 
 int crk_corrections_adjoint(crk_ctx *ctx, const crk_leaves *lv, const float *V, const float *Abar,
@@ -3310,19 +3469,21 @@ int crk_corrections_adjoint(crk_ctx *ctx, const crk_leaves *lv, const float *V, 
     if (n == 0) return CRK_OK;
     float *coef = (float *)crk_scratch(ctx, 33, sizeof(float) * kCorrCoef * (size_t)n);
     if (!coef) return crk_fail(ctx, CRK_ENOMEM, "adjoint scratch");
+    KernelOrder ko(ctx, lv, 17 + 4);
     CorrAdjP p{};
-    p.V = V;
+    p.V = ko.input(V, 1);
     p.n_singular = n_singular;
     p.n = n;
-    p.Abar = Abar;
-    p.Bbar = Bbar;
-    p.gAbar = gradAbar;
-    p.gBbar = gradBbar;
+    p.Abar = ko.input(Abar, 1);
+    p.Bbar = ko.input(Bbar, 3);
+    p.gAbar = ko.input(gradAbar, 3);
+    p.gBbar = ko.input(gradBbar, 9);
     p.coef = coef;
-    int rc;
-    if ((rc = run_stage<CorrAdjPrepStage>(ctx, lv, p, true, CRK_K_CORRECTIONS))) return rc;
-    CorrAdjSweepP q{V, coef, xbar3, Vbar, n, nullptr, nullptr};
-    return run_stage<CorrAdjStage>(ctx, lv, q, true, CRK_K_CORRECTIONS);
+    CorrAdjSweepP q{p.V, coef, ko.output(xbar3, 3), ko.output(Vbar, 1), n, nullptr, nullptr};
+    int rc = ko.begin();
+    if (!rc) rc = run_stage<CorrAdjPrepStage>(ctx, lv, p, true, CRK_K_CORRECTIONS, nullptr, ko.on);
+    if (!rc) rc = run_stage<CorrAdjStage>(ctx, lv, q, true, CRK_K_CORRECTIONS, nullptr, ko.on);
+    return ko.end(rc);
 }
 
 int crk_hydro_adjoint(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params *hp, const float *m, const float *v3,
@@ -3335,10 +3496,15 @@ int crk_hydro_adjoint(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvbar3 || !dubar || !xbar3 ||
                       !vbar3 || !ubar || !mbar || !Vbar || !rhobar || !Abar || !Bbar3 || !gradAbar3 || !gradBbar9))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    HydroAdjP p{m,      v3,     u,     V,     rho,   A,         B,         gradA,     gradB,
-                dvbar3, dubar,  xbar3, vbar3, ubar,  mbar,      Vbar,      rhobar,    Abar,
-                Bbar3,  gradAbar3, gradBbar9, hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, nullptr, nullptr};
-    return run_stage<HydroAdjStage>(ctx, lv, p, true, CRK_K_HYDRO);
+    KernelOrder ko(ctx, lv, 27 + 26);
+    HydroAdjP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
+                ko.input(gradA, 3), ko.input(gradB, 9),
+                ko.input(dvbar3, 3), ko.input(dubar, 1), ko.output(xbar3, 3), ko.output(vbar3, 3), ko.output(ubar, 1),
+                ko.output(mbar, 1), ko.output(Vbar, 1), ko.output(rhobar, 1), ko.output(Abar, 1), ko.output(Bbar3, 3),
+                ko.output(gradAbar3, 3), ko.output(gradBbar9, 9), hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n,
+                nullptr, nullptr};
+    const int rc = ko.begin();
+    return rc ? rc : ko.end(run_stage<HydroAdjStage>(ctx, lv, p, true, CRK_K_HYDRO, nullptr, ko.on));
 }
 
 template <bool kGas>
@@ -3605,26 +3771,6 @@ int grav_short_noalloc(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params
 // to the caller's order once at the end.
 namespace {
 
-// dst[c*n + q] = src[c*n + perm[q]] for c < ncomp (into kernel order)
-__global__ void to_korder_kernel(int64_t n, int ncomp, const int32_t *__restrict__ perm, const float *__restrict__ src,
-                                 float *__restrict__ dst) {
-    int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    const int64_t o = perm[q];
-    for (int c = 0; c < ncomp; ++c) dst[c * n + q] = src[c * n + o];
-}
-
-
-// One column through a permutation: dst[o] = src[perm[o]] (o in the
-// destination order).  One column per launch keeps the randomly read source
-// (n floats) about the size of L2, so each 32-byte sector is fetched from DRAM
-// about once; gathering many columns at once thrashes L2 (measured slower).
-__global__ void permute_col_kernel(int64_t n, const int32_t *__restrict__ perm, const float *__restrict__ src,
-                                   float *__restrict__ dst) {
-    int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (o < n) dst[o] = __ldg(src + perm[o]);
-}
-
 __global__ void cotangent_kernel(int64_t n, const float *__restrict__ a_g, const float4 *__restrict__ pos,
                                  float *__restrict__ abar_g, float *__restrict__ rhob_k) {
     int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -3643,24 +3789,19 @@ int crk_stage_forces(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params *
     const int64_t n = lv->n;
     if (n == 0) return CRK_OK;
     auto C = [&](int k) { return w + (size_t)k * n; };
-    cudaStream_t st = ctx->stream;
-    const int g = crk_grid(n, 256);
-    auto col = [&](float *dst, const float *src, const int32_t *perm) {
-        permute_col_kernel<<<g, 256, 0, st>>>(n, perm, src, dst);
-        ++ctx->launches;
-    };
-    col(C(K::m), m, lv->kperm);
-    for (int c = 0; c < 3; ++c) col(C(K::v) + (size_t)c * n, v3 + (size_t)c * n, lv->kperm);
-    col(C(K::u), u, lv->kperm);
-    if (gravity) col(C(K::mg), m, lv->kperm_g);
-    CRK_LAUNCH_CHECK(ctx, "stage inputs");
     int rc;
+    Bundle in, in_g;
+    in.add(m, C(K::m), 1, n);
+    in.add(v3, C(K::v), 3, n);
+    in.add(u, C(K::u), 1, n);
+    if (gravity) in_g.add(m, C(K::mg), 1, n);
+    if ((rc = permute_bundle(ctx, n, lv->kperm, in)) || (rc = permute_bundle(ctx, n, lv->kperm_g, in_g))) return rc;
     {
         GeomP p{C(K::m), C(K::V), C(K::rho), n, nullptr, nullptr};
         if ((rc = run_stage<GeomStage>(ctx, lv, p, true, CRK_K_GEOMETRY, nullptr, true))) return rc;
     }
     {
-        if (n_singular) CRK_CUDA(ctx, cudaMemsetAsync(n_singular, 0, sizeof(int32_t), st));
+        if (n_singular) CRK_CUDA(ctx, cudaMemsetAsync(n_singular, 0, sizeof(int32_t), ctx->stream));
         CorrP p{C(K::V), C(K::A), C(K::B), C(K::gA), C(K::gB), n_singular, n, nullptr};
         if ((rc = run_stage<CorrStage>(ctx, lv, p, true, CRK_K_CORRECTIONS, nullptr, true))) return rc;
     }
@@ -3700,13 +3841,10 @@ int crk_stage_energy(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params 
     auto C = [&](int k) { return w + (size_t)k * n; };
     const float *vs = C(K::v);
     if (vstar3) {
-        const int g = crk_grid(n, 256);
-        for (int c = 0; c < 3; ++c) {
-            permute_col_kernel<<<g, 256, 0, ctx->stream>>>(n, lv->kperm, vstar3 + (size_t)c * n,
-                                                           C(K::vs) + (size_t)c * n);
-            ++ctx->launches;
-        }
-        CRK_LAUNCH_CHECK(ctx, "stage v*");
+        Bundle in;
+        in.add(vstar3, C(K::vs), 3, n);
+        const int rc = permute_bundle(ctx, n, lv->kperm, in);
+        if (rc) return rc;
         vs = C(K::vs);
     }
     HydroP p{C(K::m), C(K::v), C(K::u), C(K::V), C(limited ? K::rhoR : K::rho), C(K::A), C(K::B), C(K::gA),
@@ -3747,19 +3885,14 @@ int crk_hydro_chain_adjoint(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_
     auto C = [&](int k) { return w + (size_t)k * n; };
     cudaStream_t st = ctx->stream;
     const int g = crk_grid(n, 256);
-    auto col = [&](float *dst, const float *src, const int32_t *perm) {
-        permute_col_kernel<<<g, 256, 0, st>>>(n, perm, src, dst);
-        ++ctx->launches;
-    };
-    col(C(cm), io->m, lv->kperm);
-    col(C(cu), io->u, lv->kperm);
-    col(C(cdub), io->dubar, lv->kperm);
-    for (int c = 0; c < 3; ++c) {
-        col(C(cv) + (size_t)c * n, io->v3 + (size_t)c * n, lv->kperm);
-        col(C(cdvb) + (size_t)c * n, io->dvbar3 + (size_t)c * n, lv->kperm);
-    }
-    CRK_LAUNCH_CHECK(ctx, "chain inputs");
     int rc;
+    Bundle in, outs;
+    in.add(io->m, C(cm), 1, n);
+    in.add(io->u, C(cu), 1, n);
+    in.add(io->dubar, C(cdub), 1, n);
+    in.add(io->v3, C(cv), 3, n);
+    in.add(io->dvbar3, C(cdvb), 3, n);
+    if ((rc = permute_bundle(ctx, n, lv->kperm, in))) return rc;
     {
         GeomP p{C(cm), C(cV), C(crho), n, nullptr, nullptr};
         if ((rc = run_stage<GeomStage>(ctx, lv, p, true, CRK_K_GEOMETRY, nullptr, true))) return rc;
@@ -3803,16 +3936,13 @@ int crk_hydro_chain_adjoint(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_
     add_cols_kernel<<<ge, 256, 0, st>>>(n, 1, C(cmh), C(cmh), C(cmg), nullptr);  // mbar
     ctx->launches += 2;
     CRK_LAUNCH_CHECK(ctx, "chain sums");
-    struct Out {
-        float *dst;
-        int src, comp;
-    } outs[] = {{io->dvdt3, cdv, 3}, {io->dudt, cdu, 1}, {io->xbar3, cxh, 3},
-                {io->mbar, cmh, 1},  {io->vbar3, cvb, 3}, {io->ubar, cub, 1}};
-    for (const Out &o : outs)
-        if (o.dst)
-            for (int c = 0; c < o.comp; ++c) col(o.dst + (size_t)c * n, C(o.src) + (size_t)c * n, lv->kinv);
-    CRK_LAUNCH_CHECK(ctx, "chain outputs");
-    return CRK_OK;
+    if (io->dvdt3) outs.add(C(cdv), io->dvdt3, 3, n);
+    if (io->dudt) outs.add(C(cdu), io->dudt, 1, n);
+    if (io->xbar3) outs.add(C(cxh), io->xbar3, 3, n);
+    if (io->mbar) outs.add(C(cmh), io->mbar, 1, n);
+    if (io->vbar3) outs.add(C(cvb), io->vbar3, 3, n);
+    if (io->ubar) outs.add(C(cub), io->ubar, 1, n);
+    return permute_bundle(ctx, n, lv->kinv, outs);
 }
 
 int crk_step_fused(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params *gp, const crk_hydro_params *hp,
@@ -3833,21 +3963,22 @@ int crk_step_fused(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params *gp
     cudaStream_t st = ctx->stream;
     const int g = crk_grid(n, 256);
     crk_step_mark(ctx, 0);
+    int rc;
     {
-        // inputs into the two kernel orders: m, v, u (gas order) and m (gravity order)
-        auto col = [&](float *dst, const float *src, const int32_t *perm) {
-            permute_col_kernel<<<g, 256, 0, st>>>(n, perm, src, dst);
-            ++ctx->launches;
-        };
-        col(m_k, io->m, lv->kperm);
-        for (int c = 0; c < 3; ++c) col(v_k + (size_t)c * n, io->v3 + (size_t)c * n, lv->kperm);
-        col(u_k, io->u, lv->kperm);
-        col(m_g, io->m, lv->kperm_g);
+        // inputs into the two kernel orders: m, v, u (gas order) and m (gravity order), with the
+        // caller's cotangents
+        Bundle in, in_g;
+        in.add(io->m, m_k, 1, n);
+        in.add(io->v3, v_k, 3, n);
+        in.add(io->u, u_k, 1, n);
+        if (io->rhobar) in.add(io->rhobar, rhob_k, 1, n);
+        if (io->Vbar) in.add(io->Vbar, Vb_k, 1, n);
+        in_g.add(io->m, m_g, 1, n);
+        if (io->abar3) in_g.add(io->abar3, abar_g, 3, n);
+        if ((rc = permute_bundle(ctx, n, lv->kperm, in)) || (rc = permute_bundle(ctx, n, lv->kperm_g, in_g))) return rc;
     }
-    CRK_LAUNCH_CHECK(ctx, "step inputs");
     unsigned long long *cnt = (unsigned long long *)io->pair_count;
     unsigned long long *swc = cnt ? (unsigned long long *)io->swept_count : nullptr;
-    int rc;
     {
         GeomP p{m_k, V_k, rho_k, n, cnt ? cnt + 0 : nullptr, swc ? swc + 0 : nullptr};
         if ((rc = run_stage<GeomStage>(ctx, lv, p, true, CRK_K_GEOMETRY, nullptr, true))) return rc;
@@ -3888,12 +4019,11 @@ int crk_step_fused(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params *gp
         if ((rc = run_stage<GravStage>(ctx, lv, p, false, CRK_K_GRAVITY, nullptr, true))) return rc;
     }
     crk_step_mark(ctx, 4);
-    // cotangents: the caller's (permuted into kernel order) or those of sum |a|^2 + sum_gas rho
-    if (io->abar3) to_korder_kernel<<<g, 256, 0, st>>>(n, 3, lv->kperm_g, io->abar3, abar_g);
-    if (io->rhobar) to_korder_kernel<<<g, 256, 0, st>>>(n, 1, lv->kperm, io->rhobar, rhob_k);
-    if (io->Vbar) to_korder_kernel<<<g, 256, 0, st>>>(n, 1, lv->kperm, io->Vbar, Vb_k);
-    cotangent_kernel<<<g, 256, 0, st>>>(n, a_g, lv->pos, io->abar3 ? nullptr : abar_g, io->rhobar ? nullptr : rhob_k);
-    ctx->launches += 1 + (io->abar3 != nullptr) + (io->rhobar != nullptr) + (io->Vbar != nullptr);
+    // cotangents not given by the caller: those of sum |a|^2 + sum_gas rho
+    if (!io->abar3 || !io->rhobar) {
+        cotangent_kernel<<<g, 256, 0, st>>>(n, a_g, lv->pos, io->abar3 ? nullptr : abar_g, io->rhobar ? nullptr : rhob_k);
+        ++ctx->launches;
+    }
     CRK_LAUNCH_CHECK(ctx, "step cotangents");
     {
         GravAdjP p{};
@@ -3915,24 +4045,31 @@ int crk_step_fused(crk_ctx *ctx, const crk_leaves *lv, const crk_grav_params *gp
     }
     crk_step_mark(ctx, 6);
     // outputs back to the caller's order (only those asked for)
-    struct Out {
-        float *dst;
-        const float *src;
-        int comp;
-        const int32_t *perm;
-    } outs[] = {{io->V, V_k, 1, lv->kinv},          {io->rho, rho_k, 1, lv->kinv},     {io->A, A_k, 1, lv->kinv},
-                {io->B, B_k, 3, lv->kinv},          {io->gradA, gA_k, 3, lv->kinv},    {io->gradB, gB_k, 9, lv->kinv},
-                {io->dvdt3, dv_k, 3, lv->kinv},     {io->dudt, du_k, 1, lv->kinv},     {io->a3, a_g, 3, lv->kinv_g},
-                {io->gx3_grav, gx_g, 3, lv->kinv_g}, {io->gm_grav, gm_g, 1, lv->kinv_g}, {io->gx3_geom, gx2_k, 3, lv->kinv},
-                {io->gm_geom, gm2_k, 1, lv->kinv},   {io->extras ? io->rho_r : nullptr, rhoR_k, 1, lv->kinv},
-                {io->extras ? io->dvdx : nullptr, dvdx_k, 9, lv->kinv}};
-    for (const Out &o : outs)
-        if (o.dst)
-            for (int c = 0; c < o.comp; ++c) {
-                permute_col_kernel<<<g, 256, 0, st>>>(n, o.perm, o.src + (size_t)c * n, o.dst + (size_t)c * n);
-                ++ctx->launches;
-            }
-    CRK_LAUNCH_CHECK(ctx, "step outputs");
+    {
+        Bundle out[3];
+        auto give = [&](Bundle &b, const float *src, float *dst, int comps) {
+            if (dst) b.add(src, dst, comps, n);
+        };
+        give(out[0], V_k, io->V, 1);
+        give(out[0], rho_k, io->rho, 1);
+        give(out[0], A_k, io->A, 1);
+        give(out[0], B_k, io->B, 3);
+        give(out[0], gA_k, io->gradA, 3);
+        give(out[0], gB_k, io->gradB, 9);
+        give(out[0], dv_k, io->dvdt3, 3);
+        give(out[0], du_k, io->dudt, 1);
+        give(out[0], gx2_k, io->gx3_geom, 3);
+        give(out[0], gm2_k, io->gm_geom, 1);
+        if (io->extras) {
+            give(out[1], rhoR_k, io->rho_r, 1);
+            give(out[1], dvdx_k, io->dvdx, 9);
+        }
+        give(out[2], a_g, io->a3, 3);
+        give(out[2], gx_g, io->gx3_grav, 3);
+        give(out[2], gm_g, io->gm_grav, 1);
+        for (int k = 0; k < 3; ++k)
+            if ((rc = permute_bundle(ctx, n, k < 2 ? lv->kinv : lv->kinv_g, out[k]))) return rc;
+    }
     crk_step_mark(ctx, 7);
     return CRK_OK;
 }
