@@ -108,8 +108,9 @@ struct crk_leaves {
     int32_t *kinv_g = nullptr;      // original index -> gravity kernel order position
     float4 *pos_g = nullptr;        // [n] gravity kernel order: leaf-relative x, y, z and h or 0
     // tight boxes (lo, hi; leaf-relative) of the gravity order's cells of 32: cell q of leaf a at
-    // entries 2 c, 2 c + 1 with c = leaf_start[a] / 32 + a + q (n / 32 + n_leaves + 1 cells at most)
-    float4 *gcell = nullptr;
+    // entries 2 c, 2 c + 1 with c = leaf_start[a] / 32 + a + q (n / 32 + n_leaves + 1 cells at most),
+    // and of the gas cells of 32 of the gas order, indexed alike (largest h in the first entry's w)
+    float4 *gcell = nullptr, *hcell = nullptr;
     // leaf-pair lists: per i-leaf a, entries [start[a], start[a] + count[a]) in
     // ascending j-leaf order (leaves may be laid out in any order)
     int32_t *gimg_start = nullptr, *gimg_cnt = nullptr;  // gravity images

@@ -677,8 +677,8 @@ __device__ __forceinline__ uint32_t spread10(uint32_t v) {
     return v;
 }
 
-// box of the 32 leaf-relative positions r of a warp into cell[0] (lo), cell[1] (hi): the
-// coordinates are >= 0 (-0 + 0 = 0), so their bits order like the values
+// box of the 32 leaf-relative positions r of a warp into cell[0] (lo, largest h), cell[1] (hi): the
+// coordinates and h are >= 0 (-0 + 0 = 0), so their bits order like the values
 __device__ __forceinline__ void store_cell(float4 *cell, const float4 &r, int lane) {
     const unsigned bits[3] = {__float_as_uint(r.x + 0.0f), __float_as_uint(r.y + 0.0f), __float_as_uint(r.z + 0.0f)};
     float l[3], u[3];
@@ -687,8 +687,9 @@ __device__ __forceinline__ void store_cell(float4 *cell, const float4 &r, int la
         l[k] = __uint_as_float(__reduce_min_sync(CRK_FULL_MASK, bits[k]));
         u[k] = __uint_as_float(__reduce_max_sync(CRK_FULL_MASK, bits[k]));
     }
+    const float hm = __uint_as_float(__reduce_max_sync(CRK_FULL_MASK, __float_as_uint(r.w)));
     if (lane == 0) {
-        cell[0] = make_float4(l[0], l[1], l[2], 0.0f);
+        cell[0] = make_float4(l[0], l[1], l[2], hm);
         cell[1] = make_float4(u[0], u[1], u[2], 0.0f);
     }
 }
@@ -837,7 +838,7 @@ __global__ void leaf_data_kernel(int64_t n_leaves, const int32_t *__restrict__ l
                                  int32_t *__restrict__ leaf_ngas, float *__restrict__ bbox,
                                  float *__restrict__ hmax, float4 *__restrict__ pos, int32_t *__restrict__ kperm_g,
                                  float4 *__restrict__ pos_g, int32_t *__restrict__ kinv, int32_t *__restrict__ kinv_g,
-                                 float4 *__restrict__ gcell, int32_t *__restrict__ err) {
+                                 float4 *__restrict__ gcell, float4 *__restrict__ hcell, int32_t *__restrict__ err) {
     __shared__ uint64_t key[kCap], zkey[kCap];
     __shared__ Bisect32<kCap> bs;
     __shared__ float4 pm[kCap];  // member position and h (0 for dark matter), gathered once
@@ -937,6 +938,10 @@ __global__ void leaf_data_kernel(int64_t n_leaves, const int32_t *__restrict__ l
         kperm[lo + q] = id;
         kinv[id] = lo + q;  // the inverse permutations, written here rather than by a pass of their own
         pos[lo + q] = make_float4(c.x - ox, c.y - oy, c.z - oz, c.w);
+    }
+    for (int q0 = w * 32; q0 < ngs[0]; q0 += nw * 32) {  // boxes of the gas cells of 32
+        const float4 c = pm[gsrc[q0 + lane < ngs[0] ? q0 + lane : ngs[0] - 1]];
+        store_cell(hcell + 2 * ((int64_t)(lo >> 5) + a + (q0 >> 5)), make_float4(c.x - ox, c.y - oy, c.z - oz, c.w), lane);
     }
     __syncthreads();
     // gravity order: the whole leaf bisected into groups of 32
@@ -1082,7 +1087,7 @@ __global__ void __launch_bounds__(128) leaf_data_rcb_kernel(
     const float *__restrict__ z, const uint8_t *__restrict__ sp, const float *__restrict__ h, int32_t *__restrict__ perm,
     int32_t *__restrict__ kperm, int32_t *__restrict__ leaf_ngas, float *__restrict__ bbox, float *__restrict__ hmax,
     float4 *__restrict__ pos, int32_t *__restrict__ kperm_g, float4 *__restrict__ pos_g, int32_t *__restrict__ kinv,
-    int32_t *__restrict__ kinv_g, float4 *__restrict__ gcell, int32_t *__restrict__ err) {
+    int32_t *__restrict__ kinv_g, float4 *__restrict__ gcell, float4 *__restrict__ hcell, int32_t *__restrict__ err) {
     __shared__ float4 pm[kRcbLeaf];                                  // member position and h (0 for dark matter)
     __shared__ uint4 key4[3][kRcbLeaf / 4];                          // dark matter << 31 | id; ranks along y, z
     __shared__ LeafParts lp;
@@ -1187,6 +1192,10 @@ __global__ void __launch_bounds__(128) leaf_data_rcb_kernel(
         kperm[lo + q] = id;
         kinv[id] = lo + q;
         pos[lo + q] = make_float4(c.x - ox, c.y - oy, c.z - oz, c.w);
+    }
+    for (int q0 = w * 32; q0 < ng; q0 += nw * 32) {  // boxes of the gas cells of 32
+        const float4 c = pm[gsrc[q0 + lane < ng ? q0 + lane : ng - 1]];
+        store_cell(hcell + 2 * ((int64_t)(lo >> 5) + a + (q0 >> 5)), make_float4(c.x - ox, c.y - oy, c.z - oz, c.w), lane);
     }
     __syncthreads();
     // gravity order: every member, down to cells of 8
@@ -2118,18 +2127,19 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
         ALLOC(lv->kinv, int32_t, n);
         ALLOC(lv->kinv_g, int32_t, n);
         ALLOC(lv->gcell, float4, 2 * (n / 32 + nl + 1));
+        ALLOC(lv->hcell, float4, 2 * (n / 32 + nl + 1));
         if (nl > 0) {
             if (lp->mode == 1 && shape && shape->max_leaf_size <= kRcbLeaf)
                 // two warps a leaf; four where the leaves are too few to fill the GPU
                 leaf_data_rcb_kernel<<<(unsigned)nl, nl < (int64_t)32 * ctx->num_sms ? 128 : 64, 0, st>>>(
                     lv->leaf_start, members, rank_yz[0], rank_yz[1], p->x, p->y, p->z, p->species, h, lv->perm,
                     lv->kperm, lv->leaf_ngas, lv->bbox, lv->hmax, lv->pos, lv->kperm_g, lv->pos_g, lv->kinv,
-                    lv->kinv_g, lv->gcell, flags + 4);
+                    lv->kinv_g, lv->gcell, lv->hcell, flags + 4);
             else
                 leaf_data_kernel<kMaxLeafCap><<<(unsigned)nl, 128, 0, st>>>(
                     nl, lv->leaf_start, members, p->x, p->y, p->z, p->species, h, lv->perm, lv->kperm, lv->leaf_ngas,
                     lv->bbox, lv->hmax, lv->pos, lv->kperm_g, lv->pos_g, lv->kinv, lv->kinv_g, lv->gcell,
-                    flags + 4);
+                    lv->hcell, flags + 4);
             ++ctx->launches;
         }
         KCHECK("leaf data");

@@ -233,7 +233,6 @@ struct GravP {
 struct GravStage {
     static constexpr bool kHalfWarp = true;
     static constexpr bool kGasOnly = false;
-    static constexpr bool kTag = false;
     static constexpr bool kAllVariants = true;
     using P = GravP;
     struct Rec {
@@ -363,7 +362,6 @@ struct GravAdjP {
 struct GravAdjStage {
     static constexpr bool kHalfWarp = true;
     static constexpr bool kGasOnly = false;
-    static constexpr bool kTag = false;
     static constexpr bool kAllVariants = true;
     using P = GravAdjP;
     struct __align__(16) Rec {
@@ -541,7 +539,6 @@ struct GeomStage {
     static constexpr bool kPair = false;
     static constexpr bool kGasOnly = true;
     static constexpr bool kCons = false;
-    static constexpr bool kTag = false;
     static constexpr bool kAllVariants = true;
     using P = GeomP;
     struct Rec {
@@ -591,7 +588,6 @@ struct GeomAdjStage {
     static constexpr bool kPair = false;
     static constexpr bool kGasOnly = true;
     static constexpr bool kCons = false;
-    static constexpr bool kTag = false;
     static constexpr bool kAllVariants = true;
     using P = GeomAdjP;
     struct __align__(16) Rec {
@@ -653,7 +649,6 @@ struct CorrStage {
     static constexpr bool kPair = false;
     static constexpr bool kGasOnly = true;
     static constexpr bool kCons = false;
-    static constexpr bool kTag = false;
     static constexpr bool kAllVariants = true;
     using P = CorrP;
     struct __align__(16) Rec {
@@ -1068,7 +1063,6 @@ struct CorrAdjStage {
     static constexpr bool kPair = false;
     static constexpr bool kGasOnly = true;
     static constexpr bool kCons = false;
-    static constexpr bool kTag = false;
     static constexpr bool kAllVariants = false;
     using P = CorrAdjSweepP;
     struct __align__(16) Rec {
@@ -1184,7 +1178,6 @@ struct HydroStageT {
     static constexpr bool kPair = false;
     static constexpr bool kGasOnly = true;
     static constexpr bool kCons = true;
-    static constexpr bool kTag = false;
     static constexpr bool kAllVariants = kPass == kHydroBoth;  // the step passes: lists and tiles only
     using P = HydroP;
     using Base = std::conditional_t<kLim, HydroRecLim, HydroRec>;
@@ -1440,7 +1433,6 @@ struct HydroAdjStage {
     static constexpr bool kPair = false;
     static constexpr bool kGasOnly = true;
     static constexpr bool kCons = false;
-    static constexpr bool kTag = false;
     static constexpr bool kAllVariants = false;
     using P = HydroAdjP;
     struct __align__(16) Rec : HydroRec {
@@ -1595,7 +1587,6 @@ struct ExtrasStage {
     static constexpr bool kPair = false;
     static constexpr bool kGasOnly = true;
     static constexpr bool kCons = false;
-    static constexpr bool kTag = false;
     static constexpr bool kAllVariants = true;
     using P = ExtrasP;
     struct __align__(16) Rec {
@@ -1688,82 +1679,6 @@ struct ListP {
     int32_t *overflow;                 // set when a list or a table exceeds its capacity, may be null
     int cap_rows, cap_table;           // capacity of one lane's list and of one group's table
     float rc2;
-    int64_t n;
-    unsigned long long *count;
-    unsigned long long *swept;  // counting runs: candidate pair evaluations (tiles and lists), may be NULL
-};
-
-template <bool kGas>
-struct ListStage {
-    static constexpr bool kGasOnly = kGas;
-    static constexpr bool kCons = false;
-    static constexpr bool kTag = true;
-    using P = ListP;
-    struct __align__(16) Rec {
-        float x, y, z, h;
-        uint32_t code, pad0, pad1, pad2;
-        static constexpr int kWords = 4;  // the code is set when the record is loaded
-    };
-    struct I {
-        uint16_t *out;
-        uint32_t *uout;
-        int64_t grp;
-        int c;    // this lane's list length
-        int u;    // table size (warp-uniform)
-        int cnt;
-    };
-
-    __device__ static float box_cut(const P &p, float hmax_i, const Rec &rj) {
-        return kGas ? hmax_i + rj.h : sqrtf(p.rc2);
-    }
-    __device__ static float leaf_cut(const P &p, float hmax_i, float hmax_j) {
-        return kGas ? hmax_i + hmax_j : sqrtf(p.rc2);
-    }
-    __device__ static void shift(Rec &r, float sx, float sy, float sz) { r.x += sx; r.y += sy; r.z += sz; }
-    __device__ static void tag(Rec &r, int img_local, int j_local) {
-        r.code = ((uint32_t)img_local << 10) | (uint32_t)j_local;
-    }
-    __device__ static void init(const P &p, I &s, const Rec &, int64_t a, int q, int lane, int32_t) {
-        s.c = 0;
-        s.u = 0;
-        s.cnt = 0;
-        s.grp = p.gstart[a] + q;
-        s.out = p.list ? p.list + (size_t)p.goff[s.grp] * 32 + lane : nullptr;
-        s.uout = p.ucode ? p.ucode + p.uoff[s.grp] : nullptr;
-    }
-    // called by all 32 lanes together (the sweep is warp-uniform)
-    template <bool kCount>
-    __device__ static void interact(const P &p, I &s, const Rec &ri, const Rec &rj) {
-        bool in;
-        if (kGas) {
-            float dx = ri.x - rj.x, dy = ri.y - rj.y, dz = ri.z - rj.z;
-            float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            float hs = ri.h + rj.h;
-            in = r2 < hs * hs;
-        } else {  // the gravity kernels take d = x_j - x_i
-            float dx = rj.x - ri.x, dy = rj.y - ri.y, dz = rj.z - ri.z;
-            float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            in = r2 < p.rc2;
-        }
-        const unsigned m = __ballot_sync(CRK_FULL_MASK, in);
-        if (m) {
-            if (in) {
-                if (s.out && s.c < p.cap_rows && s.u < p.cap_table) s.out[(size_t)s.c * 32] = (uint16_t)s.u;
-                ++s.c;
-            }
-            if (s.uout && (int)(threadIdx.x & 31) == __ffs(m) - 1 && s.u < p.cap_table) s.uout[s.u] = rj.code;
-            ++s.u;
-        }
-    }
-    __device__ static void finish(const P &p, I &s, const Rec &, int32_t, int64_t i) {
-        if (p.cnt) p.cnt[i] = s.c;
-        if (p.overflow && (s.c > p.cap_rows || s.u > p.cap_table)) atomicOr(p.overflow, 1);
-        if ((threadIdx.x & 31) == 0) {  // lane 0 is always active
-            if (p.ucnt) p.ucnt[s.grp] = s.u;
-            if (p.umax) atomicMax(p.umax, s.u);
-        }
-    }
-    __device__ static void finish_other(const P &, int32_t) {}
 };
 
 // --------------------------------------------------------------- framework
@@ -1834,7 +1749,6 @@ __device__ __forceinline__ void tile_group(const LeafView &lv, const typename S:
             if (jv) {
                 rj = rec[j];
                 S::shift(rj, im.sx, im.sy, im.sz);
-                if constexpr (S::kTag) S::tag(rj, e - ib, j - jlo);
                 float dx = fmaxf(fmaxf(bl0 - rj.x, rj.x - bh0), 0.f);
                 float dy = fmaxf(fmaxf(bl1 - rj.y, rj.y - bh1), 0.f);
                 float dz = fmaxf(fmaxf(bl2 - rj.z, rj.z - bh2), 0.f);
@@ -2254,30 +2168,174 @@ __device__ __forceinline__ int64_t group_count(int64_t cap, const int32_t *dgrou
     return g < cap ? g : cap;
 }
 
-// Tiles, one warp per i-group: every warp works even where a leaf holds fewer
-// groups than a block has warps (gas stages: a leaf of 128 holds about 64 gas).
-template <class S, bool kCount>
-__global__ void __launch_bounds__(kThreads) pair_group_kernel(LeafView lv, typename S::P p,
-                                                              RecView<typename S::Rec> rec,
-                                                              GroupTable gt, double *__restrict__ cons_part) {
-    using Rec = typename S::Rec;
-    __shared__ __align__(16) Rec buf[kWarps][kCap];
-    __shared__ double cons_sh[kWarps][4];
+// Builds the neighbour lists, one warp per i-group.  The j cells of 32 are
+// culled 32 at a time, one per lane, by their boxes (and largest h), the
+// particles of a cell near enough are tested against the group's box and
+// compacted; then every lane tests 32 buffered candidates against its own i in
+// straight-line packed FP32 (the kernels' own arithmetic, so the lists hold
+// exactly the pairs they would find in range) and keeps the answers as bits.
+// The union of the lanes' bits gives the candidates their table entries, and
+// each lane writes the entries of its own bits.  A ballot, a counter and two
+// predicated stores for every candidate, as before, kept the issue slots busy.
+// 2x256^3 box 11.2 -> 6.9 ms, 2x64^3 230 -> 142 us, 2x32^3 90 -> 43 us.
+template <bool kGas>
+__global__ void __launch_bounds__(kThreads) list_build_kernel(LeafView lv, ListP p, GroupTable gt,
+                                                              const float4 *__restrict__ cellbox, int log_cpl) {
+    __shared__ float4 buf[kWarps][2][32];  // candidate pairs: (x0, x1, y0, y1), (z0, z1, h0, h1)
+    __shared__ uint32_t code[kWarps][64];
+    __shared__ float4 cells[kWarps][32];   // one round's cells: shift, first particle
+    __shared__ int2 cell_n[kWarps][32];    // particles, code of the first
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double cons_acc[4] = {0.0, 0.0, 0.0, 0.0};
+    const unsigned below = lanemask_lt();
+    const int cmask = (1 << log_cpl) - 1;
+    const float rc = sqrtf(p.rc2);
     const int64_t ngroups = group_count(gt.groups, gt.dgroups);
     for (int64_t grp = next_group(lv, -1, lane); grp < ngroups; grp = next_group(lv, grp, lane)) {
         const int64_t a = gt.gleaf[grp];
         const int lo = lv.leaf_start[a];
-        const int hi = S::kGasOnly ? lo + lv.leaf_ngas[a] : lv.leaf_start[a + 1];
-        const int g0 = lo + 32 * (int)(grp - gt.gstart[a]);
-        tile_group<S, kCount>(lv, p, rec, buf[warp], a, lo, g0, hi, lane, cons_acc);
-    }
-    if constexpr (S::kCons) {
-        if (cons_part) cons_block_partial(cons_sh, cons_acc, cons_part);
+        const int hi = kGas ? lo + lv.leaf_ngas[a] : lv.leaf_start[a + 1];
+        const int g0 = lo + 32 * (int)(grp - gt.gstart[a]), i = g0 + lane;
+        const bool act = i < hi;
+        const float4 ri = lv.pos[act ? i : g0];
+        // leaf-relative coordinates and h are >= 0 (-0 + 0 = 0): their bits order like the values
+        const unsigned x[3] = {__float_as_uint(ri.x + 0.0f), __float_as_uint(ri.y + 0.0f), __float_as_uint(ri.z + 0.0f)};
+        float bl[3], bh[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            bl[k] = __uint_as_float(__reduce_min_sync(CRK_FULL_MASK, x[k]));
+            bh[k] = __uint_as_float(__reduce_max_sync(CRK_FULL_MASK, x[k]));
+        }
+        const float hm = __uint_as_float(__reduce_max_sync(CRK_FULL_MASK, __float_as_uint(ri.w)));
+        const float2 nx = make_float2(-ri.x, -ri.x), ny = make_float2(-ri.y, -ri.y), nz = make_float2(-ri.z, -ri.z),
+                     h2 = make_float2(ri.w, ri.w);
+        uint16_t *const out = p.list ? p.list + (size_t)p.goff[grp] * 32 + lane : nullptr;
+        uint32_t *const uout = p.ucode ? p.ucode + p.uoff[grp] : nullptr;
+        int c = 0, u = 0, cnt = 0;  // this lane's list length; table size and candidates (warp-uniform)
+        // the first `m` (at most 32) candidates
+        auto test = [&](int m) {
+            __syncwarp();
+            unsigned in = 0u;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const float4 q0 = buf[warp][0][k], q1 = buf[warp][1][k];
+                const float2 dx = __fadd2_rn(make_float2(q0.x, q0.y), nx), dy = __fadd2_rn(make_float2(q0.z, q0.w), ny),
+                             dz = __fadd2_rn(make_float2(q1.x, q1.y), nz);
+                const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+                float2 c2 = make_float2(p.rc2, p.rc2);
+                if constexpr (kGas) {
+                    const float2 hs = __fadd2_rn(h2, make_float2(q1.z, q1.w));
+                    c2 = __fmul2_rn(hs, hs);
+                }
+                if (r2.x < c2.x) in |= 1u << (2 * k);
+                if (r2.y < c2.y) in |= 2u << (2 * k);
+            }
+            if (m < 32) in &= (1u << m) - 1u;
+            if (!act) in = 0u;
+            const unsigned used = __reduce_or_sync(CRK_FULL_MASK, in);
+            if (uout && (used >> lane & 1u)) {
+                const int at = u + __popc(used & below);
+                if (at < p.cap_table) uout[at] = code[warp][lane];
+            }
+            while (in) {
+                const unsigned low = in & (0u - in);
+                const int at = u + __popc(used & (low - 1u));
+                if (out && c < p.cap_rows && at < p.cap_table) out[(size_t)c * 32] = (uint16_t)at;
+                ++c;
+                in ^= low;
+            }
+            u += __popc(used);
+            __syncwarp();
+        };
+        const int ib = lv.img_start[a], ie = ib + lv.img_cnt[a];
+        int q = lane & cmask;  // this lane's cell of its image's leaf
+        for (int e0 = ib; e0 < ie;) {
+            const int e = e0 + (lane >> log_cpl);
+            bool pass = false, more = false;
+            if (e < ie) {
+                const crk_image im = lv.img[e];
+                const int jlo = lv.leaf_start[im.b], jhi = kGas ? jlo + lv.leaf_ngas[im.b] : lv.leaf_start[im.b + 1];
+                const int jb = jlo + 32 * q;
+                more = jhi - jb > 32 * (cmask + 1);
+                if (jb < jhi) {
+                    const float4 *gb = cellbox + 2 * ((int64_t)(jlo >> 5) + im.b + q);
+                    const float4 l = gb[0], h = gb[1];
+                    const float gx = fmaxf(fmaxf(im.sx + l.x - bh[0], bl[0] - (im.sx + h.x)), 0.f);
+                    const float gy = fmaxf(fmaxf(im.sy + l.y - bh[1], bl[1] - (im.sy + h.y)), 0.f);
+                    const float gz = fmaxf(fmaxf(im.sz + l.z - bh[2], bl[2] - (im.sz + h.z)), 0.f);
+                    const float cut = kGas ? hm + l.w : rc;
+                    pass = fmaf(gx, gx, fmaf(gy, gy, gz * gz)) <= cut * cut * 1.0001f + 1e-6f;
+                    cells[warp][lane] = make_float4(im.sx, im.sy, im.sz, __int_as_float(jb));
+                    cell_n[warp][lane] = make_int2(min(jhi - jb, 32), ((e - ib) << 10) | (jb - jlo));
+                }
+            }
+            unsigned todo = __ballot_sync(CRK_FULL_MASK, pass);
+            if (__any_sync(CRK_FULL_MASK, more)) {  // a leaf with more cells than its lanes: once more
+                q += cmask + 1;
+            } else {
+                q = lane & cmask;
+                e0 += 32 >> log_cpl;
+            }
+            __syncwarp();
+            float4 cl = make_float4(0.f, 0.f, 0.f, 0.f), rn = cl;  // the next cell, loaded one ahead
+            int2 nn = make_int2(0, 0);
+            auto next = [&]() {
+                const int src = __ffs(todo) - 1;
+                cl = cells[warp][src];
+                nn = cell_n[warp][src];
+                if (lane < nn.x) rn = lv.pos[__float_as_int(cl.w) + lane];
+            };
+            if (todo) next();
+            while (todo) {
+                const float4 rj = make_float4(rn.x + cl.x, rn.y + cl.y, rn.z + cl.z, rn.w);
+                const bool jv = lane < nn.x;
+                const uint32_t cd = (uint32_t)(nn.y + lane);
+                todo &= todo - 1;
+                if (todo) next();
+                const float dx = fmaxf(fmaxf(bl[0] - rj.x, rj.x - bh[0]), 0.f);
+                const float dy = fmaxf(fmaxf(bl[1] - rj.y, rj.y - bh[1]), 0.f);
+                const float dz = fmaxf(fmaxf(bl[2] - rj.z, rj.z - bh[2]), 0.f);
+                const float cut = kGas ? hm + rj.w : rc;
+                const bool keep = jv && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= cut * cut * 1.0001f + 1e-6f;
+                const unsigned m = __ballot_sync(CRK_FULL_MASK, keep);
+                if (keep) {
+                    const int at = cnt + __popc(m & below);
+                    float *d0 = reinterpret_cast<float *>(&buf[warp][0][at >> 1]) + (at & 1);
+                    float *d1 = reinterpret_cast<float *>(&buf[warp][1][at >> 1]) + (at & 1);
+                    d0[0] = rj.x; d0[2] = rj.y; d1[0] = rj.z; d1[2] = rj.w;
+                    code[warp][at] = cd;
+                }
+                cnt += __popc(m);
+                if (cnt >= 32) {
+                    test(32);
+                    cnt -= 32;  // the rest (at most 31) goes to the front
+                    buf[warp][lane >> 4][lane & 15] = buf[warp][lane >> 4][16 + (lane & 15)];
+                    code[warp][lane] = code[warp][32 + lane];
+                    __syncwarp();
+                }
+            }
+            __syncwarp();
+        }
+        if (cnt) test(cnt);
+        if (p.cnt && act) p.cnt[i] = c;
+        const int cmax = (int)__reduce_max_sync(CRK_FULL_MASK, (unsigned)c);
+        if (lane == 0) {
+            if (p.overflow && (cmax > p.cap_rows || u > p.cap_table)) atomicOr(p.overflow, 1);
+            if (p.ucnt) p.ucnt[grp] = u;
+            if (p.umax) atomicMax(p.umax, u);
+        }
+        __syncwarp();
     }
 }
 
+template <bool kGas>
+void launch_list_build(crk_ctx *ctx, const crk_leaves *lv, const LeafView &v, const ListP &p, const GroupTable &gt,
+                       int64_t groups) {
+    int log_cpl = 0;  // cells of 32 per leaf, rounded up to a power of two (at most 32: one per lane)
+    while ((32 << log_cpl) < lv->max_leaf_size && log_cpl < 5) ++log_cpl;
+    const unsigned grid = (unsigned)std::max<int64_t>(1, (groups + kWarps - 1) / kWarps);
+    list_build_kernel<kGas><<<grid, kThreads, 0, ctx->stream>>>(v, p, gt, kGas ? lv->hcell : lv->gcell, log_cpl);
+    ++ctx->launches;
+}
 
 // Tiles with sub-warp i-groups: the warp's 32 i-particles form 32/G groups of
 // G consecutive (Z-ordered) particles, each with its own box and its own
@@ -2373,7 +2431,6 @@ __global__ void __launch_bounds__(kThreads) pair_kernel_sub(LeafView lv, typenam
                     if (jv) {
                         rj = rec[j];
                         S::shift(rj, im.sx, im.sy, im.sz);
-                        if constexpr (S::kTag) S::tag(rj, e - ib, j - jlo);
                     }
                     bool full = false;
 #pragma unroll
@@ -2642,7 +2699,6 @@ __global__ void __launch_bounds__(kThreads) pair_kernel_ring(LeafView lv, typena
                     if (jv) {
                         rj = rec[j];
                         S::shift(rj, im.sx, im.sy, im.sz);
-                        if constexpr (S::kTag) S::tag(rj, e - ib, j - jlo);
 #pragma unroll
                         for (int t = 0; t < 2; ++t) {
                             float dx = fmaxf(fmaxf(bl[t][0] - rj.x, rj.x - bh[t][0]), 0.f);
@@ -3546,7 +3602,6 @@ int crk_gas_groups(crk_ctx *ctx, crk_leaves *lv) {
 // smoothing lengths keep well above the largest counts; room for 1/8 more groups than this build
 // holds (a rebuild of moved particles reuses the buffers).
 int crk_gas_lists_onepass(crk_ctx *ctx, crk_leaves *lv, int32_t ngroups) {
-    using LS = ListStage<true>;
     if (no_lists(lv, true)) return CRK_OK;
     crk_nlist &out = lv->gas_lists;
     const int64_t nl = lv->n_leaves, n = lv->n;
@@ -3579,11 +3634,9 @@ int crk_gas_lists_onepass(crk_ctx *ctx, crk_leaves *lv, int32_t ngroups) {
     list_group_leaf_kernel<<<crk_grid(nl, 256), 256, 0, st>>>(nl, out.gstart, out.gleaf, capg);
     strided_offsets_kernel<<<crk_grid(capg + 1, 256), 256, 0, st>>>(capg + 1, capr, capt, out.goff, out.uoff);
     ListP pf{out.list, out.ucode, out.gstart, out.goff, out.uoff, out.cnt, out.unum, nullptr, lv->dev + 3, capr, capt,
-             lv->r_cut_grav * lv->r_cut_grav, n, nullptr};
-    const GroupTable gt{out.gstart, out.gleaf, ngroups, nullptr};
-    const unsigned gg = (unsigned)std::max<int64_t>(1, ((int64_t)ngroups + kWarps - 1) / kWarps);
-    pair_group_kernel<LS, false><<<gg, kThreads, 0, st>>>(v, pf, RecView<LS::Rec>{v.pos, n}, gt, nullptr);
-    ctx->launches += 3;
+             lv->r_cut_grav * lv->r_cut_grav};
+    launch_list_build<true>(ctx, lv, v, pf, GroupTable{out.gstart, out.gleaf, ngroups, nullptr}, ngroups);
+    ctx->launches += 2;
     CRK_LAUNCH_CHECK(ctx, "neighbour lists");
     return CRK_OK;
 }
@@ -3597,9 +3650,7 @@ static int build_lists(crk_ctx *ctx, crk_leaves *lv, crk_nlist &out, bool reuse)
     if (no_lists(lv, kGas)) return CRK_OK;
     if (reuse && (!kGas || !out.onepass)) return crk_fail(ctx, CRK_ESTATE, "rebuild: lists without fixed capacities");
     cudaStream_t st = ctx->stream;
-    using LS = ListStage<kGas>;
     const LeafView v = list_view<kGas>(lv);
-    const RecView<typename LS::Rec> rec{v.pos, n};  // a list record is the position and h
     const float rc2 = lv->r_cut_grav * lv->r_cut_grav;
     int32_t *dgroups = lv->dev + (kGas ? 1 : 2);  // this build's group count, for the kernels
     int rc;
@@ -3608,12 +3659,10 @@ static int build_lists(crk_ctx *ctx, crk_leaves *lv, crk_nlist &out, bool reuse)
         const int64_t capg = out.groups;
         list_group_leaf_kernel<<<crk_grid(nl, 256), 256, 0, st>>>(nl, out.gstart, out.gleaf, capg);
         ListP pf{out.list, out.ucode, out.gstart, out.goff, out.uoff, out.cnt, out.unum, nullptr, lv->dev + 3,
-                 kGasListCapRows, kGasTableCap, rc2, n, nullptr};
-        const GroupTable gt{out.gstart, out.gleaf, capg, dgroups};
-        const unsigned gg = (unsigned)((capg + kWarps - 1) / kWarps > 0 ? (capg + kWarps - 1) / kWarps : 1);
-        pair_group_kernel<LS, false><<<gg, kThreads, 0, st>>>(v, pf, rec, gt, nullptr);
+                 kGasListCapRows, kGasTableCap, rc2};
+        launch_list_build<kGas>(ctx, lv, v, pf, GroupTable{out.gstart, out.gleaf, capg, dgroups}, capg);
         lists_status_kernel<<<1, 1, 0, st>>>(dgroups, capg, lv->dev + 3, lv->dev);
-        ctx->launches += 3;
+        ctx->launches += 2;
         CRK_LAUNCH_CHECK(ctx, "neighbour lists");
         return CRK_OK;
     }
@@ -3635,16 +3684,15 @@ static int build_lists(crk_ctx *ctx, crk_leaves *lv, crk_nlist &out, bool reuse)
     if (!gleaf || !ucnt || !goff || !uoff || !gk) return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation");
     list_group_leaf_kernel<<<crk_grid(nl, 256), 256, 0, st>>>(nl, gstart, gleaf, ngroups);
     const GroupTable gt{gstart, gleaf, ngroups, nullptr};
-    const unsigned ggrid = (unsigned)((ngroups + kWarps - 1) / kWarps > 0 ? (ngroups + kWarps - 1) / kWarps : 1);
     CRK_CUDA(ctx, cudaMemsetAsync(ucnt, 0, sizeof(int32_t) * (size_t)(ngroups + 1), st));
     CRK_CUDA(ctx, cudaMemsetAsync(tot + 4, 0, sizeof(int32_t), st));
     ListP pc{nullptr, nullptr, gstart, nullptr, nullptr, cnt, ucnt, tot + 4, nullptr, 2147483647, 2147483647,
-             rc2, n, nullptr};
-    pair_group_kernel<LS, false><<<ggrid, kThreads, 0, st>>>(v, pc, rec, gt, nullptr);
+             rc2};
+    launch_list_build<kGas>(ctx, lv, v, pc, gt, ngroups);
     CRK_LAUNCH_CHECK(ctx, "neighbour counts");
     CRK_CUDA(ctx, cudaMemsetAsync(gk, 0, sizeof(int32_t) * (size_t)(ngroups + 1), st));
     list_group_k_kernel<<<(unsigned)nl, kThreads, 0, st>>>(nl, lv->leaf_start, lv->leaf_ngas, kGas, gstart, cnt, gk);
-    ctx->launches += 3;
+    ctx->launches += 2;
     rc = crk_exclusive_scan_i32(ctx, gk, goff, ngroups + 1, tot + 1);
     if (rc) return rc;
     rc = crk_exclusive_scan_i32(ctx, ucnt, uoff, ngroups + 1, tot + 2);
@@ -3666,9 +3714,8 @@ static int build_lists(crk_ctx *ctx, crk_leaves *lv, crk_nlist &out, bool reuse)
     if (!list || !ucode)
         return crk_fail(ctx, CRK_ENOMEM, "neighbour list allocation (%lld entries)", (long long)entries);
     ListP pf{list, ucode, gstart, goff, uoff, nullptr, nullptr, nullptr, nullptr, 2147483647, 2147483647,
-             rc2, n, nullptr};
-    pair_group_kernel<LS, false><<<ggrid, kThreads, 0, st>>>(v, pf, rec, gt, nullptr);
-    ++ctx->launches;
+             rc2};
+    launch_list_build<kGas>(ctx, lv, v, pf, gt, ngroups);
     CRK_LAUNCH_CHECK(ctx, "neighbour lists");
     out.unum = ucnt;
     out.uoff = uoff;
