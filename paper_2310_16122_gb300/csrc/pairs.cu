@@ -675,21 +675,66 @@ struct CorrStage {
     __host__ __device__ static constexpr int idx3(int a, int b, int c) {
         return a == 0 ? (b == 0 ? c : (b == 1 ? 2 + c : 5)) : (a == 1 ? (b == 1 ? 5 + c : 8) : 9);
     }
-    // the full gradient moments dm1[g][a] and dm2[g][ab] (ab packed) from m0, m1, s2, s3
-    __device__ static void grad_moments(const I &s, double m0, const double m1[3], double dm1[3][3],
-                                        double dm2[3][6]) {
+    // The FP64 part of one particle (FP64 runs at 1/64 of the FP32 rate here and bounds the finish, so
+    // the products are arranged around the symmetric sums).  With q = m0 + B.m1 = 1/A, T = s3 B (the
+    // symmetric matrix sum_b s3_abg B_b) and U = s2 + T,
+    //   dm1_g + dm2_g B = q e_g + U_g + B_g m1  (U_g: column g)  and  m2^-1 m1 = -B, so
+    //   dB_g = -m2^-1 U_g + B_g B - q m2^-1 e_g,
+    //   dm0_g + 2 B.dm1_g + B^T dm2_g B = dm0_g + 2 q B_g + ((2 s2 + T) B)_g.
+    // Matrices are packed xx xy xz yy yz zz.
+    struct Solved {
+        double Mi[6], m1[3], B[3], q, A, T[6], U[6], K[3];
+    };
+    __device__ static double at(const double m[6], int a, int b) { return m[a <= b ? idx2(a, b) : idx2(b, a)]; }
+    // row a of the symmetric matrix m times v
+    __device__ static double row(const double m[6], int a, const double v[3]) {
+        return at(m, a, 0) * v[0] + at(m, a, 1) * v[1] + at(m, a, 2) * v[2];
+    }
+    // false for a singular particle
+    template <class Sums>
+    __device__ static bool solve(const Sums &s, Solved &r) {
+        double M[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) M[q] = (double)s.m2[q] - (double)s.c2[q];
+        // cofactors of the symmetric matrix
+        r.Mi[0] = M[3] * M[5] - M[4] * M[4];
+        r.Mi[1] = M[2] * M[4] - M[1] * M[5];
+        r.Mi[2] = M[1] * M[4] - M[2] * M[3];
+        r.Mi[3] = M[0] * M[5] - M[2] * M[2];
+        r.Mi[4] = M[1] * M[2] - M[0] * M[4];
+        r.Mi[5] = M[0] * M[3] - M[1] * M[1];
+        const double det = M[0] * r.Mi[0] + M[1] * r.Mi[1] + M[2] * r.Mi[2];
+        const double tr = M[0] + M[3] + M[5];
+        if (!(det > 1e-12 * tr * tr * tr)) return false;
+        const double id = 1.0 / det;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) r.Mi[q] *= id;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) r.m1[a] = (double)s.m1[a] - (double)s.c1[a];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) r.B[a] = -row(r.Mi, a, r.m1);
+        r.q = (double)s.m0 - (double)s.c0 + (r.B[0] * r.m1[0] + r.B[1] * r.m1[1] + r.B[2] * r.m1[2]);
+        r.A = 1.0 / r.q;
+        double s2[6], s3[10], W[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) s2[k] = (double)s.s2[k];
+#pragma unroll
+        for (int k = 0; k < 10; ++k) s3[k] = (double)s.s3[k];
         const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
-        for (int g = 0; g < 3; ++g) {
-            for (int a = 0; a < 3; ++a)
-                dm1[g][a] = (a == g ? m0 : 0.0) + (double)s.s2[a < g ? idx2(a, g) : idx2(g, a)];
-            for (int q = 0; q < 6; ++q) {
-                int t0 = ia[q], t1 = ib[q], t2 = g;  // sort (a, b, g); a <= b already
-                if (t2 < t1) { t2 = t1; t1 = g; }
-                if (t1 < t0) { int u = t0; t0 = t1; t1 = u; }
-                dm2[g][q] = (ia[q] == g ? m1[ib[q]] : 0.0) + (ib[q] == g ? m1[ia[q]] : 0.0) +
-                            (double)s.s3[idx3(t0, t1, t2)];
-            }
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            r.T[k] = s3[sorted3(ia[k], ib[k], 0)] * r.B[0] + s3[sorted3(ia[k], ib[k], 1)] * r.B[1] +
+                     s3[sorted3(ia[k], ib[k], 2)] * r.B[2];
+            r.U[k] = s2[k] + r.T[k];
+            W[k] = s2[k] + r.U[k];  // 2 s2 + T
         }
+#pragma unroll
+        for (int g = 0; g < 3; ++g) r.K[g] = (double)s.dm0[g] + 2.0 * r.q * r.B[g] + row(W, g, r.B);
+        return true;
+    }
+    // packed index of the sorted axes of (a <= b) and c
+    __host__ __device__ static constexpr int sorted3(int a, int b, int c) {
+        return c >= b ? idx3(a, b, c) : (c >= a ? idx3(a, c, b) : idx3(c, a, b));
     }
     __device__ static Rec gather(const P &p, int32_t o, float4 ps) { return {ps.x, ps.y, ps.z, ps.w, p.V[o], 0, 0, 0}; }
     __device__ static float box_cut(const P &, float hmax_i, const Rec &rj) { return hmax_i + rj.h; }
@@ -739,21 +784,9 @@ struct CorrStage {
         if (kCount) s.cnt += in;
     }
     __device__ static void finish(const P &p, I &s, const Rec &, int32_t o, int64_t) {
-        double m0 = (double)s.m0 - (double)s.c0;
-        double m1[3], M[3][3];
-        for (int a = 0; a < 3; ++a) m1[a] = (double)s.m1[a] - (double)s.c1[a];
-        const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
-        for (int q = 0; q < 6; ++q) {
-            double v = (double)s.m2[q] - (double)s.c2[q];
-            M[ia[q]][ib[q]] = v;
-            M[ib[q]][ia[q]] = v;
-        }
-        double det = M[0][0] * (M[1][1] * M[2][2] - M[1][2] * M[2][1]) -
-                     M[0][1] * (M[1][0] * M[2][2] - M[1][2] * M[2][0]) +
-                     M[0][2] * (M[1][0] * M[2][1] - M[1][1] * M[2][0]);
-        double tr = M[0][0] + M[1][1] + M[2][2];
         const int64_t n = p.n;
-        if (!(det > 1e-12 * tr * tr * tr)) {
+        Solved r;
+        if (!solve(s, r)) {
             const float nan = __int_as_float(0x7fc00000);
             p.A[o] = nan;
             for (int a = 0; a < 3; ++a) { p.B[a * n + o] = nan; p.gA[a * n + o] = nan; }
@@ -761,40 +794,17 @@ struct CorrStage {
             if (p.n_singular) atomicAdd(p.n_singular, 1);
             return;
         }
-        double Mi[3][3];
-        double id = 1.0 / det;
-        Mi[0][0] = (M[1][1] * M[2][2] - M[1][2] * M[2][1]) * id;
-        Mi[0][1] = (M[0][2] * M[2][1] - M[0][1] * M[2][2]) * id;
-        Mi[0][2] = (M[0][1] * M[1][2] - M[0][2] * M[1][1]) * id;
-        Mi[1][0] = Mi[0][1];
-        Mi[1][1] = (M[0][0] * M[2][2] - M[0][2] * M[2][0]) * id;
-        Mi[1][2] = (M[0][2] * M[1][0] - M[0][0] * M[1][2]) * id;
-        Mi[2][0] = Mi[0][2];
-        Mi[2][1] = Mi[1][2];
-        Mi[2][2] = (M[0][0] * M[1][1] - M[0][1] * M[1][0]) * id;
-        double B[3];
-        for (int a = 0; a < 3; ++a) B[a] = -(Mi[a][0] * m1[0] + Mi[a][1] * m1[1] + Mi[a][2] * m1[2]);
-        double A = 1.0 / (m0 + B[0] * m1[0] + B[1] * m1[1] + B[2] * m1[2]);
-        p.A[o] = (float)A;
-        for (int a = 0; a < 3; ++a) p.B[a * n + o] = (float)B[a];
-        double dm1[3][3], dm2[3][6];
-        grad_moments(s, m0, m1, dm1, dm2);
+        p.A[o] = (float)r.A;
+        const double A2 = -r.A * r.A;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) p.B[a * n + o] = (float)r.B[a];
+#pragma unroll
         for (int g = 0; g < 3; ++g) {
-            double dM[3][3];
-            for (int q = 0; q < 6; ++q) {
-                dM[ia[q]][ib[q]] = dm2[g][q];
-                dM[ib[q]][ia[q]] = dm2[g][q];
-            }
-            double t[3], BdMB = 0.0, Bdm1 = 0.0;
-            for (int a = 0; a < 3; ++a) {
-                double dMB = dM[a][0] * B[0] + dM[a][1] * B[1] + dM[a][2] * B[2];
-                t[a] = dm1[g][a] + dMB;
-                BdMB += B[a] * dMB;
-                Bdm1 += B[a] * dm1[g][a];
-            }
-            p.gA[g * n + o] = (float)(-A * A * ((double)s.dm0[g] + 2.0 * Bdm1 + BdMB));
+            p.gA[g * n + o] = (float)(A2 * r.K[g]);
+            const double u[3] = {at(r.U, 0, g), at(r.U, 1, g), at(r.U, 2, g)};
+#pragma unroll
             for (int a = 0; a < 3; ++a)
-                p.gB[(3 * g + a) * n + o] = (float)(-(Mi[a][0] * t[0] + Mi[a][1] * t[1] + Mi[a][2] * t[2]));
+                p.gB[(3 * g + a) * n + o] = (float)(r.B[a] * r.B[g] - row(r.Mi, a, u) - r.q * at(r.Mi, a, g));
         }
     }
     __device__ static void finish_other(const P &p, int32_t o) {
@@ -826,197 +836,106 @@ struct CorrAdjP : CorrP {
 struct CorrAdjPrepStage : CorrStage {
     static constexpr bool kAllVariants = false;
     using P = CorrAdjP;
-    // The preparation sweep accumulates the gradient moments in full (30 sums, not the forward's
-    // symmetric s2/s3): with its FP64 finish the symmetric form measured slower here.
-    struct I {
-        float m0, c0;
-        float m1[3], c1[3];
-        float m2[6], c2[6];  // xx xy xz yy yz zz
-        float dm0[3];
-        float dm1[9];   // [g][a]
-        float dm2[18];  // [g][ab]
-        int cnt;
-    };
-    __device__ static void init(const P &, I &s, const Rec &, int64_t, int, int, int32_t) {
-        s.m0 = s.c0 = 0.f;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) s.m1[a] = s.c1[a] = s.dm0[a] = 0.f;
-#pragma unroll
-        for (int a = 0; a < 6; ++a) s.m2[a] = s.c2[a] = 0.f;
-#pragma unroll
-        for (int a = 0; a < 9; ++a) s.dm1[a] = 0.f;
-#pragma unroll
-        for (int a = 0; a < 18; ++a) s.dm2[a] = 0.f;
-        s.cnt = 0;
-    }
-    template <bool kCount>
-    __device__ static void interact(const P &, I &s, const Rec &ri, const Rec &rj) {
-        float x[3] = {ri.x - rj.x, ri.y - rj.y, ri.z - rj.z};  // x_ij
-        float r2 = fmaf(x[0], x[0], fmaf(x[1], x[1], x[2] * x[2]));
-        float hs = ri.h + rj.h;
-        bool in = r2 < hs * hs;
-        float W, dWr;
-        wendland(r2, 0.5f * hs, W, dWr);
-        float w = in ? rj.V * W : 0.0f;
-        float vd = in ? rj.V * dWr : 0.0f;
-        float wx[3] = {w * x[0], w * x[1], w * x[2]};
-        float dW[3] = {vd * x[0], vd * x[1], vd * x[2]};  // V_j d_g W
-        kahan_add(s.m0, s.c0, w);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) kahan_add(s.m1[a], s.c1[a], wx[a]);
-        const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
-        float xx[6];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) {
-            xx[q] = x[ia[q]] * x[ib[q]];
-            kahan_add(s.m2[q], s.c2[q], wx[ia[q]] * x[ib[q]]);
-        }
-#pragma unroll
-        for (int g = 0; g < 3; ++g) {
-            s.dm0[g] += dW[g];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) s.dm1[3 * g + a] = fmaf(x[a], dW[g], s.dm1[3 * g + a] + (a == g ? w : 0.0f));
-#pragma unroll
-            for (int q = 0; q < 6; ++q) {
-                float t = (ia[q] == g ? wx[ib[q]] : 0.0f) + (ib[q] == g ? wx[ia[q]] : 0.0f);
-                s.dm2[6 * g + q] = fmaf(xx[q], dW[g], s.dm2[6 * g + q] + t);
-            }
-        }
-        if (kCount) s.cnt += in;
-    }
+    // Reverse of CorrStage's Solved, in the sums m0, m1, m2, dm0, s2, s3 themselves, whose cotangents
+    // are the polynomial coefficients.  H_ga: the cotangent of dB_g^a (row g).  The sweep is CorrStage's
+    // and the FP64 of this finish bounds the rest: 422 -> 295 us on the 2x64^3 box against the reverse
+    // taken through the 30 unreduced sums dm1, dm2.
     __device__ static void finish(const P &p, I &s, const Rec &, int32_t o, int64_t) {
         const int64_t n = p.n;
-        const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
-        double m0 = (double)s.m0 - (double)s.c0, m1[3], M[3][3];
-        for (int a = 0; a < 3; ++a) m1[a] = (double)s.m1[a] - (double)s.c1[a];
-        for (int q = 0; q < 6; ++q) {
-            double v = (double)s.m2[q] - (double)s.c2[q];
-            M[ia[q]][ib[q]] = v;
-            M[ib[q]][ia[q]] = v;
-        }
-        double det = M[0][0] * (M[1][1] * M[2][2] - M[1][2] * M[2][1]) -
-                     M[0][1] * (M[1][0] * M[2][2] - M[1][2] * M[2][0]) +
-                     M[0][2] * (M[1][0] * M[2][1] - M[1][1] * M[2][0]);
-        double tr = M[0][0] + M[1][1] + M[2][2];
-        if (!(det > 1e-12 * tr * tr * tr)) {  // singular: contributes nothing
+        Solved r;
+        if (!solve(s, r)) {  // singular: contributes nothing
             for (int k = 0; k < kCorrCoef; ++k) p.coef[k * n + o] = 0.f;
             if (p.n_singular) atomicAdd(p.n_singular, 1);
             return;
         }
-        double Mi[3][3];
-        double id = 1.0 / det;
-        Mi[0][0] = (M[1][1] * M[2][2] - M[1][2] * M[2][1]) * id;
-        Mi[0][1] = (M[0][2] * M[2][1] - M[0][1] * M[2][2]) * id;
-        Mi[0][2] = (M[0][1] * M[1][2] - M[0][2] * M[1][1]) * id;
-        Mi[1][1] = (M[0][0] * M[2][2] - M[0][2] * M[2][0]) * id;
-        Mi[1][2] = (M[0][2] * M[1][0] - M[0][0] * M[1][2]) * id;
-        Mi[2][2] = (M[0][0] * M[1][1] - M[0][1] * M[1][0]) * id;
-        Mi[1][0] = Mi[0][1];
-        Mi[2][0] = Mi[0][2];
-        Mi[2][1] = Mi[1][2];
-        double B[3], Bb[3], Mib[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-        for (int a = 0; a < 3; ++a) B[a] = -(Mi[a][0] * m1[0] + Mi[a][1] * m1[1] + Mi[a][2] * m1[2]);
-        double A = 1.0 / (m0 + B[0] * m1[0] + B[1] * m1[1] + B[2] * m1[2]);
-        for (int a = 0; a < 3; ++a) Bb[a] = (double)p.Bbar[a * n + o];
-        double Ab = (double)p.Abar[o];
-        // moment cotangents: dm1b[g][a], dm2b[g][ab] (symmetric in ab, packed as ia/ib)
-        double m0b = 0.0, m1b[3] = {0, 0, 0}, dm0b[3], dm1b[3][3], dm2b[3][6];
-        double dm1[3][3], dm2[3][6];
+        float *coef = p.coef + o;
+        double H[3][3], Kb[3], Bb[3], Ab = (double)p.Abar[o], qb = 0.0;
+        const double A2 = -r.A * r.A;
+#pragma unroll
         for (int g = 0; g < 3; ++g) {
-            for (int a = 0; a < 3; ++a) dm1[g][a] = (double)s.dm1[3 * g + a];
-            for (int q = 0; q < 6; ++q) dm2[g][q] = (double)s.dm2[6 * g + q];
-        }
-        for (int g = 0; g < 3; ++g) {
-            double dM[3][3], t[3], tb[3], K = (double)s.dm0[g];
-            for (int q = 0; q < 6; ++q) {
-                dM[ia[q]][ib[q]] = dm2[g][q];
-                dM[ib[q]][ia[q]] = dm2[g][q];
-            }
-            for (int a = 0; a < 3; ++a) {
-                t[a] = dm1[g][a] + dM[a][0] * B[0] + dM[a][1] * B[1] + dM[a][2] * B[2];
-                K += 2.0 * B[a] * dm1[g][a] + B[a] * (dM[a][0] * B[0] + dM[a][1] * B[1] + dM[a][2] * B[2]);
-            }
-            double gb[3];
-            for (int a = 0; a < 3; ++a) gb[a] = (double)p.gBbar[(3 * g + a) * n + o];
-            for (int a = 0; a < 3; ++a) tb[a] = -(Mi[a][0] * gb[0] + Mi[a][1] * gb[1] + Mi[a][2] * gb[2]);
-            for (int a = 0; a < 3; ++a)
-                for (int b = 0; b < 3; ++b) Mib[a][b] -= gb[a] * t[b];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) H[g][a] = (double)p.gBbar[(3 * g + a) * n + o];
             const double gAb = (double)p.gAbar[g * n + o];
-            const double Kb = -A * A * gAb;
-            Ab += -2.0 * A * K * gAb;
-            dm0b[g] = Kb;
-            for (int a = 0; a < 3; ++a) {
-                dm1b[g][a] = tb[a] + 2.0 * B[a] * Kb;
-                Bb[a] += tb[0] * dM[0][a] + tb[1] * dM[1][a] + tb[2] * dM[2][a];  // dM symmetric
-                Bb[a] += 2.0 * dm1[g][a] * Kb + 2.0 * (dM[a][0] * B[0] + dM[a][1] * B[1] + dM[a][2] * B[2]) * Kb;
-            }
-            // dm2b[g][a][b] = tb_a B_b + B_a B_b Kb, summed over (a, b) and (b, a) for a packed
-            // off-diagonal entry (the moment sums are symmetric in ab)
-            for (int q = 0; q < 6; ++q) {
-                const int a = ia[q], b = ib[q];
-                double v = tb[a] * B[b] + B[a] * B[b] * Kb;
-                if (a != b) v += tb[b] * B[a] + B[b] * B[a] * Kb;
-                dm2b[g][q] = v;
-            }
+            Bb[g] = (double)p.Bbar[g * n + o];
+            Kb[g] = A2 * gAb;
+            Ab -= 2.0 * r.A * r.K[g] * gAb;
+            coef[(10 + g) * n] = (float)Kb[g];  // l1: dm0
         }
-        const double denb = -A * A * Ab;
-        m0b += denb;
-        for (int a = 0; a < 3; ++a) {
-            Bb[a] += m1[a] * denb;
-            m1b[a] += B[a] * denb;
-        }
-        for (int a = 0; a < 3; ++a) {
-            m1b[a] -= Mi[0][a] * Bb[0] + Mi[1][a] * Bb[1] + Mi[2][a] * Bb[2];
-            for (int b = 0; b < 3; ++b) Mib[a][b] -= Bb[a] * m1[b];
-        }
-        // m2b = -Mi^T Mib Mi^T = -Mi (Mib Mi) (Mi symmetric): two 3x3 products (FP64 is 1/64 rate)
-        double T[3][3], m2b[3][3];
-        for (int c = 0; c < 3; ++c)
-            for (int b = 0; b < 3; ++b) T[c][b] = Mib[c][0] * Mi[0][b] + Mib[c][1] * Mi[1][b] + Mib[c][2] * Mi[2][b];
+        // dB_g^a = B_a B_g - (Mi U)_ag - q Mi_ag and K_g = dm0_g + 2 q B_g + ((2 s2 + T) B)_g
+        double Mib[3][3], Ub[3][3];
+#pragma unroll
         for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) m2b[a][b] = -(Mi[a][0] * T[0][b] + Mi[a][1] * T[1][b] + Mi[a][2] * T[2][b]);
-        // polynomial coefficients.  dm2b enters as sum_{g,ab} dm2b[g][ab] (delta_ag x_b W +
-        // delta_bg x_a W + x_a x_b x_g dWr) with the packed (a <= b) entries carrying both orders.
-        double c[kCorrCoef];
-        c[0] = m0b + dm1b[0][0] + dm1b[1][1] + dm1b[2][2];
-        for (int e = 0; e < 3; ++e) c[1 + e] = m1b[e];
-        for (int g = 0; g < 3; ++g)
-            for (int q = 0; q < 6; ++q) {
-                const int a = ia[q], b = ib[q];
-                // delta_ag x_b + delta_bg x_a (for a = b = g: 2 x_a)
-                if (a == g) c[1 + b] += dm2b[g][q];
-                if (b == g) c[1 + a] += dm2b[g][q];
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                Mib[a][b] = -(H[0][a] * at(r.U, b, 0) + H[1][a] * at(r.U, b, 1) + H[2][a] * at(r.U, b, 2)) - r.q * H[b][a];
+                Ub[a][b] = -(at(r.Mi, a, 0) * H[b][0] + at(r.Mi, a, 1) * H[b][1] + at(r.Mi, a, 2) * H[b][2]);
+                qb -= H[b][a] * at(r.Mi, a, b);
             }
-        // q0: x^T m2b x as monomials
-        c[4] = m2b[0][0];
-        c[5] = m2b[0][1] + m2b[1][0];
-        c[6] = m2b[0][2] + m2b[2][0];
-        c[7] = m2b[1][1];
-        c[8] = m2b[1][2] + m2b[2][1];
-        c[9] = m2b[2][2];
-        for (int e = 0; e < 3; ++e) c[10 + e] = dm0b[e];
-        // q1: sum_ga dm1b[g][a] x_a x_g
-        c[13] = dm1b[0][0];
-        c[14] = dm1b[0][1] + dm1b[1][0];
-        c[15] = dm1b[0][2] + dm1b[2][0];
-        c[16] = dm1b[1][1];
-        c[17] = dm1b[1][2] + dm1b[2][1];
-        c[18] = dm1b[2][2];
-        // k: sum_{g,ab} dm2b[g][ab] x_g x_a x_b (packed entries already hold both ab orders)
-        for (int e = 0; e < 10; ++e) c[19 + e] = 0.0;
-        for (int g = 0; g < 3; ++g)
-            for (int q = 0; q < 6; ++q) {
-                int t[3] = {g, ia[q], ib[q]};
-                // sort the three axes to find the monomial
-                if (t[0] > t[1]) { int u = t[0]; t[0] = t[1]; t[1] = u; }
-                if (t[1] > t[2]) { int u = t[1]; t[1] = t[2]; t[2] = u; }
-                if (t[0] > t[1]) { int u = t[0]; t[0] = t[1]; t[1] = u; }
-                // index of (t0 <= t1 <= t2) among xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz
-                const int idx = t[0] == 0 ? (t[1] == 0 ? t[2] : (t[1] == 1 ? 2 + t[2] : 5))
-                                          : (t[0] == 1 ? (t[1] == 1 ? 6 + (t[2] - 1) : 8) : 9);
-                c[19 + idx] += dm2b[g][q];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+#pragma unroll
+            for (int g = 0; g < 3; ++g) {
+                // 2 s2 + T = s2 + U
+                Bb[a] += (H[g][a] + H[a][g]) * r.B[g] + Kb[g] * ((double)s.s2[a <= g ? idx2(a, g) : idx2(g, a)] + at(r.U, a, g));
             }
-        for (int k = 0; k < kCorrCoef; ++k) p.coef[k * n + o] = (float)c[k];
+            Bb[a] += 2.0 * r.q * Kb[a];
+            qb += 2.0 * Kb[a] * r.B[a];
+        }
+        // s2 and T cotangents, one entry per monomial x_a x_b (both orders of an off-diagonal pair)
+        double Tb[6];
+        const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const int a = ia[k], b = ib[k];
+            const double w = a == b ? Kb[a] * r.B[a] : Kb[a] * r.B[b] + Kb[b] * r.B[a];
+            Tb[k] = (a == b ? Ub[a][a] : Ub[a][b] + Ub[b][a]) + w;
+            coef[(13 + k) * n] = (float)(Tb[k] + w);  // q1: s2
+        }
+        // T = s3 B: Bb_c += sum_ab Tb_ab s3_abc, and s3's coefficients are those of (x^T Tb x)(B.x)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int k = 0; k < 6; ++k) Bb[c] += Tb[k] * (double)s.s3[sorted3(ia[k], ib[k], c)];
+        const double *B = r.B;
+        const double k3[10] = {Tb[0] * B[0],
+                               Tb[0] * B[1] + Tb[1] * B[0],
+                               Tb[0] * B[2] + Tb[2] * B[0],
+                               Tb[1] * B[1] + Tb[3] * B[0],
+                               Tb[1] * B[2] + Tb[2] * B[1] + Tb[4] * B[0],
+                               Tb[2] * B[2] + Tb[5] * B[0],
+                               Tb[3] * B[1],
+                               Tb[3] * B[2] + Tb[4] * B[1],
+                               Tb[4] * B[2] + Tb[5] * B[1],
+                               Tb[5] * B[2]};
+#pragma unroll
+        for (int k = 0; k < 10; ++k) coef[(19 + k) * n] = (float)k3[k];
+        // A = 1/q, q = m0 + B.m1, B = -Mi m1, Mi = m2^-1
+        qb += A2 * Ab;
+        coef[0] = (float)qb;  // c0: m0
+#pragma unroll
+        for (int a = 0; a < 3; ++a) Bb[a] += qb * r.m1[a];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            coef[(1 + a) * n] = (float)(qb * r.B[a] - row(r.Mi, a, Bb));  // l0: m1
+#pragma unroll
+            for (int b = 0; b < 3; ++b) Mib[a][b] -= Bb[a] * r.m1[b];
+        }
+        // m2's cotangent -Mi Mib Mi, per monomial: -Mi (Mib + Mib^T) Mi off the diagonal, half of it on it
+        double S[6], Y[3][3];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) S[k] = ia[k] == ib[k] ? 2.0 * Mib[ia[k]][ia[k]] : Mib[ia[k]][ib[k]] + Mib[ib[k]][ia[k]];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                const double c[3] = {at(r.Mi, 0, b), at(r.Mi, 1, b), at(r.Mi, 2, b)};
+                Y[a][b] = row(S, a, c);
+            }
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const double c[3] = {Y[0][ib[k]], Y[1][ib[k]], Y[2][ib[k]]};
+            coef[(4 + k) * n] = (float)((ia[k] == ib[k] ? -0.5 : -1.0) * row(r.Mi, ia[k], c));  // q0: m2
+        }
     }
     __device__ static void finish_other(const P &p, int32_t o) {
         for (int k = 0; k < kCorrCoef; ++k) p.coef[k * p.n + o] = 0.f;
@@ -2815,6 +2734,11 @@ template <>
 struct list_min_blocks<CorrStage> {
     static constexpr int value = 5;
 };
+// its reverse preparation: four blocks 295 us on the 2x64^3 box, five 299, uncapped 329
+template <>
+struct list_min_blocks<CorrAdjPrepStage> {
+    static constexpr int value = 4;
+};
 
 // index rows in flight in list_kernel<S>: 8 for the short pair terms (records of at most 32
 // bytes and few registers), 4 for the long ones
@@ -2844,6 +2768,10 @@ struct flat_tail<GeomAdjStage> {
 };
 template <>
 struct flat_tail<CorrStage> {
+    static constexpr bool value = true;
+};
+template <>
+struct flat_tail<CorrAdjPrepStage> {
     static constexpr bool value = true;
 };
 template <>
