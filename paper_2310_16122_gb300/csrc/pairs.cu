@@ -168,6 +168,74 @@ __device__ __forceinline__ void kahan_add(float &s, float &c, float v) {
     s = t;
 }
 
+// A value as the unevaluated sum h + l of two floats (h the rounded sum, 2^-47 relative): error-free
+// transformations of Dekker (1971) and Knuth, products by FMA.  4-15 FP32 instructions an operation,
+// each issued at 64 times the rate of an FP64 one.  Not for infinities or results near the subnormals.
+struct Two {
+    float h, l;
+};
+__device__ __forceinline__ Two quick_two(float a, float b) {  // |a| >= |b|, or a = 0
+    const float s = __fadd_rn(a, b);
+    return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ Two sum_two(float a, float b) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ Two prod_two(Two a, Two b) {  // not normalised
+    const float p = __fmul_rn(a.h, b.h);
+    return {p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ Two prod_two(Two a, float b) {
+    const float p = __fmul_rn(a.h, b);
+    return {p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p))};
+}
+__device__ __forceinline__ Two plus_two(Two a, Two b) {  // not normalised
+    const Two s = sum_two(a.h, b.h);
+    return {s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
+}
+__device__ __forceinline__ Two norm_two(Two a) { return quick_two(a.h, a.l); }
+__device__ __forceinline__ Two operator-(Two a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ Two operator+(Two a, Two b) { return norm_two(plus_two(a, b)); }
+__device__ __forceinline__ Two operator+(Two a, float b) {
+    const Two s = sum_two(a.h, b);
+    return quick_two(s.h, __fadd_rn(s.l, a.l));
+}
+__device__ __forceinline__ Two operator*(Two a, Two b) { return norm_two(prod_two(a, b)); }
+__device__ __forceinline__ Two operator*(Two a, float b) { return norm_two(prod_two(a, b)); }
+// the same operations in FP64, so that code over either type reads alike
+template <class B>
+__device__ __forceinline__ Two mad(Two a, B b, Two c) { return norm_two(plus_two(c, prod_two(a, b))); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+template <class B>
+__device__ __forceinline__ Two dot3(Two a0, B b0, Two a1, B b1, Two a2, B b2) {
+    return norm_two(plus_two(plus_two(prod_two(a0, b0), prod_two(a1, b1)), prod_two(a2, b2)));
+}
+__device__ __forceinline__ double dot3(double a0, double b0, double a1, double b1, double a2, double b2) {
+    return fma(a2, b2, fma(a1, b1, a0 * b0));
+}
+__device__ __forceinline__ Two twice(Two a) { return {2.0f * a.h, 2.0f * a.l}; }
+__device__ __forceinline__ double twice(double a) { return 2.0 * a; }
+__device__ __forceinline__ Two inverse(Two a) {
+    const float r = 1.0f / a.h;
+    return quick_two(r, __fmul_rn(r, __fmaf_rn(-r, a.l, __fmaf_rn(-r, a.h, 1.0f))));
+}
+__device__ __forceinline__ double inverse(double a) { return 1.0 / a; }
+__device__ __forceinline__ float rounded(Two a) { return a.h; }  // normalised values
+__device__ __forceinline__ float rounded(double a) { return (float)a; }
+// exact difference of two floats
+__device__ __forceinline__ void difference(float a, float b, Two &d) { d = sum_two(a, -b); }
+__device__ __forceinline__ void difference(double a, double b, double &d) { d = a - b; }
+// what a float is read as beside a T
+template <class T>
+struct beside {
+    using type = double;
+};
+template <>
+struct beside<Two> {
+    using type = float;
+};
+
 // 1/sqrt(x), 1/x and a/x by the hardware approximations for arguments that are normal numbers:
 // rsqrtf and __fdividef wrap the same approximation in a scaling for subnormal x, four
 // instructions per pair that no argument here needs.  Gravity's x = r^2 + eps^2 may be subnormal
@@ -675,61 +743,84 @@ struct CorrStage {
     __host__ __device__ static constexpr int idx3(int a, int b, int c) {
         return a == 0 ? (b == 0 ? c : (b == 1 ? 2 + c : 5)) : (a == 1 ? (b == 1 ? 5 + c : 8) : 9);
     }
-    // The FP64 part of one particle (FP64 runs at 1/64 of the FP32 rate here and bounds the finish, so
-    // the products are arranged around the symmetric sums).  With q = m0 + B.m1 = 1/A, T = s3 B (the
-    // symmetric matrix sum_b s3_abg B_b) and U = s2 + T,
+    // The solve of one particle.  With q = m0 + B.m1 = 1/A, T = s3 B (the symmetric matrix
+    // sum_b s3_abg B_b) and U = s2 + T,
     //   dm1_g + dm2_g B = q e_g + U_g + B_g m1  (U_g: column g)  and  m2^-1 m1 = -B, so
-    //   dB_g = -m2^-1 U_g + B_g B - q m2^-1 e_g,
+    //   dB_g = -m2^-1 (U_g + q e_g) + B_g B,
     //   dm0_g + 2 B.dm1_g + B^T dm2_g B = dm0_g + 2 q B_g + ((2 s2 + T) B)_g.
-    // Matrices are packed xx xy xz yy yz zz.
+    // Matrices are packed xx xy xz yy yz zz; Uq is U with q added on its diagonal.
+    // T = Two: lengths in units of a power of two near sqrt(tr m2), which keeps the FP32 exponents
+    // in range.  FP64 runs at 1/64 of the FP32 rate here: with it the solve took a third of the kernel
+    // (2x64^3: 164 us, now 127; 2x128^3 in the kernel order 1.15 ms, now 0.91; the reverse's
+    // preparation 295 us, now 260).  Only a particle that is close to singular (det m2 < 1e-6 tr^3,
+    // where 47 bits could show) or out of range goes through FP64.
+    template <class T>
     struct Solved {
-        double Mi[6], m1[3], B[3], q, A, T[6], U[6], K[3];
+        using F = typename beside<T>::type;
+        T Mi[6], m1[3], B[3], q, A, U[6], Uq[6], K[3];
+        F s3[10], f1, g1;  // third sums in scaled lengths; scale of a length and its inverse
     };
-    __device__ static double at(const double m[6], int a, int b) { return m[a <= b ? idx2(a, b) : idx2(b, a)]; }
+    template <class T>
+    __device__ static T at(const T m[6], int a, int b) { return m[a <= b ? idx2(a, b) : idx2(b, a)]; }
     // row a of the symmetric matrix m times v
-    __device__ static double row(const double m[6], int a, const double v[3]) {
-        return at(m, a, 0) * v[0] + at(m, a, 1) * v[1] + at(m, a, 2) * v[2];
+    template <class T>
+    __device__ static T row(const T m[6], int a, const T v[3]) {
+        return dot3(at(m, a, 0), v[0], at(m, a, 1), v[1], at(m, a, 2), v[2]);
     }
-    // false for a singular particle
-    template <class Sums>
-    __device__ static bool solve(const Sums &s, Solved &r) {
-        double M[6];
+    __device__ static void scale_of(float tr, double &f1, double &g1) { f1 = g1 = 1.0; }
+    __device__ static void scale_of(float tr, float &f1, float &g1) {
+        const int half = max((((__float_as_int(tr) >> 23) & 255) - 127) >> 1, -63);
+        f1 = __int_as_float((127 - half) << 23);
+        g1 = __int_as_float((127 + half) << 23);
+    }
+    // is det m2 large enough for T, in scaled lengths
+    __device__ static bool regular(double det, double tr, float) { return det > 1e-12 * tr * tr * tr; }
+    __device__ static bool regular(Two det, Two tr, float m0) {
+        return det.h > 1e-6f * tr.h * tr.h * tr.h && m0 > 1e-12f && m0 < 1e12f;
+    }
+    // false for a singular particle (FP64) or one that needs FP64 (Two)
+    template <class T, class Sums>
+    __device__ static bool solve(const Sums &s, Solved<T> &r) {
+        using F = typename beside<T>::type;
+        scale_of(s.m2[0] + s.m2[3] + s.m2[5], r.f1, r.g1);
+        const F f1 = r.f1, f2 = f1 * f1;
+        T M[6];
 #pragma unroll
-        for (int q = 0; q < 6; ++q) M[q] = (double)s.m2[q] - (double)s.c2[q];
+        for (int k = 0; k < 6; ++k) difference((F)s.m2[k] * f2, (F)s.c2[k] * f2, M[k]);
         // cofactors of the symmetric matrix
-        r.Mi[0] = M[3] * M[5] - M[4] * M[4];
-        r.Mi[1] = M[2] * M[4] - M[1] * M[5];
-        r.Mi[2] = M[1] * M[4] - M[2] * M[3];
-        r.Mi[3] = M[0] * M[5] - M[2] * M[2];
-        r.Mi[4] = M[1] * M[2] - M[0] * M[4];
-        r.Mi[5] = M[0] * M[3] - M[1] * M[1];
-        const double det = M[0] * r.Mi[0] + M[1] * r.Mi[1] + M[2] * r.Mi[2];
-        const double tr = M[0] + M[3] + M[5];
-        if (!(det > 1e-12 * tr * tr * tr)) return false;
-        const double id = 1.0 / det;
+        r.Mi[0] = mad(M[3], M[5], -(M[4] * M[4]));
+        r.Mi[1] = mad(M[2], M[4], -(M[1] * M[5]));
+        r.Mi[2] = mad(M[1], M[4], -(M[2] * M[3]));
+        r.Mi[3] = mad(M[0], M[5], -(M[2] * M[2]));
+        r.Mi[4] = mad(M[1], M[2], -(M[0] * M[4]));
+        r.Mi[5] = mad(M[0], M[3], -(M[1] * M[1]));
+        const T det = dot3(M[0], r.Mi[0], M[1], r.Mi[1], M[2], r.Mi[2]);
+        if (!regular(det, M[0] + M[3] + M[5], s.m0)) return false;
+        const T id = inverse(det);
 #pragma unroll
-        for (int q = 0; q < 6; ++q) r.Mi[q] *= id;
+        for (int k = 0; k < 6; ++k) r.Mi[k] = r.Mi[k] * id;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) r.m1[a] = (double)s.m1[a] - (double)s.c1[a];
+        for (int a = 0; a < 3; ++a) difference((F)s.m1[a] * f1, (F)s.c1[a] * f1, r.m1[a]);
 #pragma unroll
         for (int a = 0; a < 3; ++a) r.B[a] = -row(r.Mi, a, r.m1);
-        r.q = (double)s.m0 - (double)s.c0 + (r.B[0] * r.m1[0] + r.B[1] * r.m1[1] + r.B[2] * r.m1[2]);
-        r.A = 1.0 / r.q;
-        double s2[6], s3[10], W[6];
+        T m0;
+        difference((F)s.m0, (F)s.c0, m0);
+        r.q = m0 + dot3(r.B[0], r.m1[0], r.B[1], r.m1[1], r.B[2], r.m1[2]);
+        r.A = inverse(r.q);
+        T W[6];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) s2[k] = (double)s.s2[k];
-#pragma unroll
-        for (int k = 0; k < 10; ++k) s3[k] = (double)s.s3[k];
+        for (int k = 0; k < 10; ++k) r.s3[k] = (F)s.s3[k] * f1;
         const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            r.T[k] = s3[sorted3(ia[k], ib[k], 0)] * r.B[0] + s3[sorted3(ia[k], ib[k], 1)] * r.B[1] +
-                     s3[sorted3(ia[k], ib[k], 2)] * r.B[2];
-            r.U[k] = s2[k] + r.T[k];
-            W[k] = s2[k] + r.U[k];  // 2 s2 + T
+            const T t = dot3(r.B[0], r.s3[sorted3(ia[k], ib[k], 0)], r.B[1], r.s3[sorted3(ia[k], ib[k], 1)], r.B[2],
+                             r.s3[sorted3(ia[k], ib[k], 2)]);
+            r.U[k] = t + (F)s.s2[k];
+            r.Uq[k] = ia[k] == ib[k] ? r.U[k] + r.q : r.U[k];
+            W[k] = r.U[k] + (F)s.s2[k];  // 2 s2 + T
         }
 #pragma unroll
-        for (int g = 0; g < 3; ++g) r.K[g] = (double)s.dm0[g] + 2.0 * r.q * r.B[g] + row(W, g, r.B);
+        for (int g = 0; g < 3; ++g) r.K[g] = mad(twice(r.q), r.B[g], row(W, g, r.B)) + (F)s.dm0[g] * r.g1;
         return true;
     }
     // packed index of the sorted axes of (a <= b) and c
@@ -783,29 +874,39 @@ struct CorrStage {
         for (int k = 0; k < 10; ++k) s.s3[k] = fmaf(xx[k3q[k]], dW[k3c[k]], s.s3[k]);
         if (kCount) s.cnt += in;
     }
-    __device__ static void finish(const P &p, I &s, const Rec &, int32_t o, int64_t) {
+    // false if the particle's sums cannot be worked on in T
+    template <class T>
+    __device__ static bool finish_in(const P &p, const I &s, int32_t o) {
+        using F = typename beside<T>::type;
         const int64_t n = p.n;
-        Solved r;
-        if (!solve(s, r)) {
-            const float nan = __int_as_float(0x7fc00000);
-            p.A[o] = nan;
-            for (int a = 0; a < 3; ++a) { p.B[a * n + o] = nan; p.gA[a * n + o] = nan; }
-            for (int a = 0; a < 9; ++a) p.gB[a * n + o] = nan;
-            if (p.n_singular) atomicAdd(p.n_singular, 1);
-            return;
-        }
-        p.A[o] = (float)r.A;
-        const double A2 = -r.A * r.A;
+        Solved<T> r;
+        if (!solve(s, r)) return false;
+        float sum = 0.0f;  // NaN once a result is not finite
+        auto put = [&](float *out, float v) {
+            *out = v;
+            sum = fmaf(v, 0.0f, sum);
+        };
+        put(p.A + o, rounded(r.A));
 #pragma unroll
-        for (int a = 0; a < 3; ++a) p.B[a * n + o] = (float)r.B[a];
+        for (int a = 0; a < 3; ++a) put(p.B + a * n + o, rounded(r.B[a] * r.f1));
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
-            p.gA[g * n + o] = (float)(A2 * r.K[g]);
-            const double u[3] = {at(r.U, 0, g), at(r.U, 1, g), at(r.U, 2, g)};
+            put(p.gA + g * n + o, rounded(-(r.A * r.K[g]) * r.A * r.f1));
+            const T u[3] = {at(r.Uq, 0, g), at(r.Uq, 1, g), at(r.Uq, 2, g)};
 #pragma unroll
             for (int a = 0; a < 3; ++a)
-                p.gB[(3 * g + a) * n + o] = (float)(r.B[a] * r.B[g] - row(r.Mi, a, u) - r.q * at(r.Mi, a, g));
+                put(p.gB + (3 * g + a) * n + o, rounded(mad(r.B[a], r.B[g], -row(r.Mi, a, u)) * (r.f1 * r.f1)));
         }
+        return std::is_same<T, double>::value || sum == 0.0f;
+    }
+    __device__ static void finish(const P &p, I &s, const Rec &, int32_t o, int64_t) {
+        if (finish_in<Two>(p, s, o) || finish_in<double>(p, s, o)) return;
+        const int64_t n = p.n;
+        const float nan = __int_as_float(0x7fc00000);
+        p.A[o] = nan;
+        for (int a = 0; a < 3; ++a) { p.B[a * n + o] = nan; p.gA[a * n + o] = nan; }
+        for (int a = 0; a < 9; ++a) p.gB[a * n + o] = nan;
+        if (p.n_singular) atomicAdd(p.n_singular, 1);
     }
     __device__ static void finish_other(const P &p, int32_t o) {
         const int64_t n = p.n;
@@ -837,105 +938,115 @@ struct CorrAdjPrepStage : CorrStage {
     static constexpr bool kAllVariants = false;
     using P = CorrAdjP;
     // Reverse of CorrStage's Solved, in the sums m0, m1, m2, dm0, s2, s3 themselves, whose cotangents
-    // are the polynomial coefficients.  H_ga: the cotangent of dB_g^a (row g).  The sweep is CorrStage's
-    // and the FP64 of this finish bounds the rest: 422 -> 295 us on the 2x64^3 box against the reverse
-    // taken through the 30 unreduced sums dm1, dm2.
-    __device__ static void finish(const P &p, I &s, const Rec &, int32_t o, int64_t) {
+    // are the polynomial coefficients.  H_ga: the cotangent of dB_g^a (row g).  The sweep is CorrStage's;
+    // this finish (2,500 FP32 instructions in float pairs) is the other half of the kernel's time: 422 ->
+    // 295 us on the 2x64^3 box against the reverse taken through the 30 unreduced sums dm1, dm2, 260 us
+    // in float pairs.
+    template <class T>
+    __device__ static bool finish_in(const P &p, const I &s, int32_t o) {
+        using F = typename beside<T>::type;
         const int64_t n = p.n;
-        Solved r;
-        if (!solve(s, r)) {  // singular: contributes nothing
-            for (int k = 0; k < kCorrCoef; ++k) p.coef[k * n + o] = 0.f;
-            if (p.n_singular) atomicAdd(p.n_singular, 1);
-            return;
-        }
-        float *coef = p.coef + o;
-        double H[3][3], Kb[3], Bb[3], Ab = (double)p.Abar[o], qb = 0.0;
-        const double A2 = -r.A * r.A;
+        Solved<T> r;
+        if (!solve(s, r)) return false;
+        const F f1 = r.f1, f2 = f1 * f1;
+        float sum = 0.0f;  // NaN once a result is not finite
+        auto put = [&](int k, float v) {
+            p.coef[k * n + o] = v;
+            sum = fmaf(v, 0.0f, sum);
+        };
+        T H[3][3], Kb[3], Bb[3], Ab, qb;
+        difference((F)p.Abar[o], (F)0, Ab);
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
+            T gAb;
 #pragma unroll
-            for (int a = 0; a < 3; ++a) H[g][a] = (double)p.gBbar[(3 * g + a) * n + o];
-            const double gAb = (double)p.gAbar[g * n + o];
-            Bb[g] = (double)p.Bbar[g * n + o];
-            Kb[g] = A2 * gAb;
-            Ab -= 2.0 * r.A * r.K[g] * gAb;
-            coef[(10 + g) * n] = (float)Kb[g];  // l1: dm0
+            for (int a = 0; a < 3; ++a) difference((F)p.gBbar[(3 * g + a) * n + o] * f2, (F)0, H[g][a]);
+            difference((F)p.gAbar[g * n + o] * f1, (F)0, gAb);
+            difference((F)p.Bbar[g * n + o] * f1, (F)0, Bb[g]);
+            const T Ag = -(r.A * gAb);
+            Kb[g] = r.A * Ag;
+            Ab = mad(twice(Ag), r.K[g], Ab);
+            put(10 + g, rounded(Kb[g] * r.g1));  // l1: dm0
         }
-        // dB_g^a = B_a B_g - (Mi U)_ag - q Mi_ag and K_g = dm0_g + 2 q B_g + ((2 s2 + T) B)_g
-        double Mib[3][3], Ub[3][3];
+        // dB_g^a = B_a B_g - (Mi Uq)_ag and K_g = dm0_g + 2 q B_g + ((2 s2 + T) B)_g
+        T Mib[3][3], Uqb[3][3];
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
             for (int b = 0; b < 3; ++b) {
-                Mib[a][b] = -(H[0][a] * at(r.U, b, 0) + H[1][a] * at(r.U, b, 1) + H[2][a] * at(r.U, b, 2)) - r.q * H[b][a];
-                Ub[a][b] = -(at(r.Mi, a, 0) * H[b][0] + at(r.Mi, a, 1) * H[b][1] + at(r.Mi, a, 2) * H[b][2]);
-                qb -= H[b][a] * at(r.Mi, a, b);
+                Mib[a][b] = -dot3(H[0][a], at(r.Uq, b, 0), H[1][a], at(r.Uq, b, 1), H[2][a], at(r.Uq, b, 2));
+                Uqb[a][b] = -row(r.Mi, a, H[b]);
             }
+        qb = Uqb[0][0] + Uqb[1][1] + Uqb[2][2] + twice(dot3(Kb[0], r.B[0], Kb[1], r.B[1], Kb[2], r.B[2]));
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
 #pragma unroll
             for (int g = 0; g < 3; ++g) {
+                Bb[a] = mad(H[g][a] + H[a][g], r.B[g], Bb[a]);
                 // 2 s2 + T = s2 + U
-                Bb[a] += (H[g][a] + H[a][g]) * r.B[g] + Kb[g] * ((double)s.s2[a <= g ? idx2(a, g) : idx2(g, a)] + at(r.U, a, g));
+                Bb[a] = mad(Kb[g], at(r.U, a, g) + (F)s.s2[a <= g ? idx2(a, g) : idx2(g, a)], Bb[a]);
             }
-            Bb[a] += 2.0 * r.q * Kb[a];
-            qb += 2.0 * Kb[a] * r.B[a];
+            Bb[a] = mad(twice(r.q), Kb[a], Bb[a]);
         }
         // s2 and T cotangents, one entry per monomial x_a x_b (both orders of an off-diagonal pair)
-        double Tb[6];
+        T Tb[6];
         const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             const int a = ia[k], b = ib[k];
-            const double w = a == b ? Kb[a] * r.B[a] : Kb[a] * r.B[b] + Kb[b] * r.B[a];
-            Tb[k] = (a == b ? Ub[a][a] : Ub[a][b] + Ub[b][a]) + w;
-            coef[(13 + k) * n] = (float)(Tb[k] + w);  // q1: s2
+            const T w = a == b ? Kb[a] * r.B[a] : mad(Kb[a], r.B[b], Kb[b] * r.B[a]);
+            Tb[k] = (a == b ? Uqb[a][a] : Uqb[a][b] + Uqb[b][a]) + w;
+            put(13 + k, rounded(Tb[k] + w));  // q1: s2
         }
         // T = s3 B: Bb_c += sum_ab Tb_ab s3_abc, and s3's coefficients are those of (x^T Tb x)(B.x)
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
-            for (int k = 0; k < 6; ++k) Bb[c] += Tb[k] * (double)s.s3[sorted3(ia[k], ib[k], c)];
-        const double *B = r.B;
-        const double k3[10] = {Tb[0] * B[0],
-                               Tb[0] * B[1] + Tb[1] * B[0],
-                               Tb[0] * B[2] + Tb[2] * B[0],
-                               Tb[1] * B[1] + Tb[3] * B[0],
-                               Tb[1] * B[2] + Tb[2] * B[1] + Tb[4] * B[0],
-                               Tb[2] * B[2] + Tb[5] * B[0],
-                               Tb[3] * B[1],
-                               Tb[3] * B[2] + Tb[4] * B[1],
-                               Tb[4] * B[2] + Tb[5] * B[1],
-                               Tb[5] * B[2]};
-#pragma unroll
-        for (int k = 0; k < 10; ++k) coef[(19 + k) * n] = (float)k3[k];
+            for (int k = 0; k < 6; ++k) Bb[c] = mad(Tb[k], r.s3[sorted3(ia[k], ib[k], c)], Bb[c]);
+        const T *B = r.B;
+        put(19, rounded(Tb[0] * B[0] * f1));
+        put(20, rounded(mad(Tb[0], B[1], Tb[1] * B[0]) * f1));
+        put(21, rounded(mad(Tb[0], B[2], Tb[2] * B[0]) * f1));
+        put(22, rounded(mad(Tb[1], B[1], Tb[3] * B[0]) * f1));
+        put(23, rounded(dot3(Tb[1], B[2], Tb[2], B[1], Tb[4], B[0]) * f1));
+        put(24, rounded(mad(Tb[2], B[2], Tb[5] * B[0]) * f1));
+        put(25, rounded(Tb[3] * B[1] * f1));
+        put(26, rounded(mad(Tb[3], B[2], Tb[4] * B[1]) * f1));
+        put(27, rounded(mad(Tb[4], B[2], Tb[5] * B[1]) * f1));
+        put(28, rounded(Tb[5] * B[2] * f1));
         // A = 1/q, q = m0 + B.m1, B = -Mi m1, Mi = m2^-1
-        qb += A2 * Ab;
-        coef[0] = (float)qb;  // c0: m0
+        qb = mad(-(r.A * Ab), r.A, qb);
+        put(0, rounded(qb));  // c0: m0
 #pragma unroll
-        for (int a = 0; a < 3; ++a) Bb[a] += qb * r.m1[a];
+        for (int a = 0; a < 3; ++a) Bb[a] = mad(qb, r.m1[a], Bb[a]);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            coef[(1 + a) * n] = (float)(qb * r.B[a] - row(r.Mi, a, Bb));  // l0: m1
+            put(1 + a, rounded(mad(qb, r.B[a], -row(r.Mi, a, Bb)) * f1));  // l0: m1
 #pragma unroll
-            for (int b = 0; b < 3; ++b) Mib[a][b] -= Bb[a] * r.m1[b];
+            for (int b = 0; b < 3; ++b) Mib[a][b] = mad(-Bb[a], r.m1[b], Mib[a][b]);
         }
         // m2's cotangent -Mi Mib Mi, per monomial: -Mi (Mib + Mib^T) Mi off the diagonal, half of it on it
-        double S[6], Y[3][3];
+        T S[6], Y[3][3];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) S[k] = ia[k] == ib[k] ? 2.0 * Mib[ia[k]][ia[k]] : Mib[ia[k]][ib[k]] + Mib[ib[k]][ia[k]];
+        for (int k = 0; k < 6; ++k) S[k] = ia[k] == ib[k] ? twice(Mib[ia[k]][ia[k]]) : Mib[ia[k]][ib[k]] + Mib[ib[k]][ia[k]];
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
             for (int b = 0; b < 3; ++b) {
-                const double c[3] = {at(r.Mi, 0, b), at(r.Mi, 1, b), at(r.Mi, 2, b)};
+                const T c[3] = {at(r.Mi, 0, b), at(r.Mi, 1, b), at(r.Mi, 2, b)};
                 Y[a][b] = row(S, a, c);
             }
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const double c[3] = {Y[0][ib[k]], Y[1][ib[k]], Y[2][ib[k]]};
-            coef[(4 + k) * n] = (float)((ia[k] == ib[k] ? -0.5 : -1.0) * row(r.Mi, ia[k], c));  // q0: m2
+            const T c[3] = {Y[0][ib[k]], Y[1][ib[k]], Y[2][ib[k]]};
+            put(4 + k, rounded(row(r.Mi, ia[k], c) * ((ia[k] == ib[k] ? (F)-0.5 : (F)-1.0) * f2)));  // q0: m2
         }
+        return std::is_same<T, double>::value || sum == 0.0f;
+    }
+    __device__ static void finish(const P &p, I &s, const Rec &, int32_t o, int64_t) {
+        if (finish_in<Two>(p, s, o) || finish_in<double>(p, s, o)) return;
+        for (int k = 0; k < kCorrCoef; ++k) p.coef[k * p.n + o] = 0.f;  // singular: contributes nothing
+        if (p.n_singular) atomicAdd(p.n_singular, 1);
     }
     __device__ static void finish_other(const P &p, int32_t o) {
         for (int k = 0; k < kCorrCoef; ++k) p.coef[k * p.n + o] = 0.f;
