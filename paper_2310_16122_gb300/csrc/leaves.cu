@@ -1258,116 +1258,60 @@ __device__ __forceinline__ double sum_sq(double gx, double gy, double gz) {
     return __dadd_rn(__dadd_rn(__dmul_rn(gx, gx), __dmul_rn(gy, gy)), __dmul_rn(gz, gz));
 }
 
-// Emits the images of leaf b that lie within `cut` of leaf a; returns how many.
-template <bool kFill>
-__device__ int leaf_images(const float *__restrict__ bbox, int64_t a, int64_t b, double L, double cut2,
-                           crk_image *__restrict__ out) {
-    const float *A = bbox + 6 * a, *B = bbox + 6 * b;
-    const float Lf = (float)L, cutf = (float)sqrt(cut2) + 1e-5f * Lf + 1e-6f;
-    if (clearly_apart(A, B, Lf, (float)sqrt(cut2))) return 0;
-    // Per axis, only the shifts whose own gap is inside the cut can give an image: the FP64
-    // sum of squares is never below one of its (non-negative) terms.  An FP32 gap with a margin
-    // above its rounding skips the FP64 work for the far shifts (FP64 is slow on this GPU).
-    double g[3][3];
-    int keep[3][3], nk[3] = {0, 0, 0};
+// The gaps of two leaves per axis and box shift (-L, 0, L), in FP32.
+struct Gaps {
+    float g[3][3];
+};
+__device__ __forceinline__ float pick3(const float g[3], int k) { return k == 0 ? g[0] : (k == 1 ? g[1] : g[2]); }
+
+// The images of leaf B within cut of leaf A as bits 9 sx + 3 sy + sz (shift indices 0, 1, 2).  The
+// decision is that of the FP64 gaps, squared and summed, against cut^2.  The FP32 gaps settle every
+// image that is not within a margin far above their rounding of the cut: FP64 (1/64 of the FP32
+// rate here) only sees those; square roots of cut^2 and two FP64 gap sums per candidate and list
+// were the kernel's time before: 147 -> 62 us on the 2x64^3 box, 6.2 -> 2.6 ms on 2x256^3.
+__device__ __forceinline__ uint32_t image_mask(const float *A, const float *B, const Gaps &s, double L, double cut) {
+    const float cf = (float)cut, m = 1e-5f * (float)L + 1e-6f, hi = cf + m, lo = cf - m;
+    const float hi2 = hi * hi, lo2 = lo > 0.0f ? lo * lo : -1.0f;
+    uint32_t keep[3];
+#pragma unroll
     for (int q = 0; q < 3; ++q)
-        for (int k = 0; k < 3; ++k) {
-            const float sf = (float)(k - 1) * Lf;
-            const float g32 = fmaxf(fmaxf((B[q] + sf) - A[3 + q], (A[q] - B[3 + q]) - sf), 0.0f);
-            if (g32 > cutf) continue;
-            const double gd = axis_gap_shift(A[q], A[3 + q], B[q], B[3 + q], (double)(k - 1) * L);
-            if (!(__dmul_rn(gd, gd) < cut2)) continue;
-            g[q][nk[q]] = gd;
-            keep[q][nk[q]++] = k;
-        }
-    int cnt = 0;
-    for (int jx = 0; jx < nk[0]; ++jx)
-        for (int jy = 0; jy < nk[1]; ++jy)
-            for (int jz = 0; jz < nk[2]; ++jz) {
-                const int ix = keep[0][jx], iy = keep[1][jy], iz = keep[2][jz];
-                double d2 = sum_sq(g[0][jx], g[1][jy], g[2][jz]);
-                if (d2 < cut2) {
-                    if (kFill) {
-                        crk_image im;
-                        im.b = (int32_t)b;
-                        double sx = (ix - 1) * L, sy = (iy - 1) * L, sz = (iz - 1) * L;
-                        im.sx = (float)__dsub_rn(__dadd_rn((double)B[0], sx), (double)A[0]);
-                        im.sy = (float)__dsub_rn(__dadd_rn((double)B[1], sy), (double)A[1]);
-                        im.sz = (float)__dsub_rn(__dadd_rn((double)B[2], sz), (double)A[2]);
-                        out[cnt] = im;
-                    }
-                    ++cnt;
+        keep[q] = (s.g[q][0] > hi ? 0u : 1u) | (s.g[q][1] > hi ? 0u : 2u) | (s.g[q][2] > hi ? 0u : 4u);
+    uint32_t out = 0;
+    for (uint32_t mx = keep[0]; mx; mx &= mx - 1) {
+        const int ix = __ffs(mx) - 1;
+        const float gx = pick3(s.g[0], ix);
+        for (uint32_t my = keep[1]; my; my &= my - 1) {
+            const int iy = __ffs(my) - 1;
+            const float gy = pick3(s.g[1], iy);
+            for (uint32_t mz = keep[2]; mz; mz &= mz - 1) {
+                const int iz = __ffs(mz) - 1;
+                const float gz = pick3(s.g[2], iz), d2 = gx * gx + gy * gy + gz * gz;
+                bool in = d2 < lo2;
+                if (!in && !(d2 > hi2)) {
+                    in = sum_sq(axis_gap_shift(A[0], A[3], B[0], B[3], (double)(ix - 1) * L),
+                                axis_gap_shift(A[1], A[4], B[1], B[4], (double)(iy - 1) * L),
+                                axis_gap_shift(A[2], A[5], B[2], B[5], (double)(iz - 1) * L)) < __dmul_rn(cut, cut);
                 }
-            }
-    return cnt;
-}
-
-template <bool kFill>
-__global__ void pairs_kernel(int64_t n_leaves, const int32_t *__restrict__ leaf_start,
-                             const int32_t *__restrict__ leaf_ngas, const float *__restrict__ bbox,
-                             const float *__restrict__ hmax, TreeDev tree, int brute, int hydro, double L,
-                             double rc, double hmax_all, int32_t *__restrict__ img_cnt, int32_t *__restrict__ pair_cnt,
-                             const int32_t *__restrict__ img_ptr, crk_image *__restrict__ img,
-                             const int32_t *__restrict__ pair_ptr, int32_t *__restrict__ pair_list) {
-    int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= n_leaves) return;
-    int ni = 0, np = 0;
-    crk_image *io = kFill ? img + img_ptr[a] : nullptr;
-    int32_t *po = kFill ? pair_list + pair_ptr[a] : nullptr;
-    const bool a_ok = leaf_start[a + 1] > leaf_start[a] && (!hydro || leaf_ngas[a] > 0);
-    if (a_ok) {
-        const float *A = bbox + 6 * a;
-        const double ha = hydro ? (double)hmax[a] : 0.0;
-        auto visit_leaf = [&](int64_t b) {
-            if (leaf_start[b + 1] == leaf_start[b]) return;
-            if (hydro && leaf_ngas[b] == 0) return;
-            double cut = rc;
-            if (hydro) {
-                double hb = (double)hmax[b];
-                cut = __dmul_rn(2.0, ha > hb ? ha : hb);
-            }
-            int c = leaf_images<kFill>(bbox, a, b, L, __dmul_rn(cut, cut), kFill ? io + ni : nullptr);
-            if (c > 0) {
-                if (kFill) po[np] = (int32_t)b;
-                ni += c;
-                np += 1;
-            }
-        };
-        if (brute) {
-            for (int64_t b = 0; b < n_leaves; ++b) visit_leaf(b);
-        } else {
-            (void)hmax_all;
-            int32_t stack[64];
-            int top = 0;
-            stack[top++] = tree.root;
-            while (top > 0) {
-                int32_t nd = stack[--top];
-                const float *Nb = tree.node_box + 6 * (int64_t)nd;
-                float cutn = hydro ? 2.0f * fmaxf((float)ha, tree.node_hmax[nd]) : (float)rc;
-                if (clearly_apart(A, Nb, (float)L, cutn)) continue;
-                int32_t lf = tree.node_leaf[nd];
-                if (lf >= 0) {
-                    visit_leaf(lf);
-                } else if (top + 2 <= 64) {
-                    stack[top++] = tree.node_right[nd];
-                    stack[top++] = tree.node_left[nd];
-                }
+                if (in) out |= 1u << (9 * ix + 3 * iy + iz);
             }
         }
     }
-    if (!kFill) {
-        img_cnt[a] = ni;
-        pair_cnt[a] = np;
-    }
+    return out;
 }
 
+// the float nearest b + (k - 1) L - a, each sum rounded to FP64 first; without a shift the FP32
+// difference is that number (b - a is exact in FP64 or |b| < 2^-29 |a|)
+__device__ __forceinline__ float image_shift(float b, float a, int k, double L) {
+    if (k == 1) return __fsub_rn(__fadd_rn(b, 0.0f), a);
+    return (float)__dsub_rn(__dadd_rn((double)b, (double)(k - 1) * L), (double)a);
+}
 
 // --- warp-cooperative leaf-pair finder ---------------------------------------------
 // One warp per i-leaf.  The warp pops up to 32 tree nodes at a time from a
 // shared-memory stack, tests them in parallel (FP32, with margin, against the
 // larger of the gravity cut and the hydro cut bound), pushes the children of
 // the survivors and collects surviving leaves.  The candidates are sorted,
-// tested exactly (FP64 per periodic image, leaf_images) for both lists, and
+// tested exactly (image_mask) for both lists, and
 // the leaf's images are written with one atomic reservation per list, so each
 // leaf's lists stay in ascending j-leaf order.
 constexpr int kTravWarps = 4;
@@ -1408,13 +1352,16 @@ __global__ void __launch_bounds__(kTravWarps * 32) leaf_pairs_warp_kernel(
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int32_t *const stack = buf_a[warp], *const sorted = buf_a[warp];
     int32_t *const cand = buf_b[warp];
-    uint8_t *const ng = reinterpret_cast<uint8_t *>(buf_b[warp]), *const nh = ng + kCandCap;
+    // per sorted candidate: the number of its images, and above it the one image of a single
+    uint16_t *const ng = reinterpret_cast<uint16_t *>(buf_b[warp]), *const nh = ng + kCandCap;
     const unsigned below = (1u << lane) - 1u;
     const int64_t a = (int64_t)blockIdx.x * kTravWarps + warp;
     if (a >= n_leaves) return;  // whole warp leaves together; no block barrier below
     const bool a_any = leaf_start[a + 1] > leaf_start[a];
     const bool a_gas = leaf_ngas[a] > 0;
-    const float *A = bbox + 6 * a;
+    float A[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) A[q] = bbox[6 * a + q];
     const float ha = hmax[a];
     const int bx = leaf_box ? leaf_box[a] : 0;
     const double L = leaf_box ? (double)box_L[bx] : L0;
@@ -1497,32 +1444,40 @@ __global__ void __launch_bounds__(kTravWarps * 32) leaf_pairs_warp_kernel(
         sorted[r] = v;
     }
     __syncwarp();
-    // exact image counts of both lists
-    const double rc2 = __dmul_rn(rc, rc);
-    for (int t = lane; t < nc; t += 32) {
-        int32_t b = sorted[t];
-        int cg = leaf_images<false>(bbox, a, b, L, rc2, nullptr);
-        int ch = 0;
-        if (a_gas && leaf_ngas[b] > 0) {
-            double hb = (double)hmax[b], hA = (double)ha;
-            double cut = __dmul_rn(2.0, hA > hb ? hA : hb);
-            ch = leaf_images<false>(bbox, a, b, L, __dmul_rn(cut, cut), nullptr);
+    // the images of both lists
+    auto images = [&](int32_t b, uint32_t &mg, uint32_t &mh) {
+        const float2 *Bp = reinterpret_cast<const float2 *>(bbox + 6 * (int64_t)b);
+        const float2 b0 = Bp[0], b1 = Bp[1], b2 = Bp[2];
+        const float B[6] = {b0.x, b0.y, b1.x, b1.y, b2.x, b2.y};
+        Gaps s;
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float sf = (float)(k - 1) * Lf;
+                const float t1 = (B[q] + sf) - A[3 + q], t2 = (A[q] - B[3 + q]) - sf, g = t1 > t2 ? t1 : t2;
+                s.g[q][k] = g < 0.0f ? 0.0f : g;  // a NaN stays, and gives no image
+            }
+        mg = image_mask(A, B, s, L, rc);
+        mh = 0;
+        if (a_gas && leaf_ngas[b] > 0) mh = image_mask(A, B, s, L, (double)(2.0f * fmaxf(ha, hmax[b])));
+    };
+    auto coded = [](uint32_t m) { return (uint16_t)(__popc(m) | ((31 - __clz(m | 1u)) << 8)); };
+    // totals: images in the low half word, pairs in the high one (27 * kCandCap < 2^16)
+    unsigned tg = 0, th = 0;
+    for (int t0 = 0; t0 < nc; t0 += 32) {
+        const int t = t0 + lane;
+        uint32_t mg = 0, mh = 0;
+        if (t < nc) {
+            images(sorted[t], mg, mh);
+            ng[t] = coded(mg);
+            nh[t] = coded(mh);
         }
-        ng[t] = (uint8_t)cg;
-        nh[t] = (uint8_t)ch;
+        tg += __reduce_add_sync(CRK_FULL_MASK, (unsigned)__popc(mg) | (mg ? 0x10000u : 0u));
+        th += __reduce_add_sync(CRK_FULL_MASK, (unsigned)__popc(mh) | (mh ? 0x10000u : 0u));
     }
     __syncwarp();
-    int tot[4] = {0, 0, 0, 0};
-    for (int t0 = 0; t0 < nc; t0 += 32) {
-        int t = t0 + lane;
-        int cg = t < nc ? ng[t] : 0, ch = t < nc ? nh[t] : 0;
-        int v[4] = {cg, cg > 0, ch, ch > 0};
-        for (int k = 0; k < 4; ++k) {
-            int s;
-            warp_excl_scan(v[k], lane, s);
-            tot[k] += s;
-        }
-    }
+    const int tot[4] = {(int)(tg & 0xffffu), (int)(tg >> 16), (int)(th & 0xffffu), (int)(th >> 16)};
     unsigned long long base[4] = {0, 0, 0, 0};
     if (lane == 0)
         for (int k = 0; k < 4; ++k) base[k] = tot[k] ? atomicAdd(&o.cursor[k], (unsigned long long)tot[k]) : 0ull;
@@ -1541,28 +1496,32 @@ __global__ void __launch_bounds__(kTravWarps * 32) leaf_pairs_warp_kernel(
             o.start[k][a] = (int32_t)base[k];
             o.count[k][a] = tot[k];
         }
-    int run[4] = {0, 0, 0, 0};
+    unsigned rg = 0, rh = 0;
     for (int t0 = 0; t0 < nc; t0 += 32) {
-        int t = t0 + lane;
-        int cg = t < nc ? ng[t] : 0, ch = t < nc ? nh[t] : 0;
-        int v[4] = {cg, cg > 0, ch, ch > 0};
-        int off[4];
-        for (int k = 0; k < 4; ++k) {
-            int s;
-            off[k] = run[k] + warp_excl_scan(v[k], lane, s);
-            run[k] += s;
-        }
-        if (t < nc) {
-            int32_t b = sorted[t];
-            if (cg > 0) {
-                o.gpair[base[1] + off[1]] = b;
-                leaf_images<true>(bbox, a, b, L, rc2, o.gimg + base[0] + off[0]);
-            }
-            if (ch > 0) {
-                double hb = (double)hmax[b], hA = (double)ha;
-                double cut = __dmul_rn(2.0, hA > hb ? hA : hb);
-                o.hpair[base[3] + off[3]] = b;
-                leaf_images<true>(bbox, a, b, L, __dmul_rn(cut, cut), o.himg + base[2] + off[2]);
+        const int t = t0 + lane;
+        const unsigned vg = t < nc ? ng[t] : 0u, vh = t < nc ? nh[t] : 0u;
+        const unsigned cg = vg & 0xffu, ch = vh & 0xffu;
+        int sg, sh;
+        const unsigned og = rg + (unsigned)warp_excl_scan((int)(cg | (cg ? 0x10000u : 0u)), lane, sg);
+        const unsigned oh = rh + (unsigned)warp_excl_scan((int)(ch | (ch ? 0x10000u : 0u)), lane, sh);
+        rg += (unsigned)sg;
+        rh += (unsigned)sh;
+        if (cg | ch) {
+            const int32_t b = sorted[t];
+            uint32_t mg = cg ? 1u << (vg >> 8) : 0u, mh = ch ? 1u << (vh >> 8) : 0u;
+            if (cg > 1 || ch > 1) images(b, mg, mh);
+            if (cg) o.gpair[base[1] + (og >> 16)] = b;
+            if (ch) o.hpair[base[3] + (oh >> 16)] = b;
+            const float2 *Bp = reinterpret_cast<const float2 *>(bbox + 6 * (int64_t)b);
+            const float2 b0 = Bp[0], b1 = Bp[1];
+            float4 *gi = reinterpret_cast<float4 *>(o.gimg + base[0] + (og & 0xffffu));
+            float4 *hi = reinterpret_cast<float4 *>(o.himg + base[2] + (oh & 0xffffu));
+            for (uint32_t m = mg | mh; m; m &= m - 1) {
+                const int k = __ffs(m) - 1;
+                const float4 im = make_float4(__int_as_float(b), image_shift(b0.x, A[0], k / 9, L),
+                                              image_shift(b0.y, A[1], k / 3 % 3, L), image_shift(b1.x, A[2], k % 3, L));
+                if (mg >> k & 1u) *gi++ = im;
+                if (mh >> k & 1u) *hi++ = im;
             }
         }
     }
