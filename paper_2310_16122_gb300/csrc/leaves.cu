@@ -11,6 +11,8 @@
 // the two other lists are stably partitioned by comparing the ranks they
 // carry (a prefix sum of the left flags orders the output).  The shape of the
 // tree depends on n alone, so the host precomputes every level's segments.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -467,20 +469,28 @@ __global__ void __launch_bounds__(kPartThreads, 6) rcb_scatter3_kernel(int64_t n
 // kernels above (so the same tree, bit for bit), but a level costs a few
 // shared-memory passes instead of three DRAM passes over the six rank
 // columns.  The block ends by writing the final member order of its range.
+// The three levels before that run in clusters of up to eight such blocks per segment (at most 16384
+// entries): a streamed level is two launches that wait on chains of dependent loads, 25 us at any size
+// below 2M particles.  Three levels take 12 us more in this kernel instead of 75 on 30,011 particles and
+// 40 us instead of 80 on 2x64^3.  Only while the clusters fit in one wave of resident blocks: beyond that
+// the remote stores are slower than the streamed levels (2x256^3 5.5 ms against 4.5, 24 boxes 537 us
+// against 380).
 constexpr int kLocalCap = 2048;
 constexpr int kLocalThreads = 512;
 constexpr int kLocalBlocks = 2;                         // resident blocks per SM (shared memory: ~113 KB each)
 constexpr int kLocalItems = kLocalCap / kLocalThreads;  // consecutive positions per thread
 constexpr int kLocalLevels = 7;                         // levels one block may run
 constexpr int kLocalSegs = 1 << kLocalLevels;           // segments per block at its deepest level
+constexpr int kClusterLevels = 3;                       // levels a cluster of blocks runs before
+constexpr int kClusterBlocks = 1 << kClusterLevels;
 constexpr size_t kLocalSmem = sizeof(int32_t) * 2 * 6 * kLocalCap + sizeof(int16_t) * 2 * kLocalCap;
 static_assert(kLocalItems == 4, "positions are moved as int4");
 
 // the level tables a block walks: tab[l] = 7 columns of m[l] segments (lo, hi, k, child, node, axis, leftbase)
 struct LocalShape {
-    int32_t *tab[kLocalLevels];
-    int32_t m[kLocalLevels];
-    int nlev;
+    int32_t *tab[kClusterLevels + kLocalLevels];
+    int32_t m[kClusterLevels + kLocalLevels];
+    int pre, nlev;  // levels run by clusters of 2^pre blocks, all levels
 };
 
 struct __align__(16) LocalSeg {
@@ -494,6 +504,7 @@ __device__ __forceinline__ uint64_t pack3(unsigned f) {
 }
 __device__ __forceinline__ int field3(uint64_t v, int b) { return (int)((v >> (21 * b)) & 0x1fffffu); }
 
+template <bool kClusters>
 __global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) rcb_local_kernel(int64_t n, LocalShape sh, RankLists L, AxisOrder o,
                                                                        const float *__restrict__ x,
                                                                        const float *__restrict__ y,
@@ -510,12 +521,30 @@ __global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) rcb_local_kernel(
     int16_t *sn = sc + kLocalCap;
     __shared__ LocalSeg seg[kLocalSegs];
     __shared__ uint64_t wsum[kLocalThreads / 32];
+    __shared__ uint64_t rows[64], totals[kClusterBlocks];  // cluster levels: left counts of the rows, of the blocks,
+    __shared__ int own[kClusterBlocks + 1];                // and the positions that each block keeps
     __shared__ int bad;
-    const int s0 = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int m0 = sh.m[0];
-    const int lo = sh.tab[0][s0], cnt = sh.tab[0][m0 + s0] - lo;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const unsigned below = lanemask_lt_u();
+    // this block's segment at its first level of its own, and those of the blocks of its cluster (the
+    // children of a level's neighbouring segments follow one another)
+    const int pre = kClusters ? sh.pre : 0, top = blockIdx.x >> pre, rank = blockIdx.x - (top << pre);
+    int f = top, e = f + 1;
+    if constexpr (kClusters) {
+        for (int lev = 0; lev < pre; ++lev) {
+            const int32_t *tab = sh.tab[lev];
+            const int m = sh.m[lev], fn = tab[3 * m + f];
+            e = tab[3 * m + e - 1] + (tab[2 * m + e - 1] > 0 ? 2 : 1);
+            f = fn;
+        }
+    }
+    const int32_t *t0 = sh.tab[pre];
+    const int m0 = sh.m[pre], nown = e - f, s0 = f + rank;
+    const int lo = rank < nown ? t0[s0] : t0[m0 + e - 1], cnt = rank < nown ? t0[m0 + s0] - lo : 0;
     if (t == 0) bad = 0;
-    if (cnt > kLocalCap) {
+    bool over = nown > (1 << pre);
+    for (int r = 0; r < nown; ++r) over |= t0[m0 + f + r] - t0[f + r] > kLocalCap;
+    if (over) {  // excluded by the host's choice of levels; the whole cluster leaves
         if (t == 0) atomicAdd(err, 1);
         return;
     }
@@ -531,8 +560,148 @@ __global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) rcb_local_kernel(
     // a rank used as an index; a partition found inconsistent (reported through err) may leave
     // positions unwritten, whose values then never index out of the arrays
     auto rk = [n](int32_t r) -> int64_t { return (uint64_t)r < (uint64_t)n ? r : 0; };
-    int f = s0, e = s0 + 1;  // this block's segments at the current level
-    for (int lev = 0; lev < sh.nlev; ++lev) {
+    // The records of the ns segments from f on, positions relative to `base`: the tight box from the ends
+    // of the three list segments (entry p of list a: rank along axis (a + 1) % 3 in column 2 a), the axis
+    // and the threshold.
+    auto records = [&](int32_t *tab, int m, int f, int ns, int base, bool store, auto entry) {
+        for (int u = t; u < ns; u += kLocalThreads) {
+            const int s = f + u;
+            LocalSeg r{tab[s] - base, tab[m + s] - base, tab[2 * m + s], tab[3 * m + s] - tab[3 * m + f], 0, 0,
+                       tab[6 * m + s] - tab[6 * m + f], 0};
+            const int k = r.k;
+            if (k > 0) {
+                float blo[3], bhi[3];
+                double ext[3];
+                for (int a = 0; a < 3; ++a) {
+                    const int32_t *S = o.S[(a + 1) % 3];
+                    blo[a] = cs[a][S[rk(entry(2 * a, r.lo))]];
+                    bhi[a] = cs[a][S[rk(entry(2 * a, r.hi - 1))]];
+                    ext[a] = __dsub_rn((double)bhi[a], (double)blo[a]);
+                }
+                int axis = 0;
+                if (ext[1] > ext[axis]) axis = 1;
+                if (ext[2] > ext[axis]) axis = 2;
+                r.axis = axis;
+                r.thr = o.R[axis][o.S[(axis + 1) % 3][rk(entry(2 * axis, r.lo + k))]];
+                if (store) {
+                    tab[5 * m + s] = axis;
+                    float *nb = node_box + 6 * (int64_t)tab[4 * m + s];
+                    for (int a = 0; a < 3; ++a) {
+                        nb[a] = blo[a];
+                        nb[3 + a] = bhi[a];
+                    }
+                }
+            }
+            seg[u] = r;
+        }
+    };
+    // is entry q (relative to the segments' base; the block's entry ql) of list b in the left part
+    auto goes_left = [&](const LocalSeg &r, int b, int q, int ql) {
+        if (b == r.axis) return q - r.lo < r.k;
+        const int c = (r.axis - b + 2) % 3;  // column of list b holding ranks along the axis
+        return cur[(2 * b + c) * kLocalCap + ql] < r.thr;
+    };
+    // ---- levels of the cluster: each block keeps the positions that are its segment's in the end; entries
+    // move to their block's next columns through distributed shared memory
+    if constexpr (kClusters) {
+        const int LO = t0[f];
+        const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+        if (t <= kClusterBlocks) own[t] = (t < nown ? t0[f + t] : t0[m0 + e - 1]) - LO;
+        __syncthreads();
+        auto owner = [&](int q) {
+            int r = 0;  // own[] of the missing blocks is the end
+#pragma unroll
+            for (int d = kClusterBlocks / 2; d; d >>= 1) r += q >= own[r + d] ? d : 0;
+            return min(r, nown - 1);
+        };
+        const int to = lo - LO;
+        int fp = top, ep = top + 1;
+        for (int lev = 0; lev < pre; ++lev) {
+            int32_t *tab = sh.tab[lev];
+            const int m = sh.m[lev], ns = ep - fp;  // at most 2^lev
+            cl.sync();  // every block's columns of this level are in place
+            records(tab, m, fp, ns, LO, rank == 0, [&](int col, int q) {
+                const int b = owner(q);
+                return cl.map_shared_rank(cur, b)[col * kLocalCap + q - own[b]];
+            });
+            __syncthreads();
+            // entries in rows of one per thread, so that a warp's left-going and right-going ones are two
+            // runs of words in the other blocks' memory (remote stores cost by the packet)
+            unsigned fl[kLocalItems];
+            int sg[kLocalItems];
+#pragma unroll
+            for (int i = 0; i < kLocalItems; ++i) {
+                const int ql = i * kLocalThreads + t, q = to + ql;
+                fl[i] = 0u;
+                sg[i] = 0;
+                for (int s = 1; s < ns; ++s) sg[i] += q >= seg[s].lo;
+                const LocalSeg &r = seg[sg[i]];
+                if (ql < cnt && r.k > 0) {
+#pragma unroll
+                    for (int b = 0; b < 3; ++b) fl[i] |= (unsigned)goes_left(r, b, q, ql) << b;
+                }
+                uint64_t c3 = 0;
+#pragma unroll
+                for (int b = 0; b < 3; ++b)
+                    c3 |= (uint64_t)__popc(__ballot_sync(CRK_FULL_MASK, (fl[i] >> b) & 1u)) << (21 * b);
+                if (lane == 0) rows[i * (kLocalThreads / 32) + w] = c3;
+            }
+            __syncthreads();
+            if (w == 0) {  // exclusive scan of the rows' counts, two per lane
+                static_assert(kLocalItems * (kLocalThreads / 32) == 64, "two counts per lane");
+                const uint64_t v0 = rows[2 * lane], v = v0 + rows[2 * lane + 1];
+                uint64_t iv = v;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint64_t u = __shfl_up_sync(CRK_FULL_MASK, iv, d);
+                    if (lane >= d) iv += u;
+                }
+                rows[2 * lane] = iv - v;
+                rows[2 * lane + 1] = iv - v + v0;
+                const uint64_t total = __shfl_sync(CRK_FULL_MASK, iv, 31);
+                if (lane < (1 << pre)) cl.map_shared_rank(totals, lane)[rank] = total;
+            }
+            cl.sync();
+            uint64_t before = 0;
+            for (int r = 0; r < rank; ++r) before += totals[r];
+#pragma unroll
+            for (int i = 0; i < kLocalItems; ++i) {
+                const int ql = i * kLocalThreads + t, q = to + ql;
+                const LocalSeg &r = seg[sg[i]];
+                const uint64_t run = before + rows[i * (kLocalThreads / 32) + w];
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    const bool left = (fl[i] >> b) & 1u;
+                    const unsigned mk = __ballot_sync(CRK_FULL_MASK, left);
+                    if (ql >= cnt) continue;
+                    int np = q;
+                    if (r.k > 0) {
+                        const int lb = field3(run, b) + __popc(mk & below) - r.lb;
+                        np = left ? r.lo + lb : r.lo + r.k + (q - r.lo - lb);
+                        if (!(np >= r.lo && np < r.hi)) {
+                            bad = 1;  // as below
+                            continue;
+                        }
+                    }
+                    const int ob = owner(np);
+                    int32_t *dst = cl.map_shared_rank(nxt, ob) + np - own[ob];
+                    dst[(2 * b) * kLocalCap] = cur[(2 * b) * kLocalCap + ql];
+                    dst[(2 * b + 1) * kLocalCap] = cur[(2 * b + 1) * kLocalCap + ql];
+                }
+            }
+            int32_t *tp = cur;
+            cur = nxt;
+            nxt = tp;
+            const int fn = tab[3 * m + fp];
+            ep = tab[3 * m + ep - 1] + (tab[2 * m + ep - 1] > 0 ? 2 : 1);
+            fp = fn;
+        }
+        cl.sync();  // no block touches another one's memory from here on
+        if (rank >= nown) return;
+    }
+    f = s0;
+    e = s0 + 1;  // this block's segments at the current level
+    for (int lev = pre; lev < sh.nlev; ++lev) {
         int32_t *tab = sh.tab[lev];
         const int m = sh.m[lev];
         const int ns = e - f;
@@ -541,39 +710,10 @@ __global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) rcb_local_kernel(
             if (t == 0) atomicAdd(err, 1);
             return;
         }
-        for (int u = t; u < ns; u += kLocalThreads) {
-            const int s = f + u;
-            LocalSeg r{tab[s] - lo, tab[m + s] - lo, tab[2 * m + s], 0, 0, 0, tab[6 * m + s] - tab[6 * m + f], 0};
-            const int k = r.k;
-            if (k > 0) {
-                // tight box from the ends of the three list segments (entry p of list a: rank
-                // along axis (a + 1) % 3 in column 0)
-                float blo[3], bhi[3];
-                double ext[3];
-                for (int a = 0; a < 3; ++a) {
-                    const int32_t *S = o.S[(a + 1) % 3];
-                    blo[a] = cs[a][S[rk(cur[(2 * a) * kLocalCap + r.lo])]];
-                    bhi[a] = cs[a][S[rk(cur[(2 * a) * kLocalCap + r.hi - 1])]];
-                    ext[a] = __dsub_rn((double)bhi[a], (double)blo[a]);
-                }
-                int axis = 0;
-                if (ext[1] > ext[axis]) axis = 1;
-                if (ext[2] > ext[axis]) axis = 2;
-                r.axis = axis;
-                r.thr = o.R[axis][o.S[(axis + 1) % 3][rk(cur[(2 * axis) * kLocalCap + r.lo + k])]];
-                tab[5 * m + s] = axis;
-                float *nb = node_box + 6 * (int64_t)tab[4 * m + s];
-                for (int a = 0; a < 3; ++a) {
-                    nb[a] = blo[a];
-                    nb[3 + a] = bhi[a];
-                }
-            }
-            seg[u] = r;
-        }
+        records(tab, m, f, ns, lo, true, [&](int col, int q) { return cur[col * kLocalCap + q]; });
         // the next level's range of this block's segments
         const int fn = tab[3 * m + f];
         const int en = tab[3 * m + e - 1] + (tab[2 * m + e - 1] > 0 ? 2 : 1);
-        for (int u = t; u < ns; u += kLocalThreads) seg[u].child = tab[3 * m + f + u] - fn;
         __syncthreads();
         // left flags of this thread's kLocalItems consecutive positions (bit b: list b)
         const int q0 = t * kLocalItems;
@@ -590,16 +730,7 @@ __global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) rcb_local_kernel(
                 const LocalSeg &r = seg[sg[i]];
                 if (r.k > 0) {
 #pragma unroll
-                    for (int b = 0; b < 3; ++b) {
-                        bool left;
-                        if (b == r.axis) {
-                            left = q - r.lo < r.k;
-                        } else {
-                            const int c = (r.axis - b + 2) % 3;  // column of list b holding ranks along the axis
-                            left = cur[(2 * b + c) * kLocalCap + q] < r.thr;
-                        }
-                        fl[i] |= (unsigned)left << b;
-                    }
+                    for (int b = 0; b < 3; ++b) fl[i] |= (unsigned)goes_left(r, b, q, q) << b;
                 }
                 mine += pack3(fl[i]);
             }
@@ -2019,7 +2150,13 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
                     break;
                 }
             if (n_lev - d_local > kLocalLevels) d_local = n_lev - kLocalLevels;
-            for (int d = 0; d < d_local; ++d) {
+            // and a cluster of blocks per segment runs the last levels before d_local on the way
+            int d_mid = d_local;
+            if (d_local < n_lev) {
+                const int d = d_local - std::min(d_local, kClusterLevels);
+                if ((int64_t)shape->level_size[d] << (d_local - d) <= (int64_t)kLocalBlocks * ctx->num_sms) d_mid = d;
+            }
+            for (int d = 0; d < d_mid; ++d) {
                 int m = (int)shape->level_size[d];
                 int32_t *tab = shape->dtab + shape->level_off[d];
                 LevelDev dv{tab, tab + m, tab + 2 * m, tab + 3 * m, tab + 4 * m, tab + 5 * m, tab + 6 * m};
@@ -2050,17 +2187,30 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             if (n > 0 && d_local < n_lev) {
                 static bool smem_set = false;  // opt-in above 48 KB, once (never inside a capture: a
                 if (!smem_set) {               // rebuild always follows a fresh build)
-                    cudaFuncSetAttribute(rcb_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalSmem);
+                    cudaFuncSetAttribute(rcb_local_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalSmem);
+                    cudaFuncSetAttribute(rcb_local_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalSmem);
                     smem_set = true;
                 }
                 LocalShape ls{};
-                ls.nlev = n_lev - d_local;
+                ls.pre = d_local - d_mid;
+                ls.nlev = n_lev - d_mid;
                 for (int l = 0; l < ls.nlev; ++l) {
-                    ls.tab[l] = shape->dtab + shape->level_off[d_local + l];
-                    ls.m[l] = (int32_t)shape->level_size[d_local + l];
+                    ls.tab[l] = shape->dtab + shape->level_off[d_mid + l];
+                    ls.m[l] = (int32_t)shape->level_size[d_mid + l];
                 }
-                rcb_local_kernel<<<(unsigned)shape->level_size[d_local], kLocalThreads, kLocalSmem, st>>>(
-                    n, ls, Lfin, ord, p->x, p->y, p->z, node_box, mem, An[0][0], An[0][1], flags + 5);
+                cudaLaunchConfig_t cfg{};
+                cfg.gridDim = dim3((unsigned)shape->level_size[d_mid] << ls.pre);
+                cfg.blockDim = dim3(kLocalThreads);
+                cfg.dynamicSmemBytes = kLocalSmem;
+                cfg.stream = st;
+                cudaLaunchAttribute cluster{};
+                cluster.id = cudaLaunchAttributeClusterDimension;
+                cluster.val.clusterDim.x = 1u << ls.pre;
+                cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+                cfg.attrs = &cluster;
+                cfg.numAttrs = ls.pre > 0 ? 1 : 0;
+                cudaLaunchKernelEx(&cfg, ls.pre > 0 ? rcb_local_kernel<true> : rcb_local_kernel<false>, n, ls, Lfin, ord,
+                                   p->x, p->y, p->z, node_box, mem, An[0][0], An[0][1], flags + 5);
                 rank_yz[0] = An[0][0];
                 rank_yz[1] = An[0][1];
                 ++ctx->launches;
