@@ -134,7 +134,7 @@ int crk_set_trace(crk_ctx *ctx, int on);
 #define CRK_VARIANT_HALFWARP_SMEM 6
 #define CRK_VARIANT_HALFWARP_LOAD 7
 /* gravity kernels: the tiles sweep with 8 particles per warp, 4 lanes per particle (TILES takes
- * 16 particles and 2 lanes per particle on boxes large enough to fill the GPU that way) */
+ * 16 particles and 2 lanes per particle) */
 #define CRK_VARIANT_SPLIT8 8
 #define CRK_N_VARIANTS 9
 int crk_set_variant(crk_ctx *ctx, int kernel, int variant);

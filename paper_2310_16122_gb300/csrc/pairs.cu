@@ -1999,14 +1999,14 @@ void launch_cells_g(const crk_ctx *ctx, const crk_leaves *lv, const LeafView &v,
     else cell_kernel<S, kCount, G, 4><<<(unsigned)grid, 128, 0, ctx->stream>>>(v, p, rec, units, log_cpl, full);
 }
 
-// SPLIT8: 8 particles per warp.  TILES: 16, or 8 where units of 16 are fewer
-// than the warps the GPU holds (28 per SM at the kernels' registers): a box of
-// 8192 particles then takes 35 / 43 us (gravity / adjoint) instead of 42 / 52,
-// one of 30011 43 / 70 instead of 47 / 68, one of 65,536 80 / 125 instead of 80 / 129.
+// TILES: 16 particles per warp, SPLIT8: 8, at every size: the split decides the order of an i's sums, and
+// a box of a batch gives the same bits as the box alone.  (8 would be faster where units of 16 are fewer
+// than the warps the GPU holds: a box of 8192 particles takes 42 / 52 us, gravity / adjoint, against
+// 35 / 43 with 8, one of 30,011 47 / 68 against 43 / 70, one of 65,536 80 / 129 against 80 / 125.)
 template <class S, bool kCount>
 void launch_cells(const crk_ctx *ctx, const crk_leaves *lv, const LeafView &v, const typename S::P &p,
                   RecView<typename S::Rec> rec, bool persistent, int warps, bool split8) {
-    if (split8 || lv->n < (int64_t)16 * 28 * ctx->num_sms) launch_cells_g<S, kCount, 8>(ctx, lv, v, p, rec, persistent, warps);
+    if (split8) launch_cells_g<S, kCount, 8>(ctx, lv, v, p, rec, persistent, warps);
     else launch_cells_g<S, kCount, 16>(ctx, lv, v, p, rec, persistent, warps);
 }
 
@@ -2850,8 +2850,8 @@ __host__ __device__ constexpr int table_cap() {
 }
 
 // resident blocks per SM that list_kernel<S> is compiled for (a register cap; 0: none).
-// Corrections is latency bound: capped for five blocks (96 registers, a few bytes spilled)
-// it ran 10.1 ms on the 2x256^3 box, against 11.0 ms at four and 10.3 ms uncapped.
+// Corrections is latency bound: capped for five blocks (96 registers, a few bytes spilled) it runs
+// 0.91 ms on the 2x128^3 box, against 0.95 ms at four and 1.07 ms at six.
 template <class S>
 struct list_min_blocks {
     static constexpr int value = 0;  // no register cap
@@ -2860,7 +2860,7 @@ template <>
 struct list_min_blocks<CorrStage> {
     static constexpr int value = 5;
 };
-// its reverse preparation: four blocks 295 us on the 2x64^3 box, five 299, uncapped 329
+// its reverse preparation: four blocks 259 us on the 2x64^3 box, three 262, five 327
 template <>
 struct list_min_blocks<CorrAdjPrepStage> {
     static constexpr int value = 4;

@@ -1,8 +1,7 @@
 """Gravity cell sweeps at the edges of their units, cells and leaves.
 
-Boxes large enough for units of 16 particles per warp (the small boxes of the
-other tests take units of 8): leaves that are no multiple of a unit, leaves of
-a handful of particles, chaining-mesh cells above 256 particles (no RCB cells
+Units of 16 and of 8 particles per warp: leaves that are no multiple of a unit,
+leaves of a handful of particles, chaining-mesh cells above 256 particles (no RCB cells
 inside, more cells of 32 than one leaf of 128 holds) and leaves of up to 1024,
 against the FP64 oracle at the gates of the other gravity tests.
 """
@@ -18,7 +17,7 @@ from tests.test_gpu_parity import boundary_pairs, cut_boundary_particles
 
 pytestmark = pytest.mark.gpu
 
-N = 70001  # above the particle count that takes units of 16 on any GB300
+N = 70001
 
 BOXES = {
     "leaf37": lambda: W.random_box(N, 33.0, 0.5, 301, max_leaf=37, h=1.0),
