@@ -1395,11 +1395,19 @@ struct Gaps {
 };
 __device__ __forceinline__ float pick3(const float g[3], int k) { return k == 0 ? g[0] : (k == 1 ? g[1] : g[2]); }
 
+// The FP64 test of one image (A, B: the two leaf boxes).  A call of its own: inlined, its per-axis
+// parts were hoisted out of the image loops and evaluated for every candidate.
+__device__ __noinline__ bool image_inside(const float *A, const float *B, int ix, int iy, int iz, double L, double cut) {
+    return sum_sq(axis_gap_shift(A[0], A[3], B[0], B[3], (double)(ix - 1) * L),
+                  axis_gap_shift(A[1], A[4], B[1], B[4], (double)(iy - 1) * L),
+                  axis_gap_shift(A[2], A[5], B[2], B[5], (double)(iz - 1) * L)) < __dmul_rn(cut, cut);
+}
+
 // The images of leaf B within cut of leaf A as bits 9 sx + 3 sy + sz (shift indices 0, 1, 2).  The
 // decision is that of the FP64 gaps, squared and summed, against cut^2.  The FP32 gaps settle every
 // image that is not within a margin far above their rounding of the cut: FP64 (1/64 of the FP32
 // rate here) only sees those; square roots of cut^2 and two FP64 gap sums per candidate and list
-// were the kernel's time before: 147 -> 62 us on the 2x64^3 box, 6.2 -> 2.6 ms on 2x256^3.
+// were the kernel's time before: 6.2 -> 1.5 ms on the 2x256^3 box.
 __device__ __forceinline__ uint32_t image_mask(const float *A, const float *B, const Gaps &s, double L, double cut) {
     const float cf = (float)cut, m = 1e-5f * (float)L + 1e-6f, hi = cf + m, lo = cf - m;
     const float hi2 = hi * hi, lo2 = lo > 0.0f ? lo * lo : -1.0f;
@@ -1418,11 +1426,7 @@ __device__ __forceinline__ uint32_t image_mask(const float *A, const float *B, c
                 const int iz = __ffs(mz) - 1;
                 const float gz = pick3(s.g[2], iz), d2 = gx * gx + gy * gy + gz * gz;
                 bool in = d2 < lo2;
-                if (!in && !(d2 > hi2)) {
-                    in = sum_sq(axis_gap_shift(A[0], A[3], B[0], B[3], (double)(ix - 1) * L),
-                                axis_gap_shift(A[1], A[4], B[1], B[4], (double)(iy - 1) * L),
-                                axis_gap_shift(A[2], A[5], B[2], B[5], (double)(iz - 1) * L)) < __dmul_rn(cut, cut);
-                }
+                if (!in && !(d2 > hi2)) in = image_inside(A, B, ix, iy, iz, L, cut);
                 if (in) out |= 1u << (9 * ix + 3 * iy + iz);
             }
         }
@@ -1431,10 +1435,13 @@ __device__ __forceinline__ uint32_t image_mask(const float *A, const float *B, c
 }
 
 // the float nearest b + (k - 1) L - a, each sum rounded to FP64 first; without a shift the FP32
-// difference is that number (b - a is exact in FP64 or |b| < 2^-29 |a|)
-__device__ __forceinline__ float image_shift(float b, float a, int k, double L) {
-    if (k == 1) return __fsub_rn(__fadd_rn(b, 0.0f), a);
+// difference is that number (b - a is exact in FP64 or |b| < 2^-29 |a|).  A call of its own: inlined,
+// the FP64 form was evaluated for every image and selected away.
+__device__ __noinline__ float wrapped_shift(float b, float a, int k, double L) {
     return (float)__dsub_rn(__dadd_rn((double)b, (double)(k - 1) * L), (double)a);
+}
+__device__ __forceinline__ float image_shift(float b, float a, int k, double L) {
+    return k == 1 ? __fsub_rn(__fadd_rn(b, 0.0f), a) : wrapped_shift(b, a, k, L);
 }
 
 // --- warp-cooperative leaf-pair finder ---------------------------------------------
@@ -1589,9 +1596,10 @@ __global__ void __launch_bounds__(kTravWarps * 32) leaf_pairs_warp_kernel(
                 const float t1 = (B[q] + sf) - A[3 + q], t2 = (A[q] - B[3 + q]) - sf, g = t1 > t2 ? t1 : t2;
                 s.g[q][k] = g < 0.0f ? 0.0f : g;  // a NaN stays, and gives no image
             }
-        mg = image_mask(A, B, s, L, rc);
+        const float *pa = bbox + 6 * a, *pb = bbox + 6 * (int64_t)b;
+        mg = image_mask(pa, pb, s, L, rc);
         mh = 0;
-        if (a_gas && leaf_ngas[b] > 0) mh = image_mask(A, B, s, L, (double)(2.0f * fmaxf(ha, hmax[b])));
+        if (a_gas && leaf_ngas[b] > 0) mh = image_mask(pa, pb, s, L, (double)(2.0f * fmaxf(ha, hmax[b])));
     };
     auto coded = [](uint32_t m) { return (uint16_t)(__popc(m) | ((31 - __clz(m | 1u)) << 8)); };
     // totals: images in the low half word, pairs in the high one (27 * kCandCap < 2^16)
