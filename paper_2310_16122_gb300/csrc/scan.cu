@@ -373,8 +373,9 @@ int crk_sort_axes(crk_ctx *ctx, const float *x, const float *y, const float *z, 
                    : radix_pass<kRadixPairs, false>(ctx, in, 3, nullptr, v[at ^ 1], counts, nb);
         if (rc) return rc;
     }
-    // batches: stable by box, so the order is (box, coordinate, index)
-    for (int shift = 0; box_of && (shift == 0 || (nbox - 1) >> shift); shift += 8, at ^= 1) {
+    // batches: stable by box, so the order is (box, coordinate, index); four digits at most (a shift by the
+    // width of an int is undefined, and the loop did not end above 2^24 boxes)
+    for (int shift = 0; box_of && (shift == 0 || (shift < 32 && (nbox - 1) >> shift)); shift += 8, at ^= 1) {
         in.val = v[at];
         in.shift = shift;
         if ((rc = radix_pass<kRadixBoxes, false>(ctx, in, 3, nullptr, v[at ^ 1], counts, nb))) return rc;
