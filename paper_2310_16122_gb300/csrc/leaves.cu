@@ -2353,17 +2353,21 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             unsigned long long *cur = (unsigned long long *)(lv->dev + 16);
             // first capacities: 1.5 times the leaves of the mean size within the cut of one (clustered
             // boxes hold 34 images a leaf and list, cubes of 128 particles at r_c = 3 an estimated 38),
-            // the hydro cut taken at the largest h but at most 128 a leaf
+            // the hydro cut taken at the largest h but at most 128 a leaf; never below 48 images and 32
+            // pairs a leaf, which rebuilds of particles that have since clustered may need
             double vol = 0.0;
-            for (float side : box_side) vol += (double)side * side * side;
+            for (int b = 0; b < nbox; ++b)
+                if (box_start[b + 1] > box_start[b]) vol += (double)box_side[b] * box_side[b] * box_side[b];
             const double ls = nl > 0 ? cbrt(vol / (double)nl) : 1.0;
             auto images = [&](double cut, double most) {
                 const double w = 2.0 * ls;  // leaf boxes nearer than cut: Minkowski sum of two leaves and a ball
                 const double v = w * w * w + 6.0 * w * w * cut + 9.42 * w * cut * cut + 4.19 * cut * cut * cut;
-                return nl * (int64_t)std::min(most, 1.5 * v / (ls * ls * ls) + 16.0) + 64;
+                return (int64_t)std::min(most, 1.5 * v / (ls * ls * ls) + 16.0);
             };
-            const int64_t cg = images((double)lp->r_cut_grav, (double)kCandCap), ch = images(2.0 * lv->hmax_all, 128.0);
-            int64_t cap[4] = {cg, cg, ch, ch};
+            const int64_t ig = images((double)lp->r_cut_grav, (double)kCandCap), ih = images(2.0 * lv->hmax_all, 128.0);
+            int64_t cap[4] = {std::max<int64_t>(ig, 48), std::max<int64_t>(ig, 32), std::max<int64_t>(ih, 48),
+                              std::max<int64_t>(ih, 32)};
+            for (int64_t &c : cap) c = c * nl + 64;
             if (re)
                 for (int k = 0; k < 4; ++k) cap[k] = lv->img_cap[k];
             crk_image *gimg = lv->gimg, *himg = lv->himg;
