@@ -942,31 +942,65 @@ struct CorrAdjPrepStage : CorrStage {
     // this finish (2,500 FP32 instructions in float pairs) is the other half of the kernel's time: 422 ->
     // 295 us on the 2x64^3 box against the reverse taken through the 30 unreduced sums dm1, dm2, 260 us
     // in float pairs.
+    // The reverse is linear in the cotangents, and a float pair holds its 47 bits only while its low word is a
+    // normal number: it works on them (in scaled lengths) in units u of a power of two near the largest, c = 1/u.
+    // False where the unit or the lengths are so far from 1 that products of the scales leave the FP32 range.
+    __device__ static bool unit_of(const float *, double, double &c, double &u) {
+        c = u = 1.0;
+        return true;
+    }
+    __device__ static bool unit_of(const float cot[16], float f1, float &c, float &u) {
+        float m[3] = {fabsf(cot[0]), 0.0f, 0.0f};
+#pragma unroll
+        for (int k = 1; k < 7; ++k) m[1] = fmaxf(m[1], fabsf(cot[k]));
+#pragma unroll
+        for (int k = 7; k < 16; ++k) m[2] = fmaxf(m[2], fabsf(cot[k]));
+        c = u = 1.0f;
+        if (fmaxf(m[0], fmaxf(m[1], m[2])) == 0.0f) return true;
+        const float most = fmaxf(m[0], fmaxf(m[1], m[2] * f1) * f1);
+        if (!(most > 0x1p-60f && most < 0x1p60f && f1 > 0x1p-30f && f1 < 0x1p30f)) return false;
+        const int e = __float_as_int(most) >> 23;  // exponent + 127
+        c = __int_as_float((254 - e) << 23);
+        u = __int_as_float(e << 23);
+        return true;
+    }
     template <class T>
     __device__ static bool finish_in(const P &p, const I &s, int32_t o) {
         using F = typename beside<T>::type;
         const int64_t n = p.n;
         Solved<T> r;
         if (!solve(s, r)) return false;
-        const F f1 = r.f1, f2 = f1 * f1;
+        const F f1 = r.f1;
+        float cot[16];  // A, B, dA, dB (3g+a)
+        cot[0] = p.Abar[o];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            cot[1 + k] = p.Bbar[k * n + o];
+            cot[4 + k] = p.gAbar[k * n + o];
+        }
+#pragma unroll
+        for (int k = 0; k < 9; ++k) cot[7 + k] = p.gBbar[k * n + o];
+        F c0, u0;
+        if (!unit_of(cot, f1, c0, u0)) return false;
+        const F c1 = c0 * f1, c2 = c1 * f1, u1 = u0 * f1, u2 = u1 * f1, v1 = u0 * r.g1;
         float sum = 0.0f;  // NaN once a result is not finite
         auto put = [&](int k, float v) {
             p.coef[k * n + o] = v;
             sum = fmaf(v, 0.0f, sum);
         };
         T H[3][3], Kb[3], Bb[3], Ab, qb;
-        difference((F)p.Abar[o], (F)0, Ab);
+        difference(cot[0] * c0, (F)0, Ab);
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
             T gAb;
 #pragma unroll
-            for (int a = 0; a < 3; ++a) difference((F)p.gBbar[(3 * g + a) * n + o] * f2, (F)0, H[g][a]);
-            difference((F)p.gAbar[g * n + o] * f1, (F)0, gAb);
-            difference((F)p.Bbar[g * n + o] * f1, (F)0, Bb[g]);
+            for (int a = 0; a < 3; ++a) difference(cot[7 + 3 * g + a] * c2, (F)0, H[g][a]);
+            difference(cot[4 + g] * c1, (F)0, gAb);
+            difference(cot[1 + g] * c1, (F)0, Bb[g]);
             const T Ag = -(r.A * gAb);
             Kb[g] = r.A * Ag;
             Ab = mad(twice(Ag), r.K[g], Ab);
-            put(10 + g, rounded(Kb[g] * r.g1));  // l1: dm0
+            put(10 + g, rounded(Kb[g] * v1));  // l1: dm0
         }
         // dB_g^a = B_a B_g - (Mi Uq)_ag and K_g = dm0_g + 2 q B_g + ((2 s2 + T) B)_g
         T Mib[3][3], Uqb[3][3];
@@ -996,7 +1030,7 @@ struct CorrAdjPrepStage : CorrStage {
             const int a = ia[k], b = ib[k];
             const T w = a == b ? Kb[a] * r.B[a] : mad(Kb[a], r.B[b], Kb[b] * r.B[a]);
             Tb[k] = (a == b ? Uqb[a][a] : Uqb[a][b] + Uqb[b][a]) + w;
-            put(13 + k, rounded(Tb[k] + w));  // q1: s2
+            put(13 + k, rounded((Tb[k] + w) * u0));  // q1: s2
         }
         // T = s3 B: Bb_c += sum_ab Tb_ab s3_abc, and s3's coefficients are those of (x^T Tb x)(B.x)
 #pragma unroll
@@ -1004,24 +1038,24 @@ struct CorrAdjPrepStage : CorrStage {
 #pragma unroll
             for (int k = 0; k < 6; ++k) Bb[c] = mad(Tb[k], r.s3[sorted3(ia[k], ib[k], c)], Bb[c]);
         const T *B = r.B;
-        put(19, rounded(Tb[0] * B[0] * f1));
-        put(20, rounded(mad(Tb[0], B[1], Tb[1] * B[0]) * f1));
-        put(21, rounded(mad(Tb[0], B[2], Tb[2] * B[0]) * f1));
-        put(22, rounded(mad(Tb[1], B[1], Tb[3] * B[0]) * f1));
-        put(23, rounded(dot3(Tb[1], B[2], Tb[2], B[1], Tb[4], B[0]) * f1));
-        put(24, rounded(mad(Tb[2], B[2], Tb[5] * B[0]) * f1));
-        put(25, rounded(Tb[3] * B[1] * f1));
-        put(26, rounded(mad(Tb[3], B[2], Tb[4] * B[1]) * f1));
-        put(27, rounded(mad(Tb[4], B[2], Tb[5] * B[1]) * f1));
-        put(28, rounded(Tb[5] * B[2] * f1));
+        put(19, rounded(Tb[0] * B[0] * u1));
+        put(20, rounded(mad(Tb[0], B[1], Tb[1] * B[0]) * u1));
+        put(21, rounded(mad(Tb[0], B[2], Tb[2] * B[0]) * u1));
+        put(22, rounded(mad(Tb[1], B[1], Tb[3] * B[0]) * u1));
+        put(23, rounded(dot3(Tb[1], B[2], Tb[2], B[1], Tb[4], B[0]) * u1));
+        put(24, rounded(mad(Tb[2], B[2], Tb[5] * B[0]) * u1));
+        put(25, rounded(Tb[3] * B[1] * u1));
+        put(26, rounded(mad(Tb[3], B[2], Tb[4] * B[1]) * u1));
+        put(27, rounded(mad(Tb[4], B[2], Tb[5] * B[1]) * u1));
+        put(28, rounded(Tb[5] * B[2] * u1));
         // A = 1/q, q = m0 + B.m1, B = -Mi m1, Mi = m2^-1
         qb = mad(-(r.A * Ab), r.A, qb);
-        put(0, rounded(qb));  // c0: m0
+        put(0, rounded(qb * u0));  // c0: m0
 #pragma unroll
         for (int a = 0; a < 3; ++a) Bb[a] = mad(qb, r.m1[a], Bb[a]);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            put(1 + a, rounded(mad(qb, r.B[a], -row(r.Mi, a, Bb)) * f1));  // l0: m1
+            put(1 + a, rounded(mad(qb, r.B[a], -row(r.Mi, a, Bb)) * u1));  // l0: m1
 #pragma unroll
             for (int b = 0; b < 3; ++b) Mib[a][b] = mad(-Bb[a], r.m1[b], Mib[a][b]);
         }
@@ -1039,7 +1073,7 @@ struct CorrAdjPrepStage : CorrStage {
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             const T c[3] = {Y[0][ib[k]], Y[1][ib[k]], Y[2][ib[k]]};
-            put(4 + k, rounded(row(r.Mi, ia[k], c) * ((ia[k] == ib[k] ? (F)-0.5 : (F)-1.0) * f2)));  // q0: m2
+            put(4 + k, rounded(row(r.Mi, ia[k], c) * ((ia[k] == ib[k] ? (F)-0.5 : (F)-1.0) * u2)));  // q0: m2
         }
         return std::is_same<T, double>::value || sum == 0.0f;
     }
