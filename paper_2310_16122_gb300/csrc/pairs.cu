@@ -48,11 +48,12 @@ struct rec_words<R, std::void_t<decltype(R::kWords)>> {
 // lines per load (8 records a line and quad), where whole records cost a line
 // per lane, and in shared memory the 16-byte stride spreads random records
 // over all banks.  Whole (Rec::kWhole): records side by side, for one whose
-// gather is bound by L1 misses rather than by lookups.  Measured on the
-// 2x64^3 clustered box, whole -> planes: Extras 226 -> 172 us, corrections
-// 198 -> 178, geometry adjoint 90 -> 70, hydro adjoint 518 -> 378,
-// Acceleration 383 -> 356, Energy 393 -> 378, hydro 253 -> 260; corrections
-// adjoint (136 bytes) 300 -> 338, kept whole.
+// gather is bound by L1 misses rather than by lookups.  Single calls on the
+// 2x64^3 clustered box, whole -> planes, us: Extras 275 -> 214, corrections 206
+// -> 190, geometry adjoint 108 -> 87, hydro adjoint 687 -> 552, Energy 563 ->
+// 355 (limited 471 -> 450).  Kept whole: hydro 319 -> 327, limited 387 -> 412,
+// Acceleration 347 -> 354, limited 416 -> 430 (up to 15% on uniform boxes with
+// less gas), corrections adjoint (its second kernel 300 -> 338).
 template <class R, class = void>
 struct rec_whole : std::false_type {};
 template <class R>
@@ -1245,7 +1246,9 @@ struct HydroStageT {
     static constexpr bool kAllVariants = kPass == kHydroBoth;  // the step passes: lists and tiles only
     using P = HydroP;
     using Base = std::conditional_t<kLim, HydroRecLim, HydroRec>;
-    struct __align__(16) Rec : std::conditional_t<kPass == kHydroEnergy, HydroRecVstar<Base>, Base> {};
+    struct __align__(16) Rec : std::conditional_t<kPass == kHydroEnergy, HydroRecVstar<Base>, Base> {
+        static constexpr bool kWhole = kPass != kHydroEnergy;
+    };
     struct I {
         float fx, fy, fz, e;
         int cnt;
@@ -1493,6 +1496,7 @@ __device__ __forceinline__ void grad_wr_vjp(const R &r, const float y[3], float 
     }
 }
 
+template <bool kWholeRec>
 struct HydroAdjStage {
     static constexpr bool kPair = false;
     static constexpr bool kGasOnly = true;
@@ -1501,6 +1505,7 @@ struct HydroAdjStage {
     using P = HydroAdjP;
     struct __align__(16) Rec : HydroRec {
         float ax, ay, az, b;  // dvbar/m, dubar/m
+        static constexpr bool kWhole = kWholeRec;
     };
     struct I {
         float xb[3], vb[3], Vb, Pb, cb, rb, Ab, Bb[3], gAb[3], gBb[9], F[3], E;
@@ -3401,6 +3406,16 @@ int permute_bundle(crk_ctx *ctx, int64_t n, const int32_t *perm, const Bundle &b
     return CRK_OK;
 }
 
+// The hydro adjoint's records: planes, and whole records where gas is below an eighth of the particles (few
+// lanes of a group are active, and each reads a record of its own).  The call, whole -> planes, us: 687 -> 552
+// on the 2x64^3 box; uniform boxes of 500,009 particles, a fifth of them gas, 391 -> 339, of 300,007, a
+// twentieth, 229 -> 243, of 880,001, a fiftieth, 501 -> 532.
+int run_hydro_adjoint(crk_ctx *ctx, const crk_leaves *lv, const HydroAdjP &p, bool korder) {
+    if (lv->n_gas < lv->n / 8)
+        return run_stage<HydroAdjStage<true>>(ctx, lv, p, true, CRK_K_HYDRO, nullptr, korder);
+    return run_stage<HydroAdjStage<false>>(ctx, lv, p, true, CRK_K_HYDRO, nullptr, korder);
+}
+
 // Single calls of the gas stages on large boxes: the caller's columns are
 // permuted into the kernel order, the stage runs there and its outputs are
 // permuted back, instead of gathering and scattering every column at random
@@ -3648,7 +3663,7 @@ int crk_hydro_adjoint(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params
                 ko.output(gradAbar3, 3), ko.output(gradBbar9, 9), hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n,
                 nullptr, nullptr};
     const int rc = ko.begin();
-    return rc ? rc : ko.end(run_stage<HydroAdjStage>(ctx, lv, p, true, CRK_K_HYDRO, nullptr, ko.on));
+    return rc ? rc : ko.end(run_hydro_adjoint(ctx, lv, p, ko.on));
 }
 
 template <bool kGas>
@@ -4045,7 +4060,7 @@ int crk_hydro_chain_adjoint(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_
         HydroAdjP p{C(cm),  C(cv),  C(cu),   C(cV),   C(crho),   C(cA),  C(cB),  C(cgA),     C(cgB),
                     C(cdvb), C(cdub), C(cxh), C(cvb), C(cub), C(cmh), C(cVh), C(crhob), C(cAb),
                     C(cBb), C(cgAb), C(cgBb), hp->gamma, hp->alpha, hp->beta, hp->eta2, n, nullptr, nullptr};
-        if ((rc = run_stage<HydroAdjStage>(ctx, lv, p, true, CRK_K_HYDRO, nullptr, true))) return rc;
+        if ((rc = run_hydro_adjoint(ctx, lv, p, true))) return rc;
     }
     {
         CorrAdjP p{};
