@@ -3426,24 +3426,41 @@ int run_hydro_adjoint(crk_ctx *ctx, const crk_leaves *lv, const HydroAdjP &p, bo
 // Single calls of the gas stages on large boxes: the caller's columns are
 // permuted into the kernel order, the stage runs there and its outputs are
 // permuted back, instead of gathering and scattering every column at random
-// 4-byte places inside the stage's kernels.  Geometry, corrections and hydro,
-// direct -> permuted: 0.62 -> 0.64 ms on 524,288 particles, 1.13 -> 1.12 on
-// 1.02M, 2.17 -> 1.83 on 1.77M, 6.47 -> 4.22 on 4.19M; with Extras,
-// Acceleration and Energy 1.36 -> 1.42, 2.61 -> 2.50, 4.89 -> 4.16, 13.8 -> 9.8.
-// (The gravity calls, four columns each way, gain nothing: 8.33 -> 8.42 ms on
-// 4.19M, 68.3 -> 68.1 on 33.5M.)
+// 4-byte places inside the stage's kernels.  In units of one column streamed
+// through the rows, the permutation costs the columns in and out (all
+// particles) and about 5 more; it saves
+//   * 2 per column that the stage scatters (dark matter gets zeros, so all
+//     particles count), 6 once those columns no longer fit L2 together;
+//   * 1 per column that it gathers and share of gas (gas rows only), 3 once
+//     those columns do not fit.
+// Uniform boxes, direct -> permuted, ms, at 2%, 20%, 50% and 100% gas: hydro on
+// 900,001 particles 0.22 -> 0.28, 0.31 -> 0.35, 0.55 -> 0.57, 0.94 -> 0.94, on
+// 4M 0.71 -> 0.96, 1.37 -> 1.28, 2.73 -> 2.33, 4.68 -> 3.85; corrections on
+// 900,001 0.23 -> 0.18, 0.24 -> 0.21, 0.32 -> 0.30, 0.45 -> 0.48, on 4M 1.85 ->
+// 0.62, 1.94 -> 1.19 at 50%; Extras on 4M 1.11 -> 0.78, 2.16 -> 1.64 at 50%.
+// Where the permuted form is taken it is at most 6% slower than the direct one
+// (corrections without dark matter near 1M); the rule errs towards the direct
+// form.  The gravity calls, four columns each way, gain nothing: 8.33 -> 8.42 ms
+// on 4.19M, 68.3 -> 68.1 on 33.5M.
 constexpr int64_t kKorderMin = 900000;
+constexpr int64_t kKorderL2 = 128 << 20;
+bool kernel_order_pays(int64_t n, int64_t n_gas, int in, int out, int scattered) {
+    const int64_t written = (4 * scattered * n > kKorderL2 ? 6 : 2) * scattered * n;
+    const int64_t read = (4 * in * n > kKorderL2 ? 3 : 1) * in * n_gas;
+    return n >= kKorderMin && written + read >= (in + out + 5) * n;
+}
 struct KernelOrder {
     crk_ctx *ctx;
     const crk_leaves *lv;
     bool on;
     float *next = nullptr;
     Bundle in, out;
-    // cols: columns the call will ask for
-    KernelOrder(crk_ctx *c, const crk_leaves *l, int cols) : ctx(c), lv(l) {
-        on = lv->n >= kKorderMin;
+    // ni, no: columns the call reads and writes; scattered: columns that its kernels write in the
+    // caller's order (its intermediate ones among them)
+    KernelOrder(crk_ctx *c, const crk_leaves *l, int ni, int no, int scattered) : ctx(c), lv(l) {
+        on = kernel_order_pays(lv->n, lv->n_gas, ni, no, scattered);
         if (!on) return;
-        next = (float *)crk_scratch(ctx, 37, sizeof(float) * (size_t)cols * (size_t)lv->n);
+        next = (float *)crk_scratch(ctx, 37, sizeof(float) * (size_t)(ni + no) * (size_t)lv->n);
         on = next != nullptr;  // without room for the columns: the direct form
     }
     float *take(int comps) {
@@ -3518,7 +3535,7 @@ int crk_geometry_adjoint(crk_ctx *ctx, const crk_leaves *lv, const float *m, con
     if (!ctx) return CRK_EINVAL;
     if (!lv) return crk_fail(ctx, CRK_EINVAL, "null leaves");
     if (lv->n > 0 && (!m || !V || !rhobar || !gx3 || !gm)) return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 4 + 4);
+    KernelOrder ko(ctx, lv, Vbar ? 4 : 3, 4, 4);
     GeomAdjP p{ko.input(m, 1), ko.input(V, 1), ko.input(rhobar, 1), ko.input(Vbar, 1), ko.output(gx3, 3),
                ko.output(gm, 1), lv->n, nullptr};
     const int rc = ko.begin();
@@ -3531,7 +3548,7 @@ int crk_corrections(crk_ctx *ctx, const crk_leaves *lv, const float *V, float *A
     if (!lv) return crk_fail(ctx, CRK_EINVAL, "null leaves");
     if (lv->n > 0 && (!V || !A || !B || !gradA || !gradB)) return crk_fail(ctx, CRK_EINVAL, "null array");
     if (n_singular) CRK_CUDA(ctx, cudaMemsetAsync(n_singular, 0, sizeof(int32_t), ctx->stream));
-    KernelOrder ko(ctx, lv, 1 + 16);
+    KernelOrder ko(ctx, lv, 1, 16, 16);
     CorrP p{ko.input(V, 1), ko.output(A, 1), ko.output(B, 3), ko.output(gradA, 3), ko.output(gradB, 9), n_singular,
             lv->n, nullptr};
     const int rc = ko.begin();
@@ -3545,7 +3562,7 @@ int crk_hydro(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params *hp, co
     if (!lv || !hp) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvdt3 || !dudt))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 23 + 4);
+    KernelOrder ko(ctx, lv, 23, 4, 4);
     HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
              ko.input(gradA, 3), ko.input(gradB, 9), ko.output(dvdt3, 3), ko.output(dudt, 1), conservation,
              hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count};
@@ -3560,7 +3577,7 @@ int crk_extras(crk_ctx *ctx, const crk_leaves *lv, const float *m, const float *
     if (!lv) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !V || !A || !B || !gradA || !gradB || !rho_r || !dvdx))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 21 + 10);
+    KernelOrder ko(ctx, lv, 21, 10, 10);
     ExtrasP p{ko.input(m, 1), ko.input(v3, 3), ko.input(V, 1), ko.input(A, 1), ko.input(B, 3), ko.input(gradA, 3),
               ko.input(gradB, 9), ko.output(rho_r, 1), ko.output(dvdx, 9), lv->n, (unsigned long long *)pair_count};
     const int rc = ko.begin();
@@ -3575,7 +3592,7 @@ int crk_hydro_limited(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params
     if (!lv || !hp) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvdx || !dvdt3 || !dudt))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 32 + 4);
+    KernelOrder ko(ctx, lv, 32, 4, 4);
     HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
              ko.input(gradA, 3), ko.input(gradB, 9), ko.output(dvdt3, 3), ko.output(dudt, 1), conservation,
              hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, ko.input(dvdx, 9)};
@@ -3592,7 +3609,7 @@ int crk_hydro_accel(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params *
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvdt3))
         return crk_fail(ctx, CRK_EINVAL, "null array");
     if (!(sig_beta >= 0.0f)) return crk_fail(ctx, CRK_EINVAL, "sig_beta must be >= 0");
-    KernelOrder ko(ctx, lv, 32 + 3);
+    KernelOrder ko(ctx, lv, dvdx ? 32 : 23, 3, 3);
     HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
              ko.input(gradA, 3), ko.input(gradB, 9), ko.output(dvdt3, 3), nullptr, conservation,
              hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, ko.input(dvdx, 9)};
@@ -3612,7 +3629,7 @@ int crk_hydro_energy(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params 
     if (!lv || !hp) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !vstar3 || !dudt))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 35 + 1);
+    KernelOrder ko(ctx, lv, 23 + (dvdx ? 9 : 0) + (vstar3 == v3 ? 0 : 3), 1, 1);
     HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
              ko.input(gradA, 3), ko.input(gradB, 9), nullptr, ko.output(dudt, 1), conservation,
              hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, ko.input(dvdx, 9)};
@@ -3635,7 +3652,7 @@ int crk_corrections_adjoint(crk_ctx *ctx, const crk_leaves *lv, const float *V, 
     if (n == 0) return CRK_OK;
     float *coef = (float *)crk_scratch(ctx, 33, sizeof(float) * kCorrCoef * (size_t)n);
     if (!coef) return crk_fail(ctx, CRK_ENOMEM, "adjoint scratch");
-    KernelOrder ko(ctx, lv, 17 + 4);
+    KernelOrder ko(ctx, lv, 17, 4, 4 + kCorrCoef);
     CorrAdjP p{};
     p.V = ko.input(V, 1);
     p.n_singular = n_singular;
@@ -3662,7 +3679,7 @@ int crk_hydro_adjoint(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvbar3 || !dubar || !xbar3 ||
                       !vbar3 || !ubar || !mbar || !Vbar || !rhobar || !Abar || !Bbar3 || !gradAbar3 || !gradBbar9))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 27 + 26);
+    KernelOrder ko(ctx, lv, 27, 26, 26);
     HydroAdjP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
                 ko.input(gradA, 3), ko.input(gradB, 9),
                 ko.input(dvbar3, 3), ko.input(dubar, 1), ko.output(xbar3, 3), ko.output(vbar3, 3), ko.output(ubar, 1),
