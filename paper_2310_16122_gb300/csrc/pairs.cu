@@ -3460,6 +3460,14 @@ struct KernelOrder {
     KernelOrder(crk_ctx *c, const crk_leaves *l, int ni, int no, int scattered) : ctx(c), lv(l) {
         on = kernel_order_pays(lv->n, lv->n_gas, ni, no, scattered);
         if (!on) return;
+        // never in a captured call: its columns may not exist yet (no allocation there), and a graph must not
+        // hold scratch that a later call may grow
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess) cudaGetLastError();
+        if (cs != cudaStreamCaptureStatusNone) {
+            on = false;
+            return;
+        }
         next = (float *)crk_scratch(ctx, 37, sizeof(float) * (size_t)(ni + no) * (size_t)lv->n);
         on = next != nullptr;  // without room for the columns: the direct form
     }
