@@ -28,6 +28,12 @@
  *    synchronisation (singular moment matrices, pair counts) are written to
  *    optional device outputs instead.
  *  - Calls on one context must not run concurrently from several host threads.
+ *  - A context keeps its scratch memory until crk_destroy.  The single gas
+ *    calls on large boxes (900,000 particles and more, by columns and share of
+ *    gas) keep 4 bytes a particle and column they read or write, up to 53
+ *    columns (crk_hydro_adjoint); that part is freed when another allocation
+ *    of the context finds no room, and without room for it such a call runs
+ *    in another form with the same results.
  */
 #ifndef CRK_H
 #define CRK_H

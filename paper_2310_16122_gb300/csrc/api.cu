@@ -23,6 +23,18 @@ int crk_check_cuda(crk_ctx *ctx, cudaError_t e, const char *what) {
     return crk_fail(ctx, CRK_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+// device memory, or (nothing left) once more without the columns of earlier single calls
+static void *crk_malloc(crk_ctx *ctx, size_t bytes, int slot) {
+    void *p = nullptr;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+        cudaGetLastError();
+        if (slot == crk_ctx::kColumns || ctx->columns_live || !ctx->slot[crk_ctx::kColumns]) return nullptr;
+        crk_scratch_drop(ctx, crk_ctx::kColumns);
+    }
+    return nullptr;
+}
+
 // Growable per-slot scratch.  Growing frees the old buffer: cudaFree waits for
 // the device, so work still using it on the context stream has finished.
 void *crk_scratch(crk_ctx *ctx, int slot, size_t bytes) {
@@ -36,15 +48,19 @@ void *crk_scratch(crk_ctx *ctx, int slot, size_t bytes) {
     void *p = nullptr;
     if (cudaMalloc(&p, want) != cudaSuccess) {
         cudaGetLastError();
-        if (cudaMalloc(&p, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
         want = bytes;
+        p = crk_malloc(ctx, bytes, slot);
+        if (!p) return nullptr;
     }
     ctx->slot[slot] = p;
     ctx->slot_bytes[slot] = want;
     return p;
+}
+
+void crk_scratch_drop(crk_ctx *ctx, int slot) {
+    if (ctx->slot[slot]) cudaFree(ctx->slot[slot]);
+    ctx->slot[slot] = nullptr;
+    ctx->slot_bytes[slot] = 0;
 }
 
 void *crk_leaves_alloc(crk_ctx *ctx, crk_leaves *lv, size_t bytes) {
@@ -69,10 +85,8 @@ void *crk_leaves_alloc(crk_ctx *ctx, crk_leaves *lv, size_t bytes) {
         // drop the cache and retry once
         for (auto &b : ctx->block_cache) cudaFree(b.first);
         ctx->block_cache.clear();
-        if (cudaMalloc(&p, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
+        p = crk_malloc(ctx, bytes, -1);
+        if (!p) return nullptr;
     }
     lv->allocs.push_back({p, bytes});
     return p;

@@ -51,8 +51,10 @@ struct crk_ctx {
     static const int kSlots = 38;  // leaf build 0-16 and 19-31, radix sort 12-14, scan 15, queue 17, step 18,
                                    // integrator 32, corrections adjoint 33, adjoint chain 34, half-warp force 35,
                                    // tuner 36, single calls' kernel-order columns 37
+    static const int kColumns = 37;  // the one slot no later call relies on: given back when memory runs short
     void *slot[kSlots] = {};
     size_t slot_bytes[kSlots] = {};
+    bool columns_live = false;  // a call is using slot kColumns
     int64_t launches = 0;  // kernels this context has launched
     // device blocks released by crk_leaves_free, reused by later leaf builds
     // on this context (stream order makes the reuse safe)
@@ -145,6 +147,7 @@ struct crk_leaves {
 int crk_fail(crk_ctx *ctx, int code, const char *fmt, ...);
 int crk_check_cuda(crk_ctx *ctx, cudaError_t e, const char *what);
 void *crk_scratch(crk_ctx *ctx, int slot, size_t bytes);
+void crk_scratch_drop(crk_ctx *ctx, int slot);
 void *crk_leaves_alloc(crk_ctx *ctx, crk_leaves *lv, size_t bytes);
 void crk_rcb_shape_free(crk_ctx *ctx);
 // neighbour lists of the leaves; reuse: a rebuild into the buffers of the first build (no host

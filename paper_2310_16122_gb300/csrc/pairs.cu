@@ -3456,8 +3456,8 @@ struct KernelOrder {
     float *next = nullptr;
     Bundle in, out;
     // ni, no: columns the call reads and writes; scattered: columns that its kernels write in the
-    // caller's order (its intermediate ones among them)
-    KernelOrder(crk_ctx *c, const crk_leaves *l, int ni, int no, int scattered) : ctx(c), lv(l) {
+    // caller's order (its intermediate ones among them); record: bytes of its stage's largest record
+    KernelOrder(crk_ctx *c, const crk_leaves *l, int ni, int no, int scattered, size_t record) : ctx(c), lv(l) {
         on = kernel_order_pays(lv->n, lv->n_gas, ni, no, scattered);
         if (!on) return;
         // never in a captured call: its columns may not exist yet (no allocation there), and a graph must not
@@ -3468,9 +3468,18 @@ struct KernelOrder {
             on = false;
             return;
         }
-        next = (float *)crk_scratch(ctx, 37, sizeof(float) * (size_t)(ni + no) * (size_t)lv->n);
-        on = next != nullptr;  // without room for the columns: the direct form
+        // the columns, and the rows they pass through (later the records), before anything runs; without room:
+        // the direct form
+        const size_t row = std::max(sizeof(float4) * (size_t)((std::max(ni, no) + 3) / 4), record);
+        next = (float *)crk_scratch(ctx, crk_ctx::kColumns, sizeof(float) * (size_t)(ni + no) * (size_t)lv->n);
+        on = ctx->columns_live = next != nullptr;
+        if (on && !crk_scratch(ctx, 4, row * (size_t)lv->n)) {
+            crk_scratch_drop(ctx, crk_ctx::kColumns);
+            on = ctx->columns_live = false;
+        }
     }
+    ~KernelOrder() { ctx->columns_live = false; }
+    KernelOrder(const KernelOrder &) = delete;
     float *take(int comps) {
         float *r = next;
         next += (size_t)comps * lv->n;
@@ -3491,6 +3500,13 @@ struct KernelOrder {
     int begin() { return on ? permute_bundle(ctx, lv->n, lv->kperm, in) : CRK_OK; }
     int end(int rc) { return rc || !on ? rc : permute_bundle(ctx, lv->n, lv->kinv, out); }
 };
+
+template <class... S>
+constexpr size_t record_bytes() {
+    size_t most = 0;
+    ((most = std::max(most, (size_t)Planes<typename S::Rec>::kBytes)), ...);
+    return most;
+}
 
 }  // namespace
 
@@ -3543,7 +3559,7 @@ int crk_geometry_adjoint(crk_ctx *ctx, const crk_leaves *lv, const float *m, con
     if (!ctx) return CRK_EINVAL;
     if (!lv) return crk_fail(ctx, CRK_EINVAL, "null leaves");
     if (lv->n > 0 && (!m || !V || !rhobar || !gx3 || !gm)) return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, Vbar ? 4 : 3, 4, 4);
+    KernelOrder ko(ctx, lv, Vbar ? 4 : 3, 4, 4, record_bytes<GeomAdjStage>());
     GeomAdjP p{ko.input(m, 1), ko.input(V, 1), ko.input(rhobar, 1), ko.input(Vbar, 1), ko.output(gx3, 3),
                ko.output(gm, 1), lv->n, nullptr};
     const int rc = ko.begin();
@@ -3556,7 +3572,7 @@ int crk_corrections(crk_ctx *ctx, const crk_leaves *lv, const float *V, float *A
     if (!lv) return crk_fail(ctx, CRK_EINVAL, "null leaves");
     if (lv->n > 0 && (!V || !A || !B || !gradA || !gradB)) return crk_fail(ctx, CRK_EINVAL, "null array");
     if (n_singular) CRK_CUDA(ctx, cudaMemsetAsync(n_singular, 0, sizeof(int32_t), ctx->stream));
-    KernelOrder ko(ctx, lv, 1, 16, 16);
+    KernelOrder ko(ctx, lv, 1, 16, 16, record_bytes<CorrStage>());
     CorrP p{ko.input(V, 1), ko.output(A, 1), ko.output(B, 3), ko.output(gradA, 3), ko.output(gradB, 9), n_singular,
             lv->n, nullptr};
     const int rc = ko.begin();
@@ -3570,7 +3586,7 @@ int crk_hydro(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params *hp, co
     if (!lv || !hp) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvdt3 || !dudt))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 23, 4, 4);
+    KernelOrder ko(ctx, lv, 23, 4, 4, record_bytes<HydroStage>());
     HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
              ko.input(gradA, 3), ko.input(gradB, 9), ko.output(dvdt3, 3), ko.output(dudt, 1), conservation,
              hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count};
@@ -3585,7 +3601,7 @@ int crk_extras(crk_ctx *ctx, const crk_leaves *lv, const float *m, const float *
     if (!lv) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !V || !A || !B || !gradA || !gradB || !rho_r || !dvdx))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 21, 10, 10);
+    KernelOrder ko(ctx, lv, 21, 10, 10, record_bytes<ExtrasStage>());
     ExtrasP p{ko.input(m, 1), ko.input(v3, 3), ko.input(V, 1), ko.input(A, 1), ko.input(B, 3), ko.input(gradA, 3),
               ko.input(gradB, 9), ko.output(rho_r, 1), ko.output(dvdx, 9), lv->n, (unsigned long long *)pair_count};
     const int rc = ko.begin();
@@ -3600,7 +3616,7 @@ int crk_hydro_limited(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params
     if (!lv || !hp) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvdx || !dvdt3 || !dudt))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 32, 4, 4);
+    KernelOrder ko(ctx, lv, 32, 4, 4, record_bytes<HydroLimStage>());
     HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
              ko.input(gradA, 3), ko.input(gradB, 9), ko.output(dvdt3, 3), ko.output(dudt, 1), conservation,
              hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, ko.input(dvdx, 9)};
@@ -3617,7 +3633,7 @@ int crk_hydro_accel(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params *
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvdt3))
         return crk_fail(ctx, CRK_EINVAL, "null array");
     if (!(sig_beta >= 0.0f)) return crk_fail(ctx, CRK_EINVAL, "sig_beta must be >= 0");
-    KernelOrder ko(ctx, lv, dvdx ? 32 : 23, 3, 3);
+    KernelOrder ko(ctx, lv, dvdx ? 32 : 23, 3, 3, record_bytes<HydroAccelStage<true>>());
     HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
              ko.input(gradA, 3), ko.input(gradB, 9), ko.output(dvdt3, 3), nullptr, conservation,
              hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, ko.input(dvdx, 9)};
@@ -3637,7 +3653,7 @@ int crk_hydro_energy(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params 
     if (!lv || !hp) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !vstar3 || !dudt))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 23 + (dvdx ? 9 : 0) + (vstar3 == v3 ? 0 : 3), 1, 1);
+    KernelOrder ko(ctx, lv, 23 + (dvdx ? 9 : 0) + (vstar3 == v3 ? 0 : 3), 1, 1, record_bytes<HydroEnergyStage<true>>());
     HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
              ko.input(gradA, 3), ko.input(gradB, 9), nullptr, ko.output(dudt, 1), conservation,
              hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, ko.input(dvdx, 9)};
@@ -3660,7 +3676,7 @@ int crk_corrections_adjoint(crk_ctx *ctx, const crk_leaves *lv, const float *V, 
     if (n == 0) return CRK_OK;
     float *coef = (float *)crk_scratch(ctx, 33, sizeof(float) * kCorrCoef * (size_t)n);
     if (!coef) return crk_fail(ctx, CRK_ENOMEM, "adjoint scratch");
-    KernelOrder ko(ctx, lv, 17, 4, 4 + kCorrCoef);
+    KernelOrder ko(ctx, lv, 17, 4, 4 + kCorrCoef, record_bytes<CorrAdjPrepStage, CorrAdjStage>());
     CorrAdjP p{};
     p.V = ko.input(V, 1);
     p.n_singular = n_singular;
@@ -3687,7 +3703,7 @@ int crk_hydro_adjoint(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !dvbar3 || !dubar || !xbar3 ||
                       !vbar3 || !ubar || !mbar || !Vbar || !rhobar || !Abar || !Bbar3 || !gradAbar3 || !gradBbar9))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 27, 26, 26);
+    KernelOrder ko(ctx, lv, 27, 26, 26, record_bytes<HydroAdjStage<true>>());
     HydroAdjP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
                 ko.input(gradA, 3), ko.input(gradB, 9),
                 ko.input(dvbar3, 3), ko.input(dubar, 1), ko.output(xbar3, 3), ko.output(vbar3, 3), ko.output(ubar, 1),
