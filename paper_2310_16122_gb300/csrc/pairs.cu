@@ -3343,7 +3343,10 @@ struct Bundle {
     const float *src[kBundle];
     float *dst[kBundle];
     int k = 0;
+    bool over = false;  // more columns than the bundle holds were added
     void add(const float *s, float *d, int comps, int64_t n) {
+        over |= k + comps > kBundle;
+        if (over) return;
         for (int c = 0; c < comps; ++c, ++k) {
             src[k] = s + (size_t)c * n;
             dst[k] = d + (size_t)c * n;
@@ -3404,6 +3407,7 @@ int permute_rows(crk_ctx *ctx, int64_t n, const int32_t *perm, const Bundle &b) 
 
 // dst = src[perm] for every column of the bundle
 int permute_bundle(crk_ctx *ctx, int64_t n, const int32_t *perm, const Bundle &b) {
+    if (b.over) return crk_fail(ctx, CRK_EINVAL, "column permutation: more than %d columns", kBundle);
     if (b.k >= 3) return permute_rows<kBundle / 4>(ctx, n, perm, b);
     for (int c = 0; c < b.k; ++c) {
         permute_col_kernel<<<crk_grid(n, 256), 256, 0, ctx->stream>>>(n, perm, b.src[c], b.dst[c]);
@@ -3454,10 +3458,12 @@ struct KernelOrder {
     const crk_leaves *lv;
     bool on;
     float *next = nullptr;
+    int left;  // columns not yet taken
     Bundle in, out;
     // ni, no: columns the call reads and writes; scattered: columns that its kernels write in the
     // caller's order (its intermediate ones among them); record: bytes of its stage's largest record
-    KernelOrder(crk_ctx *c, const crk_leaves *l, int ni, int no, int scattered, size_t record) : ctx(c), lv(l) {
+    KernelOrder(crk_ctx *c, const crk_leaves *l, int ni, int no, int scattered, size_t record)
+        : ctx(c), lv(l), left(ni + no) {
         on = kernel_order_pays(lv->n, lv->n_gas, ni, no, scattered);
         if (!on) return;
         // never in a captured call: its columns may not exist yet (no allocation there), and a graph must not
@@ -3482,7 +3488,8 @@ struct KernelOrder {
     KernelOrder(const KernelOrder &) = delete;
     float *take(int comps) {
         float *r = next;
-        next += (size_t)comps * lv->n;
+        left -= comps;
+        if (left >= 0) next += (size_t)comps * lv->n;
         return r;
     }
     const float *input(const float *p, int comps) {
@@ -3497,7 +3504,11 @@ struct KernelOrder {
         out.add(r, p, comps, lv->n);
         return r;
     }
-    int begin() { return on ? permute_bundle(ctx, lv->n, lv->kperm, in) : CRK_OK; }
+    int begin() {
+        if (!on) return CRK_OK;
+        if (left < 0 || in.over || out.over) return crk_fail(ctx, CRK_EINVAL, "more columns than the call reserved");
+        return permute_bundle(ctx, lv->n, lv->kperm, in);
+    }
     int end(int rc) { return rc || !on ? rc : permute_bundle(ctx, lv->n, lv->kinv, out); }
 };
 
