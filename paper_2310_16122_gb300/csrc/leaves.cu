@@ -2320,10 +2320,15 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
                 int m = (int)shape->level_size[d];
                 int32_t *tab = shape->dtab + shape->level_off[d];
                 LevelDev dv{tab, tab + m, tab + 2 * m, tab + 3 * m, tab + 4 * m, tab + 5 * m, tab + 6 * m};
-                if (m > kTreeLevel || tl.n == kTreeLevels) {  // (levels shrink towards the root)
+                if (m > kTreeLevel) {  // (levels shrink towards the root)
                     node_hmax_kernel<<<crk_grid(m, 128), 128, 0, st>>>(m, dv, shape->left, shape->right, node_hmax);
                     ++ctx->launches;
                 } else {
+                    if (tl.n == kTreeLevels) {  // a full table runs before the levels that read its nodes
+                        tree_hmax_kernel<<<1, 1024, 0, st>>>(tl, shape->left, shape->right, node_hmax);
+                        ++ctx->launches;
+                        tl.n = 0;
+                    }
                     tl.k[tl.n] = dv.k;
                     tl.node[tl.n] = dv.node;
                     tl.m[tl.n++] = m;
