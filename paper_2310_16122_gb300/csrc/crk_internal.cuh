@@ -48,7 +48,7 @@ struct crk_ctx {
     int num_sms = 0;
     std::string err;
     // growable scratch arena: one buffer per slot
-    static const int kSlots = 38;  // leaf build 0-16 and 19-31, radix sort 12-14, scan 15, queue 17, step 18,
+    static const int kSlots = 38;  // leaf build 0-16, 19-21 and 31, radix sort 12-14, scan 15, queue 17, step 18,
                                    // integrator 32, corrections adjoint 33, adjoint chain 34, half-warp force 35,
                                    // tuner 36, single calls' kernel-order columns 37
     static const int kColumns = 37;  // the one slot no later call relies on: given back when memory runs short
@@ -200,9 +200,10 @@ int crk_exclusive_scan_i32(crk_ctx *ctx, const int32_t *in, int32_t *out, int64_
 // stable LSD radix sort of (key, value) pairs by all 32 key bits
 int crk_radix_sort_u32(crk_ctx *ctx, uint32_t *keys, int32_t *vals, int64_t n, int key_bits);
 // the stable (coordinate, index) order along each axis, in scratch memory (slots 1, 2, 13, 14), for
-// coordinates >= 0; with box_of ((device) box of each particle, nbox boxes) the (box, coordinate, index) order
+// coordinates >= 0; with box_of ((device) box of each particle, nbox boxes) the (box, coordinate, index) order.
+// spare: nine columns of n int32 in that scratch which the sort is done with
 int crk_sort_axes(crk_ctx *ctx, const float *x, const float *y, const float *z, int64_t n, const int32_t *box_of,
-                  int nbox, int32_t *order[3]);
+                  int nbox, int32_t *order[3], int32_t *spare[9]);
 // sort key of a coordinate: the IEEE bits of non-negative floats are ordered like the values
 __device__ __forceinline__ uint32_t crk_coord_key(float x) { return x == 0.0f ? 0u : __float_as_uint(x); }
 

@@ -2113,10 +2113,7 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             for (int a = 0; a < 3; ++a) {
                 Lc[a] = nullptr;
                 R[a] = (int32_t *)crk_scratch(ctx, 5 + a, nb);
-                for (int c = 0; c < 2; ++c) {
-                    Ac[a][c] = (int32_t *)crk_scratch(ctx, 19 + 2 * a + c, nb);
-                    An[a][c] = (int32_t *)crk_scratch(ctx, 25 + 2 * a + c, nb);
-                }
+                Ac[a][0] = (int32_t *)crk_scratch(ctx, 19 + a, nb);
             }
             int32_t *node_of = (int32_t *)crk_scratch(ctx, 8, nb);
             int32_t *node_nx = (int32_t *)crk_scratch(ctx, 9, nb);
@@ -2126,12 +2123,18 @@ static int build_leaves_impl(crk_ctx *ctx, const crk_particles *p, const float *
             for (size_t m : shape->level_size) max_seg = std::max(max_seg, m);
             SegRec *segs = (SegRec *)crk_scratch(ctx, 31, sizeof(SegRec) * max_seg);
             bool ok = node_of && node_nx && mem && flag && segs;
-            for (int a = 0; a < 3; ++a) ok = ok && R[a] && Ac[a][0] && Ac[a][1] && An[a][0] && An[a][1];
+            for (int a = 0; a < 3; ++a) ok = ok && R[a] && Ac[a][0];
             if (!ok) {
                 rc = crk_fail(ctx, CRK_ENOMEM, "scratch");
                 goto fail;
             }
-            TRY(crk_sort_axes(ctx, p->x, p->y, p->z, n, box_of, nbox, Lc));
+            int32_t *spare[9] = {};  // the other nine rank columns live where the sort's keys and values were
+            TRY(crk_sort_axes(ctx, p->x, p->y, p->z, n, box_of, nbox, Lc, spare));
+            for (int a = 0; a < 3; ++a) {
+                Ac[a][1] = spare[a];
+                An[a][0] = spare[3 + a];
+                An[a][1] = spare[6 + a];
+            }
             tr.mark("axis sorts");
             const AxisOrder ord{{Lc[0], Lc[1], Lc[2]}, {R[0], R[1], R[2]}};
             if (n > 0) {

@@ -352,14 +352,15 @@ int crk_radix_sort_u32(crk_ctx *ctx, uint32_t *keys, int32_t *vals, int64_t n, i
 // build and two host reads instead of four, leaf build + gravity on 30,011
 // particles went from 810 to 490 us, the whole step on 2x64^3 from 3490 to 3152 us.
 int crk_sort_axes(crk_ctx *ctx, const float *x, const float *y, const float *z, int64_t n, const int32_t *box_of,
-                  int nbox, int32_t *order[3]) {
+                  int nbox, int32_t *order[3], int32_t *spare[9]) {
     if (n <= 0) return CRK_OK;
     if (n > 2147483647LL) return crk_fail(ctx, CRK_EINVAL, "radix sort: n too large");
     const int64_t nb = (n + kSortTile - 1) / kSortTile;
-    uint32_t *k[2] = {(uint32_t *)crk_scratch(ctx, 1, sizeof(uint32_t) * 3 * (size_t)n),
-                      (uint32_t *)crk_scratch(ctx, 13, sizeof(uint32_t) * 3 * (size_t)n)};
-    int32_t *v[2] = {(int32_t *)crk_scratch(ctx, 2, sizeof(int32_t) * 3 * (size_t)n),
-                     (int32_t *)crk_scratch(ctx, 14, sizeof(int32_t) * 3 * (size_t)n)};
+    const int64_t pitch = (n + 63) & ~(int64_t)63;  // of the spare columns: each starts on a 256-byte boundary
+    uint32_t *k[2] = {(uint32_t *)crk_scratch(ctx, 1, sizeof(uint32_t) * 3 * (size_t)pitch),
+                      (uint32_t *)crk_scratch(ctx, 13, sizeof(uint32_t) * 3 * (size_t)pitch)};
+    int32_t *v[2] = {(int32_t *)crk_scratch(ctx, 2, sizeof(int32_t) * 3 * (size_t)pitch),
+                     (int32_t *)crk_scratch(ctx, 14, sizeof(int32_t) * 3 * (size_t)pitch)};
     int32_t *counts = (int32_t *)crk_scratch(ctx, 12, sizeof(int32_t) * 3 * (size_t)(nb * kRadix));
     if (!k[0] || !k[1] || !v[0] || !v[1] || !counts) return crk_fail(ctx, CRK_ENOMEM, "radix sort scratch");
     int at = 0, rc;
@@ -380,6 +381,11 @@ int crk_sort_axes(crk_ctx *ctx, const float *x, const float *y, const float *z, 
         in.shift = shift;
         if ((rc = radix_pass<kRadixBoxes, false>(ctx, in, 3, nullptr, v[at ^ 1], counts, nb))) return rc;
     }
-    for (int a = 0; a < 3; ++a) order[a] = v[at] + a * n;
+    for (int a = 0; a < 3; ++a) {
+        order[a] = v[at] + a * n;
+        spare[a] = (int32_t *)k[0] + a * pitch;
+        spare[3 + a] = (int32_t *)k[1] + a * pitch;
+        spare[6 + a] = v[at ^ 1] + a * pitch;
+    }
     return CRK_OK;
 }
