@@ -1245,7 +1245,7 @@ struct HydroRecVstar : Base {
 //                 (1/2 when u_i = u_j), so that sum_i m_i du_i = -sum_i f_i.v*_i.
 constexpr int kHydroBoth = 0, kHydroAccel = 1, kHydroEnergy = 2;
 
-template <bool kLim, int kPass = kHydroBoth>
+template <bool kLim, int kPass = kHydroBoth, bool kWholeRec = kPass != kHydroEnergy>
 struct HydroStageT {
     static constexpr bool kPair = false;
     static constexpr bool kGasOnly = true;
@@ -1254,7 +1254,7 @@ struct HydroStageT {
     using P = HydroP;
     using Base = std::conditional_t<kLim, HydroRecLim, HydroRec>;
     struct __align__(16) Rec : std::conditional_t<kPass == kHydroEnergy, HydroRecVstar<Base>, Base> {
-        static constexpr bool kWhole = kPass != kHydroEnergy;
+        static constexpr bool kWhole = kWholeRec;
     };
     struct I {
         float fx, fy, fz, e;
@@ -1645,8 +1645,8 @@ struct HydroAdjStage {
 
 template <bool kLim>
 using HydroAccelStage = HydroStageT<kLim, kHydroAccel>;
-template <bool kLim>
-using HydroEnergyStage = HydroStageT<kLim, kHydroEnergy>;
+template <bool kLim, bool kWholeRec = false>
+using HydroEnergyStage = HydroStageT<kLim, kHydroEnergy, kWholeRec>;
 
 // Extras (Sec. 5: the density and state gradients), over gas j including j = i:
 //   rhoR_i = sum_j m_j W^R_ij,   dv_i[3a+b] = sum_j V_j (v_j^a - v_i^a) (grad_i W^R_ij)^b
@@ -3417,14 +3417,21 @@ int permute_bundle(crk_ctx *ctx, int64_t n, const int32_t *perm, const Bundle &b
     return CRK_OK;
 }
 
-// The hydro adjoint's records: planes, and whole records where gas is below an eighth of the particles (few
-// lanes of a group are active, and each reads a record of its own).  The call, whole -> planes, us: 687 -> 552
-// on the 2x64^3 box; uniform boxes of 500,009 particles, a fifth of them gas, 391 -> 339, of 300,007, a
-// twentieth, 229 -> 243, of 880,001, a fiftieth, 501 -> 532.
+// The records of the Energy pass and the hydro adjoint: planes, and whole records where gas is below a sixteenth
+// (hydro adjoint: an eighth) of the particles: few lanes of a group are active, and each reads a record of its
+// own.  The hydro adjoint, whole -> planes, us: 687 -> 552 on the 2x64^3 box; uniform boxes of 500,009 particles,
+// a fifth of them gas, 391 -> 339, of 300,007, a twentieth, 229 -> 243, of 880,001, a fiftieth, 501 -> 532.
+// Energy: 563 -> 355; 500,009 particles, a tenth gas, 175 -> 157, of 650,001, a fiftieth, 201 -> 207.
+bool sparse_gas(const crk_leaves *lv, int part) { return lv->n_gas < lv->n / part; }
 int run_hydro_adjoint(crk_ctx *ctx, const crk_leaves *lv, const HydroAdjP &p, bool korder) {
-    if (lv->n_gas < lv->n / 8)
-        return run_stage<HydroAdjStage<true>>(ctx, lv, p, true, CRK_K_HYDRO, nullptr, korder);
+    if (sparse_gas(lv, 8)) return run_stage<HydroAdjStage<true>>(ctx, lv, p, true, CRK_K_HYDRO, nullptr, korder);
     return run_stage<HydroAdjStage<false>>(ctx, lv, p, true, CRK_K_HYDRO, nullptr, korder);
+}
+template <bool kLim>
+int run_energy(crk_ctx *ctx, const crk_leaves *lv, const HydroP &p, double *conservation, bool korder) {
+    if (sparse_gas(lv, 16))
+        return run_stage<HydroEnergyStage<kLim, true>>(ctx, lv, p, true, CRK_K_ENERGY, conservation, korder);
+    return run_stage<HydroEnergyStage<kLim>>(ctx, lv, p, true, CRK_K_ENERGY, conservation, korder);
 }
 
 // Single calls of the gas stages on large boxes: the caller's columns are
@@ -3664,15 +3671,15 @@ int crk_hydro_energy(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params 
     if (!lv || !hp) return crk_fail(ctx, CRK_EINVAL, "null argument");
     if (lv->n > 0 && (!m || !v3 || !u || !V || !rho || !A || !B || !gradA || !gradB || !vstar3 || !dudt))
         return crk_fail(ctx, CRK_EINVAL, "null array");
-    KernelOrder ko(ctx, lv, 23 + (dvdx ? 9 : 0) + (vstar3 == v3 ? 0 : 3), 1, 1, record_bytes<HydroEnergyStage<true>>());
+    KernelOrder ko(ctx, lv, 23 + (dvdx ? 9 : 0) + (vstar3 == v3 ? 0 : 3), 1, 1, record_bytes<HydroEnergyStage<true, true>>());
     HydroP p{ko.input(m, 1), ko.input(v3, 3), ko.input(u, 1), ko.input(V, 1), ko.input(rho, 1), ko.input(A, 1), ko.input(B, 3),
              ko.input(gradA, 3), ko.input(gradB, 9), nullptr, ko.output(dudt, 1), conservation,
              hp->gamma, hp->alpha, hp->beta, hp->eta2, lv->n, (unsigned long long *)pair_count, ko.input(dvdx, 9)};
     p.vstar = vstar3 == v3 ? p.v3 : ko.input(vstar3, 3);
     const int rc = ko.begin();
     if (rc) return rc;
-    if (dvdx) return ko.end(run_stage<HydroEnergyStage<true>>(ctx, lv, p, true, CRK_K_ENERGY, conservation, ko.on));
-    return ko.end(run_stage<HydroEnergyStage<false>>(ctx, lv, p, true, CRK_K_ENERGY, conservation, ko.on));
+    if (dvdx) return ko.end(run_energy<true>(ctx, lv, p, conservation, ko.on));
+    return ko.end(run_energy<false>(ctx, lv, p, conservation, ko.on));
 }
 
 int crk_corrections_adjoint(crk_ctx *ctx, const crk_leaves *lv, const float *V, const float *Abar,
@@ -4060,8 +4067,8 @@ int crk_stage_energy(crk_ctx *ctx, const crk_leaves *lv, const crk_hydro_params 
              C(K::gB), nullptr, C(K::du), conservation, hp->gamma, hp->alpha, hp->beta, hp->eta2, n, nullptr,
              limited ? C(K::dvdx) : nullptr};
     p.vstar = vs;
-    if (limited) return run_stage<HydroEnergyStage<true>>(ctx, lv, p, true, CRK_K_ENERGY, conservation, true);
-    return run_stage<HydroEnergyStage<false>>(ctx, lv, p, true, CRK_K_ENERGY, conservation, true);
+    if (limited) return run_energy<true>(ctx, lv, p, conservation, true);
+    return run_energy<false>(ctx, lv, p, conservation, true);
 }
 
 namespace {
