@@ -755,7 +755,6 @@ struct CorrStage {
     // (2x64^3: 164 us, now 127; 2x128^3 in the kernel order 1.15 ms, now 0.91; the reverse's
     // preparation 295 us, now 260).  Only a particle that is close to singular (det m2 < 1e-6 tr^3,
     // where 47 bits could show) or out of range goes through FP64.
-    // kWithM0: s2 holds s2 + m0 1, so that q without m0 stands beside it (both are zero inside a lattice).
     template <class T>
     struct Solved {
         using F = typename beside<T>::type;
@@ -781,7 +780,7 @@ struct CorrStage {
         return det.h > 1e-6f * tr.h * tr.h * tr.h && m0 > 1e-12f && m0 < 1e12f;
     }
     // false for a singular particle (FP64) or one that needs FP64 (Two)
-    template <bool kWithM0, class T, class Sums>
+    template <class T, class Sums>
     __device__ static bool solve(const Sums &s, Solved<T> &r) {
         using F = typename beside<T>::type;
         scale_of(s.m2[0] + s.m2[3] + s.m2[5], r.f1, r.g1);
@@ -807,9 +806,8 @@ struct CorrStage {
         for (int a = 0; a < 3; ++a) r.B[a] = -row(r.Mi, a, r.m1);
         T m0;
         difference((F)s.m0, (F)s.c0, m0);
-        const T bm = dot3(r.B[0], r.m1[0], r.B[1], r.m1[1], r.B[2], r.m1[2]), q = m0 + bm;
-        r.A = inverse(q);
-        r.q = kWithM0 ? bm : q;  // what is missing beside s2
+        r.q = m0 + dot3(r.B[0], r.m1[0], r.B[1], r.m1[1], r.B[2], r.m1[2]);
+        r.A = inverse(r.q);
         T W[6];
 #pragma unroll
         for (int k = 0; k < 10; ++k) r.s3[k] = (F)s.s3[k] * f1;
@@ -846,8 +844,7 @@ struct CorrStage {
         for (int a = 0; a < 10; ++a) s.s3[a] = 0.f;
         s.cnt = 0;
     }
-    // kWithM0: the diagonal of s2 is summed with m0, pair by pair (near cancelling terms)
-    template <bool kCount, bool kWithM0 = false>
+    template <bool kCount>
     __device__ static void interact(const P &, I &s, const Rec &ri, const Rec &rj) {
         float x[3] = {ri.x - rj.x, ri.y - rj.y, ri.z - rj.z};  // x_ij
         float r2 = fmaf(x[0], x[0], fmaf(x[1], x[1], x[2] * x[2]));
@@ -868,7 +865,7 @@ struct CorrStage {
         for (int q = 0; q < 6; ++q) {
             xx[q] = x[ia[q]] * x[ib[q]];
             kahan_add(s.m2[q], s.c2[q], wx[ia[q]] * x[ib[q]]);
-            s.s2[q] = fmaf(xx[q], vd, kWithM0 && ia[q] == ib[q] ? s.s2[q] + w : s.s2[q]);
+            s.s2[q] = fmaf(xx[q], vd, s.s2[q]);
         }
 #pragma unroll
         for (int g = 0; g < 3; ++g) s.dm0[g] += dW[g];
@@ -884,7 +881,7 @@ struct CorrStage {
         using F = typename beside<T>::type;
         const int64_t n = p.n;
         Solved<T> r;
-        if (!solve<false>(s, r)) return false;
+        if (!solve(s, r)) return false;
         float sum = 0.0f;  // NaN once a result is not finite
         auto put = [&](float *out, float v) {
             *out = v;
@@ -946,10 +943,6 @@ struct CorrAdjPrepStage : CorrStage {
     // this finish (2,500 FP32 instructions in float pairs) is the other half of the kernel's time: 422 ->
     // 295 us on the 2x64^3 box against the reverse taken through the 30 unreduced sums dm1, dm2, 260 us
     // in float pairs.
-    template <bool kCount>
-    __device__ static void interact(const P &p, I &s, const Rec &ri, const Rec &rj) {
-        CorrStage::interact<kCount, true>(p, s, ri, rj);
-    }
     // The reverse is linear in the cotangents, and a float pair holds its 47 bits only while its low word is a
     // normal number: it works on them (in scaled lengths) in units u of a power of two near the largest, c = 1/u.
     // False where the unit or the lengths are so far from 1 that products of the scales leave the FP32 range.
@@ -977,7 +970,7 @@ struct CorrAdjPrepStage : CorrStage {
         using F = typename beside<T>::type;
         const int64_t n = p.n;
         Solved<T> r;
-        if (!solve<true>(s, r)) return false;
+        if (!solve(s, r)) return false;
         const F f1 = r.f1;
         float cot[16];  // A, B, dA, dB (3g+a)
         cot[0] = p.Abar[o];
