@@ -22,7 +22,8 @@
  *  - Gas-only quantities (h, V, rho, u, A, B, ...) also have length n; their
  *    dark-matter entries are ignored on input and written as 0 on output.
  *  - Every compute call is asynchronous on the context's stream and does not
- *    synchronise.  crk_build_leaves synchronises once (it reads back sizes).
+ *    synchronise.  crk_build_leaves does (it reads back sizes: twice, and more
+ *    often where a capacity has to grow).
  *  - Every call returns CRK_OK (0) or a negative status; crk_last_error()
  *    gives a message.  Device-side results that the host cannot see without a
  *    synchronisation (singular moment matrices, pair counts) are written to
@@ -173,7 +174,7 @@ int crk_launch_count(const crk_ctx *ctx, int64_t *out);
  * the periodic shifts {-box, 0, box} of the distance between their tight
  * FP32 boxes, summed in squares in FP64.  Errors: CRK_EBOX if r_cut_grav or
  * 2 max h is not below box/2 or a position lies outside [0, box).
- * Synchronises the context stream once. */
+ * Synchronises the context stream. */
 int crk_build_leaves(crk_ctx *ctx, const crk_particles *p, const float *h, const crk_leaf_params *lp,
                      crk_leaves **out);
 
@@ -216,8 +217,9 @@ void crk_leaves_free(crk_ctx *ctx, crk_leaves *lv);
  * (same count, species, boxes and leaf parameters as the build that made lv),
  * with no host synchronisation and no allocation, so the call can be captured
  * in a CUDA graph together with the kernels that use the leaves.  Every
- * buffer keeps the size the first build gave it (the leaf-pair image lists
- * their first capacities, the gas neighbour lists 1/8 more groups than the
+ * buffer keeps the size the first build gave it (the leaf-pair lists at least
+ * 48 images and 32 pairs a leaf, or the first build's counts and 1/8 more
+ * where those did not fit; the gas neighbour lists 1/8 more groups than the
  * first build held).  What a build checks on the host becomes a bit of the
  * leaves' device status word instead: positions outside the box, gas h <= 0,
  * 2 h_max >= box/2, a changed gas count, a capacity overflow.  After a
@@ -258,7 +260,11 @@ int crk_geometry(crk_ctx *ctx, const crk_leaves *lv, const float *m, float *V, f
  * w = V_j W_ij and x = x_ij the moments m0, m1, m2 and their gradients in the
  * evaluation point give B = -m2^-1 m1, A = 1/(m0 + B.m1),
  * dA = -A^2 (dm0 + 2 B.dm1 + B^T dm2 B), dB = -m2^-1 (dm1 + dm2 B).
- * Moment sums in FP32 (compensated for m0, m1, m2); the 3x3 inverse in FP64.
+ * Moment sums in FP32 (compensated for m0, m1, m2).  The per-particle 3x3
+ * solve runs in pairs of floats (about 47 bits, lengths in units of a power of
+ * two); a particle with det(m2) <= 1e-6 tr(m2)^3, m0 outside (1e-12, 1e12) or a
+ * result that is not finite is solved in FP64, where the test for singular
+ * particles below is made.
  * Outputs A[n], B[3n], gradA[3n], gradB[9n] with gradB[(3g+a)n + i] =
  * d B^a / d x^g.  A particle with det(m2) <= 1e-12 tr(m2)^3 gets NaN outputs
  * and is counted in n_singular (device int32, may be NULL). */
@@ -407,8 +413,10 @@ int crk_geometry_adjoint(crk_ctx *ctx, const crk_leaves *lv, const float *m, con
  *   L = sum_i Abar_i A_i + Bbar_i.B_i + gradAbar_i.gradA_i + gradBbar_i:gradB_i
  * in the positions, xbar3[3n], and in the volumes, Vbar[n] (h held fixed; the
  * leaves are constant).  Pair (i, j) enters i's moments as V_j t(x_ij); each
- * particle's moment cotangents come from the closed-form reverse of its FP64
- * 3x3 step (a first sweep recomputes the moments), then
+ * particle's moment cotangents come from the closed-form reverse of its 3x3
+ * step (a first sweep recomputes the moments; precision as in crk_corrections,
+ * cotangents in units of a power of two, and FP64 also where they or the
+ * lengths are so far from 1 that those units leave the FP32 range), then
  *   xbar_i = sum_j V_j grad T_i(x_ij) - V_i grad T_j(x_ji),  Vbar_i = sum_j T_j(x_ji)
  * with T_i the moment terms weighted by i's cotangents (a second sweep; nothing
  * per pair is stored).  A singular particle contributes nothing and is

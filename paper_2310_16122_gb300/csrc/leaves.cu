@@ -950,16 +950,18 @@ __device__ int16_t *bisect32(Bisect32<kCap> &bs, int m, const float4 *pm, const 
 
 // One block per leaf: tight box, gas count, largest gas h; the canonical
 // order (gas first, then dark matter, each by index) for export; the gas
-// kernel order (gas first, then dark matter along a Z-order curve of the leaf
-// box, ties by index; the gas part bisected into groups of 32 as below); the
-// gravity kernel order (species mixed): the leaf bisected into groups of 32,
+// kernel order (gas first, then dark matter, each along a Z-order curve of the
+// leaf box, ties by index; the gas part bisected into groups of 32 as below; RCB
+// leaves of at most 128 have the kernel below, which takes both in canonical
+// order instead, so that a part of at most 32 gas particles stays in index
+// order); the gravity kernel order (species mixed): the leaf bisected into groups of 32,
 // each split along the longest extent of its part in (coordinate, index)
 // order with a multiple of 32 particles on the left, so that every group of 32
 // consecutive particles is an RCB cell (the gravity tiles sweep the
 // candidates within r_c of a group's box: at r_c = 3 such cells cut the
 // candidates per in-range pair from ~4.0 to ~3.3 against Z-order groups); and
 // the leaf-relative positions in both kernel orders.
-// kCap: the largest leaf the launch may meet (RCB leaves of at most 128 have a kernel of their own below).
+// kCap: the largest leaf the launch may meet.
 template <int kCap>
 __global__ void leaf_data_kernel(int64_t n_leaves, const int32_t *__restrict__ leaf_start,
                                  const int32_t *__restrict__ members, const float *__restrict__ x,

@@ -237,11 +237,10 @@ struct beside<Two> {
     using type = float;
 };
 
-// 1/sqrt(x), 1/x and a/x by the hardware approximations for arguments that are normal numbers:
-// rsqrtf and __fdividef wrap the same approximation in a scaling for subnormal x, four
-// instructions per pair that no argument here needs.  Gravity's x = r^2 + eps^2 may be subnormal
-// (eps = 0, r < 1e-19): x^-3/2 then overflows to infinity either way.  The same bits;
-// on the 2x128^3 box gravity 3644 -> 3272 us, its adjoint 6324 -> 6006 us.
+// 1/sqrt(x), 1/x and a/x by PTX's .approx.ftz instructions, which read a subnormal operand as zero; the
+// arguments here are normal numbers.  Gravity's x = r^2 + eps^2 may be subnormal (eps = 0, r < 1e-19):
+// x^-3/2 then overflows to infinity either way.  Against rsqrtf and __fdividef, gravity on the 2x128^3 box
+// 3644 -> 3272 us, its adjoint 6324 -> 6006 us.
 __device__ __forceinline__ float rsqrt_normal(float x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -752,8 +751,8 @@ struct CorrStage {
     // Matrices are packed xx xy xz yy yz zz; Uq is U with q added on its diagonal.
     // T = Two: lengths in units of a power of two near sqrt(tr m2), which keeps the FP32 exponents
     // in range.  FP64 runs at 1/64 of the FP32 rate here: with it the solve took a third of the kernel
-    // (2x64^3: 164 us, now 127; 2x128^3 in the kernel order 1.15 ms, now 0.91; the reverse's
-    // preparation 295 us, now 260).  Only a particle that is close to singular (det m2 < 1e-6 tr^3,
+    // (2x64^3: 164 us, now 127; 2x128^3 in the kernel order 1.15 ms, now 0.90; the reverse's
+    // preparation 295 us, now 254).  Only a particle that is close to singular (det m2 < 1e-6 tr^3,
     // where 47 bits could show) or out of range goes through FP64.
     template <class T>
     struct Solved {
@@ -939,10 +938,11 @@ struct CorrAdjPrepStage : CorrStage {
     static constexpr bool kAllVariants = false;
     using P = CorrAdjP;
     // Reverse of CorrStage's Solved, in the sums m0, m1, m2, dm0, s2, s3 themselves, whose cotangents
-    // are the polynomial coefficients.  H_ga: the cotangent of dB_g^a (row g).  The sweep is CorrStage's;
-    // this finish (2,500 FP32 instructions in float pairs) is the other half of the kernel's time: 422 ->
-    // 295 us on the 2x64^3 box against the reverse taken through the 30 unreduced sums dm1, dm2, 260 us
-    // in float pairs.
+    // are the polynomial coefficients.  H_ga: the cotangent of dB_g^a (row g).  The sweep is CorrStage's, with
+    // the very sums of the forward pass: through the chain the gradients in the positions are 4% nearer to 64
+    // bits than through the 30 unreduced sums dm1, dm2 (by themselves, for cotangents of dA, 1-2% farther off).
+    // This finish (2,500 FP32 instructions in float pairs) is half of the kernel's time: 422 -> 295 us on
+    // the 2x64^3 box against the unreduced sums, then 254 us in float pairs.
     // The reverse is linear in the cotangents, and a float pair holds its 47 bits only while its low word is a
     // normal number: it works on them (in scaled lengths) in units u of a power of two near the largest, c = 1/u.
     // False where the unit or the lengths are so far from 1 that products of the scales leave the FP32 range.
@@ -1863,8 +1863,9 @@ __device__ __forceinline__ void tile_group(const LeafView &lv, const typename S:
 }
 
 // Cell sweeps (the TILES and SPLIT8 variants of the gravity kernels).  A warp
-// takes G consecutive particles of a leaf (G = 16 or 8: an RCB cell of the
-// gravity kernel order) and all candidates within r_c of their box:
+// takes G consecutive particles of a leaf (G = 16 or 8; in RCB leaves of at most
+// 128 an RCB cell of the gravity kernel order, in larger leaves and mesh cells a
+// part of a cell of 32) and all candidates within r_c of their box:
 //   1. The j side is walked in cells of 32 (the groups of the kernel order).
 //      Their boxes are tested 32 at a time, one per lane, before any particle
 //      is loaded; the particles of a cell near enough are tested one per lane,
@@ -1875,12 +1876,13 @@ __device__ __forceinline__ void tile_group(const LeafView &lv, const typename S:
 //      works.  The sums of the 32/G streams are added by shuffles at the end
 //      (fixed order, no atomics: deterministic).
 // The FP32 pipe bounds it (56% busy; DRAM below 1%), on swept pairs: of those
-// 0.43 are in range with G = 16 on the clustered boxes, 0.34 with G = 32 and
-// 0.54 with G = 8, whose candidate tests cost more than the pairs they save.
-// 2x128^3 box, gravity / adjoint: 2.92 / 5.49 ms (G = 32: 2.97 / 5.92, G = 8:
-// 3.56 / 6.33), against 3.27 / 6.01 for a warp per group of 32 that walked the
-// leaf images one by one.  Slower: several units per warp sharing the candidate loads (3.3 / 5.7 ms and more), two i per
-// lane against one j (the j then needs register moves: 3.3 / 5.7 ms).
+// 0.43 are in range with G = 16 on the clustered boxes and 0.54 with G = 8, whose
+// candidate tests cost more than the pairs they save.  2x128^3 box, gravity /
+// adjoint: 2.92 / 5.49 ms (G = 8: 3.56 / 6.33), against 3.27 / 6.01 for a warp
+// per group of 32 that walked the leaf images one by one.  The same holds where
+// units are not RCB cells (2x48^3, that form -> G = 16, us: leaves of 256 340 /
+// 541 -> 217 / 379, of 1024 844 / 1032 -> 231 / 389; mesh cells of 128 on the
+// lattice box of 2x64^3 551 / 920 -> 454 / 852).
 template <class S, bool kCount, int G, int kW>
 __global__ void __launch_bounds__(32 * kW) cell_kernel(LeafView lv, typename S::P p, RecView<typename S::Rec> rec,
                                                        int units, int log_cpl, int full) {
@@ -2422,7 +2424,7 @@ void launch_list_build(crk_ctx *ctx, const crk_leaves *lv, const LeafView &v, co
 }
 
 // Tiles with sub-warp i-groups: the warp's 32 i-particles form 32/G groups of
-// G consecutive (Z-ordered) particles, each with its own box and its own
+// G consecutive particles of the kernel order, each with its own box and its own
 // compacted candidate buffer; lane l sweeps the buffer of group l/G.  Smaller
 // groups have smaller boxes, so a larger share of the swept pairs is in range.
 // Within one 8-lane phase of a shared-memory load every lane reads the same
@@ -2890,7 +2892,7 @@ __host__ __device__ constexpr int table_cap() {
 
 // resident blocks per SM that list_kernel<S> is compiled for (a register cap; 0: none).
 // Corrections is latency bound: capped for five blocks (96 registers, a few bytes spilled) it runs
-// 0.91 ms on the 2x128^3 box, against 0.95 ms at four and 1.07 ms at six.
+// 0.90 ms on the 2x128^3 box, against 0.95 ms at four and 1.07 ms at six.
 template <class S>
 struct list_min_blocks {
     static constexpr int value = 0;  // no register cap
@@ -2899,7 +2901,7 @@ template <>
 struct list_min_blocks<CorrStage> {
     static constexpr int value = 5;
 };
-// its reverse preparation: four blocks 259 us on the 2x64^3 box, three 262, five 327
+// its reverse preparation: four blocks 254 us on the 2x64^3 box, three 267, five 271
 template <>
 struct list_min_blocks<CorrAdjPrepStage> {
     static constexpr int value = 4;
