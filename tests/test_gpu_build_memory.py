@@ -2,8 +2,8 @@
 
 Per particle and with 1/8 headroom: 12 ints of sort buffers, 3 more rank columns, 3 ranks, 3 of node numbers
 and members, 1.4 of counts and sums (20.4 x 4.5 = 92 bytes); leaves of 20 bytes of orders, 32 of positions and 4 of
-cell boxes; and per leaf of 122 particles 2.7 KB of image and pair lists (22): 170 bytes.  Twelve further rank
-columns in scratch of their own (9 ints, 40 bytes) would exceed the limit of 200.
+cell boxes; and per leaf of 122 particles 2.7 KB of image and pair lists (22): 170 bytes.  The nine other rank
+columns in scratch of their own (40 bytes) would exceed the limit of 200.
 """
 import gc
 
